@@ -59,4 +59,40 @@ __host__ __device__ __forceinline__ bool axis_attends(int delta, int width, int 
   return x <= width - 1;
 }
 
+// Walks one axis' differences -(n - 1) .. n - 1 in order with the distance's remainder carried along (one division
+// per axis instead of one per difference: the host evaluates some 70 differences per head, at 6 ns a division) and
+// calls f(index, difference) for every attended one.
+template <class F>
+inline void for_attended(int n, int width, int offset, int stride, F f) {
+  int d = -(n - 1);
+  long long x = (long long)d - offset;            // key minus query minus offset
+  const long long dist = x < 0 ? -x : x;
+  long long r = stride ? dist % stride : dist;    // remainder of the distance
+  for (int i = 0; i < 2 * n - 1; ++i, ++d, ++x) {
+    if (r <= width - 1) f(i, d);
+    if (x < 0) {                                  // the distance falls by one
+      if (stride && r == 0) r = stride;
+      --r;
+    } else {
+      ++r;
+      if (stride && r == stride) r = 0;
+    }
+  }
+}
+
+// One axis' attended differences as a bit set, bit d + n - 1 for difference d, with the number of attended
+// coordinate pairs (n <= 64).
+struct AxisSet {
+  unsigned long long lo, hi;
+  int pairs;
+};
+inline AxisSet axis_set(int n, int width, int offset, int stride) {
+  AxisSet s = {0, 0, 0};
+  for_attended(n, width, offset, stride, [&](int i, int d) {
+    (i < 64 ? s.lo : s.hi) |= 1ull << (i & 63);
+    s.pairs += n - (d < 0 ? -d : d);
+  });
+  return s;
+}
+
 }  // namespace psa

@@ -13,7 +13,8 @@
 #include "psa_common.cuh"
 
 namespace psa {
-cudaError_t launch_mask_build(const HeadParamsArray& hp, const int* head_bases, const Geom& g, int n_heads_here,
+bool mask_build_small(const Geom& g);
+cudaError_t launch_mask_build(const HeadParamsArray& hp, const AxisSet* sets, const int* head_bases, const Geom& g, int n_heads_here,
                               uint8_t* block_mask, int* row_ptr, int* col_idx, int total_nnz_through_chunk,
                               int n_sms, cudaStream_t stream, int* launches);
 cudaError_t launch_plan(const HeadParamsArray& hp, const Geom& g, int head0, int n_heads_here, bool clear_status,
@@ -154,10 +155,8 @@ int set_text(Geom* g, long long n_text) {
 // Attended block pairs of one head: product of the two axis pair counts.
 long long head_nnz(const psa_head_params& p, const Geom& g) {
   long long ct = 0, cs = 0;
-  for (int d = -(g.Tp - 1); d <= g.Tp - 1; ++d)
-    if (axis_attends(d, p.Tw, p.To, p.Ts)) ct += g.Tp - (d < 0 ? -d : d);
-  for (int d = -(g.Sp - 1); d <= g.Sp - 1; ++d)
-    if (axis_attends(d, p.Sw, p.So, p.Ss)) cs += g.Sp - (d < 0 ? -d : d);
+  for_attended(g.Tp, p.Tw, p.To, p.Ts, [&](int, int d) { ct += g.Tp - (d < 0 ? -d : d); });
+  for_attended(g.Sp, p.Sw, p.So, p.Ss, [&](int, int d) { cs += g.Sp - (d < 0 ? -d : d); });
   return ct * cs;
 }
 
@@ -237,6 +236,10 @@ int encode_maps(TensorMaps* tm, const void* q, const void* k, const void* v, voi
   int rc;
   const int n_in = lay.shared_qkv ? 1 : n_heads_here;
   for (int last = 0; last < 2; ++last) {
+    if (last && g.n_last == kSlabTokens) {   // a block's last slab is a full one
+      tm->q[1] = tm->q[0]; tm->k[1] = tm->k[0]; tm->v[1] = tm->v[0]; tm->o[1] = tm->o[0];
+      break;
+    }
     if ((rc = encode_map(&tm->q[last], q, g, lay.in_head, lay.in_token, n_in, last != 0)) != PSA_OK) return rc;
     if ((rc = encode_map(&tm->k[last], k, g, lay.in_head, lay.in_token, n_in, last != 0)) != PSA_OK) return rc;
     if ((rc = encode_map(&tm->v[last], v, g, lay.in_head, lay.in_token, n_in, last != 0)) != PSA_OK) return rc;
@@ -358,11 +361,21 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T
   if (block_mask && !aligned16(block_mask)) return PSA_ERR_INVALID_ARG;
   if ((row_ptr && (reinterpret_cast<uintptr_t>(row_ptr) & 3u)) || (col_idx && (reinterpret_cast<uintptr_t>(col_idx) & 3u)))
     return PSA_ERR_INVALID_ARG;
-  // exclusive prefix of the per-head pair counts (host arithmetic, a few thousand operations)
+  // exclusive prefix of the per-head pair counts, and each head's axis sets where the kernel takes them (one walk over
+  // the differences gives both)
+  const bool small = mask_build_small(g);
   std::vector<long long> base(prob->n_heads + 1, 0);
+  std::vector<AxisSet> sets(small ? 2 * (size_t)prob->n_heads : 0);
   for (int h = 0; h < prob->n_heads; ++h) {
-    if (!valid_params(params[h])) return PSA_ERR_INVALID_ARG;
-    base[h + 1] = base[h] + head_nnz(params[h], g);
+    const psa_head_params& p = params[h];
+    if (!valid_params(p)) return PSA_ERR_INVALID_ARG;
+    if (small) {
+      sets[2 * h] = axis_set(g.Tp, p.Tw, p.To, p.Ts);
+      sets[2 * h + 1] = axis_set(g.Sp, p.Sw, p.So, p.Ss);
+      base[h + 1] = base[h] + (long long)sets[2 * h].pairs * sets[2 * h + 1].pairs;
+    } else {
+      base[h + 1] = base[h] + head_nnz(p, g);
+    }
   }
   const long long nnz = base[prob->n_heads];
   if (nnz >= (1ll << 31) || (long long)prob->n_heads * g.NB >= (1ll << 31) - 1) return PSA_ERR_UNSUPPORTED;
@@ -381,7 +394,7 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T
       bases[h] = (int)base[head0 + h];
     }
     int launches = 0;
-    const cudaError_t e = launch_mask_build(hp, bases, g, n_here, block_mask ? block_mask + (long long)head0 * g.NB * g.NB : nullptr,
+    const cudaError_t e = launch_mask_build(hp, small ? &sets[2 * (size_t)head0] : nullptr, bases, g, n_here, block_mask ? block_mask + (long long)head0 * g.NB * g.NB : nullptr,
                                             row_ptr ? row_ptr + (long long)head0 * g.NB : nullptr, col_idx,
                                             (int)base[head0 + n_here], ws->n_sms, static_cast<cudaStream_t>(stream), &launches);
     g_launches += launches;

@@ -339,26 +339,19 @@ mask_build_small_kernel(const HeadSets hs, const Geom g, int n_heads_here, unsig
   }
 }
 
-cudaError_t launch_mask_build(const HeadParamsArray& hp, const int* head_bases, const Geom& g, int n_heads_here,
+bool mask_build_small(const Geom& g) { return g.Tp <= 64 && g.Sp <= 32; }
+
+// sets: the two axis sets of every head (temporal, spatial), when mask_build_small(g).
+cudaError_t launch_mask_build(const HeadParamsArray& hp, const AxisSet* sets, const int* head_bases, const Geom& g, int n_heads_here,
                               uint8_t* block_mask, int* row_ptr, int* col_idx, int total_nnz_through_chunk,
                               int n_sms, cudaStream_t stream, int* launches) {
-  HeadBases hb;
-  for (int h = 0; h < kMaxHeads; ++h) hb.base[h] = h < n_heads_here ? head_bases[h] : 0;
-  if (g.Tp <= 64 && g.Sp <= 32) {
-    HeadSets hs;
-    for (int h = 0; h < kMaxHeads; ++h) {
-      unsigned long long st = 0, st_hi = 0, ss = 0;
-      if (h < n_heads_here) {
-        const psa_head_params& p = hp.p[h];
-        for (int i = 0; i < 2 * g.Tp - 1; ++i)
-          if (axis_attends(i - (g.Tp - 1), p.Tw, p.To, p.Ts)) (i < 64 ? st : st_hi) |= 1ull << (i & 63);
-        for (int i = 0; i < 2 * g.Sp - 1; ++i)
-          if (axis_attends(i - (g.Sp - 1), p.Sw, p.So, p.Ss)) ss |= 1ull << i;
-      }
-      hs.setT[h] = st;
-      hs.setT_hi[h] = st_hi;
-      hs.setS[h] = ss;
-      hs.base[h] = h < n_heads_here ? head_bases[h] : 0;
+  if (mask_build_small(g)) {
+    HeadSets hs;   // entries beyond n_heads_here are never read
+    for (int h = 0; h < n_heads_here; ++h) {
+      hs.setT[h] = sets[2 * h].lo;
+      hs.setT_hi[h] = sets[2 * h].hi;
+      hs.setS[h] = sets[2 * h + 1].lo;
+      hs.base[h] = head_bases[h];
     }
     const unsigned long long two40 = 1ull << 40;
     const unsigned long long magic_nb = (two40 + (unsigned long long)g.NB - 1ull) / (unsigned long long)g.NB;
@@ -380,6 +373,8 @@ cudaError_t launch_mask_build(const HeadParamsArray& hp, const int* head_bases, 
     ++*launches;
     return cudaGetLastError();
   }
+  HeadBases hb;
+  for (int h = 0; h < kMaxHeads; ++h) hb.base[h] = h < n_heads_here ? head_bases[h] : 0;
   const size_t smem = tables_bytes(g);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(mask_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -1,0 +1,32 @@
+"""psa_mask_sizes (host code: the incremental walk over an axis' coordinate differences) against the oracle's axis
+masks: short and long axes, strides of 1, short, longer than the axis and infinite, offsets inside and far outside."""
+import random
+
+import pytest
+
+from oracle import psa_oracle as O
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_pair_counts_match_the_axis_masks(seed):
+    from paper_2609_37001_b200 import build
+    build.build()
+    from paper_2609_37001_b200 import binding as B
+    rng = random.Random(seed)
+    for _ in range(150):
+        T, H, W = rng.choice([1, 2, 21, 64, 65, 130]), rng.randint(1, 12), rng.randint(1, 12)
+        p = (rng.randint(1, T + 3), rng.choice([0, 1, -2, T, -T, 5 * T, -(1 << 29)]), rng.choice([0, 1, 2, 3, T, T + 1, 1 << 20]),
+             rng.randint(1, H * W + 3), rng.choice([0, -1, 3, H * W, -3 * H * W]), rng.choice([0, 1, 5, 6, H * W + 7]))
+        nb, nnz = B.psa_mask_sizes([p], (T, H, W), (1, 1, 1))
+        want = int(O.axis_mask(T, *p[:3]).sum()) * int(O.axis_mask(H * W, *p[3:]).sum())
+        assert (nb, nnz) == (T * H * W, want), (p, T, H, W)
+
+
+def test_parameters_given_as_lists_or_floats():
+    from paper_2609_37001_b200 import build
+    build.build()
+    from paper_2609_37001_b200 import binding as B
+    grid, tile = (21, 45, 80), (1, 15, 16)
+    want = B.psa_mask_sizes([(4, 2, 0, 5, 1, 3)], grid, tile)
+    assert B.psa_mask_sizes([[4, 2, 0, 5, 1, 3]], grid, tile) == want
+    assert B.psa_mask_sizes([(4.0, 2.0, 0.0, 5.0, 1.0, 3.0)], grid, tile) == want

@@ -73,6 +73,9 @@ constexpr uint32_t kOffMaskS = kOffMaskT + (kMaxTp / 32) * 4;   // kMaxSp / 32 w
 constexpr uint32_t kOffSched = kOffMaskS + (kMaxSp / 32) * 4;   // two published work items
 constexpr uint32_t kOffMisc = kOffSched + 32;                   // tmem base, abort flag
 constexpr uint32_t kOffXchg = kOffMisc + 16;                    // split-KV merge: (m, l) of 128 rows
+constexpr uint32_t kPartBytes = 128 * 128 * 4;                  // cluster mode: fp32 partial output of one tile, in the ring
+static_assert(2 * kPartBytes <= kNumSlots * kSlabBytes, "the partial outputs do not fit into the ring");
+constexpr uint32_t kOffScale = kOffQ + 4096;                    // cluster mode: weight of every partial result, in the Q buffers
 constexpr uint32_t kSmemBytes = kOffXchg + 128 * 8;
 constexpr uint32_t kSmemAlloc = kSmemBytes;                     // base alignment comes from the declaration
 static_assert(kSmemAlloc <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
@@ -163,6 +166,37 @@ __device__ __forceinline__ bool mbar_wait_probe_warp(uint32_t bar_a, uint32_t pa
   return __all_sync(0xffffffffu, ok);
 }
 
+// Programmatic dependent launch: the next kernel of the stream may start once every block has triggered; it sees this
+// kernel's results after its own wait.  Both do nothing in a launch without the attribute.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// words of an axis' set of attended differences
+__host__ __device__ constexpr int axis_words(int n) { return (2 * n - 1 + 31) / 32; }
+
+// Cluster: rank and size, the shared::cluster address of a CTA's shared memory, a barrier over all threads.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* tm, uint32_t bar,
                                             int c0, int c1, int c2, int c3, int c4) {
   asm volatile(
@@ -333,54 +367,85 @@ __device__ __noinline__ bool dbg_fail(int* ws_header, int code) {
 #endif
 
 // ----------------------------------------------------------------------------- planning
-// Work order: per head, query blocks ranked by attended key-block count (largest first),
-// heads kept together so that concurrently running CTAs share K/V in L2.
-__global__ void __launch_bounds__(256)
-plan_kernel(const HeadParamsArray hp, const Geom g, int head0, int clear_status, int* __restrict__ ws_header,
+// Work order: heads by descending number of attended pairs (`place`, from the host; heads stay together so that
+// concurrently running CTAs share K/V in L2), within a head query blocks by descending number of attended key blocks.
+// Heaviest first keeps the last wave short.  Bound by latency (one block per head): axis sets by ballot, counts as
+// popcounts of windows of the sets, ranks by counting larger keys, four per shared-memory load.  2.0 us for 40 heads
+// of 315 blocks (one thread per pair of coordinates and a compare of two words per pair of blocks: 11.7 us), most of
+// it hidden behind the attention kernel's prologue, which starts when every block has reached the trigger.
+constexpr int kPlanThreads = 512;
+__global__ void __launch_bounds__(kPlanThreads)
+plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int clear_status, int* __restrict__ ws_header,
             psa_head_params* __restrict__ hp_dev, WorkItem* __restrict__ items) {
-  extern __shared__ int sm[];  // cntT[Tp], cntS[Sp], cnt[NB]
-  int* cntT = sm;
-  int* cntS = sm + g.Tp;
-  int* cnt = cntS + g.Sp;
+  extern __shared__ __align__(16) uint32_t sm[];  // key[NB rounded up to 4], cntT[Tp], cntS[Sp], setT[], setS[]
+  pdl_trigger();
+  uint32_t* key = sm;
+  const int nb4 = (g.NB + 3) & ~3;
+  uint32_t* cntT = sm + nb4;
+  uint32_t* cntS = cntT + g.Tp;
+  uint32_t* setT = cntS + g.Sp;
+  uint32_t* setS = setT + axis_words(g.Tp);
   const int h = blockIdx.x;
-  const psa_head_params p = hp.p[head0 + h];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const psa_head_params p = hp.p[h];
+  // The previous launch on this workspace may still be running; nothing is written before it has finished.
+  pdl_wait();
   // The scheduler ticket restarts with every launch; the status words are cleared only by the
   // first launch of an API call, so that a timeout recorded by an earlier launch of the same call
   // (a call may need several: more than 128 heads, chunks of a host-tensor call) survives.
   if (h == 0 && threadIdx.x < kWsHeaderWords && (clear_status || (threadIdx.x != kWsStatus && threadIdx.x != kWsDetail)))
     ws_header[threadIdx.x] = 0;
   if (threadIdx.x == 0) hp_dev[h] = p;
-  for (int a = threadIdx.x; a < g.Tp + g.Sp; a += blockDim.x) {
-    int c = 0;
-    if (a < g.Tp) {
-      for (int k = 0; k < g.Tp; ++k) c += axis_attends(k - a, p.Tw, p.To, p.Ts);
-    } else {
-      for (int k = 0; k < g.Sp; ++k) c += axis_attends(k - (a - g.Tp), p.Sw, p.So, p.Ss);
-    }
-    sm[a] = c;
+  // attended differences, bit d + n - 1 for difference d
+  const int wT = axis_words(g.Tp), wS = axis_words(g.Sp);
+  for (int w = warp; w < wT + wS; w += kPlanThreads / 32) {
+    const bool is_t = w < wT;
+    const int i = (is_t ? w : w - wT) * 32 + lane, n = is_t ? g.Tp : g.Sp;
+    const bool att = i < 2 * n - 1 && (is_t ? axis_attends(i - (n - 1), p.Tw, p.To, p.Ts) : axis_attends(i - (n - 1), p.Sw, p.So, p.Ss));
+    const unsigned m = __ballot_sync(0xffffffffu, att);
+    if (lane == 0) setT[w] = m;   // setS follows setT
   }
   __syncthreads();
-  for (int qb = threadIdx.x; qb < g.NB; qb += blockDim.x) cnt[qb] = cntT[qb / g.Sp] * cntS[qb % g.Sp];
+  // row count of coordinate x: bits n - 1 - x .. 2n - 2 - x of its set
+  for (int a = threadIdx.x; a < g.Tp + g.Sp; a += kPlanThreads) {
+    const bool is_t = a < g.Tp;
+    const uint32_t* set = is_t ? setT : setS;
+    const int n = is_t ? g.Tp : g.Sp, x = is_t ? a : a - g.Tp;
+    const int lo = n - 1 - x, hi = lo + n;   // [lo, hi)
+    int c = 0;
+    for (int w = lo >> 5; w <= (hi - 1) >> 5; ++w) {
+      uint32_t m = set[w];
+      if (w == lo >> 5) m &= 0xffffffffu << (lo & 31);
+      if (w == (hi - 1) >> 5) m &= 0xffffffffu >> (31 - ((hi - 1) & 31));
+      c += __popc(m);
+    }
+    cntT[a] = c;   // cntS follows cntT
+  }
+  __syncthreads();
+  // unique keys: larger count first, then smaller block id (counts are at most NB < 2^16 here)
+  for (int qb = threadIdx.x; qb < nb4; qb += kPlanThreads)
+    key[qb] = qb < g.NB ? cntT[qb / g.Sp] * cntS[qb % g.Sp] * (uint32_t)g.NB + (uint32_t)(g.NB - 1 - qb) : 0u;
   __syncthreads();
   const int ipb = g.items_per_block;
-  // Text-query items first: they attend every key block, so they are the heaviest of the head.
+  // Text-query items of all heads first: they attend every key block, so they are the heaviest (behind the lighter
+  // items of earlier heads the last one alone kept the launch running: 825 instead of 783 us for 7 heads of 150 blocks).
   // Two text slabs per item; a single one runs in split-KV mode.  Flag in bit 25.
-  WorkItem* head_items = items + (size_t)h * g.items_per_head;
-  for (int it = threadIdx.x; it < g.n_titems; it += blockDim.x) {
+  WorkItem* head_items = items + (size_t)hp.place[h] * g.n_titems;
+  for (int it = threadIdx.x; it < g.n_titems; it += kPlanThreads) {
     const int sub0 = 2 * it;
     const int nq = (g.n_ts - sub0) >= 2 ? 2 : 1;
     head_items[it] = make_int4(h, 0, g.NB, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
   }
-  WorkItem* out = head_items + g.n_titems;
-  for (int qb = threadIdx.x; qb < g.NB; qb += blockDim.x) {
-    const int c = cnt[qb];
-    int rank = 0;
-    for (int j = 0; j < g.NB; ++j) {
-      const int cj = cnt[j];
-      rank += (cj > c) || (cj == c && j < qb);
+  WorkItem* out = items + (size_t)gridDim.x * g.n_titems + (size_t)hp.place[h] * g.NB * ipb;
+  for (int qb = threadIdx.x; qb < g.NB; qb += kPlanThreads) {
+    const uint32_t mine = key[qb];
+    int pos = 0;
+    for (int j = 0; j < nb4; j += 4) {
+      const uint4 k4 = *reinterpret_cast<const uint4*>(key + j);
+      pos += (int)(k4.x > mine) + (int)(k4.y > mine) + (int)(k4.z > mine) + (int)(k4.w > mine);
     }
+    const int c = (int)(mine / (uint32_t)g.NB);
     // two-slab items first (heavier), then the odd single-slab items, each in rank order
-    int pos = rank;
     for (int it = 0; it < ipb; ++it) {
       const int sub0 = 2 * it;
       const int nq = (g.n_sub - sub0) >= 2 ? 2 : 1;
@@ -392,20 +457,6 @@ plan_kernel(const HeadParamsArray hp, const Geom g, int head0, int clear_status,
 }
 
 // ----------------------------------------------------------------------------- attention
-struct AttnParams {
-  Geom g;
-  const WorkItem* items;
-  const psa_head_params* hp_dev;
-  int* ws_header;
-  float* lse;     // already offset to the first head of this launch
-  int n_items;
-  int shared_qkv; // 1: every head reads head 0 of q, k, v (candidate masks of one head, PSA-Search)
-};
-
-struct TensorMaps {
-  CUtensorMap q[3], k[3], v[3], o[3];  // [0]: full 128-token slab box, [1]: a block's last slab, [2]: text slab
-};
-
 // Extents and token count of slab `sub` of a block; `last` selects the tensor-map set.
 __device__ __forceinline__ void slab_shape(const Geom& g, int sub, int& et, int& eh, int& ew, int& ntok, int& last) {
   last = (sub == g.n_sub - 1) ? 1 : 0;
@@ -443,9 +494,11 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t lo) { return ((uint64_t)k
 //   m_ref / l: running reference maximum (scaled log2 domain) and running sum.
 // The reference maximum is lazy: it moves only when the slab's maximum exceeds it by more than
 // kRescaleThreshold, so exponentials stay below 2^threshold and O is rarely rescaled.
-template <int NK>
+//   lr (kRounded): running sum of the probabilities as rounded to bf16 for P V.  A shared item's partial results are
+// weighted by it, so that the rounding of a dominant probability cancels in out = O / lr; lse comes from l.
+template <int NK, bool kRounded>
 __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uint4 meta, bool first,
-                                             float scale_log2, float& m_ref, float& l, uint32_t bar_half,
+                                             float scale_log2, float& m_ref, float& l, float& lr, uint32_t bar_half,
                                              uint32_t bar_ready) {
   constexpr int NFULL = NK / 32, REM = NK % 32;
   static_assert(NK % 16 == 0 && NK >= 64 && NK <= 128 && (REM == 0 || REM == 16), "unsupported slab width");
@@ -482,6 +535,7 @@ __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uin
     }
     if (__any_sync(0xffffffffu, grow)) {
       l *= alpha;
+      if (kRounded) lr *= alpha;
 #pragma unroll
       for (int c4 = 0; c4 < 4; ++c4) {
         uint32_t o[32];
@@ -495,7 +549,7 @@ __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uin
   }
   const float m_use = (m_ref == neg_inf) ? 0.f : m_ref;
   const uint64_t sc2 = pack2(scale_log2, scale_log2), negm2 = pack2(-m_use, -m_use);
-  uint64_t sum2 = pack2(0.f, 0.f);
+  uint64_t sum2 = pack2(0.f, 0.f), sumr2 = pack2(0.f, 0.f);
   // probabilities exp2(scale*s - m_use), bf16, written over the scores in chunks of 32 keys
   auto exp_chunk = [&](int base, int npairs, uint32_t* pk) {
 #pragma unroll
@@ -513,6 +567,7 @@ __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uin
       }
       sum2 = add2(sum2, pack2(p0, p1));
       pk[c] = pack_bf16(p0, p1);
+      if (kRounded) sumr2 = add2(sumr2, pack2(__uint_as_float(pk[c] << 16), __uint_as_float(pk[c] & 0xffff0000u)));
     }
   };
 #pragma unroll
@@ -534,11 +589,98 @@ __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uin
   float sum0, sum1;
   unpack2(sum2, sum0, sum1);
   l += sum0 + sum1;
+  if (kRounded) {
+    unpack2(sumr2, sum0, sum1);
+    lr += sum0 + sum1;
+  }
   tc_wait_st();
   tc_fence_before();
   mbar_arrive(bar_ready);
 }
 
+// Token row (within the head) of row `row` of a query slab, or -1 if the row is padding.
+__device__ __forceinline__ long long row_token(const Geom& g, bool textq, int qb, int sub, int row) {
+  if (textq) {   // text slab: rows are consecutive text tokens; they follow the L video tokens
+    const int i = sub * kSlabTokens + row;
+    return i < g.n_text ? g.L + i : -1;
+  }
+  int t0, h0, w0, et, eh, ew, ntok, last;
+  slab_origin(g, qb, sub, t0, h0, w0);
+  slab_shape(g, sub, et, eh, ew, ntok, last);
+  const int t = t0 + row / (ew * eh), hh = h0 + (row / ew) % eh, ww = w0 + row % ew;
+  return (row < ntok && t < g.T && hh < g.H && ww < g.W) ? ((long long)t * g.H + hh) * g.W + ww : -1;
+}
+
+// Merge of a cluster's partial results (the softmax warpgroups of all its CTAs, between two cluster barriers): this CTA takes
+// every cluster_size-th part of the item's query rows, reads the (m, l, lr) and O of all CTAs -- and of both tiles when
+// the item is a single query slab whose even and odd key slabs were accumulated apart -- in a fixed order, and writes
+// out and lse.
+__device__ __forceinline__ void merge_cluster(const AttnParams& prm, uint8_t* smem, uint32_t sbase) {
+  const Geom& g = prm.g;
+  const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);   // the item as the load warp published it
+  if (wi.x < 0) return;                                               // (it gave up before that)
+  const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
+  const bool textq = ((wi.w >> 25) & 1) != 0;
+  const int csize = (int)cluster_size(), crank = (int)cluster_rank();
+  const int rpc = nq * 128 / csize;                  // rows of this CTA: 16, 32, 64 or 128
+  const int r0 = crank * rpc;                        // first of them, counted over the item's query slabs
+  const int tiles = nq == 1 ? 2 : 1, n_part = tiles * csize;
+  float* scale = reinterpret_cast<float*>(smem + kOffScale);   // [n_part][rpc]
+  const float neg_inf = __int_as_float(0xff800000);
+  // tile and tile row of the item's row r, for partial result p
+  auto tile_of = [&](int r, int p) -> int { return nq == 1 ? (p & 1) : (r >> 7); };
+  auto rank_of = [&](int p) -> uint32_t { return (uint32_t)(nq == 1 ? p >> 1 : p); };
+  const int tid = (int)threadIdx.x - 32 * kFirstSoftmaxWarp, n_thr = kThreads - 32 * kFirstSoftmaxWarp;
+  for (int i = tid; i < rpc; i += n_thr) {
+    const int r = r0 + i;
+    float m_all = neg_inf, l_all = 0.f, lr_all = 0.f;
+    for (int p = 0; p < n_part; ++p) {
+      const float4 ml = ld_cluster_f4(map_rank(sbase + kOffQ + (uint32_t)(tile_of(r, p) * 128 + (r & 127)) * 16u, rank_of(p)));
+      scale[p * rpc + i] = ml.x;
+      const float m_new = fmaxf(m_all, ml.x);
+      const float wa = (m_all == neg_inf) ? 0.f : fast_exp2(m_all - m_new), wb = (ml.x == neg_inf) ? 0.f : fast_exp2(ml.x - m_new);
+      l_all = wa * l_all + wb * ml.y;
+      lr_all = wa * lr_all + wb * ml.z;
+      m_all = m_new;
+    }
+    const bool empty = !(l_all > 0.f);
+    const float inv = empty ? 0.f : 1.f / lr_all;
+    for (int p = 0; p < n_part; ++p) {
+      const float m = scale[p * rpc + i];
+      scale[p * rpc + i] = (m == neg_inf) ? 0.f : fast_exp2(m - m_all) * inv;
+    }
+    const long long tok = row_token(g, textq, qb, sub0 + (r >> 7), r & 127);
+    if (tok >= 0 && PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.Lt, 0xD15))
+      prm.lse[(long long)head * g.Lt + tok] = empty ? neg_inf : (m_all + log2f(l_all)) * 0.6931471805599453f;
+  }
+  asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32 * kFirstSoftmaxWarp) : "memory");
+  // units of one row and 8 columns, rows fastest: 16-byte reads of consecutive rows are contiguous
+  uint16_t* out = reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head;
+  for (int u = tid; u < rpc * 16; u += n_thr) {
+    const int i = u % rpc, cg = u / rpc, r = r0 + i;
+    const long long tok = row_token(g, textq, qb, sub0 + (r >> 7), r & 127);
+    if (tok < 0) continue;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int p = 0; p < n_part; ++p) {
+      const float w = scale[p * rpc + i];
+      const uint32_t at = map_rank(sbase + kOffRing + (uint32_t)tile_of(r, p) * kPartBytes + (uint32_t)(2 * cg) * 2048u + (uint32_t)(r & 127) * 16u, rank_of(p));
+      const float4 a = ld_cluster_f4(at), b = ld_cluster_f4(at + 2048u);
+      if (w != 0.f) {
+        acc[0] = fmaf(w, a.x, acc[0]); acc[1] = fmaf(w, a.y, acc[1]); acc[2] = fmaf(w, a.z, acc[2]); acc[3] = fmaf(w, a.w, acc[3]);
+        acc[4] = fmaf(w, b.x, acc[4]); acc[5] = fmaf(w, b.y, acc[5]); acc[6] = fmaf(w, b.z, acc[6]); acc[7] = fmaf(w, b.w, acc[7]);
+      }
+    }
+    if (PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.Lt, 0xD16))
+      *reinterpret_cast<uint4*>(out + tok * prm.out_token + cg * 8) =
+          make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+  }
+}
+
+// kCluster: a cluster of 2, 4 or 8 CTAs shares ONE work item (cluster i of the grid takes item i), each CTA taking
+// its share of the attended key blocks; the partial results are merged through distributed shared memory.  Otherwise
+// persistent CTAs draw whole items from the ticket.
+template <bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
   // 128-byte swizzled slabs need a 1024-byte aligned base; the declaration asks for it and the
@@ -585,6 +727,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + kOffMisc), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (threadIdx.x == 0) pdl_trigger();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -626,14 +769,26 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
     uint32_t kv_g = 0;         // key slabs issued so far
     uint32_t it_q0 = 0, it_q1 = 0; // items in which query slab i was active
     bool ok = tmem_ok;
+    pdl_wait();   // the work items are written by the planning kernel
     for (uint32_t n = 0; ok; ++n) {
       const uint32_t sslot = n & 1u;
       ok = mbar_wait_warp(bar(kBarSchedEmpty + sslot), ((n >> 1) & 1u) ^ 1u, abort_flag, 0x401);
       if (!ok) break;
       WorkItem wi = make_int4(-1, 0, 0, 0);
+      int skip = 0;   // attended key blocks before this CTA's share
       if (lane == 0) {
-        const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
-        if (ticket < prm.n_items) wi = prm.items[ticket];
+        if constexpr (kCluster) {
+          if (n == 0) {
+            const int r = (int)cluster_rank(), c = (int)cluster_size();
+            wi = prm.items[blockIdx.x / (uint32_t)c];
+            skip = (int)((long long)wi.z * r / c);
+            wi.z = (int)((long long)wi.z * (r + 1) / c) - skip;
+            if (r + 1 < c) wi.w |= 1 << 26;   // the text keys go with the last share
+          }
+        } else {
+          const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
+          if (ticket < prm.n_items) wi = prm.items[ticket];
+        }
         sched[sslot].x = wi.x; sched[sslot].y = wi.y; sched[sslot].z = wi.z; sched[sslot].w = wi.w;
         mbar_arrive(bar(kBarSchedFull + sslot));
       }
@@ -641,6 +796,11 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       wi.y = __shfl_sync(0xffffffffu, wi.y, 0);
       wi.w = __shfl_sync(0xffffffffu, wi.w, 0);
       if (wi.x < 0) break;
+      int left = 0x7fffffff;   // attended key blocks still to load
+      if constexpr (kCluster) {
+        skip = __shfl_sync(0xffffffffu, skip, 0);
+        left = __shfl_sync(0xffffffffu, wi.z, 0);
+      }
       const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
       if (!PSA_CHECKED(head < g.n_heads && qb >= 0 && qb <= g.NB && nq >= 1 && nq <= 2 &&
                        sub0 + nq <= ((wi.w >> 25) & 1 ? g.n_ts : g.n_sub), 0xD04)) {
@@ -738,16 +898,21 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
         else { bt0 = t0; bh0 = h0; bw0 = w0; blast = last; bntok = ntok; }
         ++npend;
       };
-      for (int tw = 0; ok && tw < g.Tp; tw += 32) {
+      for (int tw = 0; ok && left > 0 && tw < g.Tp; tw += 32) {
         uint32_t mt = maskT[tw >> 5];
-        while (ok && mt) {
+        while (ok && left > 0 && mt) {
           const int tk = tw + __ffs(mt) - 1;
           mt &= mt - 1;
-          for (int sw = 0; ok && sw < g.Sp; sw += 32) {
+          for (int sw = 0; ok && left > 0 && sw < g.Sp; sw += 32) {
             uint32_t ms = maskS[sw >> 5];
             while (ok && ms) {
               const int sk = sw + __ffs(ms) - 1;
               ms &= ms - 1;
+              if constexpr (kCluster) {
+                if (skip > 0) { --skip; continue; }
+                if (left == 0) break;
+                --left;
+              }
               const int kb = tk * g.Sp + sk;
               for (int sub = 0; ok && sub < g.n_sub; ++sub) {
                 int t0, h0, w0, et, eh, ew, ntok, last;
@@ -774,7 +939,8 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
         }
       }
       // text key slabs: attended by every query; tokens beyond n_text are zero-filled and masked
-      for (int ts = 0; ok && ts < g.n_ts; ++ts) {
+      const int n_ts = kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts;
+      for (int ts = 0; ok && ts < n_ts; ++ts) {
         const int tok0 = ts * kSlabTokens;
         const int nvalid = g.n_text - tok0;   // >= 1
         const uint32_t vw0 = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
@@ -881,7 +1047,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       const int nq = (wi.w >> 16) & 0xff;
       const bool split = ((wi.w >> 24) & 1) != 0;
       const int n_vid = wi.z * g.n_sub;          // video key slabs, then the text slabs (always 128 wide)
-      const int n_kv = n_vid + g.n_ts;
+      const int n_kv = n_vid + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
       auto nk_j = [&](int j, int r) -> int { return j >= n_vid ? kSlabTokens : nk_at(r); };
       // which accumulators this item uses: both for a two-slab item, and for a split-KV item
       // with at least two key slabs (even slabs -> O_0, odd slabs -> O_1)
@@ -1084,11 +1250,12 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       const bool split = ((wi.w >> 24) & 1) != 0;
       const bool textq = ((wi.w >> 25) & 1) != 0;
       const int n_vid = wi.z * g.n_sub;          // video key slabs, then the text slabs (always 128 wide)
-      const int n_kv = n_vid + g.n_ts;
+      const int n_kv = n_vid + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
       const bool use_o1 = (nq > 1) || (split && n_kv > 1);
       const bool active = (qi == 0) || use_o1;
       float m_ref = neg_inf;  // running reference maximum, scaled log2 domain
       float l = 0.f;          // running sum of exp2(s - m_ref)
+      float lr = 0.f;         // cluster mode: the same of the rounded probabilities
       if (active) {
         // key slabs of this tile: all of them, or every second one in a split-KV item
         const int j0 = split ? qi : 0, dj = split ? 2 : 1;
@@ -1107,10 +1274,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
           const uint4 m = *reinterpret_cast<const uint4*>(meta + ((kv_g + (uint32_t)j) % kMetaRing) * 8);
           const uint32_t bh = bar(kBarPHalf + qi), br = bar(kBarPReady + qi);
           const bool first = (j == j0);
-          if (nk == 128) softmax_slab<128>(tS, tO, m, first, g.scale_log2, m_ref, l, bh, br);
-          else if (nk == 112) softmax_slab<112>(tS, tO, m, first, g.scale_log2, m_ref, l, bh, br);
-          else if (nk == 96) softmax_slab<96>(tS, tO, m, first, g.scale_log2, m_ref, l, bh, br);
-          else softmax_slab<64>(tS, tO, m, first, g.scale_log2, m_ref, l, bh, br);
+          if (nk == 128) softmax_slab<128, kCluster>(tS, tO, m, first, g.scale_log2, m_ref, l, lr, bh, br);
+          else if (nk == 112) softmax_slab<112, kCluster>(tS, tO, m, first, g.scale_log2, m_ref, l, lr, bh, br);
+          else if (nk == 96) softmax_slab<96, kCluster>(tS, tO, m, first, g.scale_log2, m_ref, l, lr, bh, br);
+          else softmax_slab<64, kCluster>(tS, tO, m, first, g.scale_log2, m_ref, l, lr, bh, br);
         }
       }
       kv_g += (uint32_t)n_kv;
@@ -1118,6 +1285,35 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       const uint32_t par_o0 = it_o0 & 1u, par_o1 = it_o1 & 1u;
       ++it_o0;
       if (use_o1) ++it_o1;
+      if constexpr (kCluster) {
+        // Leave this tile's partial result in shared memory for the merge after the roles have met: (m, l, lr) of each row
+        // in the Q buffers, O as fp32 [32 column groups of 4][128 rows] in the K/V ring -- both idle once every MMA
+        // of the CTA has completed.  A tile without keys is marked by m = -inf; what is read as its O gets weight 0.
+        ok = mbar_wait_warp(bar(kBarOFull + 0), par_o0, abort_flag, 0x310);
+        if (!ok) break;
+        if (use_o1) {
+          ok = mbar_wait_warp(bar(kBarOFull + 1), par_o1, abort_flag, 0x311);
+          if (!ok) break;
+        }
+        const bool has = active && n_kv > 0;
+        *reinterpret_cast<float4*>(smem + kOffQ + (uint32_t)(qi * 128 + row) * 16u) =
+            has ? make_float4(m_ref, l, lr, 0.f) : make_float4(neg_inf, 0.f, 0.f, 0.f);
+        if (has) {
+          tc_fence_after();
+          uint8_t* part = smem + kOffRing + (uint32_t)qi * kPartBytes + (uint32_t)row * 16u;
+#pragma unroll 1
+          for (int c4 = 0; c4 < 4; ++c4) {
+            uint32_t o[32];
+            tc_ld32(tO + c4 * 32, o);
+            tc_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              *reinterpret_cast<uint4*>(part + (uint32_t)(c4 * 8 + e) * 2048u) = make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+          }
+          tc_fence_before();
+        }
+        continue;
+      }
       if (!active) continue;
 
       // ---- epilogue: out = O / l, lse = ln2 * (m_ref + log2 l).  In a split-KV item the two
@@ -1236,6 +1432,11 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
   // ------------------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
+  if constexpr (kCluster) {
+    cluster_sync_all();   // every CTA's partial results are in place
+    if (warp >= kFirstSoftmaxWarp) merge_cluster(prm, smem, sbase);   // (the first warpgroup gave its registers away)
+    cluster_sync_all();   // nobody's shared memory is read any more
+  }
   if (threadIdx.x == 0 && *abort_flag != 0) {
     if (atomicCAS(prm.ws_header + kWsStatus, 0, (int)PSA_ERR_TIMEOUT) == 0) prm.ws_header[kWsDetail] = *abort_flag;
   }
@@ -1269,37 +1470,64 @@ cudaError_t launch_wait_probe(int* ws_header, unsigned long long limit_ns, cudaS
 }
 
 // ----------------------------------------------------------------------------- launchers
-size_t plan_smem_bytes(const Geom& g) { return sizeof(int) * (size_t)(g.Tp + g.Sp + g.NB); }
+size_t plan_smem_bytes(const Geom& g) {
+  return 4 * (size_t)(((g.NB + 3) & ~3) + g.Tp + g.Sp + axis_words(g.Tp) + axis_words(g.Sp));
+}
 
-cudaError_t launch_plan(const HeadParamsArray& hp, const Geom& g, int head0, int n_heads_here, bool clear_status,
+namespace {
+// Launch that may start before its predecessor in the stream has finished (see pdl_wait), in clusters of `cluster`.
+struct LaunchConfig {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  LaunchConfig(int grid, int threads, size_t smem, cudaStream_t stream, int cluster) {
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+  }
+};
+}  // namespace
+
+// Once per device: shared-memory limits, and how many clusters of 2, 4 and 8 CTAs run at a time.
+cudaError_t attn_init(int clusters[3]) {
+  cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(attn_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc);
+  if (e != cudaSuccess) return e;
+  for (int i = 0; i < 3; ++i) {
+    LaunchConfig lc(2 << i, kThreads, kSmemAlloc, nullptr, 2 << i);
+    if ((e = cudaOccupancyMaxActiveClusters(&clusters[i], attn_fwd_kernel<true>, &lc.cfg)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, bool clear_status,
                         int* ws_header, psa_head_params* hp_dev, WorkItem* items, cudaStream_t stream) {
   const size_t smem = plan_smem_bytes(g);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  plan_kernel<<<n_heads_here, 256, smem, stream>>>(hp, g, head0, clear_status ? 1 : 0, ws_header, hp_dev, items);
-  return cudaGetLastError();
+  LaunchConfig lc(n_heads_here, kPlanThreads, smem, stream, 1);
+  return cudaLaunchKernelEx(&lc.cfg, plan_kernel, hp, g, clear_status ? 1 : 0, ws_header, hp_dev, items);
 }
 
-cudaError_t launch_attn(const TensorMaps& tm, const Geom& g, const WorkItem* items, const psa_head_params* hp_dev,
-                        int* ws_header, float* lse, int n_items, int n_sms, bool shared_qkv, cudaStream_t stream) {
-  {  // per device, cheap: set on every call
-    cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc);
-    if (e != cudaSuccess) return e;
+// cluster: CTAs per work item (1: persistent CTAs, whole items)
+cudaError_t launch_attn(const TensorMaps& tm, const AttnParams& prm, int n_sms, int cluster, cudaStream_t stream) {
+  if (prm.n_items <= 0) return cudaSuccess;
+  if (cluster > 1) {
+    LaunchConfig lc(prm.n_items * cluster, kThreads, kSmemAlloc, stream, cluster);
+    return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<true>, tm, prm);
   }
-  AttnParams prm;
-  prm.g = g;
-  prm.items = items;
-  prm.hp_dev = hp_dev;
-  prm.ws_header = ws_header;
-  prm.lse = lse;
-  prm.n_items = n_items;
-  prm.shared_qkv = shared_qkv ? 1 : 0;
-  const int grid = n_items < n_sms ? n_items : n_sms;
-  if (grid <= 0) return cudaSuccess;
-  attn_fwd_kernel<<<grid, kThreads, kSmemAlloc, stream>>>(tm, prm);
-  return cudaGetLastError();
+  LaunchConfig lc(prm.n_items < n_sms ? prm.n_items : n_sms, kThreads, kSmemAlloc, stream, 1);
+  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<false>, tm, prm);
 }
 
 }  // namespace psa

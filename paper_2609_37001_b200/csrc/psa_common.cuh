@@ -1,5 +1,6 @@
 // Shared host/device definitions of the PSA library (not part of the public ABI).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -39,10 +40,35 @@ struct HeadParamsArray {
   psa_head_params p[kMaxHeads];
 };
 
+// Arguments of the planning kernel: the heads' parameters and each head's place in the work order.
+struct PlanParams {
+  psa_head_params p[kMaxHeads];
+  uint8_t place[kMaxHeads];
+};
+
 // One unit of work of the attention kernel: up to two query slabs of one query block.
 // x = head, y = query block id, z = number of attended key blocks,
 // w = first slab index | (number of slabs << 16) | (split-KV mode << 24) | (text-query item << 25)
+// (inside a CTA of a cluster that shares one item: z = its share of the blocks, bit 26 of w = no text keys)
 typedef int4 WorkItem;
+
+// [0]: box of a full 128-token slab, [1]: of a block's last slab, [2]: of a text slab
+struct TensorMaps {
+  CUtensorMap q[3], k[3], v[3], o[3];
+};
+
+// Arguments of one attention launch; lse and out start at the launch's first head.
+struct AttnParams {
+  Geom g;
+  const WorkItem* items;
+  const psa_head_params* hp_dev;
+  int* ws_header;
+  float* lse;
+  int n_items;
+  int shared_qkv;   // 1: every head reads head 0 of q, k, v (candidate masks of one head, PSA-Search)
+  void* out;        // for rows that are stored without TMA; strides in elements
+  long long out_head, out_token;
+};
 
 // Layout of the per-device workspace (all int32 words).
 constexpr int kWsStatus = 0;     // first device-side error (0 = none)

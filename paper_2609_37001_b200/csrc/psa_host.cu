@@ -17,13 +17,10 @@ bool mask_build_small(const Geom& g);
 cudaError_t launch_mask_build(const HeadParamsArray& hp, const AxisSet* sets, const int* head_bases, const Geom& g, int n_heads_here,
                               uint8_t* block_mask, int* row_ptr, int* col_idx, int total_nnz_through_chunk,
                               int n_sms, cudaStream_t stream, int* launches);
-cudaError_t launch_plan(const HeadParamsArray& hp, const Geom& g, int head0, int n_heads_here, bool clear_status,
-                        int* ws_header, psa_head_params* hp_dev, WorkItem* items, cudaStream_t stream);
-struct TensorMaps {
-  CUtensorMap q[3], k[3], v[3], o[3];  // [0]: full 128-token slab box, [1]: a block's last slab, [2]: text slab
-};
-cudaError_t launch_attn(const TensorMaps& tm, const Geom& g, const WorkItem* items, const psa_head_params* hp_dev,
-                        int* ws_header, float* lse, int n_items, int n_sms, bool shared_qkv, cudaStream_t stream);
+cudaError_t attn_init(int clusters[3]);
+cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, bool clear_status, int* ws_header,
+                        psa_head_params* hp_dev, WorkItem* items, cudaStream_t stream);
+cudaError_t launch_attn(const TensorMaps& tm, const AttnParams& prm, int n_sms, int cluster, cudaStream_t stream);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
                                  float* losses, cudaStream_t stream, int* launches);
@@ -43,6 +40,8 @@ struct Workspace {
   size_t bytes = 0;
   int n_sms = 0;
   int cc_major = 0;
+  bool attn_ready = false;
+  int clusters[3] = {0, 0, 0};   // clusters of 2, 4 and 8 attention CTAs that run at a time
 };
 Workspace g_ws[kMaxDevices];
 
@@ -174,6 +173,17 @@ int device_info(int* dev, Workspace** ws) {
   return PSA_OK;
 }
 
+// First attention call on a device: driver entry point, kernel attributes.
+int init_attn(Workspace* w) {
+  if (w->attn_ready) return PSA_OK;
+  if (w->cc_major != 10) return PSA_ERR_UNSUPPORTED;
+  const int rc = load_driver_entry();
+  if (rc != PSA_OK) return rc;
+  if (attn_init(w->clusters) != cudaSuccess) return PSA_ERR_CUDA;
+  w->attn_ready = true;
+  return PSA_OK;
+}
+
 int ensure_workspace(Workspace* w, size_t bytes) {
   if (w->bytes >= bytes) return PSA_OK;
   if (w->base) {
@@ -254,6 +264,53 @@ int encode_maps(TensorMaps* tm, const void* q, const void* k, const void* v, voi
     tm->q[2] = tm->q[0]; tm->k[2] = tm->k[0]; tm->v[2] = tm->v[0]; tm->o[2] = tm->o[0];
   }
   return PSA_OK;
+}
+
+// Attended block pairs of every head; returns their sum.
+long long head_weights(const psa_head_params* params, int n, const Geom& g, long long* w) {
+  long long total = 0;
+  for (int h = 0; h < n; ++h) {
+    // (the samples of a batch or the heads of a group often repeat the parameters of the head before)
+    w[h] = h > 0 && std::memcmp(&params[h], &params[h - 1], sizeof(psa_head_params)) == 0 ? w[h - 1] : head_nnz(params[h], g);
+    total += w[h];
+  }
+  return total;
+}
+
+// Planning arguments of one launch: the heads' parameters and their places in the work order, heavier heads first.
+void plan_params(PlanParams* pp, const psa_head_params* params, const long long* w, int n) {
+  for (int h = 0; h < n; ++h) {
+    pp->p[h] = params[h];
+    int place = 0;
+    for (int j = 0; j < n; ++j) place += w[j] > w[h] || (w[j] == w[h] && j < h);
+    pp->place[h] = (uint8_t)place;
+  }
+}
+
+// CTAs that share a work item: 1 (persistent CTAs that draw whole items), 2, 4 or 8.  A launch takes about as many
+// rounds as its items need on the SMs, so a problem of few items, or of a few more than a whole number of rounds,
+// leaves SMs idle; sharing items makes the rounds shorter.  Times in clocks, measured: a key slab takes 3,300 for two
+// query slabs and 1,900 for one (split-KV mode), an item 9,000 beside its slabs in a persistent CTA and 18,000 in a
+// cluster (which starts its CTAs anew and merges).
+// Decided for a call as a whole (`pairs` of all its heads), so that the chunks of a host-tensor call compute what the
+// device call computes, bit for bit.
+int share_items(const Workspace& ws, const Geom& g, long long pairs, int n_heads) {
+  const int n_items = (n_heads < kMaxHeads ? n_heads : kMaxHeads) * g.items_per_head;   // of one launch
+  if (n_items > 2 * ws.n_sms) return 1;   // (beyond two rounds at most a third is to be gained)
+  const double blocks = (double)pairs / ((double)n_heads * g.NB);   // attended by the average query block
+  const int singles = g.n_sub & 1, pairs_per_block = g.n_sub >> 1;
+  const double slabs = blocks * g.n_sub + g.n_ts;
+  const double item = slabs * (3300.0 * pairs_per_block + 1900.0 * singles) / (pairs_per_block + singles);
+  auto rounds = [](int items, int at_a_time) -> double { return (double)((items + at_a_time - 1) / at_a_time); };
+  double best = rounds(n_items, ws.n_sms) * (item + 9000.0);
+  int cluster = 1;
+  for (int i = 0; i < 3; ++i) {
+    const int c = 2 << i;
+    if (ws.clusters[i] < 1 || blocks < c) break;   // a share holds at least one block
+    const double t = rounds(n_items, ws.clusters[i]) * (item / c + 18000.0);
+    if (t < 0.9 * best) { best = t; cluster = c; }
+  }
+  return cluster;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -406,14 +463,14 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T
 // Planning + attention launches for n_heads heads (in launches of at most kMaxHeads) on the cached
 // per-device workspace.  Arguments are already validated; g_mu is held by the caller.
 // clear_status: this is the first launch sequence of an API call (later ones keep the status word).
+// cluster: CTAs per work item, 0: by share_items for these heads.
 static int run_attn(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
-                    int n_heads, const Geom& g, const Layout& lay, cudaStream_t st, bool clear_status = true) {
+                    int n_heads, const Geom& g, const Layout& lay, cudaStream_t st, bool clear_status = true, int cluster = 0) {
   int dev;
   Workspace* ws;
   int rc = device_info(&dev, &ws);
   if (rc != PSA_OK) return rc;
-  if (ws->cc_major != 10) return PSA_ERR_UNSUPPORTED;
-  rc = load_driver_entry();
+  rc = init_attn(ws);
   if (rc != PSA_OK) return rc;
   const int chunk = n_heads < kMaxHeads ? n_heads : kMaxHeads;
   const size_t items_bytes = sizeof(WorkItem) * (size_t)chunk * g.items_per_head;
@@ -424,11 +481,11 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
   int* ws_header = static_cast<int*>(ws->base);
   psa_head_params* hp_dev = reinterpret_cast<psa_head_params*>(static_cast<char*>(ws->base) + hp_off);
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(ws->base) + items_off);
+  std::vector<long long> weights((size_t)n_heads);
+  const long long pairs = head_weights(head_params, n_heads, g, weights.data());
+  if (cluster == 0) cluster = share_items(*ws, g, pairs, n_heads);
   for (int head0 = 0; head0 < n_heads; head0 += kMaxHeads) {
     const int n_here = n_heads - head0 < kMaxHeads ? n_heads - head0 : kMaxHeads;
-    HeadParamsArray hp;
-    std::memset(&hp, 0, sizeof(hp));
-    for (int h = 0; h < n_here; ++h) hp.p[h] = head_params[head0 + h];
     const long long in_off = lay.shared_qkv ? 0 : (long long)head0 * lay.in_head;
     const long long out_off = (long long)head0 * lay.out_head;
     TensorMaps tm;
@@ -437,24 +494,26 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
       return rc;
     Geom gh = g;
     gh.n_heads = n_here;
-    if (launch_plan(hp, gh, 0, n_here, clear_status && head0 == 0, ws_header, hp_dev, items, st) != cudaSuccess)
+    PlanParams pp;
+    plan_params(&pp, head_params + head0, weights.data() + head0, n_here);
+    if (launch_plan(pp, gh, n_here, clear_status && head0 == 0, ws_header, hp_dev, items, st) != cudaSuccess)
       return PSA_ERR_CUDA;
     ++g_launches;
     const int n_items = n_here * g.items_per_head;
     if (g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
-    if (launch_attn(tm, gh, items, hp_dev, ws_header, lse + (long long)head0 * g.Lt, n_items, ws->n_sms, lay.shared_qkv, st) !=
-        cudaSuccess)
-      return PSA_ERR_CUDA;
+    const AttnParams prm = {gh, items, hp_dev, ws_header, lse + (long long)head0 * g.Lt, n_items, lay.shared_qkv ? 1 : 0,
+                            static_cast<uint16_t*>(out) + out_off, lay.out_head, lay.out_token};
+    if (launch_attn(tm, prm, ws->n_sms, cluster, st) != cudaSuccess) return PSA_ERR_CUDA;
     if (g_ev_start && g_ev_stop) cudaEventRecord(g_ev_stop, st);
     ++g_launches;
   }
   return PSA_OK;
 }
 
-// psa_attn_fwd with the choice of keeping the status word (chunks of one host-tensor call).
+// psa_attn_fwd with the choice of keeping the status word and of the CTAs per item (chunks of one host-tensor call).
 static int attn_fwd_checked(const void* q, const void* k, const void* v, void* out, float* lse,
                             const psa_head_params* head_params, const psa_problem* prob, int T, int H, int W, void* stream,
-                            bool clear_status) {
+                            bool clear_status, int cluster = 0) {
   Geom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
@@ -468,7 +527,7 @@ static int attn_fwd_checked(const void* q, const void* k, const void* v, void* o
     if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lock(g_mu);
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
-  return run_attn(q, k, v, out, lse, head_params, prob->n_heads, g, lay, static_cast<cudaStream_t>(stream), clear_status);
+  return run_attn(q, k, v, out, lse, head_params, prob->n_heads, g, lay, static_cast<cudaStream_t>(stream), clear_status, cluster);
 }
 
 int psa_attn_fwd(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
@@ -628,8 +687,7 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   Workspace* ws;
   rc = device_info(&dev, &ws);
   if (rc != PSA_OK) return rc;
-  if (ws->cc_major != 10) return PSA_ERR_UNSUPPORTED;
-  rc = load_driver_entry();
+  rc = init_attn(ws);
   if (rc != PSA_OK) return rc;
   void* base = nullptr;
   rc = noalloc_scratch(dev, &base);
@@ -639,18 +697,20 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(base) + kNoAllocItemsOff);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  HeadParamsArray hp;
-  std::memset(&hp, 0, sizeof(hp));
-  for (int h = 0; h < prob->n_heads; ++h) hp.p[h] = head_params[h];
   TensorMaps tm;
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
   if ((rc = encode_maps(&tm, q, k, v, out, g, lay, prob->n_heads)) != PSA_OK) return rc;
   // The planning kernel clears the header words (status, ticket) and rewrites the parameter
   // records and every work item of this call, so nothing of the previous call is read.
-  if (launch_plan(hp, g, 0, prob->n_heads, true, header, hp_dev, items, st) != cudaSuccess) return PSA_ERR_CUDA;
+  PlanParams pp;
+  long long weights[kMaxHeads];
+  const long long pairs = head_weights(head_params, prob->n_heads, g, weights);
+  plan_params(&pp, head_params, weights, prob->n_heads);
+  if (launch_plan(pp, g, prob->n_heads, true, header, hp_dev, items, st) != cudaSuccess) return PSA_ERR_CUDA;
   ++g_launches;
-  if (launch_attn(tm, g, items, hp_dev, header, lse, (int)n_items_ll, ws->n_sms, false, st) != cudaSuccess)
-    return PSA_ERR_CUDA;
+  const int n_items = (int)n_items_ll;
+  const AttnParams prm = {g, items, hp_dev, header, lse, n_items, 0, out, lay.out_head, lay.out_token};
+  if (launch_attn(tm, prm, ws->n_sms, share_items(*ws, g, pairs, prob->n_heads), st) != cudaSuccess) return PSA_ERR_CUDA;
   ++g_launches;
   if (status_detail) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return PSA_ERR_CUDA;
@@ -715,16 +775,25 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
   Chunk chunks[kHostChunks];
   int n_list = 0;
   int last1 = -1, last2 = -1;   // lightest and second-lightest head
+  Geom g;
+  int rc = make_geom(prob, T, H, W, true, &g);
+  if (rc != PSA_OK) return rc;
+  for (int h = 0; h < prob->n_heads; ++h)
+    if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
+  std::vector<long long> weights((size_t)prob->n_heads);
+  const long long pairs = head_weights(head_params, prob->n_heads, g, weights.data());
+  int cluster;
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    Workspace* ws;
+    if ((rc = device_info(&dev, &ws)) != PSA_OK || (rc = init_attn(ws)) != PSA_OK) return rc;
+    cluster = share_items(*ws, g, pairs, prob->n_heads);
+  }
   if (n_edge) {
-    Geom g;
-    const int rcg = make_geom(prob, T, H, W, true, &g);
-    if (rcg != PSA_OK) return rcg;
-    long long w1 = 0, w2 = 0;
     for (int h = 0; h < prob->n_heads; ++h) {
-      if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
-      const long long w = head_nnz(head_params[h], g);
-      if (last1 < 0 || w < w1) { last2 = last1; w2 = w1; last1 = h; w1 = w; }
-      else if (last2 < 0 || w < w2) { last2 = h; w2 = w; }
+      const long long w = weights[h];
+      if (last1 < 0 || w < weights[last1]) { last2 = last1; last1 = h; }
+      else if (last2 < 0 || w < weights[last2]) last2 = h;
     }
   }
   {
@@ -758,7 +827,7 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
     if (cudaStreamWaitEvent(st, pipe->ev_in[c], 0) != cudaSuccess) return PSA_ERR_CUDA;
     psa_problem sub = *prob;
     sub.n_heads = nh;
-    const int rc = attn_fwd_checked(dq, dk, dv, dout, d_lse + (size_t)h0 * L, head_params + h0, &sub, T, H, W, stream, c == 0);
+    rc = attn_fwd_checked(dq, dk, dv, dout, d_lse + (size_t)h0 * L, head_params + h0, &sub, T, H, W, stream, c == 0, cluster);
     if (rc != PSA_OK) return rc;
     if (cudaEventRecord(pipe->ev_done[c], st) != cudaSuccess) return PSA_ERR_CUDA;
     if (cudaStreamWaitEvent(pipe->d2h, pipe->ev_done[c], 0) != cudaSuccess) return PSA_ERR_CUDA;

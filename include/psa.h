@@ -203,7 +203,8 @@ int psa_search_select_at_sparsity(const float* losses, const float* sparsity, in
 
 /* Synchronises the current device, then returns the status word the last psa_attn_fwd
  * on it left behind: PSA_OK, or PSA_ERR_TIMEOUT if a bounded wait inside the kernel
- * expired (outputs are then undefined).  *detail (optional, host) receives a
+ * expired (outputs are then undefined); also what a replay of a call captured in a CUDA graph
+ * reported since the last query.  *detail (optional, host) receives a
  * diagnostic code naming the wait that gave up. */
 int psa_last_device_status(int32_t* detail);
 

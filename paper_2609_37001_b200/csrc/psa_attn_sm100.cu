@@ -73,9 +73,9 @@ constexpr uint32_t kOffMaskS = kOffMaskT + (kMaxTp / 32) * 4;   // kMaxSp / 32 w
 constexpr uint32_t kOffSched = kOffMaskS + (kMaxSp / 32) * 4;   // two published work items
 constexpr uint32_t kOffMisc = kOffSched + 32;                   // tmem base, abort flag
 constexpr uint32_t kOffXchg = kOffMisc + 16;                    // split-KV merge: (m, l) of 128 rows
-constexpr uint32_t kPartBytes = 128 * 128 * 4;                  // cluster mode: fp32 partial output of one tile, in the ring
-static_assert(2 * kPartBytes <= kNumSlots * kSlabBytes, "the partial outputs do not fit into the ring");
-constexpr uint32_t kOffScale = kOffQ + 4096;                    // cluster mode: weight of every partial result, in the Q buffers
+static_assert(256 * 128 * 4 <= kNumSlots * kSlabBytes, "the partial outputs do not fit into the ring");
+constexpr uint32_t kOffPartTmp = kOffQ + 16384;                 // cluster mode: (m, l, lr) of the two tiles of one query slab
+constexpr uint32_t kOffRowTok = kOffXchg;                       // cluster mode: token of every row that this CTA merges
 constexpr uint32_t kSmemBytes = kOffXchg + 128 * 8;
 constexpr uint32_t kSmemAlloc = kSmemBytes;                     // base alignment comes from the declaration
 static_assert(kSmemAlloc <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
@@ -192,11 +192,13 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
+__device__ __forceinline__ void st_cluster_u4(uint32_t addr, const uint32_t* v) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
+__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* tm, uint32_t bar,
                                             int c0, int c1, int c2, int c3, int c4) {
   asm volatile(
@@ -352,16 +354,25 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
+// First error of API call `call_id` into the status words.  Nothing clears them: the host takes them as an answer only
+// if they carry the id of the call that it asks about.
+__device__ __forceinline__ void report_status(int* ws_header, int call_id, int status, int detail) {
+  if (atomicExch(ws_header + kWsCallId, call_id) != call_id) {
+    ws_header[kWsDetail] = detail;
+    ws_header[kWsStatus] = status;
+  }
+}
+
 // Checked build (-DPSA_DEBUG_CHECKS; the stand-in for a memory checker): every global store index,
 // TMA coordinate, ring / table index and TMEM column range computed by the kernel is verified before
 // use.  A violation records PSA_ERR_INTERNAL with a code naming the site in the status word and the
 // access is skipped -- nothing traps.  In the regular build the checks compile to `true`.
 #ifdef PSA_DEBUG_CHECKS
-__device__ __noinline__ bool dbg_fail(int* ws_header, int code) {
-  if (atomicCAS(ws_header + kWsStatus, 0, (int)PSA_ERR_INTERNAL) == 0) ws_header[kWsDetail] = code;
+__device__ __noinline__ bool dbg_fail(int* ws_header, int call_id, int code) {
+  report_status(ws_header, call_id, PSA_ERR_INTERNAL, code);
   return false;
 }
-#define PSA_CHECKED(cond, code) ((cond) ? true : dbg_fail(prm.ws_header, (code)))
+#define PSA_CHECKED(cond, code) ((cond) ? true : dbg_fail(prm.ws_header, prm.call_id, (code)))
 #else
 #define PSA_CHECKED(cond, code) true
 #endif
@@ -375,7 +386,7 @@ __device__ __noinline__ bool dbg_fail(int* ws_header, int code) {
 // it hidden behind the attention kernel's prologue, which starts when every block has reached the trigger.
 constexpr int kPlanThreads = 512;
 __global__ void __launch_bounds__(kPlanThreads)
-plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int clear_status, int* __restrict__ ws_header,
+plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict__ ws_header,
             psa_head_params* __restrict__ hp_dev, WorkItem* __restrict__ items) {
   extern __shared__ __align__(16) uint32_t sm[];  // key[NB rounded up to 4], cntT[Tp], cntS[Sp], setT[], setS[]
   pdl_trigger();
@@ -390,11 +401,7 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int clear_statu
   const psa_head_params p = hp.p[h];
   // The previous launch on this workspace may still be running; nothing is written before it has finished.
   pdl_wait();
-  // The scheduler ticket restarts with every launch; the status words are cleared only by the
-  // first launch of an API call, so that a timeout recorded by an earlier launch of the same call
-  // (a call may need several: more than 128 heads, chunks of a host-tensor call) survives.
-  if (h == 0 && threadIdx.x < kWsHeaderWords && (clear_status || (threadIdx.x != kWsStatus && threadIdx.x != kWsDetail)))
-    ws_header[threadIdx.x] = 0;
+  if (h == 0 && threadIdx.x == 0) ws_header[kWsCounter] = 0;   // the scheduler ticket restarts with every launch
   if (threadIdx.x == 0) hp_dev[h] = p;
   // attended differences, bit d + n - 1 for difference d
   const int wT = axis_words(g.Tp), wS = axis_words(g.Sp);
@@ -611,80 +618,99 @@ __device__ __forceinline__ long long row_token(const Geom& g, bool textq, int qb
   return (row < ntok && t < g.T && hh < g.H && ww < g.W) ? ((long long)t * g.H + hh) * g.W + ww : -1;
 }
 
-// Merge of a cluster's partial results (the softmax warpgroups of all its CTAs, between two cluster barriers): this CTA takes
-// every cluster_size-th part of the item's query rows, reads the (m, l, lr) and O of all CTAs -- and of both tiles when
-// the item is a single query slab whose even and odd key slabs were accumulated apart -- in a fixed order, and writes
-// out and lse.
-__device__ __forceinline__ void merge_cluster(const AttnParams& prm, uint8_t* smem, uint32_t sbase) {
+// Item i of a launch without planning (every item runs at once, so their order does not matter); its number of
+// attended key blocks is left to the load warp.
+__device__ __forceinline__ WorkItem direct_item(const Geom& g, int i) {
+  const int n_text_items = g.n_heads * g.n_titems;
+  if (i < n_text_items) {
+    const int head = i / g.n_titems, sub0 = 2 * (i % g.n_titems);
+    const int nq = (g.n_ts - sub0) >= 2 ? 2 : 1;
+    return make_int4(head, 0, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
+  }
+  i -= n_text_items;
+  const int per_head = g.NB * g.items_per_block;
+  const int head = i / per_head, r = i - head * per_head, sub0 = 2 * (r / g.NB);
+  const int nq = (g.n_sub - sub0) >= 2 ? 2 : 1;
+  return make_int4(head, r % g.NB, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
+}
+
+// Cluster mode: CTA d of the cluster merges query rows d * rpc .. (d + 1) * rpc - 1 of the item (rpc = nq * 128 /
+// cluster size), and every CTA pushes its partial results of those rows into d's shared memory: (m, l, lr) to
+// kOffQ [source][row], O as fp32 to kOffRing [source][32 groups of 4 columns][row].  Remote stores are posted; reading
+// the partial results from where they were computed took 5 to 9 us at 8 x 128 rows, against 2 for pushing them.
+struct Share {
+  uint32_t ml, o, step;   // shared::cluster addresses of this thread's row in the merging CTA, bytes between column groups
+};
+__device__ __forceinline__ Share share_of_row(uint32_t sbase, int r, int nq) {
+  const int rpc = nq * 128 / (int)cluster_size(), i = r & (rpc - 1);
+  const uint32_t d = (uint32_t)(r / rpc), src = cluster_rank();
+  return Share{map_rank(sbase + kOffQ + (src * (uint32_t)rpc + (uint32_t)i) * 16u, d),
+               map_rank(sbase + kOffRing + (src * 32u * (uint32_t)rpc + (uint32_t)i) * 16u, d), (uint32_t)rpc * 16u};
+}
+
+// The merge itself, by the softmax warpgroups, once all partial results have arrived: sums over the sources in a fixed
+// order, out and lse written.
+__device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8_t* smem) {
   const Geom& g = prm.g;
   const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);   // the item as the load warp published it
   if (wi.x < 0) return;                                               // (it gave up before that)
-  const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
-  const bool textq = ((wi.w >> 25) & 1) != 0;
-  const int csize = (int)cluster_size(), crank = (int)cluster_rank();
-  const int rpc = nq * 128 / csize;                  // rows of this CTA: 16, 32, 64 or 128
-  const int r0 = crank * rpc;                        // first of them, counted over the item's query slabs
-  const int tiles = nq == 1 ? 2 : 1, n_part = tiles * csize;
-  float* scale = reinterpret_cast<float*>(smem + kOffScale);   // [n_part][rpc]
+  const int head = wi.x, nq = (wi.w >> 16) & 0xff;
+  const int csize = (int)cluster_size();
+  constexpr int kMergeThreads = kThreads - 32 * kFirstSoftmaxWarp;
+  const int tid = (int)threadIdx.x - 32 * kFirstSoftmaxWarp;
+  const int rpc = nq * 128 / csize;    // 16, 32, 64 or 128
+  const int i = tid & (rpc - 1);       // this thread's row
+  const int tok = *reinterpret_cast<const int*>(smem + kOffRowTok + i * 4);
+  if (tok < 0) return;
   const float neg_inf = __int_as_float(0xff800000);
-  // tile and tile row of the item's row r, for partial result p
-  auto tile_of = [&](int r, int p) -> int { return nq == 1 ? (p & 1) : (r >> 7); };
-  auto rank_of = [&](int p) -> uint32_t { return (uint32_t)(nq == 1 ? p >> 1 : p); };
-  const int tid = (int)threadIdx.x - 32 * kFirstSoftmaxWarp, n_thr = kThreads - 32 * kFirstSoftmaxWarp;
-  for (int i = tid; i < rpc; i += n_thr) {
-    const int r = r0 + i;
-    float m_all = neg_inf, l_all = 0.f, lr_all = 0.f;
-    for (int p = 0; p < n_part; ++p) {
-      const float4 ml = ld_cluster_f4(map_rank(sbase + kOffQ + (uint32_t)(tile_of(r, p) * 128 + (r & 127)) * 16u, rank_of(p)));
-      scale[p * rpc + i] = ml.x;
-      const float m_new = fmaxf(m_all, ml.x);
-      const float wa = (m_all == neg_inf) ? 0.f : fast_exp2(m_all - m_new), wb = (ml.x == neg_inf) ? 0.f : fast_exp2(ml.x - m_new);
-      l_all = wa * l_all + wb * ml.y;
-      lr_all = wa * lr_all + wb * ml.z;
-      m_all = m_new;
-    }
-    const bool empty = !(l_all > 0.f);
-    const float inv = empty ? 0.f : 1.f / lr_all;
-    for (int p = 0; p < n_part; ++p) {
-      const float m = scale[p * rpc + i];
-      scale[p * rpc + i] = (m == neg_inf) ? 0.f : fast_exp2(m - m_all) * inv;
-    }
-    const long long tok = row_token(g, textq, qb, sub0 + (r >> 7), r & 127);
-    if (tok >= 0 && PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.Lt, 0xD15))
-      prm.lse[(long long)head * g.Lt + tok] = empty ? neg_inf : (m_all + log2f(l_all)) * 0.6931471805599453f;
+  const float4* ml = reinterpret_cast<const float4*>(smem + kOffQ) + i;
+  float m_all = neg_inf, l_all = 0.f, lr_all = 0.f;
+  for (int p = 0; p < csize; ++p) m_all = fmaxf(m_all, ml[p * rpc].x);
+  for (int p = 0; p < csize; ++p) {
+    const float4 v = ml[p * rpc];
+    const float w = (v.x == neg_inf) ? 0.f : fast_exp2(v.x - m_all);
+    l_all += w * v.y;
+    lr_all += w * v.z;
   }
-  asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32 * kFirstSoftmaxWarp) : "memory");
-  // units of one row and 8 columns, rows fastest: 16-byte reads of consecutive rows are contiguous
-  uint16_t* out = reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head;
-  for (int u = tid; u < rpc * 16; u += n_thr) {
-    const int i = u % rpc, cg = u / rpc, r = r0 + i;
-    const long long tok = row_token(g, textq, qb, sub0 + (r >> 7), r & 127);
-    if (tok < 0) continue;
+  const bool empty = !(l_all > 0.f);
+  const float inv = empty ? 0.f : 1.f / lr_all;
+  if (tid < rpc && PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.Lt, 0xD15))
+    prm.lse[(long long)head * g.Lt + tok] = empty ? neg_inf : (m_all + log2f(l_all)) * 0.6931471805599453f;
+  // units of 8 columns of the row; the lanes of a warp read consecutive rows
+  for (int cg = tid / rpc; cg < 16; cg += kMergeThreads / rpc) {
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float4* o = reinterpret_cast<const float4*>(smem + kOffRing) + 2 * cg * rpc + i;
 #pragma unroll 4
-    for (int p = 0; p < n_part; ++p) {
-      const float w = scale[p * rpc + i];
-      const uint32_t at = map_rank(sbase + kOffRing + (uint32_t)tile_of(r, p) * kPartBytes + (uint32_t)(2 * cg) * 2048u + (uint32_t)(r & 127) * 16u, rank_of(p));
-      const float4 a = ld_cluster_f4(at), b = ld_cluster_f4(at + 2048u);
-      if (w != 0.f) {
-        acc[0] = fmaf(w, a.x, acc[0]); acc[1] = fmaf(w, a.y, acc[1]); acc[2] = fmaf(w, a.z, acc[2]); acc[3] = fmaf(w, a.w, acc[3]);
-        acc[4] = fmaf(w, b.x, acc[4]); acc[5] = fmaf(w, b.y, acc[5]); acc[6] = fmaf(w, b.z, acc[6]); acc[7] = fmaf(w, b.w, acc[7]);
-      }
+    for (int p = 0; p < csize; ++p, o += 32 * rpc) {
+      const float m = ml[p * rpc].x;
+      if (m == neg_inf) continue;   // a share without keys left nothing behind
+      const float w = fast_exp2(m - m_all);
+      const float4 a = o[0], b = o[rpc];
+      acc[0] = fmaf(w, a.x, acc[0]); acc[1] = fmaf(w, a.y, acc[1]); acc[2] = fmaf(w, a.z, acc[2]); acc[3] = fmaf(w, a.w, acc[3]);
+      acc[4] = fmaf(w, b.x, acc[4]); acc[5] = fmaf(w, b.y, acc[5]); acc[6] = fmaf(w, b.z, acc[6]); acc[7] = fmaf(w, b.w, acc[7]);
     }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] *= inv;
     if (PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.Lt, 0xD16))
-      *reinterpret_cast<uint4*>(out + tok * prm.out_token + cg * 8) =
+      *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head + (long long)tok * prm.out_token + cg * 8) =
           make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
   }
 }
 
-// kCluster: a cluster of 2, 4 or 8 CTAs shares ONE work item (cluster i of the grid takes item i), each CTA taking
-// its share of the attended key blocks; the partial results are merged through distributed shared memory.  Otherwise
-// persistent CTAs draw whole items from the ticket.
-template <bool kCluster>
+// How a launch hands out its work items.
+//   kTicket   persistent CTAs draw planned items (heaviest first) from a ticket
+//   kDirect   CTA i runs item i: all items run at once, nothing is planned
+//   kShared   cluster i (2, 4 or 8 CTAs) runs planned item i, each CTA taking its share of the attended key blocks
+//   kSharedDirect   the same without planning
+// (Separate instantiations: the ticket kernel's slab loop is sensitive to what else is compiled with it -- one kernel
+// with the mode as an argument was 1.5 to 2 % slower on the 720p layers.)
+enum Mode { kTicket, kDirect, kShared, kSharedDirect };
+template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
-attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
+attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ HeadParamsArray heads, const AttnParams prm) {
   // 128-byte swizzled slabs need a 1024-byte aligned base; the declaration asks for it and the
   // kernel checks it (a misaligned base is reported through the status word, no work is done).
+  constexpr bool kCluster = kMode == kShared || kMode == kSharedDirect, kPlanned = kMode == kTicket || kMode == kShared;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
   const uint32_t sbase = smem_u32(smem);
@@ -700,9 +726,11 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
 
   // A short query slab leaves its last rows of the Q buffer unwritten; keep them finite.
-  for (uint32_t off = threadIdx.x * 16u; off < 2u * kSlabBytes; off += kThreads * 16u)
-    *reinterpret_cast<uint4*>(smem + kOffQ + off) = make_uint4(0u, 0u, 0u, 0u);
-  fence_async_smem();
+  if (kMode == kTicket || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
+    for (uint32_t off = threadIdx.x * 16u; off < 2u * kSlabBytes; off += kThreads * 16u)
+      *reinterpret_cast<uint4*>(smem + kOffQ + off) = make_uint4(0u, 0u, 0u, 0u);
+    fence_async_smem();
+  }
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int i = 0; i < 2; ++i) {
@@ -775,32 +803,35 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       ok = mbar_wait_warp(bar(kBarSchedEmpty + sslot), ((n >> 1) & 1u) ^ 1u, abort_flag, 0x401);
       if (!ok) break;
       WorkItem wi = make_int4(-1, 0, 0, 0);
-      int skip = 0;   // attended key blocks before this CTA's share
-      if (lane == 0) {
+      int skip = 0, left = 0x7fffffff;   // attended key blocks before this CTA's share, and those still to load
+      // This CTA's share of the item's attended key blocks; the text keys go with the last share.
+      auto take_share = [&]() {
         if constexpr (kCluster) {
-          if (n == 0) {
-            const int r = (int)cluster_rank(), c = (int)cluster_size();
-            wi = prm.items[blockIdx.x / (uint32_t)c];
-            skip = (int)((long long)wi.z * r / c);
-            wi.z = (int)((long long)wi.z * (r + 1) / c) - skip;
-            if (r + 1 < c) wi.w |= 1 << 26;   // the text keys go with the last share
-          }
-        } else {
-          const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
-          if (ticket < prm.n_items) wi = prm.items[ticket];
+          const int r = (int)cluster_rank(), c = (int)cluster_size();
+          skip = (int)((long long)wi.z * r / c);
+          left = wi.z = (int)((long long)wi.z * (r + 1) / c) - skip;
+          if (r + 1 < c) wi.w |= 1 << 26;
         }
+      };
+      auto publish = [&]() {   // by lane 0
         sched[sslot].x = wi.x; sched[sslot].y = wi.y; sched[sslot].z = wi.z; sched[sslot].w = wi.w;
         mbar_arrive(bar(kBarSchedFull + sslot));
+      };
+      if constexpr (kMode == kTicket) {
+        if (lane == 0) {
+          const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
+          if (ticket < prm.n_items) wi = prm.items[ticket];
+          publish();
+        }
+        wi.x = __shfl_sync(0xffffffffu, wi.x, 0);
+        wi.y = __shfl_sync(0xffffffffu, wi.y, 0);
+        wi.w = __shfl_sync(0xffffffffu, wi.w, 0);
+      } else {
+        if (n == 0) wi = kPlanned ? prm.items[blockIdx.x / cluster_size()] : direct_item(g, (int)(blockIdx.x / cluster_size()));
+        if constexpr (kPlanned) take_share();
+        if (lane == 0 && (kPlanned || n > 0)) publish();
       }
-      wi.x = __shfl_sync(0xffffffffu, wi.x, 0);
-      wi.y = __shfl_sync(0xffffffffu, wi.y, 0);
-      wi.w = __shfl_sync(0xffffffffu, wi.w, 0);
       if (wi.x < 0) break;
-      int left = 0x7fffffff;   // attended key blocks still to load
-      if constexpr (kCluster) {
-        skip = __shfl_sync(0xffffffffu, skip, 0);
-        left = __shfl_sync(0xffffffffu, wi.z, 0);
-      }
       const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
       if (!PSA_CHECKED(head < g.n_heads && qb >= 0 && qb <= g.NB && nq >= 1 && nq <= 2 &&
                        sub0 + nq <= ((wi.w >> 25) & 1 ? g.n_ts : g.n_sub), 0xD04)) {
@@ -811,20 +842,32 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       const int lag = ((wi.w >> 24) & 1) ? 2 : 1;   // V_j travels with K_{j+lag} (2 in split-KV mode)
       const bool textq = ((wi.w >> 25) & 1) != 0;   // the queries are text tokens: every key is attended
       const int head_ld = prm.shared_qkv ? 0 : head;   // head coordinate of the q, k, v loads
-      const psa_head_params p = prm.hp_dev[head];
-      const int tq = qb / g.Sp, sq = qb % g.Sp;
-      // attended key-block coordinates of this query block, one bit per block coordinate
-      for (int b = 0; b < g.Tp; b += 32) {
-        const int tk = b + lane;
-        const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
-        if (lane == 0) maskT[b >> 5] = m;
-      }
-      for (int b = 0; b < g.Sp; b += 32) {
-        const int sk = b + lane;
-        const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
-        if (lane == 0) maskS[b >> 5] = m;
-      }
-      __syncwarp();
+      auto eval_masks = [&]() {
+        const psa_head_params p = kPlanned ? prm.hp_dev[head] : heads.p[head];
+        const int tq = qb / g.Sp, sq = qb % g.Sp;
+        int cnt_t = 0, cnt_s = 0;
+        // attended key-block coordinates of this query block, one bit per block coordinate
+        for (int b = 0; b < g.Tp; b += 32) {
+          const int tk = b + lane;
+          const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
+          if (lane == 0) maskT[b >> 5] = m;
+          cnt_t += __popc(m);
+        }
+        for (int b = 0; b < g.Sp; b += 32) {
+          const int sk = b + lane;
+          const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
+          if (lane == 0) maskS[b >> 5] = m;
+          cnt_s += __popc(m);
+        }
+        __syncwarp();
+        if constexpr (!kPlanned) {   // the item is complete only now
+          wi.z = cnt_t * cnt_s;
+          take_share();
+          if (lane == 0) publish();
+        }
+      };
+      // (a CTA that only starts up loads the queries first)
+      if constexpr (kMode == kTicket) eval_masks();
       // query slabs
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -852,6 +895,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
         if (i == 0) ++it_q0; else ++it_q1;
       }
       if (!ok) break;
+      if constexpr (kMode != kTicket) eval_masks();
       // key / value slabs in ascending key-block id.  Up to `lag` slabs wait for their V load.
       int npend = 0;
       int at0 = 0, ah0 = 0, aw0 = 0, alast = 0, antok = kSlabTokens;  // oldest pending slab
@@ -1227,7 +1271,20 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       }
     }
     __syncwarp();
+  } else if constexpr (kCluster) {
+    // ======================================================================= idle warps: tokens of the rows to merge
+    // (the divisions take a microsecond, which the merge need not wait for)
+    if (tmem_ok && mbar_wait_warp(bar(kBarSchedFull), 0u, abort_flag, 0x402)) {
+      const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);
+      const int nq = (wi.w >> 16) & 0xff, rpc = nq * 128 / (int)cluster_size(), r0 = (int)cluster_rank() * rpc;
+      if (wi.x >= 0)
+        for (int i = (int)threadIdx.x - 64; i < rpc; i += 64)
+          *reinterpret_cast<int*>(smem + kOffRowTok + (uint32_t)i * 4u) =
+              (int)row_token(g, ((wi.w >> 25) & 1) != 0, wi.y, (wi.w & 0xffff) + ((r0 + i) >> 7), (r0 + i) & 127);
+    }
+    __syncwarp();
   }
+  if constexpr (kCluster) cluster_sync_all();   // the barrier that the softmax warps meet at before they push
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
     // ======================================================================= softmax warps
@@ -1239,7 +1296,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
     uint32_t it_o0 = 0, it_o1 = 0, cnt_s = 0, kv_g = 0;
     uint32_t n_stage = 0;   // output slabs staged by this warpgroup so far
     uint32_t n_merge = 0;   // split-KV merges so far
-    bool ok = true;
+    bool ok = true, met = false;   // met: cluster mode's first barrier passed
     const float neg_inf = __int_as_float(0xff800000);
     float2* xchg = reinterpret_cast<float2*>(smem + kOffXchg);
 
@@ -1286,9 +1343,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       ++it_o0;
       if (use_o1) ++it_o1;
       if constexpr (kCluster) {
-        // Leave this tile's partial result in shared memory for the merge after the roles have met: (m, l, lr) of each row
-        // in the Q buffers, O as fp32 [32 column groups of 4][128 rows] in the K/V ring -- both idle once every MMA
-        // of the CTA has completed.  A tile without keys is marked by m = -inf; what is read as its O gets weight 0.
+        // Push this CTA's partial results to the CTAs that merge them.  The receiving Q buffers and K/V ring are idle
+        // once every MMA of the cluster has completed: the first cluster barrier.  A share without keys is marked by
+        // m = -inf.  The two tiles of a single query slab (even / odd key slabs) are merged here first: each warpgroup
+        // takes 64 columns of both.
         ok = mbar_wait_warp(bar(kBarOFull + 0), par_o0, abort_flag, 0x310);
         if (!ok) break;
         if (use_o1) {
@@ -1296,22 +1354,53 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
           if (!ok) break;
         }
         const bool has = active && n_kv > 0;
-        *reinterpret_cast<float4*>(smem + kOffQ + (uint32_t)(qi * 128 + row) * 16u) =
-            has ? make_float4(m_ref, l, lr, 0.f) : make_float4(neg_inf, 0.f, 0.f, 0.f);
-        if (has) {
-          tc_fence_after();
-          uint8_t* part = smem + kOffRing + (uint32_t)qi * kPartBytes + (uint32_t)row * 16u;
+        cluster_sync_all();
+        met = true;
+        tc_fence_after();
+        const float4 mine = has ? make_float4(m_ref, l, lr, 0.f) : make_float4(neg_inf, 0.f, 0.f, 0.f);
+        if (split) {
+          float4* tmp = reinterpret_cast<float4*>(smem + kOffPartTmp) + row;   // [2][128]
+          tmp[qi * 128] = mine;
+          mbar_arrive(bar(kBarStage + qi));
+          ok = mbar_wait_warp(bar(kBarStage + (qi ^ 1)), 0u, abort_flag, 0x313);
+          if (!ok) break;
+          const float4 a = tmp[0], b = tmp[128];
+          const float m_all = fmaxf(a.x, b.x);
+          const float wa = (a.x == neg_inf) ? 0.f : fast_exp2(a.x - m_all), wb = (b.x == neg_inf) ? 0.f : fast_exp2(b.x - m_all);
+          const Share sh = share_of_row(sbase, row, 1);
+          if (qi == 0) st_cluster_f4(sh.ml, make_float4(m_all, wa * a.y + wb * b.y, wa * a.z + wb * b.z, 0.f));
+          const uint32_t tO0 = tmem + lane_addr + 256u;
+          if (n_kv > 0) {
 #pragma unroll 1
-          for (int c4 = 0; c4 < 4; ++c4) {
-            uint32_t o[32];
-            tc_ld32(tO + c4 * 32, o);
-            tc_wait_ld();
+            for (int c4 = 2 * qi; c4 < 2 * qi + 2; ++c4) {
+              uint32_t o[32], o1[32];
+              tc_ld32(tO0 + c4 * 32, o);
+              tc_ld32(tO0 + 128u + c4 * 32, o1);
+              tc_wait_ld();
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-              *reinterpret_cast<uint4*>(part + (uint32_t)(c4 * 8 + e) * 2048u) = make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+              for (int c = 0; c < 32; ++c)   // (an accumulator without keys holds left-overs)
+                o[c] = __float_as_uint((wa != 0.f ? wa * __uint_as_float(o[c]) : 0.f) + (wb != 0.f ? wb * __uint_as_float(o1[c]) : 0.f));
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                st_cluster_u4(sh.o + (uint32_t)(c4 * 8 + e) * sh.step, o + 4 * e);
+            }
           }
-          tc_fence_before();
+        } else {
+          const Share sh = share_of_row(sbase, qi * 128 + row, 2);
+          st_cluster_f4(sh.ml, mine);
+          if (n_kv > 0) {
+#pragma unroll 1
+            for (int c4 = 0; c4 < 4; ++c4) {
+              uint32_t o[32];
+              tc_ld32(tO + c4 * 32, o);
+              tc_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                st_cluster_u4(sh.o + (uint32_t)(c4 * 8 + e) * sh.step, o + 4 * e);
+            }
+          }
         }
+        tc_fence_before();
         continue;
       }
       if (!active) continue;
@@ -1426,19 +1515,22 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
       }
       ++n_stage;
     }
-    if ((warp & 3) == 0 && lane == 0) tma_store_wait_all();
+    if constexpr (kCluster) {
+      if (!met) cluster_sync_all();
+    } else {
+      if ((warp & 3) == 0 && lane == 0) tma_store_wait_all();
+    }
   }
 
   // ------------------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
   if constexpr (kCluster) {
-    cluster_sync_all();   // every CTA's partial results are in place
-    if (warp >= kFirstSoftmaxWarp) merge_cluster(prm, smem, sbase);   // (the first warpgroup gave its registers away)
-    cluster_sync_all();   // nobody's shared memory is read any more
+    cluster_sync_all();   // every partial result has arrived; no CTA writes into another one any more
+    if (warp >= kFirstSoftmaxWarp) merge_cluster(prm, smem);   // (the first warpgroup gave its registers away)
   }
   if (threadIdx.x == 0 && *abort_flag != 0) {
-    if (atomicCAS(prm.ws_header + kWsStatus, 0, (int)PSA_ERR_TIMEOUT) == 0) prm.ws_header[kWsDetail] = *abort_flag;
+    report_status(prm.ws_header, prm.call_id, PSA_ERR_TIMEOUT, *abort_flag);
   }
   if (warp == kWarpMma) {
     tc_fence_after();
@@ -1448,7 +1540,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const AttnParams prm) {
 
 // One warp waits, with the kernel's own bounded wait, on a barrier that nothing arrives on.
 // The wait must give up after limit_ns, record PSA_ERR_TIMEOUT and return normally.
-__global__ void wait_probe_kernel(int* ws_header, unsigned long long limit_ns) {
+__global__ void wait_probe_kernel(int* ws_header, int call_id, unsigned long long limit_ns) {
   __shared__ __align__(8) unsigned long long probe_bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -1459,13 +1551,11 @@ __global__ void wait_probe_kernel(int* ws_header, unsigned long long limit_ns) {
   __syncwarp();
   const bool ok = mbar_wait(smem_u32(&probe_bar), 0, &abort_flag, 0x7e57, limit_ns);
   __syncwarp();
-  if (threadIdx.x == 0 && !ok) {
-    if (atomicCAS(ws_header + kWsStatus, 0, (int)PSA_ERR_TIMEOUT) == 0) ws_header[kWsDetail] = abort_flag;
-  }
+  if (threadIdx.x == 0 && !ok) report_status(ws_header, call_id, PSA_ERR_TIMEOUT, abort_flag);
 }
 
-cudaError_t launch_wait_probe(int* ws_header, unsigned long long limit_ns, cudaStream_t stream) {
-  wait_probe_kernel<<<1, 32, 0, stream>>>(ws_header, limit_ns);
+cudaError_t launch_wait_probe(int* ws_header, int call_id, unsigned long long limit_ns, cudaStream_t stream) {
+  wait_probe_kernel<<<1, 32, 0, stream>>>(ws_header, call_id, limit_ns);
   return cudaGetLastError();
 }
 
@@ -1497,37 +1587,42 @@ struct LaunchConfig {
 
 // Once per device: shared-memory limits, and how many clusters of 2, 4 and 8 CTAs run at a time.
 cudaError_t attn_init(int clusters[3]) {
-  cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attn_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc);
-  if (e != cudaSuccess) return e;
+  const void* kernels[] = {(const void*)attn_fwd_kernel<kTicket>, (const void*)attn_fwd_kernel<kDirect>,
+                           (const void*)attn_fwd_kernel<kShared>, (const void*)attn_fwd_kernel<kSharedDirect>};
+  cudaError_t e = cudaSuccess;
+  for (const void* k : kernels)
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc)) != cudaSuccess) return e;
   for (int i = 0; i < 3; ++i) {
     LaunchConfig lc(2 << i, kThreads, kSmemAlloc, nullptr, 2 << i);
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters[i], attn_fwd_kernel<true>, &lc.cfg)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveClusters(&clusters[i], attn_fwd_kernel<kSharedDirect>, &lc.cfg)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, bool clear_status,
-                        int* ws_header, psa_head_params* hp_dev, WorkItem* items, cudaStream_t stream) {
+cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header,
+                        psa_head_params* hp_dev, WorkItem* items, cudaStream_t stream) {
   const size_t smem = plan_smem_bytes(g);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   LaunchConfig lc(n_heads_here, kPlanThreads, smem, stream, 1);
-  return cudaLaunchKernelEx(&lc.cfg, plan_kernel, hp, g, clear_status ? 1 : 0, ws_header, hp_dev, items);
+  return cudaLaunchKernelEx(&lc.cfg, plan_kernel, hp, g, ws_header, hp_dev, items);
 }
 
 // cluster: CTAs per work item (1: persistent CTAs, whole items)
-cudaError_t launch_attn(const TensorMaps& tm, const AttnParams& prm, int n_sms, int cluster, cudaStream_t stream) {
+// heads: read by launches without planning only.  cluster: CTAs per work item, 1: whole items.  direct: all items run
+// at once, nothing was planned.
+cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster, bool direct,
+                        cudaStream_t stream) {
   if (prm.n_items <= 0) return cudaSuccess;
-  if (cluster > 1) {
-    LaunchConfig lc(prm.n_items * cluster, kThreads, kSmemAlloc, stream, cluster);
-    return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<true>, tm, prm);
-  }
-  LaunchConfig lc(prm.n_items < n_sms ? prm.n_items : n_sms, kThreads, kSmemAlloc, stream, 1);
-  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<false>, tm, prm);
+  const int ctas = cluster > 1 || direct ? prm.n_items * cluster : (prm.n_items < n_sms ? prm.n_items : n_sms);
+  LaunchConfig lc(ctas, kThreads, kSmemAlloc, stream, cluster);
+  if (cluster > 1)
+    return direct ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kSharedDirect>, tm, heads, prm)
+                  : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kShared>, tm, heads, prm);
+  return direct ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kDirect>, tm, heads, prm)
+                : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicket>, tm, heads, prm);
 }
 
 }  // namespace psa

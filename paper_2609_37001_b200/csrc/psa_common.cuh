@@ -65,14 +65,16 @@ struct AttnParams {
   int* ws_header;
   float* lse;
   int n_items;
+  int call_id;      // id of the API call, for the status words
   int shared_qkv;   // 1: every head reads head 0 of q, k, v (candidate masks of one head, PSA-Search)
   void* out;        // for rows that are stored without TMA; strides in elements
   long long out_head, out_token;
 };
 
 // Layout of the per-device workspace (all int32 words).
-constexpr int kWsStatus = 0;     // first device-side error (0 = none)
+constexpr int kWsStatus = 0;     // first device-side error of call kWsCallId
 constexpr int kWsDetail = 1;     // diagnostic of that error
+constexpr int kWsCallId = 3;     // API call that reported an error last (0 = none yet)
 constexpr int kWsCounter = 2;    // dynamic scheduler ticket
 constexpr int kWsHeaderWords = 16;
 

@@ -18,13 +18,14 @@ cudaError_t launch_mask_build(const HeadParamsArray& hp, const AxisSet* sets, co
                               uint8_t* block_mask, int* row_ptr, int* col_idx, int total_nnz_through_chunk,
                               int n_sms, cudaStream_t stream, int* launches);
 cudaError_t attn_init(int clusters[3]);
-cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, bool clear_status, int* ws_header,
-                        psa_head_params* hp_dev, WorkItem* items, cudaStream_t stream);
-cudaError_t launch_attn(const TensorMaps& tm, const AttnParams& prm, int n_sms, int cluster, cudaStream_t stream);
+cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
+                        WorkItem* items, cudaStream_t stream);
+cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster,
+                        bool direct, cudaStream_t stream);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
                                  float* losses, cudaStream_t stream, int* launches);
-cudaError_t launch_wait_probe(int* ws_header, unsigned long long limit_ns, cudaStream_t stream);
+cudaError_t launch_wait_probe(int* ws_header, int call_id, unsigned long long limit_ns, cudaStream_t stream);
 }  // namespace psa
 
 namespace {
@@ -40,10 +41,21 @@ struct Workspace {
   size_t bytes = 0;
   int n_sms = 0;
   int cc_major = 0;
+  int last_call = 0;             // id of the last API call whose kernels report to the status words
   bool attn_ready = false;
   int clusters[3] = {0, 0, 0};   // clusters of 2, 4 and 8 attention CTAs that run at a time
 };
 Workspace g_ws[kMaxDevices];
+
+// Id of a new API call on `stream` (g_mu held).  Never 0, which is what untouched status words hold.  A call that is
+// being captured has kCapturedCall set: its kernels run again whenever the graph is replayed.
+constexpr int kCapturedCall = 1 << 30;
+int g_calls = 0;
+int next_call_id(cudaStream_t stream) {
+  g_calls = g_calls + 1 == kCapturedCall ? 1 : g_calls + 1;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive ? g_calls | kCapturedCall : g_calls;
+}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -61,6 +73,21 @@ int load_driver_entry() {
   }
   g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   return PSA_OK;
+}
+
+// What call `call_id`, or a replay of a captured call, reported in the status words at `header` (its work has finished);
+// what a replay reported is cleared.
+int read_status(void* header, int call_id, int32_t* detail) {
+  int hdr[4] = {0, 0, 0, 0};
+  if (cudaMemcpy(hdr, header, sizeof(hdr), cudaMemcpyDeviceToHost) != cudaSuccess) return PSA_ERR_CUDA;
+  const int from = hdr[kWsCallId];
+  const bool mine = from != 0 && (from == call_id || (from & kCapturedCall));
+  if (detail) *detail = mine ? hdr[kWsDetail] : 0;
+  if (!mine) return PSA_OK;
+  const int zero = 0;
+  if ((from & kCapturedCall) && cudaMemcpy(static_cast<int*>(header) + kWsCallId, &zero, sizeof(zero), cudaMemcpyHostToDevice) != cudaSuccess)
+    return PSA_ERR_CUDA;
+  return hdr[kWsStatus];
 }
 
 bool valid_params(const psa_head_params& p) {
@@ -266,15 +293,12 @@ int encode_maps(TensorMaps* tm, const void* q, const void* k, const void* v, voi
   return PSA_OK;
 }
 
-// Attended block pairs of every head; returns their sum.
-long long head_weights(const psa_head_params* params, int n, const Geom& g, long long* w) {
-  long long total = 0;
+// Attended block pairs of every head.
+void head_weights(const psa_head_params* params, int n, const Geom& g, long long* w) {
   for (int h = 0; h < n; ++h) {
     // (the samples of a batch or the heads of a group often repeat the parameters of the head before)
     w[h] = h > 0 && std::memcmp(&params[h], &params[h - 1], sizeof(psa_head_params)) == 0 ? w[h - 1] : head_nnz(params[h], g);
-    total += w[h];
   }
-  return total;
 }
 
 // Planning arguments of one launch: the heads' parameters and their places in the work order, heavier heads first.
@@ -289,28 +313,65 @@ void plan_params(PlanParams* pp, const psa_head_params* params, const long long*
 
 // CTAs that share a work item: 1 (persistent CTAs that draw whole items), 2, 4 or 8.  A launch takes about as many
 // rounds as its items need on the SMs, so a problem of few items, or of a few more than a whole number of rounds,
-// leaves SMs idle; sharing items makes the rounds shorter.  Times in clocks, measured: a key slab takes 3,300 for two
-// query slabs and 1,900 for one (split-KV mode), an item 9,000 beside its slabs in a persistent CTA and 18,000 in a
-// cluster (which starts its CTAs anew and merges).
-// Decided for a call as a whole (`pairs` of all its heads), so that the chunks of a host-tensor call compute what the
-// device call computes, bit for bit.
-int share_items(const Workspace& ws, const Geom& g, long long pairs, int n_heads) {
+// leaves SMs idle; sharing items makes the rounds shorter.  Clocks, from time stamps in the kernel: a key slab takes
+// 3,300 for two query slabs and 1,900 for one (split-KV mode); start-up, epilogue and exit take 15,000 in a persistent
+// CTA and 21,000 in a cluster (which also merges).
+// Decided for a call as a whole, so that the chunks of a host-tensor call compute what the device call computes, bit
+// for bit.  weights: attended block pairs of every head.
+int share_items(const Workspace& ws, const Geom& g, const long long* weights, int n_heads) {
   const int n_items = (n_heads < kMaxHeads ? n_heads : kMaxHeads) * g.items_per_head;   // of one launch
   if (n_items > 2 * ws.n_sms) return 1;   // (beyond two rounds at most a third is to be gained)
-  const double blocks = (double)pairs / ((double)n_heads * g.NB);   // attended by the average query block
-  const int singles = g.n_sub & 1, pairs_per_block = g.n_sub >> 1;
-  const double slabs = blocks * g.n_sub + g.n_ts;
-  const double item = slabs * (3300.0 * pairs_per_block + 1900.0 * singles) / (pairs_per_block + singles);
-  auto rounds = [](int items, int at_a_time) -> double { return (double)((items + at_a_time - 1) / at_a_time); };
-  double best = rounds(n_items, ws.n_sms) * (item + 9000.0);
+  long long total = 0, most = 0;
+  for (int h = 0; h < n_heads; ++h) {
+    total += weights[h];
+    if (weights[h] > most) most = weights[h];
+  }
+  // blocks attended by the average query block, of all heads and of the heaviest
+  const double avg = (double)total / ((double)n_heads * g.NB), heavy = (double)most / g.NB;
+  const int singles = g.n_sub & 1, doubles = g.n_sub >> 1;
+  const double per_slab = (3300.0 * doubles + 1900.0 * singles) / (doubles + singles);
+  auto time = [&](int at_a_time, int c, double fixed) -> double {
+    if (n_items <= at_a_time) return (heavy * g.n_sub + g.n_ts) * per_slab / c + fixed;   // one round: the longest item
+    return (double)((n_items + at_a_time - 1) / at_a_time) * ((avg * g.n_sub + g.n_ts) * per_slab / c + fixed);
+  };
+  double best = time(ws.n_sms, 1, 15000.0);
   int cluster = 1;
   for (int i = 0; i < 3; ++i) {
     const int c = 2 << i;
-    if (ws.clusters[i] < 1 || blocks < c) break;   // a share holds at least one block
-    const double t = rounds(n_items, ws.clusters[i]) * (item / c + 18000.0);
-    if (t < 0.9 * best) { best = t; cluster = c; }
+    if (ws.clusters[i] < 1 || heavy < c) break;   // a share of a heavy item holds at least one block
+    const double t = time(ws.clusters[i], c, 21000.0);
+    if (t < 0.95 * best) { best = t; cluster = c; }
   }
   return cluster;
+}
+
+// Whether every item of a launch runs at the same time.  Then their order does not matter and no planning is needed:
+// one kernel instead of two (a 2,048-token call is bound by such latencies).
+bool runs_at_once(const Workspace& ws, int n_items, int cluster) {
+  const int at_once = cluster == 1 ? ws.n_sms : ws.clusters[cluster == 2 ? 0 : (cluster == 4 ? 1 : 2)];
+  return n_items <= at_once;
+}
+
+// Planning (unless the launch is direct) and attention.
+cudaError_t launch_call(const TensorMaps& tm, const AttnParams& prm, const psa_head_params* params, const long long* weights,
+                        const Workspace& ws, int cluster, bool record, cudaStream_t st) {
+  HeadParamsArray heads;   // entries beyond the launch's heads are never read, nor any of a planned launch
+  const int n = prm.g.n_heads;
+  const bool direct = runs_at_once(ws, prm.n_items, cluster);
+  if (direct) {
+    std::memcpy(heads.p, params, sizeof(psa_head_params) * (size_t)n);
+  } else {
+    PlanParams pp;
+    plan_params(&pp, params, weights, n);
+    const cudaError_t e = launch_plan(pp, prm.g, n, prm.ws_header, const_cast<psa_head_params*>(prm.hp_dev),
+                                      const_cast<WorkItem*>(prm.items), st);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+  }
+  if (record && g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
+  const cudaError_t e = launch_attn(tm, heads, prm, ws.n_sms, cluster, direct, st);
+  if (e == cudaSuccess) ++g_launches;
+  return e;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -340,7 +401,7 @@ HostPipe* host_pipe(int dev) {   // caller holds g_mu; returns nullptr if the st
 }
 
 // ---- scratch of psa_attn_fwd_noalloc ------------------------------------------------------
-// Layout: 16 int32 header words (status, detail, scheduler ticket), kMaxHeads head parameter
+// Layout: 16 int32 header words (status, detail, scheduler ticket, reporting call), kMaxHeads head parameter
 // records, then up to kNoAllocMaxItems work items.  It lives in every GPU that loads the
 // library, from load to exit.
 constexpr int kNoAllocMaxItems = 16384;
@@ -462,10 +523,11 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T
 
 // Planning + attention launches for n_heads heads (in launches of at most kMaxHeads) on the cached
 // per-device workspace.  Arguments are already validated; g_mu is held by the caller.
-// clear_status: this is the first launch sequence of an API call (later ones keep the status word).
+// new_call: this is the first launch sequence of an API call (later ones report under the same id, so that an error of
+// an earlier one -- more than 128 heads, chunks of a host-tensor call, samples of a batched call -- is not lost).
 // cluster: CTAs per work item, 0: by share_items for these heads.
 static int run_attn(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
-                    int n_heads, const Geom& g, const Layout& lay, cudaStream_t st, bool clear_status = true, int cluster = 0) {
+                    int n_heads, const Geom& g, const Layout& lay, cudaStream_t st, bool new_call = true, int cluster = 0) {
   int dev;
   Workspace* ws;
   int rc = device_info(&dev, &ws);
@@ -482,8 +544,9 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
   psa_head_params* hp_dev = reinterpret_cast<psa_head_params*>(static_cast<char*>(ws->base) + hp_off);
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(ws->base) + items_off);
   std::vector<long long> weights((size_t)n_heads);
-  const long long pairs = head_weights(head_params, n_heads, g, weights.data());
-  if (cluster == 0) cluster = share_items(*ws, g, pairs, n_heads);
+  head_weights(head_params, n_heads, g, weights.data());
+  if (cluster == 0) cluster = share_items(*ws, g, weights.data(), n_heads);
+  if (new_call) ws->last_call = next_call_id(st);
   for (int head0 = 0; head0 < n_heads; head0 += kMaxHeads) {
     const int n_here = n_heads - head0 < kMaxHeads ? n_heads - head0 : kMaxHeads;
     const long long in_off = lay.shared_qkv ? 0 : (long long)head0 * lay.in_head;
@@ -494,26 +557,19 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
       return rc;
     Geom gh = g;
     gh.n_heads = n_here;
-    PlanParams pp;
-    plan_params(&pp, head_params + head0, weights.data() + head0, n_here);
-    if (launch_plan(pp, gh, n_here, clear_status && head0 == 0, ws_header, hp_dev, items, st) != cudaSuccess)
-      return PSA_ERR_CUDA;
-    ++g_launches;
     const int n_items = n_here * g.items_per_head;
-    if (g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
-    const AttnParams prm = {gh, items, hp_dev, ws_header, lse + (long long)head0 * g.Lt, n_items, lay.shared_qkv ? 1 : 0,
-                            static_cast<uint16_t*>(out) + out_off, lay.out_head, lay.out_token};
-    if (launch_attn(tm, prm, ws->n_sms, cluster, st) != cudaSuccess) return PSA_ERR_CUDA;
+    const AttnParams prm = {gh, items, hp_dev, ws_header, lse + (long long)head0 * g.Lt, n_items,
+                            ws->last_call, lay.shared_qkv ? 1 : 0, static_cast<uint16_t*>(out) + out_off, lay.out_head, lay.out_token};
+    if (launch_call(tm, prm, head_params + head0, weights.data() + head0, *ws, cluster, true, st) != cudaSuccess) return PSA_ERR_CUDA;
     if (g_ev_start && g_ev_stop) cudaEventRecord(g_ev_stop, st);
-    ++g_launches;
   }
   return PSA_OK;
 }
 
-// psa_attn_fwd with the choice of keeping the status word and of the CTAs per item (chunks of one host-tensor call).
+// psa_attn_fwd with the choice of continuing an API call and of the CTAs per item (chunks of one host-tensor call).
 static int attn_fwd_checked(const void* q, const void* k, const void* v, void* out, float* lse,
                             const psa_head_params* head_params, const psa_problem* prob, int T, int H, int W, void* stream,
-                            bool clear_status, int cluster = 0) {
+                            bool new_call, int cluster = 0) {
   Geom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
@@ -527,7 +583,7 @@ static int attn_fwd_checked(const void* q, const void* k, const void* v, void* o
     if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lock(g_mu);
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
-  return run_attn(q, k, v, out, lse, head_params, prob->n_heads, g, lay, static_cast<cudaStream_t>(stream), clear_status, cluster);
+  return run_attn(q, k, v, out, lse, head_params, prob->n_heads, g, lay, static_cast<cudaStream_t>(stream), new_call, cluster);
 }
 
 int psa_attn_fwd(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
@@ -638,7 +694,9 @@ int psa_search_losses(const void* q, const void* k, const void* v, const psa_hea
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::lock_guard<std::mutex> lock(g_mu);
   const Layout lay = {0, prob->stride_token, g.L * kHeadDim, kHeadDim, true};
-  rc = run_attn(q, k, v, outs, lse, params.data(), n_cand + 1, g, lay, st);
+  // whole items: with n_cand + 1 of them per block they are rarely few, and every candidate's output is then rounded as
+  // a plain call's is (the losses are differences of outputs)
+  rc = run_attn(q, k, v, outs, lse, params.data(), n_cand + 1, g, lay, st, true, 1);
   if (rc != PSA_OK) return rc;
   int launches = 0;
   const cudaError_t e = launch_search_losses(outs, outs + (long long)n_cand * g.L * kHeadDim, g.L * kHeadDim, n_cand, partial,
@@ -700,24 +758,16 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   TensorMaps tm;
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
   if ((rc = encode_maps(&tm, q, k, v, out, g, lay, prob->n_heads)) != PSA_OK) return rc;
-  // The planning kernel clears the header words (status, ticket) and rewrites the parameter
-  // records and every work item of this call, so nothing of the previous call is read.
-  PlanParams pp;
+  // What the kernels read of the scratch is written by this call's planning kernel; nothing of the previous call is read.
   long long weights[kMaxHeads];
-  const long long pairs = head_weights(head_params, prob->n_heads, g, weights);
-  plan_params(&pp, head_params, weights, prob->n_heads);
-  if (launch_plan(pp, g, prob->n_heads, true, header, hp_dev, items, st) != cudaSuccess) return PSA_ERR_CUDA;
-  ++g_launches;
-  const int n_items = (int)n_items_ll;
-  const AttnParams prm = {g, items, hp_dev, header, lse, n_items, 0, out, lay.out_head, lay.out_token};
-  if (launch_attn(tm, prm, ws->n_sms, share_items(*ws, g, pairs, prob->n_heads), st) != cudaSuccess) return PSA_ERR_CUDA;
-  ++g_launches;
+  head_weights(head_params, prob->n_heads, g, weights);
+  const int cluster = share_items(*ws, g, weights, prob->n_heads), n_items = (int)n_items_ll, call_id = next_call_id(st);
+  const AttnParams prm = {g, items, hp_dev, header, lse, n_items, call_id, 0,
+                          out, lay.out_head, lay.out_token};
+  if (launch_call(tm, prm, head_params, weights, *ws, cluster, false, st) != cudaSuccess) return PSA_ERR_CUDA;
   if (status_detail) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return PSA_ERR_CUDA;
-    int hdr[2] = {0, 0};
-    if (cudaMemcpy(hdr, header, sizeof(hdr), cudaMemcpyDeviceToHost) != cudaSuccess) return PSA_ERR_CUDA;
-    *status_detail = hdr[1];
-    return hdr[0];
+    return read_status(header, call_id, status_detail);
   }
   return PSA_OK;
 }
@@ -781,13 +831,13 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
   for (int h = 0; h < prob->n_heads; ++h)
     if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
   std::vector<long long> weights((size_t)prob->n_heads);
-  const long long pairs = head_weights(head_params, prob->n_heads, g, weights.data());
+  head_weights(head_params, prob->n_heads, g, weights.data());
   int cluster;
   {
     std::lock_guard<std::mutex> lock(g_mu);
     Workspace* ws;
     if ((rc = device_info(&dev, &ws)) != PSA_OK || (rc = init_attn(ws)) != PSA_OK) return rc;
-    cluster = share_items(*ws, g, pairs, prob->n_heads);
+    cluster = share_items(*ws, g, weights.data(), prob->n_heads);
   }
   if (n_edge) {
     for (int h = 0; h < prob->n_heads; ++h) {
@@ -853,8 +903,8 @@ int psa_selftest_wait_timeout(int limit_ms, void* stream) {
   rc = ensure_workspace(ws, 4096);
   if (rc != PSA_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ws->base, 0, sizeof(int) * kWsHeaderWords, st) != cudaSuccess) return PSA_ERR_CUDA;
-  if (launch_wait_probe(static_cast<int*>(ws->base), 1000000ull * (unsigned long long)limit_ms, st) != cudaSuccess)
+  ws->last_call = next_call_id(st);
+  if (launch_wait_probe(static_cast<int*>(ws->base), ws->last_call, 1000000ull * (unsigned long long)limit_ms, st) != cudaSuccess)
     return PSA_ERR_CUDA;
   ++g_launches;
   return PSA_OK;
@@ -869,10 +919,7 @@ int psa_last_device_status(int32_t* detail) {
   if (cudaDeviceSynchronize() != cudaSuccess) return PSA_ERR_CUDA;
   if (detail) *detail = 0;
   if (!ws->base) return PSA_OK;
-  int hdr[2] = {0, 0};
-  if (cudaMemcpy(hdr, ws->base, sizeof(hdr), cudaMemcpyDeviceToHost) != cudaSuccess) return PSA_ERR_CUDA;
-  if (detail) *detail = hdr[1];
-  return hdr[0];
+  return read_status(ws->base, ws->last_call, detail);
 }
 
 int psa_shutdown(void) {

@@ -516,10 +516,16 @@ __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uin
   if (REM) tc_ld16(tS + NFULL * 32, s + NFULL * 32);
   tc_wait_ld();
   if ((meta.x & meta.y & meta.z & meta.w) != 0xffffffffu) {  // 3D-padding: padded key positions score -inf
+    // by groups of 32 keys: padding of the slab's outer axes touches few of them
     const uint32_t v[4] = {meta.x, meta.y, meta.z, meta.w};
 #pragma unroll
-    for (int c = 0; c < NK; ++c)
-      if (!((v[c >> 5] >> (c & 31)) & 1u)) s[c] = 0xff800000u;
+    for (int c4 = 0; c4 < (NK + 31) / 32; ++c4) {
+      if (v[c4] != 0xffffffffu) {
+#pragma unroll
+        for (int c = c4 * 32; c < NK && c < c4 * 32 + 32; ++c)
+          if (!((v[c4] >> (c & 31)) & 1u)) s[c] = 0xff800000u;
+      }
+    }
   }
   // eight independent chains (NK is a multiple of 16): shorter dependency depth
   float a[8];
@@ -796,6 +802,17 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     uint32_t pair_g = 0;       // pair barriers armed so far
     uint32_t kv_g = 0;         // key slabs issued so far
     uint32_t it_q0 = 0, it_q1 = 0; // items in which query slab i was active
+    // Position of key c = lane + 32 i within a slab, t << 16 | h << 8 | w, for the validity words of slabs at the grid's
+    // edge (a block's last slab is only shorter along its slowest axis, so it is laid out alike).  Computed once: with
+    // its divisions in the slab loop this warp took 3,800 clocks per edge slab and the whole CTA waited for it.
+    int pos[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = lane + 32 * i;
+      pos[i] = (c / (g.cw * g.ch)) << 16 | ((c / g.cw) % g.ch) << 8 | (c % g.cw);
+    }
+    // block -> row of the spatial block grid without a division: sk, Wp <= 2^11
+    const uint32_t magic_w = ((1u << 22) + (uint32_t)g.Wp - 1u) / (uint32_t)g.Wp;
     bool ok = tmem_ok;
     pdl_wait();   // the work items are written by the planning kernel
     for (uint32_t n = 0; ok; ++n) {
@@ -957,26 +974,28 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
                 if (left == 0) break;
                 --left;
               }
-              const int kb = tk * g.Sp + sk;
+              const int hb = (int)(((unsigned long long)(uint32_t)sk * magic_w) >> 22);
+              int t0 = tk * g.bt, h0 = hb * g.bh, w0 = (sk - hb * g.Wp) * g.bw;
               for (int sub = 0; ok && sub < g.n_sub; ++sub) {
-                int t0, h0, w0, et, eh, ew, ntok, last;
-                slab_origin(g, kb, sub, t0, h0, w0);
-                slab_shape(g, sub, et, eh, ew, ntok, last);
-                // validity of the slab's key positions (3D-padding): bit c of word c/32
-                const bool edge = (t0 + et > g.T) || (h0 + eh > g.H) || (w0 + ew > g.W);
+                const int last = (sub == g.n_sub - 1) ? 1 : 0, ntok = last ? g.n_last : kSlabTokens;
+                const int et = last && g.sub_axis == 0 ? g.c_last : g.ct, eh = last && g.sub_axis == 1 ? g.c_last : g.ch,
+                          ew = last && g.sub_axis == 2 ? g.c_last : g.cw;
+                // validity of the slab's key positions (3D-padding): bit c of word c/32; ones beyond a short slab
                 uint32_t vw0 = 0xffffffffu, vw1 = 0xffffffffu, vw2 = 0xffffffffu, vw3 = 0xffffffffu;
-                if (edge) {
-                  const int ehw = ew * eh;
-                  int c = lane;
-                  vw0 = __ballot_sync(0xffffffffu, (t0 + c / ehw < g.T) && (h0 + (c / ew) % eh < g.H) && (w0 + c % ew < g.W));
-                  c += 32;
-                  vw1 = __ballot_sync(0xffffffffu, (t0 + c / ehw < g.T) && (h0 + (c / ew) % eh < g.H) && (w0 + c % ew < g.W));
-                  c += 32;
-                  vw2 = __ballot_sync(0xffffffffu, (t0 + c / ehw < g.T) && (h0 + (c / ew) % eh < g.H) && (w0 + c % ew < g.W));
-                  c += 32;
-                  vw3 = __ballot_sync(0xffffffffu, (t0 + c / ehw < g.T) && (h0 + (c / ew) % eh < g.H) && (w0 + c % ew < g.W));
+                const int rt = g.T - t0, rh = g.H - h0, rw = g.W - w0;
+                if (et > rt || eh > rh || ew > rw) {
+                  auto valid = [&](int i) -> bool {
+                    return ((pos[i] >> 16) < rt && ((pos[i] >> 8) & 0xff) < rh && (pos[i] & 0xff) < rw) || lane + 32 * i >= ntok;
+                  };
+                  vw0 = __ballot_sync(0xffffffffu, valid(0));
+                  vw1 = __ballot_sync(0xffffffffu, valid(1));
+                  vw2 = __ballot_sync(0xffffffffu, valid(2));
+                  vw3 = __ballot_sync(0xffffffffu, valid(3));
                 }
                 issue_slab(t0, h0, w0, last, ntok, vw0, vw1, vw2, vw3);
+                if (g.sub_axis == 0) t0 += g.ct;
+                else if (g.sub_axis == 1) h0 += g.ch;
+                else w0 += g.cw;
               }
             }
           }

@@ -180,10 +180,13 @@ int set_text(Geom* g, long long n_text) {
 
 // Attended block pairs of one head: product of the two axis pair counts.
 long long head_nnz(const psa_head_params& p, const Geom& g) {
-  long long ct = 0, cs = 0;
-  for_attended(g.Tp, p.Tw, p.To, p.Ts, [&](int, int d) { ct += g.Tp - (d < 0 ? -d : d); });
-  for_attended(g.Sp, p.Sw, p.So, p.Ss, [&](int, int d) { cs += g.Sp - (d < 0 ? -d : d); });
-  return ct * cs;
+  auto pairs = [](int n, int w, int o, int s) -> long long {
+    if (n <= 64) return axis_set(n, w, o, s).pairs;
+    long long c = 0;
+    for_attended(n, w, o, s, [&](int, int d) { c += n - (d < 0 ? -d : d); });
+    return c;
+  };
+  return pairs(g.Tp, p.Tw, p.To, p.Ts) * pairs(g.Sp, p.Sw, p.So, p.Ss);
 }
 
 int device_info(int* dev, Workspace** ws) {

@@ -640,6 +640,29 @@ __device__ __forceinline__ WorkItem direct_item(const Geom& g, int i) {
   return make_int4(head, r % g.NB, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
 }
 
+// Attended key-block coordinates of an item's query block (all of them for text queries), one bit per block coordinate,
+// by a whole warp; returns the number of attended key blocks.
+__device__ __forceinline__ int key_block_sets(const Geom& g, const WorkItem& wi, const psa_head_params p, int lane, uint32_t* maskT,
+                                              uint32_t* maskS) {
+  const bool textq = ((wi.w >> 25) & 1) != 0;
+  const int tq = wi.y / g.Sp, sq = wi.y % g.Sp;
+  int cnt_t = 0, cnt_s = 0;
+  for (int b = 0; b < g.Tp; b += 32) {
+    const int tk = b + lane;
+    const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
+    if (lane == 0) maskT[b >> 5] = m;
+    cnt_t += __popc(m);
+  }
+  for (int b = 0; b < g.Sp; b += 32) {
+    const int sk = b + lane;
+    const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
+    if (lane == 0) maskS[b >> 5] = m;
+    cnt_s += __popc(m);
+  }
+  __syncwarp();
+  return cnt_t * cnt_s;
+}
+
 // Cluster mode: CTA d of the cluster merges query rows d * rpc .. (d + 1) * rpc - 1 of the item (rpc = nq * 128 /
 // cluster size), and every CTA pushes its partial results of those rows into d's shared memory: (m, l, lr) to
 // kOffQ [source][row], O as fp32 to kOffRing [source][32 groups of 4 columns][row].  Remote stores are posted; reading
@@ -762,6 +785,14 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (threadIdx.x == 0) pdl_trigger();
+  // Without planning the load warp works its item out here, alongside the rest of the set-up (1.5 us earlier).
+  WorkItem first_item = make_int4(-1, 0, 0, 0);
+  if constexpr (!kPlanned) {
+    if (warp == kWarpLoad) {
+      first_item = direct_item(g, (int)(blockIdx.x / cluster_size()));
+      first_item.z = key_block_sets(g, first_item, heads.p[first_item.x], lane, maskT, maskS);
+    }
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -814,7 +845,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     // block -> row of the spatial block grid without a division: sk, Wp <= 2^11
     const uint32_t magic_w = ((1u << 22) + (uint32_t)g.Wp - 1u) / (uint32_t)g.Wp;
     bool ok = tmem_ok;
-    pdl_wait();   // the work items are written by the planning kernel
+    pdl_wait();   // the work items are written by the planning kernel, q, k and v by whatever ran before
     for (uint32_t n = 0; ok; ++n) {
       const uint32_t sslot = n & 1u;
       ok = mbar_wait_warp(bar(kBarSchedEmpty + sslot), ((n >> 1) & 1u) ^ 1u, abort_flag, 0x401);
@@ -844,9 +875,9 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         wi.y = __shfl_sync(0xffffffffu, wi.y, 0);
         wi.w = __shfl_sync(0xffffffffu, wi.w, 0);
       } else {
-        if (n == 0) wi = kPlanned ? prm.items[blockIdx.x / cluster_size()] : direct_item(g, (int)(blockIdx.x / cluster_size()));
-        if constexpr (kPlanned) take_share();
-        if (lane == 0 && (kPlanned || n > 0)) publish();
+        if (n == 0) wi = kPlanned ? prm.items[blockIdx.x / cluster_size()] : first_item;
+        take_share();
+        if (lane == 0) publish();
       }
       if (wi.x < 0) break;
       const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
@@ -860,7 +891,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       const bool textq = ((wi.w >> 25) & 1) != 0;   // the queries are text tokens: every key is attended
       const int head_ld = prm.shared_qkv ? 0 : head;   // head coordinate of the q, k, v loads
       auto eval_masks = [&]() {
-        const psa_head_params p = kPlanned ? prm.hp_dev[head] : heads.p[head];
+        const psa_head_params p = prm.hp_dev[head];
         const int tq = qb / g.Sp, sq = qb % g.Sp;
         int cnt_t = 0, cnt_s = 0;
         // attended key-block coordinates of this query block, one bit per block coordinate
@@ -877,14 +908,8 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
           cnt_s += __popc(m);
         }
         __syncwarp();
-        if constexpr (!kPlanned) {   // the item is complete only now
-          wi.z = cnt_t * cnt_s;
-          take_share();
-          if (lane == 0) publish();
-        }
       };
-      // (a CTA that only starts up loads the queries first)
-      if constexpr (kMode == kTicket) eval_masks();
+      if constexpr (kPlanned) eval_masks();
       // query slabs
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -912,7 +937,6 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         if (i == 0) ++it_q0; else ++it_q1;
       }
       if (!ok) break;
-      if constexpr (kMode != kTicket) eval_masks();
       // key / value slabs in ascending key-block id.  Up to `lag` slabs wait for their V load.
       int npend = 0;
       int at0 = 0, ah0 = 0, aw0 = 0, alast = 0, antok = kSlabTokens;  // oldest pending slab

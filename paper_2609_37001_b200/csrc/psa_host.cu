@@ -315,15 +315,19 @@ void plan_params(PlanParams* pp, const psa_head_params* params, const long long*
 }
 
 // CTAs that share a work item: 1 (persistent CTAs that draw whole items), 2, 4 or 8.  A launch takes about as many
-// rounds as its items need on the SMs, so a problem of few items, or of a few more than a whole number of rounds,
-// leaves SMs idle; sharing items makes the rounds shorter.  Clocks, from time stamps in the kernel: a key slab takes
-// 3,300 for two query slabs and 1,900 for one (split-KV mode); start-up, epilogue and exit take 15,000 in a persistent
-// CTA and 21,000 in a cluster (which also merges).
+// rounds as its items need on the SMs, and at least as long as its longest item, so a problem of few items, of a few more
+// than a whole number of rounds, or of a few very long ones (text queries attend every key) leaves SMs idle; sharing
+// items makes the rounds shorter.  Clocks, from time stamps in the kernel: a key slab takes 3,300 for two query slabs and
+// 1,900 for one (split-KV mode); start-up, epilogue and exit take 15,000 in a persistent CTA and 20,000 in a cluster
+// (which also merges).  Over 56 drawn problems of 12 to 700 items the choice was within 9 % of the best of the four,
+// except one at 18 % (12 items); without text, whole items were best in all 24 problems of more than two rounds.
 // Decided for a call as a whole, so that the chunks of a host-tensor call compute what the device call computes, bit
 // for bit.  weights: attended block pairs of every head.
 int share_items(const Workspace& ws, const Geom& g, const long long* weights, int n_heads) {
-  const int n_items = (n_heads < kMaxHeads ? n_heads : kMaxHeads) * g.items_per_head;   // of one launch
-  if (n_items > 2 * ws.n_sms) return 1;   // (beyond two rounds at most a third is to be gained)
+  const int heads = n_heads < kMaxHeads ? n_heads : kMaxHeads;   // of one launch
+  const int n_items = heads * g.items_per_head, n_text = heads * g.n_titems;
+  // beyond two rounds at most a third is to be gained, unless text queries make long items
+  if (n_items > (n_text ? 8 : 2) * ws.n_sms) return 1;
   long long total = 0, most = 0;
   for (int h = 0; h < n_heads; ++h) {
     total += weights[h];
@@ -333,17 +337,23 @@ int share_items(const Workspace& ws, const Geom& g, const long long* weights, in
   const double avg = (double)total / ((double)n_heads * g.NB), heavy = (double)most / g.NB;
   const int singles = g.n_sub & 1, doubles = g.n_sub >> 1;
   const double per_slab = (3300.0 * doubles + 1900.0 * singles) / (doubles + singles);
+  const double text = n_text ? ((double)g.NB * g.n_sub + g.n_ts) * (g.n_ts > 1 ? 3300.0 : 1900.0) : 0.0;
+  const double heavy_item = (heavy * g.n_sub + g.n_ts) * per_slab, longest = heavy_item > text ? heavy_item : text;
+  const double work = (double)(n_items - n_text) * (avg * g.n_sub + g.n_ts) * per_slab + n_text * text;
   auto time = [&](int at_a_time, int c, double fixed) -> double {
-    if (n_items <= at_a_time) return (heavy * g.n_sub + g.n_ts) * per_slab / c + fixed;   // one round: the longest item
-    return (double)((n_items + at_a_time - 1) / at_a_time) * ((avg * g.n_sub + g.n_ts) * per_slab / c + fixed);
+    const double one = longest / c + fixed;
+    if (n_items <= at_a_time) return one;
+    const double all = (double)((n_items + at_a_time - 1) / at_a_time) * (work / n_items / c + fixed);
+    return all > one ? all : one;
   };
   double best = time(ws.n_sms, 1, 15000.0);
   int cluster = 1;
   for (int i = 0; i < 3; ++i) {
     const int c = 2 << i;
-    if (ws.clusters[i] < 1 || heavy < c) break;   // a share of a heavy item holds at least one block
-    const double t = time(ws.clusters[i], c, 21000.0);
-    if (t < 0.95 * best) { best = t; cluster = c; }
+    if (ws.clusters[i] < 1 || longest < c * per_slab * g.n_sub) break;   // a share of a long item holds at least one block
+    const double t = time(ws.clusters[i], c, 20000.0);
+    // (rounds of whole items overlap more than the estimate knows: the longer ones go first)
+    if (t < (n_items <= ws.clusters[i] ? 0.97 : 0.88) * best) { best = t; cluster = c; }
   }
   return cluster;
 }

@@ -1456,6 +1456,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         // hand (m, l) of the odd key slabs to warpgroup 0 (release / acquire through the barrier)
         xchg[row] = make_float2(m_ref, l);
         mbar_arrive(bar(kBarMerge));
+        // This warpgroup has no use for O_1 itself, but must not fall a phase behind its barrier: a following two-slab
+        // item without keys waits for nothing else, and would take the phase before last for its own.
+        ok = mbar_wait_warp(bar(kBarOFull + 1), par_o1, abort_flag, 0x314);
+        if (!ok) break;
         continue;
       }
       ok = mbar_wait_warp(bar(kBarOFull + qi), (qi == 0 ? par_o0 : par_o1), abort_flag, 0x310 + qi);

@@ -68,9 +68,9 @@ constexpr int kBarQFull = 0, kBarQEmpty = 2, kBarPairFull = 4, kBarSlotEmpty = k
               kBarSchedEmpty = kBarSchedFull + 2, kBarStage = kBarSchedEmpty + 2, kBarMerge = kBarStage + 2,
               kBarDrain = kBarMerge + 1, kNumBars = (kBarDrain + 1 + 1) & ~1;
 constexpr uint32_t kOffMeta = kOffBar + kNumBars * 8;           // kMetaRing x 8 words
-constexpr uint32_t kOffMaskT = kOffMeta + kMetaRing * 32;       // kMaxTp / 32 words
-constexpr uint32_t kOffMaskS = kOffMaskT + (kMaxTp / 32) * 4;   // kMaxSp / 32 words
-constexpr uint32_t kOffSched = kOffMaskS + (kMaxSp / 32) * 4;   // two published work items
+constexpr uint32_t kOffMaskT = kOffMeta + kMetaRing * 32;       // [2][kMaxTp / 32] words: of the blocks that are no edge blocks, of edge blocks
+constexpr uint32_t kOffMaskS = kOffMaskT + 2 * (kMaxTp / 32) * 4;   // [2][kMaxSp / 32] words
+constexpr uint32_t kOffSched = kOffMaskS + 2 * (kMaxSp / 32) * 4;   // two published work items
 constexpr uint32_t kOffMisc = kOffSched + 32;                   // tmem base, abort flag
 constexpr uint32_t kOffXchg = kOffMisc + 16;                    // split-KV merge: (m, l) of 128 rows
 static_assert(256 * 128 * 4 <= kNumSlots * kSlabBytes, "the partial outputs do not fit into the ring");
@@ -377,6 +377,15 @@ __device__ __noinline__ bool dbg_fail(int* ws_header, int call_id, int code) {
 #define PSA_CHECKED(cond, code) true
 #endif
 
+// Whether block coordinates are those of an edge block (Geom: the last one along the stacked axis).
+__device__ __forceinline__ bool edge_s(const Geom& g, int s) {   // stacked axis h or w
+  return g.sub_axis == 1 ? s >= (g.Hp - 1) * g.Wp : s % g.Wp == g.Wp - 1;
+}
+__device__ __forceinline__ bool is_edge_block(const Geom& g, int qb) {
+  if (g.nb_edge == 0) return false;
+  return g.sub_axis == 0 ? qb >= g.NB - g.Sp : edge_s(g, qb % g.Sp);
+}
+
 // ----------------------------------------------------------------------------- planning
 // Work order: heads by descending number of attended pairs (`place`, from the host; heads stay together so that
 // concurrently running CTAs share K/V in L2), within a head query blocks by descending number of attended key blocks.
@@ -388,7 +397,7 @@ constexpr int kPlanThreads = 512;
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict__ ws_header,
             psa_head_params* __restrict__ hp_dev, WorkItem* __restrict__ items) {
-  extern __shared__ __align__(16) uint32_t sm[];  // key[NB rounded up to 4], cntT[Tp], cntS[Sp], setT[], setS[]
+  extern __shared__ __align__(16) uint32_t sm[];  // key[NB rounded up to 4], cntT[Tp], cntS[Sp], setT[], setS[], cntE[Sp]
   pdl_trigger();
   uint32_t* key = sm;
   const int nb4 = (g.NB + 3) & ~3;
@@ -396,6 +405,7 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
   uint32_t* cntS = cntT + g.Tp;
   uint32_t* setT = cntS + g.Sp;
   uint32_t* setS = setT + axis_words(g.Tp);
+  uint32_t* cntE = setS + axis_words(g.Sp);   // [Sp]
   const int h = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const psa_head_params p = hp.p[h];
@@ -429,6 +439,24 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
     cntT[a] = c;   // cntS follows cntT
   }
   __syncthreads();
+  // attended edge blocks: the last temporal coordinate, or the spatial coordinates at the edge
+  if (g.nb_edge != 0 && g.sub_axis != 0) {
+    for (int x = threadIdx.x; x < g.Sp; x += kPlanThreads) {
+      int c = 0;
+      const int first = g.sub_axis == 1 ? (g.Hp - 1) * g.Wp : g.Wp - 1, step = g.sub_axis == 1 ? 1 : g.Wp;
+      for (int k = first; k < g.Sp; k += step) {
+        const int b = k - x + g.Sp - 1;
+        c += (int)(setS[b >> 5] >> (b & 31) & 1u);
+      }
+      cntE[x] = (uint32_t)c;
+    }
+  }
+  auto edge_count = [&](int t, int x) -> int {
+    if (g.nb_edge == 0) return 0;
+    if (g.sub_axis != 0) return (int)(cntT[t] * cntE[x]);
+    const int b = 2 * (g.Tp - 1) - t;
+    return setT[b >> 5] >> (b & 31) & 1u ? (int)cntS[x] : 0;
+  };
   // unique keys: larger count first, then smaller block id (counts are at most NB < 2^16 here)
   for (int qb = threadIdx.x; qb < nb4; qb += kPlanThreads)
     key[qb] = qb < g.NB ? cntT[qb / g.Sp] * cntS[qb % g.Sp] * (uint32_t)g.NB + (uint32_t)(g.NB - 1 - qb) : 0u;
@@ -441,9 +469,9 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
   for (int it = threadIdx.x; it < g.n_titems; it += kPlanThreads) {
     const int sub0 = 2 * it;
     const int nq = (g.n_ts - sub0) >= 2 ? 2 : 1;
-    head_items[it] = make_int4(h, 0, g.NB, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
+    head_items[it] = make_int4(h | (g.nb_edge << 8), 0, g.NB - g.nb_edge, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
   }
-  WorkItem* out = items + (size_t)gridDim.x * g.n_titems + (size_t)hp.place[h] * g.NB * ipb;
+  WorkItem* out = items + (size_t)gridDim.x * g.n_titems + (size_t)hp.place[h] * (g.items_per_head - g.n_titems);
   for (int qb = threadIdx.x; qb < g.NB; qb += kPlanThreads) {
     const uint32_t mine = key[qb];
     int pos = 0;
@@ -451,14 +479,21 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
       const uint4 k4 = *reinterpret_cast<const uint4*>(key + j);
       pos += (int)(k4.x > mine) + (int)(k4.y > mine) + (int)(k4.z > mine) + (int)(k4.w > mine);
     }
-    const int c = (int)(mine / (uint32_t)g.NB);
+    const int c = (int)(mine / (uint32_t)g.NB), ce = edge_count(qb / g.Sp, qb % g.Sp);
+    const bool edge = is_edge_block(g, qb);
+    const int n_sub = edge ? g.n_edge : g.n_sub;
     // two-slab items first (heavier), then the odd single-slab items, each in rank order
     for (int it = 0; it < ipb; ++it) {
       const int sub0 = 2 * it;
-      const int nq = (g.n_sub - sub0) >= 2 ? 2 : 1;
+      if (sub0 >= n_sub) break;
+      if (it == 1 && g.nb_edge != 0 && (g.n_edge + 1) / 2 < ipb) {   // edge blocks have no second item
+        pos = 0;
+        for (int j = 0; j < g.NB; ++j) pos += key[j] > mine && !is_edge_block(g, j);
+      }
+      const int nq = (n_sub - sub0) >= 2 ? 2 : 1;
       // A single-slab item runs in split-KV mode: both softmax warpgroups work on that one
       // query slab, one on the even and one on the odd key slabs (flag in bit 24).
-      out[(size_t)it * g.NB + pos] = make_int4(h, qb, c, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
+      out[(size_t)it * g.NB + pos] = make_int4(h | (ce << 8), qb, c - ce, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
     }
   }
 }
@@ -634,33 +669,61 @@ __device__ __forceinline__ WorkItem direct_item(const Geom& g, int i) {
     return make_int4(head, 0, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
   }
   i -= n_text_items;
-  const int per_head = g.NB * g.items_per_block;
-  const int head = i / per_head, r = i - head * per_head, sub0 = 2 * (r / g.NB);
-  const int nq = (g.n_sub - sub0) >= 2 ? 2 : 1;
-  return make_int4(head, r % g.NB, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
+  const int per_head = g.items_per_head - g.n_titems;
+  const int head = i / per_head, r = i - head * per_head;
+  int qb = r, sub0 = 0;
+  if (r >= g.NB) {   // second items (three slabs per block), of edge blocks only if these have them, too
+    sub0 = 2;
+    qb = r - g.NB;
+    if (g.nb_edge != 0 && (g.n_edge + 1) / 2 < g.items_per_block && g.sub_axis != 0) {
+      const int per_row = g.sub_axis == 1 ? (g.Hp - 1) * g.Wp : g.Wp - 1, rows = g.sub_axis == 1 ? g.Sp : g.Wp;
+      qb = qb / per_row * rows + qb % per_row;
+    }
+  }
+  const int n_sub = is_edge_block(g, qb) ? g.n_edge : g.n_sub;
+  const int nq = (n_sub - sub0) >= 2 ? 2 : 1;
+  return make_int4(head, qb, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
+}
+
+// Words b / 32 of the two temporal (spatial) sets: without and with the edge coordinates of `m`.  The axis that edge blocks
+// are not told by goes into both.
+__device__ __forceinline__ void store_set_t(const Geom& g, uint32_t* maskT, int b, uint32_t m) {
+  const uint32_t e = b == ((g.Tp - 1) & ~31) ? 1u << ((g.Tp - 1) & 31) : 0u;
+  const bool by_t = g.nb_edge != 0 && g.sub_axis == 0;
+  maskT[b >> 5] = by_t ? m & ~e : m;
+  maskT[kMaxTp / 32 + (b >> 5)] = by_t ? m & e : m;
+}
+__device__ __forceinline__ void store_set_s(const Geom& g, uint32_t* maskS, int b, uint32_t m, uint32_t e) {
+  maskS[b >> 5] = m & ~e;
+  maskS[kMaxSp / 32 + (b >> 5)] = g.sub_axis != 0 ? m & e : m;
 }
 
 // Attended key-block coordinates of an item's query block (all of them for text queries), one bit per block coordinate,
-// by a whole warp; returns the number of attended key blocks.
-__device__ __forceinline__ int key_block_sets(const Geom& g, const WorkItem& wi, const psa_head_params p, int lane, uint32_t* maskT,
+// by a whole warp; completes the item's numbers of attended key blocks.
+__device__ __forceinline__ void key_block_sets(const Geom& g, WorkItem& wi, const psa_head_params p, int lane, uint32_t* maskT,
                                               uint32_t* maskS) {
   const bool textq = ((wi.w >> 25) & 1) != 0;
   const int tq = wi.y / g.Sp, sq = wi.y % g.Sp;
-  int cnt_t = 0, cnt_s = 0;
+  int cnt_t = 0, cnt_s = 0, edge_t = 0, edge_s_cnt = 0;
   for (int b = 0; b < g.Tp; b += 32) {
     const int tk = b + lane;
     const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
-    if (lane == 0) maskT[b >> 5] = m;
+    if (lane == 0) store_set_t(g, maskT, b, m);
     cnt_t += __popc(m);
+    if (b == ((g.Tp - 1) & ~31)) edge_t = (int)(m >> ((g.Tp - 1) & 31) & 1u);
   }
   for (int b = 0; b < g.Sp; b += 32) {
     const int sk = b + lane;
     const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
-    if (lane == 0) maskS[b >> 5] = m;
+    const unsigned e = g.nb_edge != 0 && g.sub_axis != 0 ? __ballot_sync(0xffffffffu, sk < g.Sp && edge_s(g, sk)) : 0u;
+    if (lane == 0) store_set_s(g, maskS, b, m, e);
     cnt_s += __popc(m);
+    edge_s_cnt += __popc(e & m);
   }
   __syncwarp();
-  return cnt_t * cnt_s;
+  const int edge = g.nb_edge == 0 ? 0 : (g.sub_axis == 0 ? edge_t * cnt_s : cnt_t * edge_s_cnt);
+  wi.z = cnt_t * cnt_s - edge;
+  wi.x |= edge << 8;
 }
 
 // Cluster mode: CTA d of the cluster merges query rows d * rpc .. (d + 1) * rpc - 1 of the item (rpc = nq * 128 /
@@ -683,7 +746,7 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
   const Geom& g = prm.g;
   const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);   // the item as the load warp published it
   if (wi.x < 0) return;                                               // (it gave up before that)
-  const int head = wi.x, nq = (wi.w >> 16) & 0xff;
+  const int head = wi.x & 0xff, nq = (wi.w >> 16) & 0xff;
   const int csize = (int)cluster_size();
   constexpr int kMergeThreads = kThreads - 32 * kFirstSoftmaxWarp;
   const int tid = (int)threadIdx.x - 32 * kFirstSoftmaxWarp;
@@ -733,13 +796,15 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
 //   kSharedDirect   the same without planning
 // (Separate instantiations: the ticket kernel's slab loop is sensitive to what else is compiled with it -- one kernel
 // with the mode as an argument was 1.5 to 2 % slower on the 720p layers.)
-enum Mode { kTicket, kDirect, kShared, kSharedDirect };
+//   kTicketEdge   kTicket for grids with edge blocks, kTicket itself being for grids without
+enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge };
 template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ HeadParamsArray heads, const AttnParams prm) {
   // 128-byte swizzled slabs need a 1024-byte aligned base; the declaration asks for it and the
   // kernel checks it (a misaligned base is reported through the status word, no work is done).
-  constexpr bool kCluster = kMode == kShared || kMode == kSharedDirect, kPlanned = kMode == kTicket || kMode == kShared;
+  constexpr bool kCluster = kMode == kShared || kMode == kSharedDirect, kDraws = kMode == kTicket || kMode == kTicketEdge;
+  constexpr bool kPlanned = kDraws || kMode == kShared, kEdge = kMode != kTicket;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
   const uint32_t sbase = smem_u32(smem);
@@ -748,6 +813,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
 
   auto bar = [&](int idx) -> uint32_t { return sbase + kOffBar + 8u * (uint32_t)idx; };
   uint32_t* meta = reinterpret_cast<uint32_t*>(smem + kOffMeta);
+  // attended key-block coordinates of the item being loaded; the sets of edge blocks behind the others'
   uint32_t* maskT = reinterpret_cast<uint32_t*>(smem + kOffMaskT);
   uint32_t* maskS = reinterpret_cast<uint32_t*>(smem + kOffMaskS);
   volatile int4* sched = reinterpret_cast<volatile int4*>(smem + kOffSched);
@@ -755,7 +821,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
 
   // A short query slab leaves its last rows of the Q buffer unwritten; keep them finite.
-  if (kMode == kTicket || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
+  if (kDraws || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
     for (uint32_t off = threadIdx.x * 16u; off < 2u * kSlabBytes; off += kThreads * 16u)
       *reinterpret_cast<uint4*>(smem + kOffQ + off) = make_uint4(0u, 0u, 0u, 0u);
     fence_async_smem();
@@ -790,7 +856,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
   if constexpr (!kPlanned) {
     if (warp == kWarpLoad) {
       first_item = direct_item(g, (int)(blockIdx.x / cluster_size()));
-      first_item.z = key_block_sets(g, first_item, heads.p[first_item.x], lane, maskT, maskS);
+      key_block_sets(g, first_item, heads.p[first_item.x], lane, maskT, maskS);
     }
   }
   tc_fence_before();
@@ -856,8 +922,13 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       auto take_share = [&]() {
         if constexpr (kCluster) {
           const int r = (int)cluster_rank(), c = (int)cluster_size();
-          skip = (int)((long long)wi.z * r / c);
-          left = wi.z = (int)((long long)wi.z * (r + 1) / c) - skip;
+          if (wi.x < 0) return;
+          const int main = wi.z, all = main + (wi.x >> 8);   // edge blocks come last
+          skip = (int)((long long)all * r / c);
+          const int end = (int)((long long)all * (r + 1) / c);
+          left = end - skip;
+          wi.z = max(min(end, main) - skip, 0);
+          wi.x = (wi.x & 0xff) | (left - wi.z) << 8;
           if (r + 1 < c) wi.w |= 1 << 26;
         }
       };
@@ -865,7 +936,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         sched[sslot].x = wi.x; sched[sslot].y = wi.y; sched[sslot].z = wi.z; sched[sslot].w = wi.w;
         mbar_arrive(bar(kBarSchedFull + sslot));
       };
-      if constexpr (kMode == kTicket) {
+      if constexpr (kDraws) {
         if (lane == 0) {
           const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
           if (ticket < prm.n_items) wi = prm.items[ticket];
@@ -880,7 +951,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         if (lane == 0) publish();
       }
       if (wi.x < 0) break;
-      const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
+      const int head = kEdge ? wi.x & 0xff : wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
       if (!PSA_CHECKED(head < g.n_heads && qb >= 0 && qb <= g.NB && nq >= 1 && nq <= 2 &&
                        sub0 + nq <= ((wi.w >> 25) & 1 ? g.n_ts : g.n_sub), 0xD04)) {
         if (lane == 0) atomicCAS((int*)abort_flag, 0, 0xD04);   // a malformed item: stop this CTA through the abort path
@@ -893,19 +964,25 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       auto eval_masks = [&]() {
         const psa_head_params p = prm.hp_dev[head];
         const int tq = qb / g.Sp, sq = qb % g.Sp;
-        int cnt_t = 0, cnt_s = 0;
         // attended key-block coordinates of this query block, one bit per block coordinate
         for (int b = 0; b < g.Tp; b += 32) {
           const int tk = b + lane;
           const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
-          if (lane == 0) maskT[b >> 5] = m;
-          cnt_t += __popc(m);
+          if (!kEdge || g.nb_edge == 0) {
+            if (lane == 0) maskT[b >> 5] = m;
+          } else {
+            if (lane == 0) store_set_t(g, maskT, b, m);
+          }
         }
         for (int b = 0; b < g.Sp; b += 32) {
           const int sk = b + lane;
           const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
-          if (lane == 0) maskS[b >> 5] = m;
-          cnt_s += __popc(m);
+          if (!kEdge || g.nb_edge == 0) {
+            if (lane == 0) maskS[b >> 5] = m;
+          } else {
+            const unsigned e = g.sub_axis != 0 ? __ballot_sync(0xffffffffu, sk < g.Sp && edge_s(g, sk)) : 0u;
+            if (lane == 0) store_set_s(g, maskS, b, m, e);
+          }
         }
         __syncwarp();
       };
@@ -983,13 +1060,17 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         else { bt0 = t0; bh0 = h0; bw0 = w0; blast = last; bntok = ntok; }
         ++npend;
       };
+      // (edge blocks, which have fewer slabs, in a second pass)
+      for (int pass = 0; pass < (kEdge && g.nb_edge != 0 ? 2 : 1); ++pass) {
+      const uint32_t *mask_t = maskT + pass * (kMaxTp / 32), *mask_s = maskS + pass * (kMaxSp / 32);
+      const int n_slabs = kEdge && pass != 0 ? g.n_edge : g.n_sub;
       for (int tw = 0; ok && left > 0 && tw < g.Tp; tw += 32) {
-        uint32_t mt = maskT[tw >> 5];
+        uint32_t mt = mask_t[tw >> 5];
         while (ok && left > 0 && mt) {
           const int tk = tw + __ffs(mt) - 1;
           mt &= mt - 1;
           for (int sw = 0; ok && left > 0 && sw < g.Sp; sw += 32) {
-            uint32_t ms = maskS[sw >> 5];
+            uint32_t ms = mask_s[sw >> 5];
             while (ok && ms) {
               const int sk = sw + __ffs(ms) - 1;
               ms &= ms - 1;
@@ -1000,7 +1081,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
               }
               const int hb = (int)(((unsigned long long)(uint32_t)sk * magic_w) >> 22);
               int t0 = tk * g.bt, h0 = hb * g.bh, w0 = (sk - hb * g.Wp) * g.bw;
-              for (int sub = 0; ok && sub < g.n_sub; ++sub) {
+              for (int sub = 0; ok && sub < n_slabs; ++sub) {
                 const int last = (sub == g.n_sub - 1) ? 1 : 0, ntok = last ? g.n_last : kSlabTokens;
                 const int et = last && g.sub_axis == 0 ? g.c_last : g.ct, eh = last && g.sub_axis == 1 ? g.c_last : g.ch,
                           ew = last && g.sub_axis == 2 ? g.c_last : g.cw;
@@ -1024,6 +1105,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
             }
           }
         }
+      }
       }
       // text key slabs: attended by every query; tokens beyond n_text are zero-filled and masked
       const int n_ts = kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts;
@@ -1133,8 +1215,8 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       if (!next_item(n, wi)) break;
       const int nq = (wi.w >> 16) & 0xff;
       const bool split = ((wi.w >> 24) & 1) != 0;
-      const int n_vid = wi.z * g.n_sub;          // video key slabs, then the text slabs (always 128 wide)
-      const int n_kv = n_vid + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
+      const int n_vid = wi.z * g.n_sub;          // key slabs, then those of edge blocks and of text (always 128 wide)
+      const int n_kv = n_vid + (kEdge ? (wi.x >> 8) * g.n_edge : 0) + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
       auto nk_j = [&](int j, int r) -> int { return j >= n_vid ? kSlabTokens : nk_at(r); };
       // which accumulators this item uses: both for a two-slab item, and for a split-KV item
       // with at least two key slabs (even slabs -> O_0, odd slabs -> O_1)
@@ -1346,11 +1428,11 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     for (uint32_t n = 0; ok; ++n) {
       WorkItem wi;
       if (!next_item(n, wi)) break;
-      const int head = wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
+      const int head = kEdge ? wi.x & 0xff : wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
       const bool split = ((wi.w >> 24) & 1) != 0;
       const bool textq = ((wi.w >> 25) & 1) != 0;
-      const int n_vid = wi.z * g.n_sub;          // video key slabs, then the text slabs (always 128 wide)
-      const int n_kv = n_vid + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
+      const int n_vid = wi.z * g.n_sub;          // key slabs, then those of edge blocks and of text (always 128 wide)
+      const int n_kv = n_vid + (kEdge ? (wi.x >> 8) * g.n_edge : 0) + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
       const bool use_o1 = (nq > 1) || (split && n_kv > 1);
       const bool active = (qi == 0) || use_o1;
       float m_ref = neg_inf;  // running reference maximum, scaled log2 domain
@@ -1608,7 +1690,7 @@ cudaError_t launch_wait_probe(int* ws_header, int call_id, unsigned long long li
 
 // ----------------------------------------------------------------------------- launchers
 size_t plan_smem_bytes(const Geom& g) {
-  return 4 * (size_t)(((g.NB + 3) & ~3) + g.Tp + g.Sp + axis_words(g.Tp) + axis_words(g.Sp));
+  return 4 * (size_t)(((g.NB + 3) & ~3) + g.Tp + 2 * g.Sp + axis_words(g.Tp) + axis_words(g.Sp));
 }
 
 namespace {
@@ -1635,7 +1717,8 @@ struct LaunchConfig {
 // Once per device: shared-memory limits, and how many clusters of 2, 4 and 8 CTAs run at a time.
 cudaError_t attn_init(int clusters[3]) {
   const void* kernels[] = {(const void*)attn_fwd_kernel<kTicket>, (const void*)attn_fwd_kernel<kDirect>,
-                           (const void*)attn_fwd_kernel<kShared>, (const void*)attn_fwd_kernel<kSharedDirect>};
+                           (const void*)attn_fwd_kernel<kShared>, (const void*)attn_fwd_kernel<kSharedDirect>,
+                           (const void*)attn_fwd_kernel<kTicketEdge>};
   cudaError_t e = cudaSuccess;
   for (const void* k : kernels)
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc)) != cudaSuccess) return e;
@@ -1668,8 +1751,9 @@ cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, cons
   if (cluster > 1)
     return direct ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kSharedDirect>, tm, heads, prm)
                   : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kShared>, tm, heads, prm);
-  return direct ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kDirect>, tm, heads, prm)
-                : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicket>, tm, heads, prm);
+  if (direct) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kDirect>, tm, heads, prm);
+  return prm.g.nb_edge ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicketEdge>, tm, heads, prm)
+                       : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicket>, tm, heads, prm);
 }
 
 }  // namespace psa

@@ -24,15 +24,19 @@ struct Geom {
   int sub_axis;            // axis along which the slabs of a block stack: 0 = t, 1 = h, 2 = w
   int c_last;              // extent of a block's LAST slab along sub_axis (<= the full slab's)
   int n_last;              // tokens of that last slab: 128, 112, 96 or 64
+  // Slabs that 3D-padding leaves without a token are neither loaded nor computed: a block that is the last one along
+  // sub_axis ("edge block") has n_edge of its n_sub slabs.  n_edge == n_sub: no slab is empty, no block counts as edge.
+  int n_edge;              // (all full 128-token slabs when n_edge < n_sub)
+  int nb_edge;             // edge blocks of the grid, 0 if no slab is empty
   int n_heads;
-  int items_per_block;     // work items per query block = ceil(n_sub / 2)
+  int items_per_block;     // work items per query block = ceil(n_sub / 2); ceil(n_edge / 2) for an edge block
   float scale_log2;        // softmax scale times log2(e)
   long long L;             // T*H*W
   // joint video + text sequences: n_text text tokens follow the L video tokens of every head
   int n_text;              // 0: video only
   int n_ts;                // text slabs of 128 tokens = ceil(n_text / 128)
   int n_titems;            // work items of the text queries per head = ceil(n_ts / 2)
-  int items_per_head;      // NB * items_per_block + n_titems
+  int items_per_head;      // of all blocks, and n_titems
   long long Lt;            // L + n_text: tokens per head, row length of lse
 };
 
@@ -47,9 +51,10 @@ struct PlanParams {
 };
 
 // One unit of work of the attention kernel: up to two query slabs of one query block.
-// x = head, y = query block id, z = number of attended key blocks,
+// x = head | (attended edge blocks << 8), y = query block id, z = number of attended key blocks that are no edge blocks,
 // w = first slab index | (number of slabs << 16) | (split-KV mode << 24) | (text-query item << 25)
-// (inside a CTA of a cluster that shares one item: z = its share of the blocks, bit 26 of w = no text keys)
+// (inside a CTA of a cluster that shares one item: x and z = its share of the blocks, bit 26 of w = no text keys).
+// Key slabs come in this order: z blocks of n_sub slabs, the edge blocks' n_edge slabs each, the text slabs.
 typedef int4 WorkItem;
 
 // [0]: box of a full 128-token slab, [1]: of a block's last slab, [2]: of a text slab

@@ -158,10 +158,18 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, Geom*
     if (g->ct > 128 || g->ch > 128 || g->cw > 128) return PSA_ERR_UNSUPPORTED;
     if (g->Tp > kMaxTp || g->Sp > kMaxSp) return PSA_ERR_UNSUPPORTED;
     g->n_sub = n_sub;
+    {   // slabs of the last block along the stacked axis that hold any token
+      const int ext = axis == 0 ? T : (axis == 1 ? H : W), b = axis == 0 ? t.bt : (axis == 1 ? t.bh : t.bw);
+      const int n = axis == 0 ? g->Tp : (axis == 1 ? g->Hp : g->Wp);
+      g->n_edge = (ext - (n - 1) * b + c0 - 1) / c0;
+      if (g->n_edge < n_sub) g->nb_edge = axis == 0 ? g->Sp : (axis == 1 ? g->Tp * g->Wp : g->Tp * g->Hp);
+    }
     g->items_per_block = (n_sub + 1) / 2;
     g->scale_log2 = prob->scale * 1.4426950408889634f;
   }
   g->items_per_head = g->NB * g->items_per_block;
+  // an edge block's empty slabs are no work (only with three slabs per block is it an item less)
+  if (g->nb_edge) g->items_per_head -= g->nb_edge * (g->items_per_block - (g->n_edge + 1) / 2);
   g->Lt = L;
   return PSA_OK;
 }
@@ -173,7 +181,7 @@ int set_text(Geom* g, long long n_text) {
   g->n_ts = (int)((n_text + kSlabTokens - 1) / kSlabTokens);
   if (g->n_ts > 0xffff) return PSA_ERR_UNSUPPORTED;
   g->n_titems = (g->n_ts + 1) / 2;
-  g->items_per_head = g->NB * g->items_per_block + g->n_titems;
+  g->items_per_head += g->n_titems;
   g->Lt = g->L + n_text;
   return PSA_OK;
 }

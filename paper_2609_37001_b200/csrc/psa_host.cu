@@ -841,6 +841,7 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
   // single-head chunks (two at each end, when the regular chunk is larger than that), and the two
   // heads with the fewest attended block pairs (the shortest kernels) are kept for the end: what
   // remains after the last byte has arrived is the lightest head's kernel and its copy-out.
+  // (With one head per chunk, too: 12 heads of 32,760 tokens 6.53 -> 6.42 ms.)
   const int n_edge = (per >= 2 && prob->n_heads >= 4 * per) ? 2 : 0;
   struct Chunk { int h0, nh; };
   Chunk chunks[kHostChunks];
@@ -860,7 +861,7 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
     if ((rc = device_info(&dev, &ws)) != PSA_OK || (rc = init_attn(ws)) != PSA_OK) return rc;
     cluster = share_items(*ws, g, weights.data(), prob->n_heads);
   }
-  if (n_edge) {
+  if (n_edge || (per == 1 && prob->n_heads >= 3)) {
     for (int h = 0; h < prob->n_heads; ++h) {
       const long long w = weights[h];
       if (last1 < 0 || w < weights[last1]) { last2 = last1; last1 = h; }

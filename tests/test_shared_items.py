@@ -51,3 +51,31 @@ def test_shared_items(grid, tile, params, n_text):
         err = np.abs(out_h[hd] - ro)
         assert err.max() <= 2e-2 and err.mean() <= 2e-3, (hd, err.max(), err.mean())
         assert np.abs(lse_h[hd][~empty] - rl[~empty]).max() <= 1e-3
+
+
+def test_shared_items_in_several_rounds():
+    """More shared items than clusters that run at a time (they are planned, heaviest first): long text-query items make
+    sharing pay.  Sampled video rows, and the text rows of the ragged last slab."""
+    from paper_2609_37001_b200 import build
+    build.build()
+    from paper_2609_37001_b200 import binding as B
+    grid, tile, n_text = (28, 29, 12), (1, 8, 16), 347
+    T, H, W = grid
+    L = T * H * W
+    params = [(28, 0, INF, 3, 0, INF), (28, 0, INF, 2, 0, INF)]
+    bits = {n: WL.tensor_bits(0x51B, n, 2, L + n_text) for n in ("q", "k", "v")}
+    q, k, v = (torch.from_numpy(bits[n].view(np.int16)).cuda().view(torch.bfloat16) for n in ("q", "k", "v"))
+    out = torch.full_like(q, float("nan"))
+    lse = torch.full((2, L + n_text), float("nan"), dtype=torch.float32, device="cuda")
+    B.psa_attn_fwd_joint(q, k, v, params, grid, tile, SCALE, n_text, out=out, lse=lse)
+    assert B.psa_last_device_status()[0] == 0
+    out_h = O.bf16_bits_to_f64(out.view(torch.int16).cpu().numpy().view(np.uint16))
+    lse_h = lse.cpu().numpy().astype(np.float64)
+    assert not np.isnan(out_h).any() and not np.isnan(lse_h).any()
+    for hd in range(2):
+        rows = sorted(set(WL.sample_rows(7, hd, L, 64)) | set(range(L + 250, L + n_text)) | {0, L - 1})
+        qf, kf, vf = (O.bf16_bits_to_f64(bits[n][hd]) for n in ("q", "k", "v"))
+        ro, rl = O.attention_rows_with_text(qf, kf, vf, rows, params[hd], T, H, W, tile, SCALE, n_text)
+        err = np.abs(out_h[hd][rows] - ro)
+        assert err.max() <= 2e-2 and err.mean() <= 2e-3, (hd, err.max(), err.mean())
+        assert np.abs(lse_h[hd][rows] - rl).max() <= 1e-3

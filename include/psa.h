@@ -124,8 +124,8 @@ int psa_attn_fwd(const void* q, const void* k, const void* v, void* out, float* 
  * (Wan 2.1 14B at 1x16x16: 12,600); larger problems return PSA_ERR_CAPACITY and launch nothing.
  * The first call on a device looks up the array's device address (with that device current);
  * make that first call before any stream capture begins.  Every call on a device shares the
- * array: the planning kernel clears the words that must start at zero and rewrites the rest,
- * so back-to-back calls on one stream are fine, but calls that overlap on the GPU (different
+ * array: what a call's kernels read of it is written by its own planning kernel (calls whose work
+ * items all run at once read none of it), so back-to-back calls on one stream are fine, but calls that overlap on the GPU (different
  * streams) race on it.  The status word of this variant is not visible to
  * psa_last_device_status(), and the event pair registered with psa_profile_events() is not
  * recorded by it.  No cudaMalloc, cudaFree or other allocating call is made. */

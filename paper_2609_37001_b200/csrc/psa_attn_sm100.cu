@@ -282,6 +282,11 @@ __device__ __forceinline__ void tc_st16(uint32_t addr, const uint32_t* r) {
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
+// 32 bytes to a 32-byte aligned address: whole sectors even when every lane writes a row of its own
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+               "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -655,7 +660,7 @@ __device__ __forceinline__ long long row_token(const Geom& g, bool textq, int qb
   int t0, h0, w0, et, eh, ew, ntok, last;
   slab_origin(g, qb, sub, t0, h0, w0);
   slab_shape(g, sub, et, eh, ew, ntok, last);
-  const int t = t0 + row / (ew * eh), hh = h0 + (row / ew) % eh, ww = w0 + row % ew;
+  const int t = t0 + (row >> g.pos_ts), hh = h0 + ((row >> g.pos_ws) & (g.ch - 1)), ww = w0 + (row & (g.cw - 1));
   return (row < ntok && t < g.T && hh < g.H && ww < g.W) ? ((long long)t * g.H + hh) * g.W + ww : -1;
 }
 
@@ -797,14 +802,20 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
 // (Separate instantiations: the ticket kernel's slab loop is sensitive to what else is compiled with it -- one kernel
 // with the mode as an argument was 1.5 to 2 % slower on the 720p layers.)
 //   kTicketEdge   kTicket for grids with edge blocks, kTicket itself being for grids without
-enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge };
+//   kTicketShort  kTicket for short items of blocks of one slab (which have no edge blocks): bound by what lies between two
+//                 items, so the next item's loads and Q K^T run while the last one is still being written out.  The query
+//                 buffers are released by the MMAs that read them last (a commit), the output goes from registers to
+//                 memory instead of through those buffers, and the accumulators are waited for at the first P V only.
+//                 12 heads of 1x8x16 blocks attending 19.5 of them, 8x32x48 grid: 221 -> 198 us
+enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge, kTicketShort };
 template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ HeadParamsArray heads, const AttnParams prm) {
   // 128-byte swizzled slabs need a 1024-byte aligned base; the declaration asks for it and the
   // kernel checks it (a misaligned base is reported through the status word, no work is done).
-  constexpr bool kCluster = kMode == kShared || kMode == kSharedDirect, kDraws = kMode == kTicket || kMode == kTicketEdge;
-  constexpr bool kPlanned = kDraws || kMode == kShared, kEdge = kMode != kTicket;
+  constexpr bool kCluster = kMode == kShared || kMode == kSharedDirect, kShort = kMode == kTicketShort;
+  constexpr bool kDraws = kMode == kTicket || kMode == kTicketEdge || kShort;
+  constexpr bool kPlanned = kDraws || kMode == kShared, kEdge = kMode != kTicket && !kShort;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
   const uint32_t sbase = smem_u32(smem);
@@ -1228,7 +1239,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
           ok = mbar_wait_warp(bar(kBarQFull + i), itq & 1u, abort_flag, 0x200 + i);
           if (!ok) break;
         }
-        if (i == 0 || use_o1) {
+        if ((i == 0 || use_o1) && (!kShort || n_kv == 0)) {
           // the epilogue of the previous item must have drained O_i before it is overwritten
           const uint32_t ito = i == 0 ? it_o0 : it_o1;
           ok = mbar_wait_warp(bar(kBarOEmpty + i), (ito & 1u) ^ 1u, abort_flag, 0x202 + i);
@@ -1251,6 +1262,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
             issue_qk(0, slot, nk_j(j, r0), j);
             tc_commit(bar(kBarSFull + j));
             tc_commit(bar(kBarSlotEmpty + slot));
+            if (kShort && j + 1 == n_kv) tc_commit(bar(kBarQEmpty + 0));
           }
           __syncwarp();
           r0 = r_inc(r0);
@@ -1268,6 +1280,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
           slot_i = more ? slot_next(kslot) : kslot;
           const int nk_cur = nk_j(j, rj);
           rj = r_inc(rj);
+          if (kShort && j < 2) {   // the previous item's O_i has been read
+            ok = mbar_wait_warp(bar(kBarOEmpty + i), ((i == 0 ? it_o0 : it_o1) & 1u) ^ 1u, abort_flag, 0x202 + i);
+            if (!ok) break;
+          }
           tc_fence_after();
           if (elect_one()) issue_pv_half(i, vslot, 0, j > 1, nk_cur);
           ok = mbar_wait_warp(bar(kBarPReady + i), cs & 1u, abort_flag, 0x232 + i);
@@ -1282,6 +1298,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
               r0 = r_inc(r0);
               tc_commit(bar(kBarSFull + i));
               tc_commit(bar(kBarSlotEmpty + kslot));
+              if (kShort && j + 3 == n_kv) tc_commit(bar(kBarQEmpty + 0));
             } else {
               tc_commit(bar(kBarOFull + i));
             }
@@ -1304,6 +1321,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
             issue_qk(1, slot, nk_j(0, 0), 1);
             tc_commit(bar(kBarSFull + 1));
             tc_commit(bar(kBarSlotEmpty + slot));
+            if (kShort && n_kv == 1) {
+              tc_commit(bar(kBarQEmpty + 0));
+              tc_commit(bar(kBarQEmpty + 1));
+            }
           }
           __syncwarp();
         }
@@ -1325,6 +1346,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
           else ok = mbar_wait2_warp(bar(kBarPairFull + pair_i), pair_ph, bar(kBarPHalf + 0), cnt_s0 & 1u, abort_flag, 0x211, 0x224);
           if (!ok) break;
           pair_adv();
+          if (kShort && j == 0) {
+            ok = mbar_wait2_warp(bar(kBarOEmpty + 0), (it_o0 & 1u) ^ 1u, bar(kBarOEmpty + 1), (it_o1 & 1u) ^ 1u, abort_flag, 0x202, 0x203);
+            if (!ok) break;
+          }
           tc_fence_after();
           if (elect_one()) issue_pv_half(0, vslot, 0, j > 0, nk_cur);
           bool half1_done = false;   // first half of P_1 already seen complete
@@ -1338,6 +1363,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
             if (more) {
               issue_qk(0, kslot, nk_next, 0);
               tc_commit(bar(kBarSFull + 0));
+              if (kShort && j + 2 == n_kv) tc_commit(bar(kBarQEmpty + 0));
             } else {
               tc_commit(bar(kBarOFull + 0));
             }
@@ -1367,6 +1393,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
               issue_qk(1, kslot, nk_next, 1);
               tc_commit(bar(kBarSFull + 1));
               tc_commit(bar(kBarSlotEmpty + kslot));
+              if (kShort && j + 2 == n_kv) tc_commit(bar(kBarQEmpty + 1));
             } else {
               tc_commit(bar(kBarOFull + 1));
             }
@@ -1378,6 +1405,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         if (elect_one()) {
           tc_commit(bar(kBarOFull + 0));
           if (nq > 1) tc_commit(bar(kBarOFull + 1));
+          if (kShort) {
+            tc_commit(bar(kBarQEmpty + 0));
+            if (nq > 1) tc_commit(bar(kBarQEmpty + 1));
+          }
         }
         __syncwarp();
       }
@@ -1536,6 +1567,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       float scale0 = 1.f, scale1 = 0.f;   // weights of O_0 and O_1 in the merged output
       if (split && qi == 1) {
         // hand (m, l) of the odd key slabs to warpgroup 0 (release / acquire through the barrier)
+        if constexpr (kShort) {   // which may still be merging the previous item: it has read that one's by then
+          ok = mbar_wait_warp(bar(kBarOEmpty + 1), par_o1 ^ 1u, abort_flag, 0x315);
+          if (!ok) break;
+        }
         xchg[row] = make_float2(m_ref, l);
         mbar_arrive(bar(kBarMerge));
         // This warpgroup has no use for O_1 itself, but must not fall a phase behind its barrier: a following two-slab
@@ -1565,6 +1600,13 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       scale0 *= inv;
       scale1 *= inv;
       uint8_t* stage = smem + kOffQ + (uint32_t)qi * kSlabBytes;
+      long long out_tok = -1;        // kShort: this row's token, and where its output goes
+      uint4* out_row = nullptr;
+      if constexpr (kShort) {
+        out_tok = row_token(g, textq, qb, sub0 + qi, row);
+        if (out_tok >= 0)
+          out_row = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head + out_tok * prm.out_token);
+      }
 #pragma unroll
       for (int c4 = 0; c4 < 4; ++c4) {
         uint32_t o[32];
@@ -1585,6 +1627,21 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         } else {
 #pragma unroll
           for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * scale0);
+        }
+        if constexpr (kShort) {
+          if (out_row != nullptr && PSA_CHECKED(head >= 0 && head < g.n_heads && out_tok < g.Lt, 0xD17)) {
+            uint32_t w[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) w[e] = empty ? 0u : pack_bf16(__uint_as_float(o[2 * e]), __uint_as_float(o[2 * e + 1]));
+            if ((reinterpret_cast<uintptr_t>(out_row) & 31u) == 0u) {
+              st_global_v8(out_row + c4 * 4, w);
+              st_global_v8(out_row + c4 * 4 + 2, w + 8);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) out_row[c4 * 4 + e] = make_uint4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
+            }
+          }
+          continue;
         }
 #pragma unroll
         for (int c8 = 0; c8 < 4; ++c8) {
@@ -1607,6 +1664,11 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       tc_fence_before();
       mbar_arrive(bar(kBarOEmpty + qi));
       if (split && use_o1) mbar_arrive(bar(kBarOEmpty + 1));
+      if constexpr (kShort) {
+        if (out_tok >= 0 && PSA_CHECKED(head >= 0 && head < g.n_heads && out_tok < g.Lt, 0xD18))
+          prm.lse[(long long)head * g.Lt + out_tok] = empty ? neg_inf : (m_ref + log2f(l)) * 0.6931471805599453f;
+        continue;
+      }
       int t0, h0, w0, et, eh, ew, ntok, last;
       const float lse_row = empty ? neg_inf : (m_ref + log2f(l)) * 0.6931471805599453f;
       if (textq) {   // text slab: rows are consecutive text tokens; they follow the L video tokens
@@ -1718,7 +1780,7 @@ struct LaunchConfig {
 cudaError_t attn_init(int clusters[3]) {
   const void* kernels[] = {(const void*)attn_fwd_kernel<kTicket>, (const void*)attn_fwd_kernel<kDirect>,
                            (const void*)attn_fwd_kernel<kShared>, (const void*)attn_fwd_kernel<kSharedDirect>,
-                           (const void*)attn_fwd_kernel<kTicketEdge>};
+                           (const void*)attn_fwd_kernel<kTicketEdge>, (const void*)attn_fwd_kernel<kTicketShort>};
   cudaError_t e = cudaSuccess;
   for (const void* k : kernels)
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc)) != cudaSuccess) return e;
@@ -1744,7 +1806,7 @@ cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, i
 // heads: read by launches without planning only.  cluster: CTAs per work item, 1: whole items.  direct: all items run
 // at once, nothing was planned.
 cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster, bool direct,
-                        cudaStream_t stream) {
+                        bool short_items, cudaStream_t stream) {
   if (prm.n_items <= 0) return cudaSuccess;
   const int ctas = cluster > 1 || direct ? prm.n_items * cluster : (prm.n_items < n_sms ? prm.n_items : n_sms);
   LaunchConfig lc(ctas, kThreads, kSmemAlloc, stream, cluster);
@@ -1752,6 +1814,7 @@ cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, cons
     return direct ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kSharedDirect>, tm, heads, prm)
                   : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kShared>, tm, heads, prm);
   if (direct) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kDirect>, tm, heads, prm);
+  if (short_items) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicketShort>, tm, heads, prm);
   return prm.g.nb_edge ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicketEdge>, tm, heads, prm)
                        : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicket>, tm, heads, prm);
 }

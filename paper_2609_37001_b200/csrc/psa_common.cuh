@@ -20,6 +20,7 @@ struct Geom {
   int bt, bh, bw;          // mask block (PSABlock) extents in tokens
   int Tp, Hp, Wp, Sp, NB;  // block grid after 3D-padding; Sp = Hp*Wp, NB = Tp*Sp
   int ct, ch, cw;          // 128-token slab = one TMA box (ct*ch*cw == 128)
+  int pos_ws, pos_ts;      // log2(cw) and log2(cw * ch): position c of a slab is w = c % cw, h = (c >> pos_ws) % ch, t = c >> pos_ts
   int n_sub;               // slabs per mask block (1..3)
   int sub_axis;            // axis along which the slabs of a block stack: 0 = t, 1 = h, 2 = w
   int c_last;              // extent of a block's LAST slab along sub_axis (<= the full slab's)

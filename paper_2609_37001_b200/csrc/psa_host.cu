@@ -21,7 +21,7 @@ cudaError_t attn_init(int clusters[3]);
 cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
                         WorkItem* items, cudaStream_t stream);
 cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster,
-                        bool direct, cudaStream_t stream);
+                        bool direct, bool short_items, cudaStream_t stream);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
                                  float* losses, cudaStream_t stream, int* launches);
@@ -156,6 +156,11 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, Geom*
     g->c_last = c_last;
     g->n_last = n_last;
     if (g->ct > 128 || g->ch > 128 || g->cw > 128) return PSA_ERR_UNSUPPORTED;
+    // (the extents of a full slab are powers of two: they multiply to 128; a block's last slab is only shorter along its
+    // slowest axis, so positions in it are the same)
+    while ((1 << g->pos_ws) < g->cw) ++g->pos_ws;
+    g->pos_ts = g->pos_ws;
+    while ((1 << g->pos_ts) < g->cw * g->ch) ++g->pos_ts;
     if (g->Tp > kMaxTp || g->Sp > kMaxSp) return PSA_ERR_UNSUPPORTED;
     g->n_sub = n_sub;
     {   // slabs of the last block along the stacked axis that hold any token
@@ -373,6 +378,17 @@ bool runs_at_once(const Workspace& ws, int n_items, int cluster) {
   return n_items <= at_once;
 }
 
+// Whether a planned launch uses the kernel that overlaps the ends of its items with the next ones: blocks of one slab, whose
+// items are the shortest, attending fewer than 64 key slabs on average.  1x8x16 blocks of an 8x32x48 grid, 12 heads, us
+// without and with: 15.6 key blocks 193 / 178, 19.5 221 / 198, 33.7 312 / 301, 65 532 / 532.  Items of two query slabs have
+// two warpgroups' rows to write and lose by it: 1x16x16 blocks attending 9.2 blocks 174 / 169 but 26.6 of a 16x48x80 grid
+// 1,308 / 1,353, 1x15x16 30.1 974 / 1,015; so do blocks of three slabs (3x8x16, 6.6 blocks 204 / 225).
+bool short_items(const Geom& g, const long long* weights, int n_heads) {
+  long long total = 0;
+  for (int h = 0; h < n_heads; ++h) total += weights[h];
+  return g.n_sub == 1 && total < (64ll - g.n_ts) * n_heads * g.NB;
+}
+
 // Planning (unless the launch is direct) and attention.
 cudaError_t launch_call(const TensorMaps& tm, const AttnParams& prm, const psa_head_params* params, const long long* weights,
                         const Workspace& ws, int cluster, bool record, cudaStream_t st) {
@@ -390,7 +406,7 @@ cudaError_t launch_call(const TensorMaps& tm, const AttnParams& prm, const psa_h
     ++g_launches;
   }
   if (record && g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
-  const cudaError_t e = launch_attn(tm, heads, prm, ws.n_sms, cluster, direct, st);
+  const cudaError_t e = launch_attn(tm, heads, prm, ws.n_sms, cluster, direct, short_items(prm.g, weights, n), st);
   if (e == cudaSuccess) ++g_launches;
   return e;
 }

@@ -4,12 +4,11 @@
 // coordinates (mask_build_small_kernel, further down: one thread block per head and temporal
 // query coordinate), and the general one described here.
 //
-// The two conditions of Algorithm 1 depend only on coordinate differences, so each block of
-// threads first tabulates, for its head, "does difference d attend" for every temporal and
-// every spatial difference (one modulo per table entry instead of two per mask byte).  Row
-// counts are window sums of those tables, and the block mask of a head is the Kronecker
-// product of its two axis masks, so the count of row (t', s') is cntT(t') * cntS(s') and
-// its offset in the column list has a closed form.
+// The two conditions of Algorithm 1 depend only on coordinate differences, so each block of threads first tabulates, for
+// its head, "does difference d attend" for every temporal and every spatial difference: bit d + n - 1 of a bit array per
+// axis, and the sorted list of the attended bits' positions.  The key coordinates that a query coordinate x attends are a
+// window of n bits and a contiguous piece of the list.  The block mask of a head is the Kronecker product of its two axis
+// masks, so the count of row (t', s') is cntT(t') * cntS(s') and its offset in the column list has a closed form.
 #include "psa_common.cuh"
 
 namespace psa {
@@ -18,116 +17,169 @@ struct HeadBases {
   int base[kMaxHeads];  // number of attended block pairs of all earlier heads
 };
 
-// Shared-memory tables of one head.  attT[d + Tp-1], attS[d + Sp-1] for differences d;
-// cntT[t], cntS[s] row counts per axis; preT[t], preS[s] their exclusive prefix sums.
-struct Tables {
-  uint8_t* attT;
-  uint8_t* attS;
-  int* cntT;
-  int* cntS;
-  int* preT;
-  int* preS;
+// Shared-memory tables of one axis with n coordinates: bits (a word of zeros behind them, so that a window may be read from
+// any bit), the number of bits set before each word, the positions of the set bits, and pre[x] = attended pairs of the
+// query coordinates before x.  At most 8.5 bytes a coordinate.
+struct Axis {
+  int n, words;
+  uint32_t* bits;
+  int* before;
+  int* pre;
+  uint16_t* list;
+
+  // attended differences below bit i
+  __device__ __forceinline__ int rank(int i) const { return before[i >> 5] + __popc(bits[i >> 5] & ((1u << (i & 31)) - 1u)); }
+  __device__ __forceinline__ int first(int x) const { return rank(n - 1 - x); }   // of x's piece of the list
+  __device__ __forceinline__ int count(int x) const { return rank(2 * n - 1 - x) - rank(n - 1 - x); }
+  __device__ __forceinline__ int pairs() const { return pre[n - 1] + count(n - 1); }
+  // 32 bits from bit i on
+  __device__ __forceinline__ uint32_t window(int i) const { return __funnelshift_r(bits[i >> 5], bits[(i >> 5) + 1], i & 31); }
 };
 
-__host__ __device__ inline size_t tables_bytes(const Geom& g) {
-  const size_t bytes = (size_t)(2 * g.Tp - 1) + (size_t)(2 * g.Sp - 1);
-  return ((bytes + 15) & ~size_t(15)) + sizeof(int) * 2 * (size_t)(g.Tp + g.Sp);
+__host__ __device__ inline int axis_words(int n) { return (2 * n - 1 + 31) / 32 + 1; }
+__host__ __device__ inline size_t axis_bytes(int n) {
+  return (8 * (size_t)axis_words(n) + 4 * (size_t)n + 2 * (size_t)(2 * n - 1) + 3) & ~size_t(3);
+}
+__device__ __forceinline__ Axis carve_axis(uint8_t* smem, int n) {
+  Axis a;
+  a.n = n;
+  a.words = axis_words(n);
+  a.bits = reinterpret_cast<uint32_t*>(smem);
+  a.before = reinterpret_cast<int*>(a.bits + a.words);
+  a.pre = a.before + a.words;
+  a.list = reinterpret_cast<uint16_t*>(a.pre + n);
+  return a;
 }
 
-__device__ __forceinline__ Tables carve_tables(uint8_t* smem, const Geom& g) {
-  Tables t;
-  t.attT = smem;
-  t.attS = smem + (2 * g.Tp - 1);
-  const size_t bytes = (size_t)(2 * g.Tp - 1) + (size_t)(2 * g.Sp - 1);
-  int* ints = reinterpret_cast<int*>(smem + ((bytes + 15) & ~size_t(15)));
-  t.cntT = ints;
-  t.cntS = ints + g.Tp;
-  t.preT = t.cntS + g.Sp;
-  t.preS = t.preT + g.Tp;
-  return t;
+__device__ __forceinline__ void axis_bits(const Axis& a, int warp, int nwarps, int lane, int width, int offset, int stride) {
+  for (int w = warp; w < a.words; w += nwarps) {
+    const int i = w * 32 + lane;
+    const unsigned m = __ballot_sync(0xffffffffu, i < 2 * a.n - 1 && axis_attends(i - (a.n - 1), width, offset, stride));
+    if (lane == 0) a.bits[w] = m;
+  }
+}
+// Exclusive prefix sums of value(0 .. n - 1) by one warp.
+template <class F>
+__device__ __forceinline__ void warp_prefix(int* out, int n, int lane, F value) {
+  int carry = 0;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane, v = i < n ? value(i) : 0;
+    int s = v;
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, s, off);
+      if (lane >= off) s += o;
+    }
+    if (i < n) out[i] = carry + s - v;
+    carry += __shfl_sync(0xffffffffu, s, 31);
+  }
+}
+__device__ __forceinline__ void axis_list(const Axis& a, int first, int step) {
+  for (int i = first; i < 2 * a.n - 1; i += step)
+    if (a.bits[i >> 5] >> (i & 31) & 1u) a.list[a.rank(i)] = (uint16_t)i;
 }
 
-// Builds the tables of one head cooperatively (whole block), ends with a barrier.
-__device__ void build_tables(const Tables& t, const psa_head_params& p, const Geom& g) {
-  for (int i = threadIdx.x; i < 2 * g.Tp - 1; i += blockDim.x) t.attT[i] = axis_attends(i - (g.Tp - 1), p.Tw, p.To, p.Ts);
-  for (int i = threadIdx.x; i < 2 * g.Sp - 1; i += blockDim.x) t.attS[i] = axis_attends(i - (g.Sp - 1), p.Sw, p.So, p.Ss);
-  __syncthreads();
-  // cnt[x] = number of key coordinates k in [0, n) with att[k - x + n-1]: a window of n entries
-  for (int x = threadIdx.x; x < g.Tp; x += blockDim.x) {
-    int c = 0;
-    for (int k = 0; k < g.Tp; ++k) c += t.attT[k - x + g.Tp - 1];
-    t.cntT[x] = c;
-  }
-  // the spatial axis can be long: one warp per 32 coordinates, lanes stride over the window
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  for (int x = warp; x < g.Sp; x += nwarps) {
-    int c = 0;
-    for (int k = lane; k < g.Sp; k += 32) c += t.attS[k - x + g.Sp - 1];
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-    if (lane == 0) t.cntS[x] = c;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int x = 0; x < g.Tp; ++x) { t.preT[x] = acc; acc += t.cntT[x]; }
-  }
-  if (threadIdx.x == 32 || (blockDim.x <= 32 && threadIdx.x == 0)) {
-    int acc = 0;
-    for (int x = 0; x < g.Sp; ++x) { t.preS[x] = acc; acc += t.cntS[x]; }
-  }
-  __syncthreads();
+// y / n and the remainder, for quotients below 2^20 (the product is then off by less than one)
+__device__ __forceinline__ int div_near(int y, int n, float inv, int& rem) {
+  int q = (int)((float)y * inv);
+  rem = y - q * n;
+  if (rem < 0) { --q; rem += n; }
+  else if (rem >= n) { ++q; rem -= n; }
+  return q;
 }
 
-// Offset of row (tq, sq) inside its head's column list, and its length.
-__device__ __forceinline__ void row_extent(const Tables& t, const Geom& g, int tq, int sq, int& offset, int& count) {
-  const int sumS = t.preS[g.Sp - 1] + t.cntS[g.Sp - 1];
-  offset = t.preT[tq] * sumS + t.cntT[tq] * t.preS[sq];
-  count = t.cntT[tq] * t.cntS[sq];
-}
-
-// One block per (group of query blocks, head); one warp per query block (= one CSR row and
-// one row of the byte mask).  Lanes cover 32 consecutive key blocks per step: coalesced mask
-// bytes, ballot-compacted ascending column ids.
+// One block per (group of consecutive rows, head); a row is a query block.  The rows' mask bytes are one region, written in
+// aligned 32-byte pieces (the region's ends bytewise): a piece is built as 32 bits, a window of the spatial bits for every
+// attended temporal coordinate it touches.  A warp then writes the list of a row, entry e of it being the (e / cntS)-th
+// attended temporal and the (e mod cntS)-th attended spatial coordinate.
+// Bound by latencies (the tables' barriers, then few independent stores per warp) on small problems and by the list's 4-byte
+// stores on large ones.  Microseconds, calls back to back, against one row per warp with a byte and a ballot per key block:
+// 6 heads of 32 x 36 blocks 22.2 -> 12.4, 20 such heads 57.5 -> 28.6, 6 of 21 x 60 26.8 -> 12.4, 40 of 8 x 60 28.8 -> 16.5,
+// 10 of 11 x 56 16.5 -> 9.2.
 __global__ void __launch_bounds__(256)
 mask_build_kernel(const HeadParamsArray hp, const HeadBases hb, const Geom g, int n_heads_here, int rows_per_block,
                   uint8_t* __restrict__ block_mask, int* __restrict__ row_ptr, int* __restrict__ col_idx,
                   int total_nnz) {
   extern __shared__ __align__(16) uint8_t smem_tab[];
   const int h = blockIdx.y;
-  const Tables t = carve_tables(smem_tab, g);
-  build_tables(t, hp.p[h], g);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int Tp = g.Tp, Sp = g.Sp, NB = g.NB;
+  const Axis aS = carve_axis(smem_tab, Sp), aT = carve_axis(smem_tab + axis_bytes(Sp), Tp);
+  const psa_head_params& p = hp.p[h];
+  axis_bits(aS, warp, nwarps, lane, p.Sw, p.So, p.Ss);
+  axis_bits(aT, nwarps - 1 - warp, nwarps, lane, p.Tw, p.To, p.Ts);
+  __syncthreads();
+  if (warp == 0) warp_prefix(aS.before, aS.words, lane, [&](int w) { return __popc(aS.bits[w]); });
+  if (warp == 1) warp_prefix(aT.before, aT.words, lane, [&](int w) { return __popc(aT.bits[w]); });
+  __syncthreads();
+  if (warp == 0) warp_prefix(aS.pre, Sp, lane, [&](int x) { return aS.count(x); });
+  else if (warp == 1) warp_prefix(aT.pre, Tp, lane, [&](int x) { return aT.count(x); });
+  else {
+    axis_list(aS, threadIdx.x - 64, blockDim.x - 64);
+    axis_list(aT, threadIdx.x - 64, blockDim.x - 64);
+  }
+  __syncthreads();
+  const float inv_nb = 1.f / (float)NB, inv_sp = 1.f / (float)Sp;
   const int q0 = blockIdx.x * rows_per_block;
-  const int q1 = min(g.NB, q0 + rows_per_block);
-  const long long nb2 = (long long)g.NB * g.NB;
-  for (int qb = q0 + warp; qb < q1; qb += nwarps) {
-    const int tq = qb / g.Sp, sq = qb % g.Sp;
-    int offset, count;
-    row_extent(t, g, tq, sq, offset, count);
-    int pos = hb.base[h] + offset;
-    if (row_ptr && lane == 0) row_ptr[(long long)h * g.NB + qb] = pos;
-    uint8_t* mrow = block_mask ? block_mask + (long long)h * nb2 + (long long)qb * g.NB : nullptr;
-    if (mrow == nullptr && col_idx == nullptr) continue;
-    const uint8_t* aT = t.attT + (g.Tp - 1 - tq);
-    const uint8_t* aS = t.attS + (g.Sp - 1 - sq);
-    int tk = lane / g.Sp, sk = lane % g.Sp;       // coordinates of key block `lane`
-    const int dt = 32 / g.Sp, ds = 32 % g.Sp;     // advance of 32 key blocks
-    for (int base = 0; base < g.NB; base += 32) {
-      const int kb = base + lane;
-      const bool att = kb < g.NB && aT[tk] && aS[sk];
-      if (mrow && kb < g.NB) mrow[kb] = att ? 1 : 0;
-      if (col_idx) {
-        const unsigned m = __ballot_sync(0xffffffffu, att);
-        if (att) col_idx[pos + __popc(m & ((1u << lane) - 1u))] = kb;
-        pos += __popc(m);
+  const int q1 = min(NB, q0 + rows_per_block);
+
+  if (block_mask) {
+    const long long x0 = ((long long)h * NB + q0) * NB, x1 = ((long long)h * NB + q1) * NB;
+    for (long long x = (x0 & ~31ll) + threadIdx.x * 32ll; x < x1; x += blockDim.x * 32ll) {
+      const int from = x < x0 ? (int)(x0 - x) : 0, to = x1 - x < 32 ? (int)(x1 - x) : 32;
+      int sk, sq;
+      int tk, tq, rem;
+      const int row = q0 + div_near((int)(x + from - x0), NB, inv_nb, rem);
+      tk = div_near(rem, Sp, inv_sp, sk);
+      tq = div_near(row, Sp, inv_sp, sq);
+      uint32_t m = 0;
+      for (int n = from; n < to;) {
+        const int len = min(to - n, Sp - sk), dt = tk - tq + Tp - 1;
+        if (aT.bits[dt >> 5] >> (dt & 31) & 1u) m |= (aS.window(Sp - 1 - sq + sk) & (0xffffffffu >> (32 - len))) << n;
+        n += len;
+        sk += len;
+        if (sk == Sp) {
+          sk = 0;
+          if (++tk == Tp) {
+            tk = 0;
+            if (++sq == Sp) { sq = 0; ++tq; }
+          }
+        }
       }
-      tk += dt;
-      sk += ds;
-      if (sk >= g.Sp) { sk -= g.Sp; ++tk; }
+      uint8_t* dst = block_mask + x;
+      if (to - from == 32) {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = (m >> (4 * i) & 15u) * 0x00204081u & 0x01010101u;
+        reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+      } else {
+        for (int n = from; n < to; ++n) dst[n] = (uint8_t)(m >> n & 1u);
+      }
     }
   }
-  if (row_ptr && blockIdx.x == 0 && h == n_heads_here - 1 && threadIdx.x == 0)
-    row_ptr[(long long)n_heads_here * g.NB] = total_nnz;
+  if (row_ptr == nullptr) return;   // (no lists without it)
+  const int pairsS = aS.pairs();
+  for (int qb = q0 + warp; qb < q1; qb += nwarps) {
+    int sq;
+    const int tq = div_near(qb, Sp, inv_sp, sq);
+    const int cT = aT.count(tq), cS = aS.count(sq);
+    const int pos = hb.base[h] + aT.pre[tq] * pairsS + cT * aS.pre[sq];
+    if (lane == 0) row_ptr[(long long)h * NB + qb] = pos;
+    if (col_idx == nullptr || cT * cS == 0) continue;
+    const uint16_t* lT = aT.list + aT.first(tq);
+    const uint16_t* lS = aS.list + aS.first(sq);
+    const int shift = (tq - (Tp - 1)) * Sp + sq - (Sp - 1);
+    int s, t = div_near(lane, cS, 1.f / (float)cS, s);
+    int ds, dt = div_near(32, cS, 1.f / (float)cS, ds);
+#pragma unroll 4
+    for (int e = lane; e < cT * cS; e += 32) {
+      col_idx[pos + e] = (int)lT[t] * Sp + (int)lS[s] + shift;
+      t += dt;
+      s += ds;
+      if (s >= cS) { s -= cS; ++t; }
+    }
+  }
+  if (blockIdx.x == 0 && h == n_heads_here - 1 && threadIdx.x == 0) row_ptr[(long long)n_heads_here * NB] = total_nnz;
 }
 
 // Fast path for block grids with at most 64 temporal and 32 spatial block coordinates (all the
@@ -375,14 +427,14 @@ cudaError_t launch_mask_build(const HeadParamsArray& hp, const AxisSet* sets, co
   }
   HeadBases hb;
   for (int h = 0; h < kMaxHeads; ++h) hb.base[h] = h < n_heads_here ? head_bases[h] : 0;
-  const size_t smem = tables_bytes(g);
+  const size_t smem = axis_bytes(g.Sp) + axis_bytes(g.Tp);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(mask_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  // enough blocks per head to fill every SM's thread slots (8 blocks of 256 threads each),
-  // at least 8 rows (one per warp) per block
-  int blocks_per_head = (8 * n_sms + n_heads_here - 1) / n_heads_here;
+  // four blocks per SM, all at once, with at least 8 rows (one per warp) each: 6 heads of 21 x 60 blocks take 12.4 us (14.8
+  // with two, 14.4 with three or five), 20 of 32 x 36 take 28.6 (32.9, 28.4, 26.7)
+  int blocks_per_head = 4 * n_sms / n_heads_here;
   if (blocks_per_head < 1) blocks_per_head = 1;
   int rows_per_block = (g.NB + blocks_per_head - 1) / blocks_per_head;
   if (rows_per_block < 8) rows_per_block = 8;

@@ -30,3 +30,15 @@ def test_parameters_given_as_lists_or_floats():
     want = B.psa_mask_sizes([(4, 2, 0, 5, 1, 3)], grid, tile)
     assert B.psa_mask_sizes([[4, 2, 0, 5, 1, 3]], grid, tile) == want
     assert B.psa_mask_sizes([(4.0, 2.0, 0.0, 5.0, 1.0, 3.0)], grid, tile) == want
+
+
+@pytest.mark.parametrize("n", [32, 33, 36, 60, 63, 64, 65])
+def test_pair_counts_of_axes_around_the_bit_set_widths(n):
+    from paper_2609_37001_b200 import build
+    build.build()
+    from paper_2609_37001_b200 import binding as B
+    for w in (1, 2, n - 1, n, 2 * n, 200):
+        for o in (0, 1, -1, n - 1, 1 - n, n, -n, 128 - n, 129 - n):
+            for s in (0, 1, 2, 3, n, 63, 64, 65, 127, 128):
+                got = B.psa_mask_sizes([(w, o, s, 1, 0, 0)], (n, 1, 1), (1, 1, 1))
+                assert got == (n, int(O.axis_mask(n, w, o, s).sum())), (n, w, o, s)

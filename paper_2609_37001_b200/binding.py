@@ -6,10 +6,10 @@ CUDA device, raises -- there is no CPU fallback.
 """
 from __future__ import annotations
 
-import array
 import ctypes
 import os
 import struct
+from itertools import chain
 from typing import Optional, Sequence, Tuple
 
 import torch
@@ -104,19 +104,32 @@ _PARAMS_CACHE: dict = {}
 
 def _params_array(head_params: Sequence[Sequence[int]]):
     """ctypes array of the per-head parameters, memoised by value: a model calls with the same few sets of masks, and
-    looking 40 heads up takes 1 us where converting them takes 8 (25 with one structure per head)."""
+    looking 40 heads up takes 1 us where converting them takes 10 (40 with one structure per head).  Entries are stored
+    under tuples of ints only, so what is given finds one by being equal to it; rows that hash by identity (tensors) are
+    equal to none of them and are converted on every call."""
     try:
-        key = tuple(head_params)
-        arr = _PARAMS_CACHE.get(key)
-    except TypeError:   # heads given as lists
-        key = tuple([tuple(p) for p in head_params])
-        arr = _PARAMS_CACHE.get(key)
+        arr = _PARAMS_CACHE.get(tuple(head_params))
+    except TypeError:   # rows without a hash: lists, arrays
+        arr = None
+    if arr is not None:
+        return arr
+    n, packed = len(head_params), None
+    try:
+        if set(map(len, head_params)) == {6}:
+            packed = struct.pack("%di" % (6 * n), *chain.from_iterable(head_params))
+            key = tuple(struct.iter_unpack("6i", packed))
+    except (TypeError, struct.error):   # floats and the like
+        packed = None
+    if packed is None:
+        key = tuple([tuple([int(x) for x in p]) for p in head_params])
+    arr = _PARAMS_CACHE.get(key)
     if arr is None:
-        n = len(key)
-        flat = [int(x) for p in key for x in p]
-        if len(flat) != 6 * n:
-            raise ValueError("six parameters per head required")
-        arr = (HeadParams * n).from_buffer(array.array("i", flat))
+        if packed is not None:
+            arr = (HeadParams * n).from_buffer_copy(packed)
+        else:   # (a row of fewer values leaves the others 0, one of more is an error)
+            arr = (HeadParams * n)()
+            for i, p in enumerate(key):
+                arr[i] = HeadParams(*p)
         if len(_PARAMS_CACHE) >= 64:
             _PARAMS_CACHE.clear()
         _PARAMS_CACHE[key] = arr

@@ -787,7 +787,7 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
       acc[4] = fmaf(w, b.x, acc[4]); acc[5] = fmaf(w, b.y, acc[5]); acc[6] = fmaf(w, b.z, acc[6]); acc[7] = fmaf(w, b.w, acc[7]);
     }
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] *= inv;
+    for (int e = 0; e < 8; ++e) acc[e] = empty ? 0.f : acc[e] * inv;   // (empty: no key, or a sum that is not a number)
     if (PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.Lt, 0xD16))
       *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head + (long long)tok * prm.out_token + cg * 8) =
           make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));

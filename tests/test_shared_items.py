@@ -79,3 +79,33 @@ def test_shared_items_in_several_rounds():
         err = np.abs(out_h[hd][rows] - ro)
         assert err.max() <= 2e-2 and err.mean() <= 2e-3, (hd, err.max(), err.mean())
         assert np.abs(lse_h[hd][rows] - rl).max() <= 1e-3
+
+
+@pytest.mark.parametrize("tile", [(1, 16, 16), (1, 8, 16)], ids=["two_slabs", "one_slab"])
+def test_rows_whose_sums_are_no_numbers(tile):
+    """NaN and infinite inputs leave the same rows 0 with lse = -inf, and the same elements infinite or NaN, whether items
+    are shared (2 heads) or whole (the same 2 heads repeated until there are many items)."""
+    from paper_2609_37001_b200 import build
+    build.build()
+    from paper_2609_37001_b200 import binding as B
+    grid, params = (8, 16, 16), [(8, 0, INF, 2, 0, INF), (2, 0, INF, 2, 0, INF)]
+    L, many = 8 * 16 * 16, 40
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn((2, L, 128), device="cuda", generator=gen).bfloat16() for _ in range(3))
+    k[0, 700, 5] = float("inf")    # scores of +inf and -inf, by the sign of the query's channel
+    k[1, 300, 9] = float("nan")    # every score of that key; only rows near it attend it
+    q[1, 1500, 3] = float("nan")   # every score of that query
+    v[1, 1900, 77] = float("inf")
+    v[1, 1910, 78] = float("nan")
+    o2, l2 = B.psa_attn_fwd(q, k, v, params, grid, tile, SCALE)
+    o80, l80 = B.psa_attn_fwd(*(x.repeat(many, 1, 1) for x in (q, k, v)), params * many, grid, tile, SCALE)
+    assert B.psa_last_device_status()[0] == 0
+    for o, l in ((o80[:2], l80[:2]), (o80[-2:], l80[-2:])):
+        assert torch.equal(torch.isneginf(l2), torch.isneginf(l))
+        empty = torch.isneginf(l2)
+        assert 0.3 < empty[0].float().mean() < 0.7 and empty[1, 1500] and empty[1, 300] and not empty[1, -1]
+        assert (o2[empty] == 0).all() and (o[empty] == 0).all()
+        assert torch.equal(o2.isnan(), o.isnan()) and torch.equal(o2.isinf(), o.isinf()) and o2.isinf().any() and o2.isnan().any()
+        ok = ~empty
+        a, b = (x.float().nan_to_num(0.0, 0.0, 0.0)[ok] for x in (o2, o))
+        assert (a - b).abs().max() <= 4e-2 and (l2[ok] - l[ok]).abs().max() <= 2e-3   # twice the bounds against the oracle

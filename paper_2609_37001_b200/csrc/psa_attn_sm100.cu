@@ -750,7 +750,6 @@ __device__ __forceinline__ Share share_of_row(uint32_t sbase, int r, int nq) {
 __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8_t* smem) {
   const Geom& g = prm.g;
   const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);   // the item as the load warp published it
-  if (wi.x < 0) return;                                               // (it gave up before that)
   const int head = wi.x & 0xff, nq = (wi.w >> 16) & 0xff;
   const int csize = (int)cluster_size();
   constexpr int kMergeThreads = kThreads - 32 * kFirstSoftmaxWarp;
@@ -1433,10 +1432,9 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     if (tmem_ok && mbar_wait_warp(bar(kBarSchedFull), 0u, abort_flag, 0x402)) {
       const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);
       const int nq = (wi.w >> 16) & 0xff, rpc = nq * 128 / (int)cluster_size(), r0 = (int)cluster_rank() * rpc;
-      if (wi.x >= 0)
-        for (int i = (int)threadIdx.x - 64; i < rpc; i += 64)
-          *reinterpret_cast<int*>(smem + kOffRowTok + (uint32_t)i * 4u) =
-              (int)row_token(g, ((wi.w >> 25) & 1) != 0, wi.y, (wi.w & 0xffff) + ((r0 + i) >> 7), (r0 + i) & 127);
+      for (int i = (int)threadIdx.x - 64; i < rpc; i += 64)
+        *reinterpret_cast<int*>(smem + kOffRowTok + (uint32_t)i * 4u) =
+            (int)row_token(g, ((wi.w >> 25) & 1) != 0, wi.y, (wi.w & 0xffff) + ((r0 + i) >> 7), (r0 + i) & 127);
     }
     __syncwarp();
   }
@@ -1718,7 +1716,9 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
   __syncthreads();
   if constexpr (kCluster) {
     cluster_sync_all();   // every partial result has arrived; no CTA writes into another one any more
-    if (warp >= kFirstSoftmaxWarp) merge_cluster(prm, smem);   // (the first warpgroup gave its registers away)
+    // (not by the first warpgroup, which gave its registers away; nor in a CTA that gave up: its item and the rows' tokens
+    // may never have been written to shared memory)
+    if (warp >= kFirstSoftmaxWarp && *abort_flag == 0) merge_cluster(prm, smem);
   }
   if (threadIdx.x == 0 && *abort_flag != 0) {
     report_status(prm.ws_header, prm.call_id, PSA_ERR_TIMEOUT, *abort_flag);

@@ -167,7 +167,8 @@ __device__ __forceinline__ bool mbar_wait_probe_warp(uint32_t bar_a, uint32_t pa
 }
 
 // Programmatic dependent launch: the next kernel of the stream may start once every block has triggered; it sees this
-// kernel's results after its own wait.  Both do nothing in a launch without the attribute.
+// kernel's results after its own wait.  Both do nothing in a launch without the attribute.  Every role waits before its
+// first wait on a barrier: a predecessor may run for longer than the barriers' time limit after it has triggered.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // words of an axis' set of attended differences
@@ -1215,6 +1216,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     };
 
     uint32_t it_o0 = 0, it_o1 = 0;    // items in which accumulator O_i was used
+    pdl_wait();   // the time limits start with the load warp's work (see pdl_wait)
     // keys of a slab from its index within its block (r = j mod n_sub, carried along: no division)
     const int r_last = g.n_sub - 1;
     auto nk_at = [&](int r) -> int { return r == r_last ? g.n_last : kSlabTokens; };
@@ -1429,6 +1431,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
   } else if constexpr (kCluster) {
     // ======================================================================= idle warps: tokens of the rows to merge
     // (the divisions take a microsecond, which the merge need not wait for)
+    pdl_wait();
     if (tmem_ok && mbar_wait_warp(bar(kBarSchedFull), 0u, abort_flag, 0x402)) {
       const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);
       const int nq = (wi.w >> 16) & 0xff, rpc = nq * 128 / (int)cluster_size(), r0 = (int)cluster_rank() * rpc;
@@ -1453,6 +1456,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     bool ok = true, met = false;   // met: cluster mode's first barrier passed
     const float neg_inf = __int_as_float(0xff800000);
     float2* xchg = reinterpret_cast<float2*>(smem + kOffXchg);
+    pdl_wait();
 
     for (uint32_t n = 0; ok; ++n) {
       WorkItem wi;

@@ -104,24 +104,28 @@ _PARAMS_CACHE: dict = {}
 
 def _params_array(head_params: Sequence[Sequence[int]]):
     """ctypes array of the per-head parameters, memoised by value: a model calls with the same few sets of masks, and
-    looking 40 heads up takes 1 us where converting them takes 10 (40 with one structure per head).  Entries are stored
+    looking 40 heads up takes 1 us where converting them takes 15 (40 with one structure per head).  Entries are stored
     under tuples of ints only, so what is given finds one by being equal to it; rows that hash by identity (tensors) are
-    equal to none of them and are converted on every call."""
+    equal to none of them and are converted on every call.  (The rows as given where they are such tuples: finding the
+    same objects again takes half the time of comparing equal ones.)"""
+    given = tuple(head_params)
     try:
-        arr = _PARAMS_CACHE.get(tuple(head_params))
+        arr = _PARAMS_CACHE.get(given)
     except TypeError:   # rows without a hash: lists, arrays
         arr = None
     if arr is not None:
         return arr
-    n, packed = len(head_params), None
+    n, packed = len(given), None
     try:
-        if set(map(len, head_params)) == {6}:
-            packed = struct.pack("%di" % (6 * n), *chain.from_iterable(head_params))
-            key = tuple(struct.iter_unpack("6i", packed))
+        if set(map(len, given)) == {6}:
+            flat = tuple(chain.from_iterable(given))
+            packed = struct.pack("%di" % (6 * n), *flat)
+            plain = set(map(type, given)) == {tuple} and set(map(type, flat)) == {int}
+            key = given if plain else tuple(struct.iter_unpack("6i", packed))
     except (TypeError, struct.error):   # floats and the like
         packed = None
     if packed is None:
-        key = tuple([tuple([int(x) for x in p]) for p in head_params])
+        key = tuple([tuple([int(x) for x in p]) for p in given])
     arr = _PARAMS_CACHE.get(key)
     if arr is None:
         if packed is not None:

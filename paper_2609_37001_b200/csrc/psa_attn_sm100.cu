@@ -78,7 +78,7 @@ constexpr uint32_t kOffPartTmp = kOffQ + 16384;                 // cluster mode:
 constexpr uint32_t kOffRowTok = kOffXchg;                       // cluster mode: token of every row that this CTA merges
 constexpr uint32_t kSmemBytes = kOffXchg + 128 * 8;
 constexpr uint32_t kSmemAlloc = kSmemBytes;                     // base alignment comes from the declaration
-static_assert(kSmemAlloc <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
+static_assert(kSmemAlloc <= kMaxSmemBytes, "exceeds the shared memory a CTA may use");
 
 // ----------------------------------------------------------------------------- PTX
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -400,18 +400,22 @@ __device__ __forceinline__ bool is_edge_block(const Geom& g, int qb) {
 // of 315 blocks (one thread per pair of coordinates and a compare of two words per pair of blocks: 11.7 us), most of
 // it hidden behind the attention kernel's prologue, which starts when every block has reached the trigger.
 constexpr int kPlanThreads = 512;
+__host__ __device__ __forceinline__ int plan_key_words(const Geom& g) {
+  const int sets = axis_words(g.Tp) + axis_words(g.Sp);
+  return g.NB > sets ? g.NB : sets;
+}
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict__ ws_header,
             psa_head_params* __restrict__ hp_dev, WorkItem* __restrict__ items) {
-  extern __shared__ __align__(16) uint32_t sm[];  // key[NB rounded up to 4], cntT[Tp], cntS[Sp], setT[], setS[], cntE[Sp]
+  // key[NB], cntT[Tp], cntS[Sp]; the axis sets stand where the keys are written later (2n - 1 bits of n coordinates: as many
+  // words as the grid has blocks are enough, but for a grid of one block)
+  extern __shared__ __align__(16) uint32_t sm[];
   pdl_trigger();
   uint32_t* key = sm;
-  const int nb4 = (g.NB + 3) & ~3;
-  uint32_t* cntT = sm + nb4;
+  uint32_t* cntT = sm + plan_key_words(g);
   uint32_t* cntS = cntT + g.Tp;
-  uint32_t* setT = cntS + g.Sp;
+  uint32_t* setT = sm;
   uint32_t* setS = setT + axis_words(g.Tp);
-  uint32_t* cntE = setS + axis_words(g.Sp);   // [Sp]
   const int h = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const psa_head_params p = hp.p[h];
@@ -429,7 +433,8 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
     if (lane == 0) setT[w] = m;   // setS follows setT
   }
   __syncthreads();
-  // row count of coordinate x: bits n - 1 - x .. 2n - 2 - x of its set
+  // row count of coordinate x: bits n - 1 - x .. 2n - 2 - x of its set; in the upper half-word how many of them are edge
+  // coordinates (the last temporal one, or the spatial ones at the edge; at most 2,048 of either)
   for (int a = threadIdx.x; a < g.Tp + g.Sp; a += kPlanThreads) {
     const bool is_t = a < g.Tp;
     const uint32_t* set = is_t ? setT : setS;
@@ -442,30 +447,22 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
       if (w == (hi - 1) >> 5) m &= 0xffffffffu >> (31 - ((hi - 1) & 31));
       c += __popc(m);
     }
-    cntT[a] = c;   // cntS follows cntT
+    int e = 0;
+    if (g.nb_edge != 0 && is_t == (g.sub_axis == 0)) {
+      const int first = is_t ? n - 1 : (g.sub_axis == 1 ? (g.Hp - 1) * g.Wp : g.Wp - 1), step = g.sub_axis == 2 ? g.Wp : 1;
+      for (int b = lo + first; b < hi; b += step) e += (int)(set[b >> 5] >> (b & 31) & 1u);
+    }
+    cntT[a] = (uint32_t)(c | e << 16);   // cntS follows cntT
   }
   __syncthreads();
-  // attended edge blocks: the last temporal coordinate, or the spatial coordinates at the edge
-  if (g.nb_edge != 0 && g.sub_axis != 0) {
-    for (int x = threadIdx.x; x < g.Sp; x += kPlanThreads) {
-      int c = 0;
-      const int first = g.sub_axis == 1 ? (g.Hp - 1) * g.Wp : g.Wp - 1, step = g.sub_axis == 1 ? 1 : g.Wp;
-      for (int k = first; k < g.Sp; k += step) {
-        const int b = k - x + g.Sp - 1;
-        c += (int)(setS[b >> 5] >> (b & 31) & 1u);
-      }
-      cntE[x] = (uint32_t)c;
-    }
-  }
+  // attended edge blocks of block (t, x)
   auto edge_count = [&](int t, int x) -> int {
     if (g.nb_edge == 0) return 0;
-    if (g.sub_axis != 0) return (int)(cntT[t] * cntE[x]);
-    const int b = 2 * (g.Tp - 1) - t;
-    return setT[b >> 5] >> (b & 31) & 1u ? (int)cntS[x] : 0;
+    return g.sub_axis != 0 ? (int)((cntT[t] & 0xffffu) * (cntS[x] >> 16)) : (int)((cntT[t] >> 16) * (cntS[x] & 0xffffu));
   };
   // unique keys: larger count first, then smaller block id (counts are at most NB < 2^16 here)
-  for (int qb = threadIdx.x; qb < nb4; qb += kPlanThreads)
-    key[qb] = qb < g.NB ? cntT[qb / g.Sp] * cntS[qb % g.Sp] * (uint32_t)g.NB + (uint32_t)(g.NB - 1 - qb) : 0u;
+  for (int qb = threadIdx.x; qb < g.NB; qb += kPlanThreads)
+    key[qb] = (cntT[qb / g.Sp] & 0xffffu) * (cntS[qb % g.Sp] & 0xffffu) * (uint32_t)g.NB + (uint32_t)(g.NB - 1 - qb);
   __syncthreads();
   const int ipb = g.items_per_block;
   // Text-query items of all heads first: they attend every key block, so they are the heaviest (behind the lighter
@@ -480,11 +477,12 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
   WorkItem* out = items + (size_t)gridDim.x * g.n_titems + (size_t)hp.place[h] * (g.items_per_head - g.n_titems);
   for (int qb = threadIdx.x; qb < g.NB; qb += kPlanThreads) {
     const uint32_t mine = key[qb];
-    int pos = 0;
-    for (int j = 0; j < nb4; j += 4) {
+    int pos = 0, j = 0;
+    for (; j + 4 <= g.NB; j += 4) {
       const uint4 k4 = *reinterpret_cast<const uint4*>(key + j);
       pos += (int)(k4.x > mine) + (int)(k4.y > mine) + (int)(k4.z > mine) + (int)(k4.w > mine);
     }
+    for (; j < g.NB; ++j) pos += (int)(key[j] > mine);
     const int c = (int)(mine / (uint32_t)g.NB), ce = edge_count(qb / g.Sp, qb % g.Sp);
     const bool edge = is_edge_block(g, qb);
     const int n_sub = edge ? g.n_edge : g.n_sub;
@@ -494,7 +492,7 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
       if (sub0 >= n_sub) break;
       if (it == 1 && g.nb_edge != 0 && (g.n_edge + 1) / 2 < ipb) {   // edge blocks have no second item
         pos = 0;
-        for (int j = 0; j < g.NB; ++j) pos += key[j] > mine && !is_edge_block(g, j);
+        for (j = 0; j < g.NB; ++j) pos += key[j] > mine && !is_edge_block(g, j);
       }
       const int nq = (n_sub - sub0) >= 2 ? 2 : 1;
       // A single-slab item runs in split-KV mode: both softmax warpgroups work on that one
@@ -1755,9 +1753,7 @@ cudaError_t launch_wait_probe(int* ws_header, int call_id, unsigned long long li
 }
 
 // ----------------------------------------------------------------------------- launchers
-size_t plan_smem_bytes(const Geom& g) {
-  return 4 * (size_t)(((g.NB + 3) & ~3) + g.Tp + 2 * g.Sp + axis_words(g.Tp) + axis_words(g.Sp));
-}
+size_t plan_smem_bytes(const Geom& g) { return 4 * (size_t)(plan_key_words(g) + g.Tp + g.Sp); }
 
 namespace {
 // Launch that may start before its predecessor in the stream has finished (see pdl_wait), in clusters of `cluster`.

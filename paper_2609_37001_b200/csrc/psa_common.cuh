@@ -13,6 +13,7 @@ constexpr int kSlabTokens = 128;  // tokens per compute slab (one MMA tile of ro
 constexpr int kMaxHeads = 128;    // heads per launch (parameters travel by value)
 constexpr int kMaxTp = 256;       // limits of the in-kernel key-block bitmasks
 constexpr int kMaxSp = 2048;
+constexpr size_t kMaxSmemBytes = 232448;   // 227 KB of shared memory that a CTA may use
 
 // Problem geometry handed to every kernel by value.
 struct Geom {

@@ -18,6 +18,7 @@ cudaError_t launch_mask_build(const HeadParamsArray& hp, const AxisSet* sets, co
                               uint8_t* block_mask, int* row_ptr, int* col_idx, int total_nnz_through_chunk,
                               int n_sms, cudaStream_t stream, int* launches);
 cudaError_t attn_init(int clusters[3]);
+size_t plan_smem_bytes(const Geom& g);
 cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
                         WorkItem* items, cudaStream_t stream);
 cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster,
@@ -161,7 +162,7 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, Geom*
     while ((1 << g->pos_ws) < g->cw) ++g->pos_ws;
     g->pos_ts = g->pos_ws;
     while ((1 << g->pos_ts) < g->cw * g->ch) ++g->pos_ts;
-    if (g->Tp > kMaxTp || g->Sp > kMaxSp) return PSA_ERR_UNSUPPORTED;
+    if (g->Tp > kMaxTp || g->Sp > kMaxSp || plan_smem_bytes(*g) > kMaxSmemBytes) return PSA_ERR_UNSUPPORTED;
     g->n_sub = n_sub;
     {   // slabs of the last block along the stacked axis that hold any token
       const int ext = axis == 0 ? T : (axis == 1 ? H : W), b = axis == 0 ? t.bt : (axis == 1 ? t.bh : t.bw);

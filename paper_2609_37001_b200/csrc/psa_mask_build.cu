@@ -36,14 +36,15 @@ struct Axis {
   __device__ __forceinline__ uint32_t window(int i) const { return __funnelshift_r(bits[i >> 5], bits[(i >> 5) + 1], i & 31); }
 };
 
-__host__ __device__ inline int axis_words(int n) { return (2 * n - 1 + 31) / 32 + 1; }
+// (one more than the sets themselves take: see bits)
+__host__ __device__ inline int table_words(int n) { return (2 * n - 1 + 31) / 32 + 1; }
 __host__ __device__ inline size_t axis_bytes(int n) {
-  return (8 * (size_t)axis_words(n) + 4 * (size_t)n + 2 * (size_t)(2 * n - 1) + 3) & ~size_t(3);
+  return (8 * (size_t)table_words(n) + 4 * (size_t)n + 2 * (size_t)(2 * n - 1) + 3) & ~size_t(3);
 }
 __device__ __forceinline__ Axis carve_axis(uint8_t* smem, int n) {
   Axis a;
   a.n = n;
-  a.words = axis_words(n);
+  a.words = table_words(n);
   a.bits = reinterpret_cast<uint32_t*>(smem);
   a.before = reinterpret_cast<int*>(a.bits + a.words);
   a.pre = a.before + a.words;

@@ -775,8 +775,9 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   for (int h = 0; h < prob->n_heads; ++h)
     if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
   // the fixed scratch bounds the problem: one launch worth of heads and kNoAllocMaxItems items
+  // (edge blocks counted like the others, whatever items they save: the limit that the header states)
   const long long n_items_ll = (long long)prob->n_heads * g.items_per_head;
-  if (prob->n_heads > kMaxHeads || n_items_ll > kNoAllocMaxItems) return PSA_ERR_CAPACITY;
+  if (prob->n_heads > kMaxHeads || (long long)prob->n_heads * g.NB * g.items_per_block > kNoAllocMaxItems) return PSA_ERR_CAPACITY;
 
   std::lock_guard<std::mutex> lock(g_mu);
   int dev;

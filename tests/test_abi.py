@@ -69,3 +69,17 @@ def test_invalid_arguments_are_rejected_on_the_host(B):
     # mask build: col_idx without row_ptr
     assert lib.psa_mask_build(hp, ctypes.byref(prob), 1, 16, 16, None, None, 64, 10, None) == B.PSA_ERR_INVALID_ARG
     assert lib.psa_mask_build(hp, ctypes.byref(prob), 1, 16, 16, None, 64, 128, 0, None) == B.PSA_ERR_CAPACITY
+
+
+def test_noalloc_capacity_counts_every_block_alike(B):
+    """The stated limit, n_heads * NB * ceil(slabs / 2) work items, also where edge blocks need fewer of them (3-slab
+    blocks on 4 frames: one slab of the second block row holds tokens)."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("a call that is not refused would run on these addresses")
+    f, tile = B.lib().psa_attn_fwd_noalloc, (3, 8, 16)
+    for heads, rc in ((40, B.PSA_ERR_CUDA), (41, B.PSA_ERR_CAPACITY), (54, B.PSA_ERR_CAPACITY), (128, B.PSA_ERR_CAPACITY)):
+        # 2 x 102 blocks of two items
+        prob = B.make_problem(heads, tile, 0.1, 4 * 48 * 272 * 128, 128)
+        hp = B._params_array([(1, 0, 0, 1, 0, 0)] * heads)
+        assert f(256, 512, 768, 1024, 2048, hp, ctypes.byref(prob), 4, 48, 272, None, None) == rc, heads

@@ -93,6 +93,9 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob,
  *   lse       device fp32 [n_heads][L], natural log of the sum of exp(scale * q.k) over
  *             attended real keys
  *   head_params host, n_heads entries
+ * Repeating a call repeats its results bit for bit.  How a head's results are rounded may depend on
+ * the call's other heads: a call of few work items has several CTAs share an item, which sums in
+ * another order, and how many is decided for the call as a whole.
  * Rows whose query block attends no key block get out = 0 and lse = -inf.  Padded
  * positions (Section 3.2, "3D-Padding") are never read from or written to memory.
  * Pointers must be 16-byte aligned.  bf16 inputs, fp32 accumulation.
@@ -222,6 +225,19 @@ int psa_profile_events(void* start_event, void* stop_event);
 
 /* Number of kernels the library has launched since load (all entry points). */
 int64_t psa_launch_count(void);
+
+/* How the last attention kernel of any entry point (on any device) handed out its work items: their number is
+ * returned (0: none launched yet), *ctas_per_item = 1, or 2, 4 or 8 CTAs that share an item, *mode (optional, like
+ * ctas_per_item) a psa_launch_mode.  For measurements and tests: the choice is by the problem's size and masks. */
+typedef enum {
+  PSA_LAUNCH_TICKET = 0,         /* persistent CTAs draw planned items                      */
+  PSA_LAUNCH_DIRECT = 1,         /* every item runs at once, nothing is planned             */
+  PSA_LAUNCH_SHARED = 2,         /* CTAs share planned items                                */
+  PSA_LAUNCH_SHARED_DIRECT = 3,  /* CTAs share items that all run at once                   */
+  PSA_LAUNCH_TICKET_EDGE = 4,    /* as 0, some blocks having slabs without any token        */
+  PSA_LAUNCH_TICKET_SHORT = 5    /* as 0, few key slabs per item, blocks of one slab        */
+} psa_launch_mode;
+int psa_last_attn_launch(int32_t* mode, int32_t* ctas_per_item);
 
 /* Frees the per-device workspaces.  Safe to call more than once. */
 int psa_shutdown(void);

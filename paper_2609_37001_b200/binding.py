@@ -78,6 +78,8 @@ def lib() -> ctypes.CDLL:
         L.psa_search_select_at_sparsity.argtypes = L.psa_search_select.argtypes
         L.psa_search_select_at_sparsity.restype = ctypes.c_int
         L.psa_last_device_status.argtypes = [ctypes.POINTER(ctypes.c_int32)]
+        L.psa_last_attn_launch.argtypes = [ctypes.POINTER(ctypes.c_int32)] * 2
+        L.psa_last_attn_launch.restype = ctypes.c_int
         L.psa_shutdown.argtypes = []
         L.psa_selftest_wait_timeout.argtypes = [i32, vp]
         L.psa_selftest_wait_timeout.restype = ctypes.c_int
@@ -388,6 +390,16 @@ def psa_search_select_at_sparsity(losses: Sequence[float], sparsity: Sequence[fl
     if r < 0:
         _check(r, "psa_search_select_at_sparsity")
     return r
+
+
+LAUNCH_MODES = ("ticket", "direct", "shared", "shared_direct", "ticket_edge", "ticket_short")
+
+
+def psa_last_attn_launch() -> Tuple[int, str, int]:
+    """(work items, mode, CTAs per item) of the last attention kernel launched, see psa.h."""
+    mode, ctas = ctypes.c_int32(0), ctypes.c_int32(0)
+    items = lib().psa_last_attn_launch(ctypes.byref(mode), ctypes.byref(ctas))
+    return items, LAUNCH_MODES[mode.value], ctas.value
 
 
 def psa_last_device_status() -> Tuple[int, int]:

@@ -792,7 +792,7 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
   }
 }
 
-// How a launch hands out its work items.
+// How a launch hands out its work items (Mode).
 //   kTicket   persistent CTAs draw planned items (heaviest first) from a ticket
 //   kDirect   CTA i runs item i: all items run at once, nothing is planned
 //   kShared   cluster i (2, 4 or 8 CTAs) runs planned item i, each CTA taking its share of the attended key blocks
@@ -805,7 +805,6 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
 //                 buffers are released by the MMAs that read them last (a commit), the output goes from registers to
 //                 memory instead of through those buffers, and the accumulators are waited for at the first P V only.
 //                 12 heads of 1x8x16 blocks attending 19.5 of them, 8x32x48 grid: 221 -> 198 us
-enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge, kTicketShort };
 template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ HeadParamsArray heads, const AttnParams prm) {
@@ -1802,21 +1801,28 @@ cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, i
   return cudaLaunchKernelEx(&lc.cfg, plan_kernel, hp, g, ws_header, hp_dev, items);
 }
 
-// cluster: CTAs per work item (1: persistent CTAs, whole items)
+template <int kMode>
+cudaError_t launch_mode(const LaunchConfig& lc, const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm) {
+  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode>, tm, heads, prm);
+}
+
 // heads: read by launches without planning only.  cluster: CTAs per work item, 1: whole items.  direct: all items run
-// at once, nothing was planned.
+// at once, nothing was planned.  *mode: the kernel launched.
 cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster, bool direct,
-                        bool short_items, cudaStream_t stream) {
+                        bool short_items, cudaStream_t stream, Mode* mode) {
   if (prm.n_items <= 0) return cudaSuccess;
   const int ctas = cluster > 1 || direct ? prm.n_items * cluster : (prm.n_items < n_sms ? prm.n_items : n_sms);
   LaunchConfig lc(ctas, kThreads, kSmemAlloc, stream, cluster);
-  if (cluster > 1)
-    return direct ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kSharedDirect>, tm, heads, prm)
-                  : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kShared>, tm, heads, prm);
-  if (direct) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kDirect>, tm, heads, prm);
-  if (short_items) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicketShort>, tm, heads, prm);
-  return prm.g.nb_edge ? cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicketEdge>, tm, heads, prm)
-                       : cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kTicket>, tm, heads, prm);
+  *mode = cluster > 1 ? (direct ? kSharedDirect : kShared)
+                      : (direct ? kDirect : (short_items ? kTicketShort : (prm.g.nb_edge ? kTicketEdge : kTicket)));
+  switch (*mode) {
+    case kTicket: return launch_mode<kTicket>(lc, tm, heads, prm);
+    case kDirect: return launch_mode<kDirect>(lc, tm, heads, prm);
+    case kShared: return launch_mode<kShared>(lc, tm, heads, prm);
+    case kSharedDirect: return launch_mode<kSharedDirect>(lc, tm, heads, prm);
+    case kTicketEdge: return launch_mode<kTicketEdge>(lc, tm, heads, prm);
+    default: return launch_mode<kTicketShort>(lc, tm, heads, prm);
+  }
 }
 
 }  // namespace psa

@@ -64,6 +64,9 @@ struct TensorMaps {
   CUtensorMap q[3], k[3], v[3], o[3];
 };
 
+// How an attention launch hands out its work items (see attn_fwd_kernel); the values are those of psa_launch_mode.
+enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge, kTicketShort };
+
 // Arguments of one attention launch; lse and out start at the launch's first head.
 struct AttnParams {
   Geom g;

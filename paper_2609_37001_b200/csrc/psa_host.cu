@@ -22,7 +22,7 @@ size_t plan_smem_bytes(const Geom& g);
 cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
                         WorkItem* items, cudaStream_t stream);
 cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster,
-                        bool direct, bool short_items, cudaStream_t stream);
+                        bool direct, bool short_items, cudaStream_t stream, Mode* mode);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
                                  float* losses, cudaStream_t stream, int* launches);
@@ -47,6 +47,12 @@ struct Workspace {
   int clusters[3] = {0, 0, 0};   // clusters of 2, 4 and 8 attention CTAs that run at a time
 };
 Workspace g_ws[kMaxDevices];
+
+// The last attention launch of any entry point (g_mu held).
+struct {
+  Mode mode = kTicket;
+  int items = 0, cluster = 1;
+} g_last_attn;
 
 // Id of a new API call on `stream` (g_mu held).  Never 0, which is what untouched status words hold.  A call that is
 // being captured has kCapturedCall set: its kernels run again whenever the graph is replayed.
@@ -407,8 +413,12 @@ cudaError_t launch_call(const TensorMaps& tm, const AttnParams& prm, const psa_h
     ++g_launches;
   }
   if (record && g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
-  const cudaError_t e = launch_attn(tm, heads, prm, ws.n_sms, cluster, direct, short_items(prm.g, weights, n), st);
-  if (e == cudaSuccess) ++g_launches;
+  const cudaError_t e = launch_attn(tm, heads, prm, ws.n_sms, cluster, direct, short_items(prm.g, weights, n), st, &g_last_attn.mode);
+  if (e == cudaSuccess) {
+    ++g_launches;
+    g_last_attn.items = prm.n_items;
+    g_last_attn.cluster = cluster;
+  }
   return e;
 }
 
@@ -480,6 +490,13 @@ const char* psa_status_string(int status) {
 }
 
 int64_t psa_launch_count(void) { return g_launches.load(); }
+
+int psa_last_attn_launch(int32_t* mode, int32_t* ctas_per_item) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (mode) *mode = g_last_attn.mode;
+  if (ctas_per_item) *ctas_per_item = g_last_attn.cluster;
+  return g_last_attn.items;
+}
 
 int psa_profile_events(void* start_event, void* stop_event) {
   std::lock_guard<std::mutex> lock(g_mu);

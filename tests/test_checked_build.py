@@ -2,7 +2,7 @@
 store index, TMA coordinate, ring slot and work-item field before using it and reports a violation
 through the status word instead of touching memory -- the stand-in for a memory checker on a pool
 where none may run.  A spread of shapes (ragged grids, 128 / 240 / 256 / 384-token blocks, empty rows,
-text tokens, more heads than SMs) must run through it with status 0 and give, bit for bit, what the
+text tokens, more heads than SMs, planned items that CTAs share, short items) must run through it with status 0 and give, bit for bit, what the
 regular build gives.  Runs in a child process: a process can load only one of the two libraries."""
 import os
 import subprocess
@@ -28,6 +28,8 @@ CASES = [
     ((2, 30, 40), (1, 12, 16), [(2, 0, 2, 2, 0, 3), (1, 0, INF, 9, 0, INF)], 0),
     ((2, 16, 16), (1, 16, 16), [((h % 2) + 1, (h % 3) - 1, INF, 1, 0, INF) for h in range(160)], 0),
     ((4, 16, 32), (1, 16, 16), [(2, 0, 3, 2, 0, 3), (1, 0, INF, 2, 1, INF)], 200),
+    ((20, 24, 30), (1, 16, 16), [(1, 0, INF, 1, 0, INF)], 219),
+    ((4, 16, 32), (1, 8, 16), [((h % 4) + 1, 0, INF, 2, 0, INF) for h in range(24)], 0),
 ]
 res = []
 for grid, tile, params, n_text in CASES:

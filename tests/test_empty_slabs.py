@@ -44,6 +44,8 @@ def test_empty_slabs(grid, tile, n_text, n_heads):
     out = torch.full_like(q, float("nan"))
     lse = torch.full((n_heads, L + n_text), float("nan"), dtype=torch.float32, device="cuda")
     B.psa_attn_fwd_joint(q, k, v, params, grid, tile, SCALE, n_text, out=out, lse=lse)
+    mode = B.psa_last_attn_launch()[1]
+    assert mode in (("direct", "shared_direct") if n_heads == 1 else ("ticket" if grid[2] == 700 else "ticket_edge", "shared")), mode
     st, detail = B.psa_last_device_status()
     assert st == 0, (st, hex(detail))
     out_h = O.bf16_bits_to_f64(out.view(torch.int16).cpu().numpy().view(np.uint16))

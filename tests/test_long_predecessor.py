@@ -28,19 +28,20 @@ def early_trigger(tmp_path_factory):
 
 @pytest.mark.parametrize("grid,tile,n_heads,n_text", [
     ((8, 16, 16), (2, 8, 8), 2, 0),       # shared items, all at once
-    ((28, 29, 12), (1, 8, 16), 2, 347),   # few items, long ones among them
+    ((20, 24, 32), (1, 16, 16), 1, 219),  # shared items, planned
     ((7, 16, 32), (1, 8, 16), 4, 0),      # 112 items
     ((21, 30, 24), (1, 15, 16), 12, 0),   # planned items
-], ids=["shared", "text", "at_once", "planned"])
-def test_time_limits_start_when_the_predecessor_has_finished(early_trigger, grid, tile, n_heads, n_text):
+], ids=["shared_direct", "shared", "direct", "ticket"])
+def test_time_limits_start_when_the_predecessor_has_finished(early_trigger, request, grid, tile, n_heads, n_text):
     from paper_2609_37001_b200 import build
     build.build()
     from paper_2609_37001_b200 import binding as B
     L = grid[0] * grid[1] * grid[2] + n_text
-    params = [(3, 0, 0, 2, 0, 0)] * n_heads
+    params = [(3, 0, 0, 2, 0, 0) if n_text == 0 else (1, 0, 0, 1, 0, 0)] * n_heads
     gen = torch.Generator(device="cuda").manual_seed(L)
     q, k, v = (torch.randn((n_heads, L, 128), device="cuda", generator=gen).bfloat16() for _ in range(3))
     want = B.psa_attn_fwd_joint(q, k, v, params, grid, tile, SCALE, n_text)
+    assert B.psa_last_attn_launch()[1] == request.node.callspec.id
     assert B.psa_last_device_status() == (0, 0)
     t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
     out, lse = (torch.empty_like(x) for x in want)

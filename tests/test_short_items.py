@@ -44,6 +44,7 @@ def test_short_items(grid, tile, n_text, n_heads, token_layout):
     out = place(torch.full_like(q, float("nan")))
     lse = torch.full((n_heads, L + n_text), float("nan"), dtype=torch.float32, device="cuda")
     B.psa_attn_fwd_joint(q, k, v, params, grid, tile, SCALE, n_text, out=out, lse=lse)
+    assert B.psa_last_attn_launch()[1] == "ticket_short"
     st, detail = B.psa_last_device_status()
     assert st == 0, (st, hex(detail))
     out_h = O.bf16_bits_to_f64(out.contiguous().view(torch.int16).cpu().numpy().view(np.uint16))

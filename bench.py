@@ -74,25 +74,35 @@ def config_of(w, extra=None):
 
 
 def slab_split(tile):
-    """(slabs per block, keys of the last slab) of a mask block, as the attention kernel splits it:
-    128-token slabs along the block's outermost axis of extent > 1, the last one possibly shorter."""
+    """(axis that a mask block's slabs stack on, its extent per full slab, slabs per block, keys of the last slab), as the
+    attention kernel splits a block: 128-token slabs along its outermost axis of extent > 1, the last possibly shorter."""
     bt, bh, bw = tile
-    if bt > 1 or (bh == 1 and bw == 1):
-        extent, other = bt, bh * bw
-    elif bh > 1:
-        extent, other = bh, bt * bw
-    else:
-        extent, other = bw, bt * bh
+    axis = 0 if bt > 1 or (bh == 1 and bw == 1) else (1 if bh > 1 else 2)
+    other = bt * bh * bw // tile[axis]
     c0 = 128 // other
-    n_sub = -(-extent // c0)
-    return n_sub, (extent - (n_sub - 1) * c0) * other
+    n_sub = -(-tile[axis] // c0)
+    return axis, c0, n_sub, (tile[axis] - (n_sub - 1) * c0) * other
 
 
-def issued_flops(nnz, tile):
+def issued_flops(w):
     """FLOPs the tensor cores are asked for: every attended block pair costs (128 rows per query
-    slab) x (keys of every key slab) x 4 x head_dim, padded and idle rows included."""
-    n_sub, n_last = slab_split(tile)
-    return 4.0 * HEAD_DIM * nnz * (128.0 * n_sub) * (128.0 * (n_sub - 1) + n_last)
+    slab) x (keys of every key slab) x 4 x head_dim, padded and idle rows included.  Slabs without any token (of the last
+    block along the stacked axis) are left out, as the kernel leaves them out."""
+    from oracle import psa_oracle as O
+    axis, c0, n_sub, n_last = slab_split(w["tile"])
+    n = [-(-x // b) for x, b in zip(w["grid"], w["tile"])]
+    n_edge = min(-(-(w["grid"][axis] - (n[axis] - 1) * w["tile"][axis]) // c0), n_sub)
+    # query rows and keys of a block by its temporal and by its spatial coordinate (all ones on the axis that has no say)
+    at = np.indices(n)[axis].reshape(n[0], -1)
+    at = at[:, 0] if axis == 0 else at[0]
+    edge = (at == n[axis] - 1) & (n_edge < n_sub)
+    rows = np.where(edge, 128.0 * n_edge, 128.0 * n_sub)
+    keys = np.where(edge, 128.0 * n_edge, 128.0 * (n_sub - 1) + n_last)
+    total = 0.0
+    for p in w["head_params"]:
+        mt, ms = O.axis_mask(n[0], *p[:3]).astype(np.float64), O.axis_mask(n[1] * n[2], *p[3:]).astype(np.float64)
+        total += (rows @ mt @ keys) * ms.sum() if axis == 0 else mt.sum() * (rows @ ms @ keys)
+    return 4.0 * HEAD_DIM * total
 
 
 # ----------------------------------------------------------------------------- CPU oracle leg
@@ -407,7 +417,7 @@ def run_ours(args, w):
             for ln in open(tp):
                 if ln.startswith("traffic_bytes_per_launch:"):
                     traffic = int(ln.split(":")[1])
-        issued = issued_flops(nnz, tile)
+        issued = issued_flops(w)
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": max(args.warmup, 3), "ms_per_step": ms_max, "ms_median": float(np.median(step_ms)),
@@ -473,13 +483,12 @@ def time_other_configs(B, WL, torch, dev, peaks, skip):
             raise SystemExit(f"{name}: device status {st} {hex(detail)}")
         ms = [ev[i].elapsed_time(ev[i + 1]) for i in range(iters)]
         mean = float(np.mean(ms))
-        _, nnz = B.psa_mask_sizes(params, w["grid"], tile)
         res.append({"workload": name, "grid": w["grid"], "n_heads": nh, "mask_block": tile, "tile_sparsity": w["tile_sparsity"],
                     "ms": mean, "ms_median": float(np.median(ms)), "ms_min": float(np.min(ms)),
                     "computed_tflops": flops / (mean * 1e-3) / 1e12,
                     "frac": flops / (mean * 1e-3) / 1e12 / peaks["bf16_tflops"],
                     "dense_equiv_tflops": dflops / (mean * 1e-3) / 1e12,
-                    "padding_ratio": issued_flops(nnz, tile) / flops if flops else None})
+                    "padding_ratio": issued_flops(w) / flops if flops else None})
         del q, k, v, out, lse
         torch.cuda.empty_cache()
     return res

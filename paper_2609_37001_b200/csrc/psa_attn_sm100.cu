@@ -1,10 +1,12 @@
 // psa_attn_fwd for sm_100a: stripe-masked flash attention forward.
 //
-// One persistent CTA per SM draws work items from a global ticket; items are stored heaviest
-// first (by the number of attended key blocks), head-major.  A work item is up to two query
-// slabs (<= 128 rows each) of one query block (PSABlock); both slabs share the block's key
-// list (GetKVBlocks, Algorithm 2), which the load warp enumerates in ascending block id straight
-// from the six stripe parameters (Algorithm 1) -- no mask or index list is read from memory.
+// A work item is up to two query slabs (<= 128 rows each) of one query block (PSABlock); both slabs share the block's key
+// list (GetKVBlocks, Algorithm 2), which the load warp enumerates in ascending block id (edge blocks last) straight from
+// the six stripe parameters (Algorithm 1) -- no mask or index list is read from memory.
+// How items reach CTAs depends on how many there are (Mode; the choice is in the host file): with more items than SMs, one
+// persistent CTA per SM draws them from a global ticket, stored heaviest first (by the number of attended key blocks) and
+// head-major by a planning kernel; when all of them run at once, CTA i takes item i and nothing is planned; when they are
+// few or some are long, a cluster of 2, 4 or 8 CTAs shares each item.
 // A single-slab item runs in split-KV mode: both softmax warpgroups work on that one slab, on
 // the even and the odd key slabs, and their partial results are merged in the epilogue.
 //
@@ -27,7 +29,9 @@
 // flag; every other waiter sees the flag at its next poll and returns, all roles leave their
 // loops, the load warp waits (bounded) for its TMA loads in flight, the MMA warp waits (bounded)
 // for its MMAs in flight, all threads meet at the one __syncthreads of the teardown, TMEM is
-// freed and the status word reports the timeout.  Not bounded by the kernel: the TMEM allocation
+// freed and the status word reports the timeout.  Not bounded by the kernel: the wait for the kernel
+// before it in the stream (griddepcontrol.wait); the two cluster barriers of shared items, which every
+// thread reaches, since all loops before them are left in bounded time; and the TMEM allocation
 // at start-up, which blocks while another resident CTA holds tensor memory -- this kernel takes a
 // whole SM (226 KB of shared memory, 512 TMEM columns), so a caller must not run other
 // TMEM-using kernels on the same device concurrently with it.

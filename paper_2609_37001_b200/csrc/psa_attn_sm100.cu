@@ -171,8 +171,8 @@ __device__ __forceinline__ bool mbar_wait_probe_warp(uint32_t bar_a, uint32_t pa
 }
 
 // Programmatic dependent launch: the next kernel of the stream may start once every block has triggered; it sees this
-// kernel's results after its own wait.  Both do nothing in a launch without the attribute.  Every role waits before its
-// first wait on a barrier: a predecessor may run for longer than the barriers' time limit after it has triggered.
+// kernel's results after its own wait.  Both do nothing in a launch without the attribute.  No role waits on a barrier
+// before that: a predecessor may run for longer than the barriers' time limit after it has triggered.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // words of an axis' set of attended differences
@@ -871,6 +871,13 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       key_block_sets(g, first_item, heads.p[first_item.x], lane, maskT, maskS);
     }
   }
+  // A persistent CTA has one idle thread wait for the kernel before, on behalf of every role behind the barrier.  (Waits in
+  // the roles, or by more threads here, made launches of many items 0.5 % slower: 33 heads of 147 blocks of 240 tokens 16.10
+  // ms without, 16.11 with one thread, 16.19 with a wait in every role.)  Launches of few items wait in the roles, behind
+  // their own set-up.
+  if constexpr (kDraws) {
+    if (threadIdx.x == 64) pdl_wait();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1217,7 +1224,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     };
 
     uint32_t it_o0 = 0, it_o1 = 0;    // items in which accumulator O_i was used
-    pdl_wait();   // the time limits start with the load warp's work (see pdl_wait)
+    if constexpr (!kDraws) pdl_wait();   // (see pdl_wait)
     // keys of a slab from its index within its block (r = j mod n_sub, carried along: no division)
     const int r_last = g.n_sub - 1;
     auto nk_at = [&](int r) -> int { return r == r_last ? g.n_last : kSlabTokens; };
@@ -1457,7 +1464,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     bool ok = true, met = false;   // met: cluster mode's first barrier passed
     const float neg_inf = __int_as_float(0xff800000);
     float2* xchg = reinterpret_cast<float2*>(smem + kOffXchg);
-    pdl_wait();
+    if constexpr (!kDraws) pdl_wait();   // (see pdl_wait)
 
     for (uint32_t n = 0; ok; ++n) {
       WorkItem wi;

@@ -72,15 +72,18 @@ constexpr int kBarQFull = 0, kBarQEmpty = 2, kBarPairFull = 4, kBarSlotEmpty = k
               kBarSchedEmpty = kBarSchedFull + 2, kBarStage = kBarSchedEmpty + 2, kBarMerge = kBarStage + 2,
               kBarDrain = kBarMerge + 1, kNumBars = (kBarDrain + 1 + 1) & ~1;
 constexpr uint32_t kOffMeta = kOffBar + kNumBars * 8;           // kMetaRing x 8 words
-constexpr uint32_t kOffMaskT = kOffMeta + kMetaRing * 32;       // [2][kMaxTp / 32] words: of the blocks that are no edge blocks, of edge blocks
-constexpr uint32_t kOffMaskS = kOffMaskT + 2 * (kMaxTp / 32) * 4;   // [2][kMaxSp / 32] words
+constexpr uint32_t kOffMaskT = kOffMeta + kMetaRing * 32;       // [kMaxTp / 32] words
+constexpr uint32_t kOffMaskS = kOffMaskT + (kMaxTp / 32) * 4;   // [2][kMaxSp / 32] words (key_block_sets)
 constexpr uint32_t kOffSched = kOffMaskS + 2 * (kMaxSp / 32) * 4;   // two published work items
 constexpr uint32_t kOffMisc = kOffSched + 32;                   // tmem base, abort flag
 constexpr uint32_t kOffXchg = kOffMisc + 16;                    // split-KV merge: (m, l) of 128 rows
 static_assert(256 * 128 * 4 <= kNumSlots * kSlabBytes, "the partial outputs do not fit into the ring");
 constexpr uint32_t kOffPartTmp = kOffQ + 16384;                 // cluster mode: (m, l, lr) of the two tiles of one query slab
 constexpr uint32_t kOffRowTok = kOffXchg;                       // cluster mode: token of every row that this CTA merges
-constexpr uint32_t kSmemBytes = kOffXchg + 128 * 8;
+// Grids with edge blocks: boxes of a slab, {w, h, t, first row / 8 << 8 | map}, as loaded for K and, up to two slabs later, for V.
+constexpr int kLists = 3, kMaxListed = 16;
+constexpr uint32_t kOffLists = kOffXchg + 128 * 8;
+constexpr uint32_t kSmemBytes = kOffLists + kLists * kMaxListed * 16;
 constexpr uint32_t kSmemAlloc = kSmemBytes;                     // base alignment comes from the declaration
 static_assert(kSmemAlloc <= kMaxSmemBytes, "exceeds the shared memory a CTA may use");
 
@@ -387,13 +390,21 @@ __device__ __noinline__ bool dbg_fail(int* ws_header, int call_id, int code) {
 #define PSA_CHECKED(cond, code) true
 #endif
 
-// Whether block coordinates are those of an edge block (Geom: the last one along the stacked axis).
-__device__ __forceinline__ bool edge_s(const Geom& g, int s) {   // stacked axis h or w
-  return g.sub_axis == 1 ? s >= (g.Hp - 1) * g.Wp : s % g.Wp == g.Wp - 1;
+// The lowest n bits, none if n < 0.
+__device__ __forceinline__ uint32_t low_bits(int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : (1u << n) - 1u); }
+
+// Class of the block at block coordinates (t, s) (EdgeClass).
+__device__ __forceinline__ int block_class(const Geom& g, int t, int s) {
+  int c = 0;
+  if ((g.edge_axes & 1) && t == g.Tp - 1) c |= 1;
+  if ((g.edge_axes & 2) && s >= g.s_edge) c |= 2;
+  if ((g.edge_axes & 4) && s % g.Wp == g.Wp - 1) c |= 4;
+  return c;
 }
-__device__ __forceinline__ bool is_edge_block(const Geom& g, int qb) {
-  if (g.nb_edge == 0) return false;
-  return g.sub_axis == 0 ? qb >= g.NB - g.Sp : edge_s(g, qb % g.Sp);
+// Of spatial block coordinates b .. b + 31, those in the last row, if its blocks are edge blocks.
+__device__ __forceinline__ uint32_t last_row_word(const Geom& g, int b) {
+  const int d = g.s_edge - b;
+  return !(g.edge_axes & 2) || d >= 32 ? 0u : (d <= 0 ? 0xffffffffu : 0xffffffffu << d);
 }
 
 // ----------------------------------------------------------------------------- planning
@@ -437,8 +448,7 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
     if (lane == 0) setT[w] = m;   // setS follows setT
   }
   __syncthreads();
-  // row count of coordinate x: bits n - 1 - x .. 2n - 2 - x of its set; in the upper half-word how many of them are edge
-  // coordinates (the last temporal one, or the spatial ones at the edge; at most 2,048 of either)
+  // row count of coordinate x: bits n - 1 - x .. 2n - 2 - x of its set
   for (int a = threadIdx.x; a < g.Tp + g.Sp; a += kPlanThreads) {
     const bool is_t = a < g.Tp;
     const uint32_t* set = is_t ? setT : setS;
@@ -451,22 +461,12 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
       if (w == (hi - 1) >> 5) m &= 0xffffffffu >> (31 - ((hi - 1) & 31));
       c += __popc(m);
     }
-    int e = 0;
-    if (g.nb_edge != 0 && is_t == (g.sub_axis == 0)) {
-      const int first = is_t ? n - 1 : (g.sub_axis == 1 ? (g.Hp - 1) * g.Wp : g.Wp - 1), step = g.sub_axis == 2 ? g.Wp : 1;
-      for (int b = lo + first; b < hi; b += step) e += (int)(set[b >> 5] >> (b & 31) & 1u);
-    }
-    cntT[a] = (uint32_t)(c | e << 16);   // cntS follows cntT
+    cntT[a] = (uint32_t)c;   // cntS follows cntT
   }
   __syncthreads();
-  // attended edge blocks of block (t, x)
-  auto edge_count = [&](int t, int x) -> int {
-    if (g.nb_edge == 0) return 0;
-    return g.sub_axis != 0 ? (int)((cntT[t] & 0xffffu) * (cntS[x] >> 16)) : (int)((cntT[t] >> 16) * (cntS[x] & 0xffffu));
-  };
   // unique keys: larger count first, then smaller block id (counts are at most NB < 2^16 here)
   for (int qb = threadIdx.x; qb < g.NB; qb += kPlanThreads)
-    key[qb] = (cntT[qb / g.Sp] & 0xffffu) * (cntS[qb % g.Sp] & 0xffffu) * (uint32_t)g.NB + (uint32_t)(g.NB - 1 - qb);
+    key[qb] = cntT[qb / g.Sp] * cntS[qb % g.Sp] * (uint32_t)g.NB + (uint32_t)(g.NB - 1 - qb);
   __syncthreads();
   const int ipb = g.items_per_block;
   // Text-query items of all heads first: they attend every key block, so they are the heaviest (behind the lighter
@@ -476,7 +476,7 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
   for (int it = threadIdx.x; it < g.n_titems; it += kPlanThreads) {
     const int sub0 = 2 * it;
     const int nq = (g.n_ts - sub0) >= 2 ? 2 : 1;
-    head_items[it] = make_int4(h | (g.nb_edge << 8), 0, g.NB - g.nb_edge, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
+    head_items[it] = make_int4(h, 0, g.NB, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24) | (1 << 25));
   }
   WorkItem* out = items + (size_t)gridDim.x * g.n_titems + (size_t)hp.place[h] * (g.items_per_head - g.n_titems);
   for (int qb = threadIdx.x; qb < g.NB; qb += kPlanThreads) {
@@ -487,21 +487,25 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
       pos += (int)(k4.x > mine) + (int)(k4.y > mine) + (int)(k4.z > mine) + (int)(k4.w > mine);
     }
     for (; j < g.NB; ++j) pos += (int)(key[j] > mine);
-    const int c = (int)(mine / (uint32_t)g.NB), ce = edge_count(qb / g.Sp, qb % g.Sp);
-    const bool edge = is_edge_block(g, qb);
-    const int n_sub = edge ? g.n_edge : g.n_sub;
+    const int c = (int)(mine / (uint32_t)g.NB);
+    const int n_sub = g.slabs_of[block_class(g, qb / g.Sp, qb % g.Sp)];
     // two-slab items first (heavier), then the odd single-slab items, each in rank order
     for (int it = 0; it < ipb; ++it) {
       const int sub0 = 2 * it;
       if (sub0 >= n_sub) break;
-      if (it == 1 && g.nb_edge != 0 && (g.n_edge + 1) / 2 < ipb) {   // edge blocks have no second item
-        pos = 0;
-        for (j = 0; j < g.NB; ++j) pos += key[j] > mine && !is_edge_block(g, j);
+      if (it == 1 && g.edge_axes != 0) {   // not all edge blocks have a second item: the rank among the blocks that have one
+        pos = j = 0;
+        for (int tj = 0; tj < g.Tp; ++tj)
+          for (int sj = 0, wj = 0; sj < g.Sp; ++sj, ++j) {
+            const int cj = g.edge_axes & ((tj == g.Tp - 1 ? 1 : 0) | (sj >= g.s_edge ? 2 : 0) | (wj == g.Wp - 1 ? 4 : 0));
+            pos += (int)(g.slabs_of[cj] > 2 && key[j] > mine);
+            wj = wj == g.Wp - 1 ? 0 : wj + 1;
+          }
       }
       const int nq = (n_sub - sub0) >= 2 ? 2 : 1;
       // A single-slab item runs in split-KV mode: both softmax warpgroups work on that one
       // query slab, one on the even and one on the odd key slabs (flag in bit 24).
-      out[(size_t)it * g.NB + pos] = make_int4(h | (ce << 8), qb, c - ce, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
+      out[(size_t)it * g.NB + pos] = make_int4(h, qb, c, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
     }
   }
 }
@@ -654,11 +658,22 @@ __device__ __forceinline__ void softmax_slab(uint32_t tS, uint32_t tO, const uin
   mbar_arrive(bar_ready);
 }
 
-// Token row (within the head) of row `row` of a query slab, or -1 if the row is padding.
-__device__ __forceinline__ long long row_token(const Geom& g, bool textq, int qb, int sub, int row) {
+// Token (within the head) of row `row` of a query slab, or -1 if the row is padding.
+template <bool kBoxes, class Params>
+__device__ __forceinline__ long long row_token(const Params& prm, bool textq, int qb, int sub, int row) {
+  const Geom& g = prm.g;
   if (textq) {   // text slab: rows are consecutive text tokens; they follow the L video tokens
     const int i = sub * kSlabTokens + row;
     return i < g.n_text ? g.L + i : -1;
+  }
+  if constexpr (kBoxes) {
+    const int tb = qb / g.Sp, sb = qb % g.Sp;
+    const EdgeClass& e = prm.cls[block_class(g, tb, sb)];
+    const int r = sub * e.step + row;
+    if (row >= e.step || r >= e.rows) return -1;
+    const int f = r / e.frame, y = r - f * e.frame;
+    const int t = tb * g.bt + f, hh = (sb / g.Wp) * g.bh + (y >> e.lw), ww = (sb % g.Wp) * g.bw + (y & ((1 << e.lw) - 1));
+    return t < g.T && hh < g.H && ww < g.W ? ((long long)t * g.H + hh) * g.W + ww : -1;
   }
   int t0, h0, w0, et, eh, ew, ntok, last;
   slab_origin(g, qb, sub, t0, h0, w0);
@@ -667,9 +682,10 @@ __device__ __forceinline__ long long row_token(const Geom& g, bool textq, int qb
   return (row < ntok && t < g.T && hh < g.H && ww < g.W) ? ((long long)t * g.H + hh) * g.W + ww : -1;
 }
 
-// Item i of a launch without planning (every item runs at once, so their order does not matter); its number of
-// attended key blocks is left to the load warp.
-__device__ __forceinline__ WorkItem direct_item(const Geom& g, int i) {
+// Item i of a launch without planning (every item runs at once, so their order does not matter), by a whole warp; its numbers
+// of attended key blocks are left to key_block_sets.
+template <bool kEdge>
+__device__ __forceinline__ WorkItem direct_item(const Geom& g, int i, int lane) {
   const int n_text_items = g.n_heads * g.n_titems;
   if (i < n_text_items) {
     const int head = i / g.n_titems, sub0 = 2 * (i % g.n_titems);
@@ -680,59 +696,72 @@ __device__ __forceinline__ WorkItem direct_item(const Geom& g, int i) {
   const int per_head = g.items_per_head - g.n_titems;
   const int head = i / per_head, r = i - head * per_head;
   int qb = r, sub0 = 0;
-  if (r >= g.NB) {   // second items (three slabs per block), of edge blocks only if these have them, too
+  if (r >= g.NB) {   // second items of the blocks that have three slabs
     sub0 = 2;
     qb = r - g.NB;
-    if (g.nb_edge != 0 && (g.n_edge + 1) / 2 < g.items_per_block && g.sub_axis != 0) {
-      const int per_row = g.sub_axis == 1 ? (g.Hp - 1) * g.Wp : g.Wp - 1, rows = g.sub_axis == 1 ? g.Sp : g.Wp;
-      qb = qb / per_row * rows + qb % per_row;
+    if (kEdge) {
+      int skip = qb;   // such blocks in front of it
+      for (int b = 0; b < g.NB; b += 32) {
+        const int j = b + lane;
+        uint32_t m = __ballot_sync(0xffffffffu, j < g.NB && g.slabs_of[block_class(g, j / g.Sp, j % g.Sp)] > 2);
+        if (skip >= __popc(m)) { skip -= __popc(m); continue; }
+        for (; skip > 0; --skip) m &= m - 1;
+        qb = b + __ffs(m) - 1;
+        break;
+      }
     }
   }
-  const int n_sub = is_edge_block(g, qb) ? g.n_edge : g.n_sub;
+  const int n_sub = kEdge ? g.slabs_of[block_class(g, qb / g.Sp, qb % g.Sp)] : g.n_sub;
   const int nq = (n_sub - sub0) >= 2 ? 2 : 1;
   return make_int4(head, qb, 0, sub0 | (nq << 16) | ((nq == 1 ? 1 : 0) << 24));
 }
 
-// Words b / 32 of the two temporal (spatial) sets: without and with the edge coordinates of `m`.  The axis that edge blocks
-// are not told by goes into both.
-__device__ __forceinline__ void store_set_t(const Geom& g, uint32_t* maskT, int b, uint32_t m) {
-  const uint32_t e = b == ((g.Tp - 1) & ~31) ? 1u << ((g.Tp - 1) & 31) : 0u;
-  const bool by_t = g.nb_edge != 0 && g.sub_axis == 0;
-  maskT[b >> 5] = by_t ? m & ~e : m;
-  maskT[kMaxTp / 32 + (b >> 5)] = by_t ? m & e : m;
-}
-__device__ __forceinline__ void store_set_s(const Geom& g, uint32_t* maskS, int b, uint32_t m, uint32_t e) {
-  maskS[b >> 5] = m & ~e;
-  maskS[kMaxSp / 32 + (b >> 5)] = g.sub_axis != 0 ? m & e : m;
-}
+// Numbers of attended block coordinates, packed: temporal ones without and with the edge one (16 bits each); spatial ones of classes
+// 0 and 2, and of classes 4 and 6.
+struct Attended {
+  uint32_t t, s, s4;
+  __device__ __forceinline__ int blocks(int c) const {
+    const uint32_t x = c & 4 ? s4 : s;
+    return (int)((c & 1 ? t >> 16 : t & 0xffffu) * (c & 2 ? x >> 16 : x & 0xffffu));
+  }
+};
 
-// Attended key-block coordinates of an item's query block (all of them for text queries), one bit per block coordinate,
-// by a whole warp; completes the item's numbers of attended key blocks.
-__device__ __forceinline__ void key_block_sets(const Geom& g, WorkItem& wi, const psa_head_params p, int lane, uint32_t* maskT,
-                                              uint32_t* maskS) {
-  const bool textq = ((wi.w >> 25) & 1) != 0;
-  const int tq = wi.y / g.Sp, sq = wi.y % g.Sp;
-  int cnt_t = 0, cnt_s = 0, edge_t = 0, edge_s_cnt = 0;
+// Attended key-block coordinates of an item's query block (all of them for text queries), one bit per block coordinate, by a
+// whole warp; spatial coordinates in the last column behind the others if these are edge blocks.
+template <bool kEdge>
+__device__ __forceinline__ Attended key_block_sets(const Geom& g, bool textq, int qb, const psa_head_params& p, int lane, uint32_t* maskT,
+                                                   uint32_t* maskS) {
+  const int tq = qb / g.Sp, sq = qb % g.Sp;
+  Attended a = {0u, 0u, 0u};
   for (int b = 0; b < g.Tp; b += 32) {
     const int tk = b + lane;
     const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
-    if (lane == 0) store_set_t(g, maskT, b, m);
-    cnt_t += __popc(m);
-    if (b == ((g.Tp - 1) & ~31)) edge_t = (int)(m >> ((g.Tp - 1) & 31) & 1u);
+    if (lane == 0) maskT[b >> 5] = m;
+    a.t += (uint32_t)__popc(m);
+    if (kEdge && (g.edge_axes & 1) && b == ((g.Tp - 1) & ~31)) a.t += (m >> ((g.Tp - 1) & 31) & 1u) * 0xffffu;   // one from the lower to the upper half
   }
   for (int b = 0; b < g.Sp; b += 32) {
     const int sk = b + lane;
     const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
-    const unsigned e = g.nb_edge != 0 && g.sub_axis != 0 ? __ballot_sync(0xffffffffu, sk < g.Sp && edge_s(g, sk)) : 0u;
-    if (lane == 0) store_set_s(g, maskS, b, m, e);
-    cnt_s += __popc(m);
-    edge_s_cnt += __popc(e & m);
+    if (!kEdge) {
+      if (lane == 0) maskS[b >> 5] = m;
+      a.s += (uint32_t)__popc(m);
+      continue;
+    }
+    const unsigned col = g.edge_axes & 4 ? __ballot_sync(0xffffffffu, sk % g.Wp == g.Wp - 1) : 0u, row = last_row_word(g, b);
+    if (lane == 0) {
+      maskS[b >> 5] = m & ~col;
+      maskS[kMaxSp / 32 + (b >> 5)] = m & col;
+    }
+    a.s += (uint32_t)(__popc(m & ~col & ~row) | __popc(m & ~col & row) << 16);
+    a.s4 += (uint32_t)(__popc(m & col & ~row) | __popc(m & col & row) << 16);
   }
   __syncwarp();
-  const int edge = g.nb_edge == 0 ? 0 : (g.sub_axis == 0 ? edge_t * cnt_s : cnt_t * edge_s_cnt);
-  wi.z = cnt_t * cnt_s - edge;
-  wi.x |= edge << 8;
+  return a;
 }
+
+// Slabs of `n` edge blocks of a class.
+__device__ __forceinline__ int class_slabs(const EdgeClass& e, int n) { return e.together > 1 ? (n + e.together - 1) / e.together : n * e.n_slabs; }
 
 // Cluster mode: CTA d of the cluster merges query rows d * rpc .. (d + 1) * rpc - 1 of the item (rpc = nq * 128 /
 // cluster size), and every CTA pushes its partial results of those rows into d's shared memory: (m, l, lr) to
@@ -750,7 +779,8 @@ __device__ __forceinline__ Share share_of_row(uint32_t sbase, int r, int nq) {
 
 // The merge itself, by the softmax warpgroups, once all partial results have arrived: sums over the sources in a fixed
 // order, out and lse written.
-__device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8_t* smem) {
+template <class Params>
+__device__ __forceinline__ void merge_cluster(const Params& prm, const uint8_t* smem) {
   const Geom& g = prm.g;
   const int4 wi = *reinterpret_cast<const int4*>(smem + kOffSched);   // the item as the load warp published it
   const int head = wi.x & 0xff, nq = (wi.w >> 16) & 0xff;
@@ -803,20 +833,30 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& prm, const uint8
 //   kSharedDirect   the same without planning
 // (Separate instantiations: the ticket kernel's slab loop is sensitive to what else is compiled with it -- one kernel
 // with the mode as an argument was 1.5 to 2 % slower on the 720p layers.)
-//   kTicketEdge   kTicket for grids with edge blocks, kTicket itself being for grids without
-//   kTicketShort  kTicket for short items of blocks of one slab (which have no edge blocks): bound by what lies between two
+//   kTicketShort  kTicket for short items of blocks of one slab: bound by what lies between two
 //                 items, so the next item's loads and Q K^T run while the last one is still being written out.  The query
 //                 buffers are released by the MMAs that read them last (a commit), the output goes from registers to
 //                 memory instead of through those buffers, and the accumulators are waited for at the first P V only.
 //                 12 heads of 1x8x16 blocks attending 19.5 of them, 8x32x48 grid: 221 -> 198 us
-template <int kMode>
+// kGrid: what the grid's edge asks for.
+//   kWhole    nothing: the block divides the grid, and no slab has padding except beyond the text
+//   kPadded   blocks at the edge have the slabs of ordinary ones, or fewer; padding is masked
+//   kCut      some blocks at the edge are cut to their tokens (EdgeClass)
+// (A slab of a cut grid goes through a list of boxes, which costs the load warp some 700 clocks: more than it has in split-KV mode.
+// 2 heads of 5x16x63 with 1x30x8 blocks, one slab each, took 28.6 us as a cut grid and take 23.6 as a padded one.)
+template <int kGrid> struct ArgsOf { typedef TensorMaps maps; typedef AttnParamsEdge params; };
+template <> struct ArgsOf<kWhole> { typedef TensorMaps maps; typedef AttnParams params; };
+template <> struct ArgsOf<kCut> { typedef TensorMapsEdge maps; typedef AttnParamsEdge params; };
+template <int kMode, int kGrid>
 __global__ void __launch_bounds__(kThreads, 1)
-attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ HeadParamsArray heads, const AttnParams prm) {
+attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const __grid_constant__ HeadParamsArray heads,
+                const __grid_constant__ typename ArgsOf<kGrid>::params prm) {
   // 128-byte swizzled slabs need a 1024-byte aligned base; the declaration asks for it and the
   // kernel checks it (a misaligned base is reported through the status word, no work is done).
   constexpr bool kCluster = kMode == kShared || kMode == kSharedDirect, kShort = kMode == kTicketShort;
-  constexpr bool kDraws = kMode == kTicket || kMode == kTicketEdge || kShort;
-  constexpr bool kPlanned = kDraws || kMode == kShared, kEdge = kMode != kTicket && !kShort;
+  constexpr bool kEdge = kGrid != kWhole, kBoxes = kGrid == kCut;
+  constexpr bool kDraws = kMode == kTicket || kShort;
+  constexpr bool kPlanned = kDraws || kMode == kShared;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
   const uint32_t sbase = smem_u32(smem);
@@ -825,7 +865,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
 
   auto bar = [&](int idx) -> uint32_t { return sbase + kOffBar + 8u * (uint32_t)idx; };
   uint32_t* meta = reinterpret_cast<uint32_t*>(smem + kOffMeta);
-  // attended key-block coordinates of the item being loaded; the sets of edge blocks behind the others'
+  // attended key-block coordinates of the item being loaded
   uint32_t* maskT = reinterpret_cast<uint32_t*>(smem + kOffMaskT);
   uint32_t* maskS = reinterpret_cast<uint32_t*>(smem + kOffMaskS);
   volatile int4* sched = reinterpret_cast<volatile int4*>(smem + kOffSched);
@@ -833,7 +873,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
 
   // A short query slab leaves its last rows of the Q buffer unwritten; keep them finite.
-  if (kDraws || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
+  if (kDraws || kEdge || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
     for (uint32_t off = threadIdx.x * 16u; off < 2u * kSlabBytes; off += kThreads * 16u)
       *reinterpret_cast<uint4*>(smem + kOffQ + off) = make_uint4(0u, 0u, 0u, 0u);
     fence_async_smem();
@@ -865,10 +905,11 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
   if (threadIdx.x == 0) pdl_trigger();
   // Without planning the load warp works its item out here, alongside the rest of the set-up (1.5 us earlier).
   WorkItem first_item = make_int4(-1, 0, 0, 0);
+  Attended attended = {0u, 0u, 0u};   // (load warp) by the item's query block
   if constexpr (!kPlanned) {
     if (warp == kWarpLoad) {
-      first_item = direct_item(g, (int)(blockIdx.x / cluster_size()));
-      key_block_sets(g, first_item, heads.p[first_item.x], lane, maskT, maskS);
+      first_item = direct_item<kEdge>(g, (int)(blockIdx.x / cluster_size()), lane);
+      attended = key_block_sets<kEdge>(g, ((first_item.w >> 25) & 1) != 0, first_item.y, heads.p[first_item.x], lane, maskT, maskS);
     }
   }
   // A persistent CTA has one idle thread wait for the kernel before, on behalf of every role behind the barrier.  (Waits in
@@ -914,21 +955,32 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     // Ring tiles are issued in the order K_0, V_0, K_1, V_1, ...; the MMA warp needs V_j and
     // K_{j+1} at the same moment, so those two travel under one "pair" barrier
     // (K_0 and the last V of an item travel alone).
-    uint32_t tile_g = 0;       // ring tiles issued so far
+    uint32_t slot_i = 0, slot_ph = 1;   // ring slot of the next tile and the parity its wait needs; pair barrier of the next arrival
+    uint32_t pair_i = 0;
     uint32_t pair_g = 0;       // pair barriers armed so far
     uint32_t kv_g = 0;         // key slabs issued so far
     uint32_t it_q0 = 0, it_q1 = 0; // items in which query slab i was active
-    // Position of key c = lane + 32 i within a slab, t << 16 | h << 8 | w, for the validity words of slabs at the grid's
+    // kPadded: position of key c = lane + 32 i within a slab, t << 16 | h << 8 | w, for the validity words of slabs at the grid's
     // edge (a block's last slab is only shorter along its slowest axis, so it is laid out alike).  Computed once: with
     // its divisions in the slab loop this warp took 3,800 clocks per edge slab and the whole CTA waited for it.
     int pos[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 4 && kGrid == kPadded; ++i) {
       const int c = lane + 32 * i;
       pos[i] = (c / (g.cw * g.ch)) << 16 | ((c / g.cw) % g.ch) << 8 | (c % g.cw);
     }
     // block -> row of the spatial block grid without a division: sk, Wp <= 2^11
     const uint32_t magic_w = ((1u << 22) + (uint32_t)g.Wp - 1u) / (uint32_t)g.Wp;
+    auto class_at = [&](int i) -> int {
+      if constexpr (kEdge) return prm.order[i];
+      return 0;
+    };
+    int n_classes = 1;
+    if constexpr (kEdge) n_classes = prm.n_classes;
+    auto block_rows = [&](int c) -> int {
+      if constexpr (kEdge) return prm.cls[c].rows;
+      return g.bt * g.bh * g.bw;
+    };
     bool ok = tmem_ok;
     pdl_wait();   // the work items are written by the planning kernel, q, k and v by whatever ran before
     for (uint32_t n = 0; ok; ++n) {
@@ -936,20 +988,42 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       ok = mbar_wait_warp(bar(kBarSchedEmpty + sslot), ((n >> 1) & 1u) ^ 1u, abort_flag, 0x401);
       if (!ok) break;
       WorkItem wi = make_int4(-1, 0, 0, 0);
-      int skip = 0, left = 0x7fffffff;   // attended key blocks before this CTA's share, and those still to load
-      // This CTA's share of the item's attended key blocks; the text keys go with the last share.
-      auto take_share = [&]() {
+      // The attended blocks of class c that are this CTA's (all of them, or its share: by rows, cut between blocks; text keys go with
+      // the last share), and how many others come before them.  `before`: rows of the classes before, carried along.
+      auto blocks_of = [&](int c, long long all, long long& before, int* skip) -> int {
+        const int n = attended.blocks(c);
+        *skip = 0;
         if constexpr (kCluster) {
-          const int r = (int)cluster_rank(), c = (int)cluster_size();
-          if (wi.x < 0) return;
-          const int main = wi.z, all = main + (wi.x >> 8);   // edge blocks come last
-          skip = (int)((long long)all * r / c);
-          const int end = (int)((long long)all * (r + 1) / c);
-          left = end - skip;
-          wi.z = max(min(end, main) - skip, 0);
-          wi.x = (wi.x & 0xff) | (left - wi.z) << 8;
-          if (r + 1 < c) wi.w |= 1 << 26;
+          const int per = block_rows(c), r = (int)cluster_rank(), size = (int)cluster_size();
+          auto upto = [&](long long rows) -> int { return rows <= before ? 0 : (int)min((rows - before) / per, (long long)n); };
+          const int from = upto(all * r / size), to = upto(all * (r + 1) / size);
+          before += (long long)n * per;
+          *skip = from;
+          return to - from;
         }
+        return n;
+      };
+      long long all_rows = 0;
+      auto take_share = [&]() {   // (every lane)
+        if constexpr (kCluster) {
+          for (int i = 0; i < n_classes; ++i) all_rows += (long long)attended.blocks(class_at(i)) * block_rows(class_at(i));
+          if (cluster_rank() + 1 < cluster_size()) wi.w |= 1 << 26;
+        }
+        long long before = 0;
+        int edge_slabs = 0, skip;
+        wi.z = 0;
+#pragma unroll 1
+        for (int i = 0; i < n_classes; ++i) {
+          const int c = class_at(i), n = blocks_of(c, all_rows, before, &skip);
+          if constexpr (kEdge) {
+            if (!prm.cls[c].in_pattern) {
+              edge_slabs += n ? class_slabs(prm.cls[c], n) : 0;
+              continue;
+            }
+          }
+          wi.z += n;
+        }
+        if (kEdge) wi.x |= edge_slabs << 8;
       };
       auto publish = [&]() {   // by lane 0
         sched[sslot].x = wi.x; sched[sslot].y = wi.y; sched[sslot].z = wi.z; sched[sslot].w = wi.w;
@@ -959,14 +1033,17 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         if (lane == 0) {
           const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
           if (ticket < prm.n_items) wi = prm.items[ticket];
-          publish();
+          if (!kEdge) publish();
         }
         wi.x = __shfl_sync(0xffffffffu, wi.x, 0);
         wi.y = __shfl_sync(0xffffffffu, wi.y, 0);
         wi.w = __shfl_sync(0xffffffffu, wi.w, 0);
-      } else {
-        if (n == 0) wi = kPlanned ? prm.items[blockIdx.x / cluster_size()] : first_item;
-        take_share();
+      } else if (n == 0) {
+        wi = kPlanned ? prm.items[blockIdx.x / cluster_size()] : first_item;
+      }
+      if (kPlanned && wi.x >= 0) attended = key_block_sets<kEdge>(g, ((wi.w >> 25) & 1) != 0, wi.y, prm.hp_dev[wi.x], lane, maskT, maskS);
+      if (kEdge || !kDraws) {
+        if (wi.x >= 0) take_share();
         if (lane == 0) publish();
       }
       if (wi.x < 0) break;
@@ -980,32 +1057,39 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       const int lag = ((wi.w >> 24) & 1) ? 2 : 1;   // V_j travels with K_{j+lag} (2 in split-KV mode)
       const bool textq = ((wi.w >> 25) & 1) != 0;   // the queries are text tokens: every key is attended
       const int head_ld = prm.shared_qkv ? 0 : head;   // head coordinate of the q, k, v loads
-      auto eval_masks = [&]() {
-        const psa_head_params p = prm.hp_dev[head];
-        const int tq = qb / g.Sp, sq = qb % g.Sp;
-        // attended key-block coordinates of this query block, one bit per block coordinate
-        for (int b = 0; b < g.Tp; b += 32) {
-          const int tk = b + lane;
-          const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
-          if (!kEdge || g.nb_edge == 0) {
-            if (lane == 0) maskT[b >> 5] = m;
-          } else {
-            if (lane == 0) store_set_t(g, maskT, b, m);
-          }
+      // A box into a tile, at a multiple of 8 rows.
+      auto load_box = [&](uint32_t dst, const CUtensorMap* map, uint32_t pb, int t, int h, int w) {
+        tma_load_5d(dst, map, pb, 0, w, h, t, head_ld);
+        tma_load_5d(dst + kHalfBytes, map, pb, 64, w, h, t, head_ld);
+      };
+      // kBoxes: every slab is a list of boxes; list `list` is the one being made.
+      int4* lists = reinterpret_cast<int4*>(smem + kOffLists);
+      int list = 0;
+      // The first nv boxes of list lv into a tile of V, the first nk of list lk into one of K (or of Q), by a whole warp.  The lists
+      // are read at once, by box_of: a shared-memory round trip takes 150 to 450 clocks while the tensor core is busy.
+      auto box_of = [&](int lv, int lk) -> int4 { return lists[(lane < kMaxListed ? lv : lk) * kMaxListed + (lane & (kMaxListed - 1))]; };
+      auto load_lists = [&](const int4& mine, uint32_t pb, const CUtensorMap* maps_v, uint32_t dv, int nv, const CUtensorMap* maps_k, uint32_t dk, int nk) {
+#pragma unroll 1
+        for (int b = 0; b < nv + nk; ++b) {
+          const int from = b < nv ? b : kMaxListed + b - nv;
+          const int w = __shfl_sync(0xffffffffu, mine.x, from), h = __shfl_sync(0xffffffffu, mine.y, from), t = __shfl_sync(0xffffffffu, mine.z, from),
+                    to = __shfl_sync(0xffffffffu, mine.w, from);
+          if (lane == 0 && PSA_CHECKED(nv <= kMaxListed && nk <= kMaxListed && (to & 255) < kMaxMaps && (to >> 8) < 16 && w >= 0 && h >= 0 && t >= 0 && t <= g.T, 0xD07))
+            load_box((b < nv ? dv : dk) + ((uint32_t)to >> 8) * 1024u, (b < nv ? maps_v : maps_k) + (to & 255), pb, t, h, w);
         }
-        for (int b = 0; b < g.Sp; b += 32) {
-          const int sk = b + lane;
-          const unsigned m = __ballot_sync(0xffffffffu, sk < g.Sp && (textq || axis_attends(sk - sq, p.Sw, p.So, p.Ss)));
-          if (!kEdge || g.nb_edge == 0) {
-            if (lane == 0) maskS[b >> 5] = m;
-          } else {
-            const unsigned e = g.sub_axis != 0 ? __ballot_sync(0xffffffffu, sk < g.Sp && edge_s(g, sk)) : 0u;
-            if (lane == 0) store_set_s(g, maskS, b, m, e);
-          }
+      };
+      // The boxes of slab `sub` of a block; their number.
+      auto list_boxes = [&](const EdgeClass& e, int sub, int t0, int h0, int w0) -> int {
+        const int first = e.first_box[sub], n = e.first_box[sub + 1] - first;
+        if (lane < n) {
+          const EdgeBox x = e.box[first + lane];
+          const int4 zeros = make_int4(0, 0, g.T, x.row8 << 8 | x.map);
+          lists[list * kMaxListed + lane] = x.t == kZeros ? zeros : make_int4(w0 + x.w, h0 + x.h, t0 + x.t, zeros.w);
         }
         __syncwarp();
+        return n;
       };
-      if constexpr (kPlanned) eval_masks();
+      const int qcls = kBoxes && !textq ? block_class(g, qb / g.Sp, qb % g.Sp) : 0;
       // query slabs
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -1013,8 +1097,19 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         const uint32_t itq = i == 0 ? it_q0 : it_q1;
         ok = mbar_wait_warp(bar(kBarQEmpty + i), (itq & 1u) ^ 1u, abort_flag, 0x100 + i);
         if (!ok) break;
-        if (lane == 0) {
-          int t0, h0, w0, et, eh, ew, ntok, last;
+        int t0, h0, w0, et, eh, ew, ntok, last, n_boxes = 0;
+        if constexpr (kBoxes) {
+          if (!textq) {
+            const EdgeClass& e = prm.cls[qcls];
+            slab_origin(g, qb, 0, t0, h0, w0);
+            n_boxes = list_boxes(e, sub0 + i, t0, h0, w0);
+            const bool whole = sub0 + i + 1 < e.n_slabs || !(e.in_pattern || e.together > 1);
+            if (e.together > 1) n_boxes = 1;   // (a block alone: no box of zeros)
+            if (lane == 0) mbar_expect_tx(bar(kBarQFull + i), whole ? kSlabBytes : (uint32_t)(e.together > 1 ? e.rows : prm.main_last) * 256u);
+            load_lists(box_of(list, list), bar(kBarQFull + i), tms.q, 0u, 0, tms.q, sbase + kOffQ + (uint32_t)i * kSlabBytes, n_boxes);
+          }
+        }
+        if (lane == 0 && n_boxes == 0) {   // (n_boxes: kBoxes, video queries)
           if (textq) {   // text slab: 128 tokens from the text map, token index in the second coordinate
             t0 = 0; h0 = 0; w0 = (sub0 + i) * kSlabTokens; ntok = kSlabTokens; last = 2;
           } else {
@@ -1026,8 +1121,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
                           ntok > 0 && ntok <= kSlabTokens &&
                           (textq || (w0 < g.Wp * g.bw && h0 < g.Hp * g.bh && t0 < g.Tp * g.bt)), 0xD01)) {   // inside the padded grid
             mbar_expect_tx(bar(kBarQFull + i), (uint32_t)ntok * 256u);
-            tma_load_5d(dst, &tms.q[last], bar(kBarQFull + i), 0, w0, h0, t0, head_ld);
-            tma_load_5d(dst + kHalfBytes, &tms.q[last], bar(kBarQFull + i), 64, w0, h0, t0, head_ld);
+            load_box(dst, &tms.q[last], bar(kBarQFull + i), t0, h0, w0);
           }
         }
         if (i == 0) ++it_q0; else ++it_q1;
@@ -1035,42 +1129,31 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       if (!ok) break;
       // key / value slabs in ascending key-block id.  Up to `lag` slabs wait for their V load.
       int npend = 0;
-      int at0 = 0, ah0 = 0, aw0 = 0, alast = 0, antok = kSlabTokens;  // oldest pending slab
+      int at0 = 0, ah0 = 0, aw0 = 0, alast = 0, antok = kSlabTokens;  // oldest pending slab (kBoxes: at0 boxes)
       int bt0 = 0, bh0 = 0, bw0 = 0, blast = 0, bntok = kSlabTokens;  // newer pending slab (lag 2)
-      // One key slab: K now, V of the slab issued `lag` slabs earlier under the same barrier.
-      auto issue_slab = [&](int t0, int h0, int w0, int last, int ntok, uint32_t vw0, uint32_t vw1, uint32_t vw2,
-                            uint32_t vw3) {
-        // slots: [V of the oldest pending slab,] K of this slab
-        const bool with_v = (npend == lag);
-        const uint32_t v_slot = tile_g % kNumSlots, v_use = tile_g / kNumSlots;
-        const uint32_t k_tile = tile_g + (with_v ? 1u : 0u);
-        const uint32_t k_slot = k_tile % kNumSlots, k_use = k_tile / kNumSlots;
-        if (with_v) {
-          ok = mbar_wait_warp(bar(kBarSlotEmpty + v_slot), (v_use & 1u) ^ 1u, abort_flag, 0x111);
-          if (!ok) return;
-        }
-        ok = mbar_wait_warp(bar(kBarSlotEmpty + k_slot), (k_use & 1u) ^ 1u, abort_flag, 0x110);
-        if (!ok) return;
-        if (lane == 0 && PSA_CHECKED(v_slot < (uint32_t)kNumSlots && k_slot < (uint32_t)kNumSlots && t0 >= 0 && h0 >= 0 && w0 >= 0 &&
-                                     last >= 0 && last <= 2 && ntok > 0 && ntok <= kSlabTokens &&
-                                     (!with_v || (at0 >= 0 && ah0 >= 0 && aw0 >= 0 && alast >= 0 && alast <= 2)), 0xD02)) {
-          uint32_t* m = meta + (kv_g % kMetaRing) * 8;
-          m[0] = vw0; m[1] = vw1; m[2] = vw2; m[3] = vw3;
-          const uint32_t pb = bar(kBarPairFull + pair_g % kNumPairBars);
-          mbar_expect_tx(pb, (uint32_t)((with_v ? antok : 0) + ntok) * 256u);
-          if (with_v) {
-            const uint32_t dv = sbase + kOffRing + v_slot * kSlabBytes;
-            tma_load_5d(dv, &tms.v[alast], pb, 0, aw0, ah0, at0, head_ld);
-            tma_load_5d(dv + kHalfBytes, &tms.v[alast], pb, 64, aw0, ah0, at0, head_ld);
-          }
-          const uint32_t dk = sbase + kOffRing + k_slot * kSlabBytes;
-          tma_load_5d(dk, &tms.k[last], pb, 0, w0, h0, t0, head_ld);
-          tma_load_5d(dk + kHalfBytes, &tms.k[last], pb, 64, w0, h0, t0, head_ld);
-        }
-        tile_g = k_tile + 1;
+      // Slots of the next tiles, V of the oldest pending slab (if it is due) and K of the new one.
+      bool with_v;
+      uint32_t v_slot, k_slot, k_par;
+      auto slot_next = [&](uint32_t sl, uint32_t& ph) -> uint32_t {
+        ph ^= sl + 1u == (uint32_t)kNumSlots ? 1u : 0u;
+        return sl + 1u == (uint32_t)kNumSlots ? 0u : sl + 1u;
+      };
+      auto wait_slots = [&]() {
+        with_v = npend == lag;
+        const uint32_t v_par = slot_ph;
+        v_slot = k_slot = slot_i;
+        k_par = slot_ph;
+        if (with_v) k_slot = slot_next(k_slot, k_par);
+        ok = with_v ? mbar_wait2_warp(bar(kBarSlotEmpty + v_slot), v_par, bar(kBarSlotEmpty + k_slot), k_par, abort_flag, 0x111, 0x110)
+                    : mbar_wait_warp(bar(kBarSlotEmpty + k_slot), k_par, abort_flag, 0x110);
+      };
+      // The tiles are on their way: queue this slab's V.
+      auto issued = [&](int t0, int h0, int w0, int last, int ntok) {
+        slot_ph = k_par;
+        slot_i = slot_next(k_slot, slot_ph);
         ++pair_g;
+        pair_i = pair_i + 1u == (uint32_t)kNumPairBars ? 0u : pair_i + 1u;
         ++kv_g;
-        // queue this slab's V
         if (with_v) {
           if (lag == 2) { at0 = bt0; ah0 = bh0; aw0 = bw0; alast = blast; antok = bntok; }
           --npend;
@@ -1079,47 +1162,135 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         else { bt0 = t0; bh0 = h0; bw0 = w0; blast = last; bntok = ntok; }
         ++npend;
       };
-      // (edge blocks, which have fewer slabs, in a second pass)
-      for (int pass = 0; pass < (kEdge && g.nb_edge != 0 ? 2 : 1); ++pass) {
-      const uint32_t *mask_t = maskT + pass * (kMaxTp / 32), *mask_s = maskS + pass * (kMaxSp / 32);
-      const int n_slabs = kEdge && pass != 0 ? g.n_edge : g.n_sub;
+      // One key slab: K now, V of the slab issued `lag` slabs earlier under the same barrier.
+      auto issue_slab = [&](int t0, int h0, int w0, int last, int ntok, uint32_t vw0, uint32_t vw1, uint32_t vw2,
+                            uint32_t vw3) {
+        wait_slots();
+        if (!ok) return;
+        if (lane == 0 && PSA_CHECKED(v_slot < (uint32_t)kNumSlots && k_slot < (uint32_t)kNumSlots && t0 >= 0 && h0 >= 0 && w0 >= 0 &&
+                                     last >= 0 && last <= 2 && ntok > 0 && ntok <= kSlabTokens &&
+                                     (!with_v || (at0 >= 0 && ah0 >= 0 && aw0 >= 0 && alast >= 0 && alast <= 2)), 0xD02)) {
+          uint32_t* m = meta + (kv_g % kMetaRing) * 8;
+          m[0] = vw0; m[1] = vw1; m[2] = vw2; m[3] = vw3;
+          const uint32_t pb = bar(kBarPairFull + pair_i);
+          mbar_expect_tx(pb, (uint32_t)((with_v ? antok : 0) + ntok) * 256u);
+          if (with_v) load_box(sbase + kOffRing + v_slot * kSlabBytes, &tms.v[alast], pb, at0, ah0, aw0);
+          load_box(sbase + kOffRing + k_slot * kSlabBytes, &tms.k[last], pb, t0, h0, w0);
+        }
+        issued(t0, h0, w0, last, ntok);
+      };
+      // The same for the slab of the n boxes of the list; vw: word `lane` of its validity bits, in lanes 0 to 3.
+      auto issue_list = [&](int n, int ntok, uint32_t vw) {
+        __syncwarp();
+        const int4 mine = box_of(list < lag ? list + kLists - lag : list - lag, list);
+        wait_slots();
+        if (!ok) return;
+        if (lane < 4) meta[(kv_g % kMetaRing) * 8 + lane] = vw;
+        __syncwarp();
+        if (PSA_CHECKED(v_slot < (uint32_t)kNumSlots && k_slot < (uint32_t)kNumSlots && ntok > 0 && ntok <= kSlabTokens, 0xD09)) {
+          const uint32_t pb = bar(kBarPairFull + pair_i);
+          if (lane == 0) mbar_expect_tx(pb, (uint32_t)((with_v ? antok : 0) + ntok) * 256u);
+          load_lists(mine, pb, tms.v, sbase + kOffRing + v_slot * kSlabBytes, with_v ? at0 : 0, tms.k, sbase + kOffRing + k_slot * kSlabBytes, n);
+        }
+        issued(n, 0, 0, 0, ntok);
+        list = list == kLists - 1 ? 0 : list + 1;
+      };
+      // classes in turn
+      long long before = 0;
+#pragma unroll 1
+      for (int ci = 0; ok && ci < n_classes; ++ci) {
+      const int c = class_at(ci);
+      int skip, left = blocks_of(c, all_rows, before, &skip);   // blocks before this CTA's share, and those still to load
+      const uint32_t* mask_s = maskS + (kEdge && (c & 4) ? kMaxSp / 32 : 0);
+      int listed = 0;
+      // The class in registers (constants by a computed index are slow): lane b holds box b, lane 4 s + i word i of slab s's validity.
+      int rows = 0, n_slabs = 1, together = 1, n_full = 0;
+      uint32_t first_box = 0, valid = 0, last_keys = kSlabTokens;
+      EdgeBox mine_box = {};
+      if constexpr (kEdge) n_slabs = prm.cls[c].n_slabs;
+      else n_slabs = g.n_sub;
+      if constexpr (kBoxes) {
+        const EdgeClass& e = prm.cls[c];
+        rows = e.rows;
+        together = e.together;
+        n_full = e.together + e.n_boxes - 1;
+        first_box = *reinterpret_cast<const uint32_t*>(e.first_box);
+        if (e.in_pattern) last_keys = (uint32_t)prm.main_last;
+        if (lane < 12) valid = e.valid[lane >> 2][lane & 3];
+        if (lane < kMaxEdgeBoxes) mine_box = e.box[lane];
+      }
       for (int tw = 0; ok && left > 0 && tw < g.Tp; tw += 32) {
-        uint32_t mt = mask_t[tw >> 5];
+        uint32_t mt = maskT[tw >> 5];
+        if (kEdge && (g.edge_axes & 1)) {
+          const uint32_t edge = tw == ((g.Tp - 1) & ~31) ? 1u << ((g.Tp - 1) & 31) : 0u;
+          mt &= c & 1 ? edge : ~edge;
+        }
         while (ok && left > 0 && mt) {
           const int tk = tw + __ffs(mt) - 1;
           mt &= mt - 1;
           for (int sw = 0; ok && left > 0 && sw < g.Sp; sw += 32) {
             uint32_t ms = mask_s[sw >> 5];
+            if (kEdge) ms &= c & 2 ? last_row_word(g, sw) : ~last_row_word(g, sw);
             while (ok && ms) {
               const int sk = sw + __ffs(ms) - 1;
               ms &= ms - 1;
               if constexpr (kCluster) {
                 if (skip > 0) { --skip; continue; }
                 if (left == 0) break;
-                --left;
               }
+              if (kCluster || kEdge) --left;
               const int hb = (int)(((unsigned long long)(uint32_t)sk * magic_w) >> 22);
               int t0 = tk * g.bt, h0 = hb * g.bh, w0 = (sk - hb * g.Wp) * g.bw;
+              if constexpr (kBoxes) {
+                int4* const to = lists + list * kMaxListed;
+                if (together > 1) {
+                  if (lane == 0 && PSA_CHECKED(listed < kMaxListed && list < kLists, 0xD06)) to[listed] = make_int4(w0, h0, t0, listed * rows << 5 | mine_box.map);
+                  if (++listed < together && left > 0) continue;
+                  // zeros in the place of what a full slab has more of
+                  const int map0 = __shfl_sync(0xffffffffu, (int)mine_box.map, 0);
+                  if (lane >= listed && lane < together) to[lane] = make_int4(0, 0, g.T, lane * rows << 5 | map0);
+                  if (lane == 1 && n_full > together) to[together] = make_int4(0, 0, g.T, mine_box.row8 << 8 | mine_box.map);
+                }
+#pragma unroll 1
+                for (int sub = 0; ok && sub < n_slabs; ++sub) {
+                  const int first = (int)(first_box >> (8 * sub) & 255u);
+                  int n = (int)(first_box >> (8 * sub + 8) & 255u) - first;
+                  uint32_t vw = __shfl_sync(0xffffffffu, valid, 4 * sub + (lane & 3));
+                  if (together > 1) {
+                    n = n_full;
+                    vw &= low_bits(listed * rows - 32 * (lane & 3));
+                    listed = 0;
+                  } else if (lane >= first && lane < first + n) {
+                    const bool zeros = mine_box.t == kZeros;
+                    lists[list * kMaxListed + lane - first] = make_int4(zeros ? 0 : w0 + mine_box.w, zeros ? 0 : h0 + mine_box.h, zeros ? g.T : t0 + mine_box.t,
+                                                                        mine_box.row8 << 8 | mine_box.map);
+                  }
+                  issue_list(n, sub + 1 == n_slabs ? (int)last_keys : kSlabTokens, vw);
+                }
+              } else {
               for (int sub = 0; ok && sub < n_slabs; ++sub) {
                 const int last = (sub == g.n_sub - 1) ? 1 : 0, ntok = last ? g.n_last : kSlabTokens;
-                const int et = last && g.sub_axis == 0 ? g.c_last : g.ct, eh = last && g.sub_axis == 1 ? g.c_last : g.ch,
-                          ew = last && g.sub_axis == 2 ? g.c_last : g.cw;
                 // validity of the slab's key positions (3D-padding): bit c of word c/32; ones beyond a short slab
                 uint32_t vw0 = 0xffffffffu, vw1 = 0xffffffffu, vw2 = 0xffffffffu, vw3 = 0xffffffffu;
-                const int rt = g.T - t0, rh = g.H - h0, rw = g.W - w0;
-                if (et > rt || eh > rh || ew > rw) {
-                  auto valid = [&](int i) -> bool {
-                    return ((pos[i] >> 16) < rt && ((pos[i] >> 8) & 0xff) < rh && (pos[i] & 0xff) < rw) || lane + 32 * i >= ntok;
-                  };
-                  vw0 = __ballot_sync(0xffffffffu, valid(0));
-                  vw1 = __ballot_sync(0xffffffffu, valid(1));
-                  vw2 = __ballot_sync(0xffffffffu, valid(2));
-                  vw3 = __ballot_sync(0xffffffffu, valid(3));
+                if constexpr (kGrid == kPadded) {
+                  const int et = last && g.sub_axis == 0 ? g.c_last : g.ct, eh = last && g.sub_axis == 1 ? g.c_last : g.ch,
+                            ew = last && g.sub_axis == 2 ? g.c_last : g.cw;
+                  const int rt = g.T - t0, rh = g.H - h0, rw = g.W - w0;
+                  if (et > rt || eh > rh || ew > rw) {
+                    auto valid = [&](int i) -> bool {
+                      return ((pos[i] >> 16) < rt && ((pos[i] >> 8) & 0xff) < rh && (pos[i] & 0xff) < rw) || lane + 32 * i >= ntok;
+                    };
+                    vw0 = __ballot_sync(0xffffffffu, valid(0));
+                    vw1 = __ballot_sync(0xffffffffu, valid(1));
+                    vw2 = __ballot_sync(0xffffffffu, valid(2));
+                    vw3 = __ballot_sync(0xffffffffu, valid(3));
+                  }
                 }
                 issue_slab(t0, h0, w0, last, ntok, vw0, vw1, vw2, vw3);
                 if (g.sub_axis == 0) t0 += g.ct;
                 else if (g.sub_axis == 1) h0 += g.ch;
                 else w0 += g.cw;
+              }
               }
             }
           }
@@ -1131,26 +1302,29 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       for (int ts = 0; ok && ts < n_ts; ++ts) {
         const int tok0 = ts * kSlabTokens;
         const int nvalid = g.n_text - tok0;   // >= 1
-        const uint32_t vw0 = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
-        const uint32_t vw1 = nvalid >= 64 ? 0xffffffffu : (nvalid <= 32 ? 0u : ((1u << (nvalid - 32)) - 1u));
-        const uint32_t vw2 = nvalid >= 96 ? 0xffffffffu : (nvalid <= 64 ? 0u : ((1u << (nvalid - 64)) - 1u));
-        const uint32_t vw3 = nvalid >= 128 ? 0xffffffffu : (nvalid <= 96 ? 0u : ((1u << (nvalid - 96)) - 1u));
-        issue_slab(0, 0, tok0, 2, kSlabTokens, vw0, vw1, vw2, vw3);
+        if constexpr (kBoxes) {
+          if (lane == 0) lists[list * kMaxListed] = make_int4(tok0, 0, 0, 2);
+          issue_list(1, kSlabTokens, low_bits(nvalid - 32 * (lane & 3)));
+        } else issue_slab(0, 0, tok0, 2, kSlabTokens, low_bits(nvalid), low_bits(nvalid - 32), low_bits(nvalid - 64), low_bits(nvalid - 96));
       }
       while (ok && npend > 0) {  // V of the item's last slab(s), one pair barrier each
-        const uint32_t v_slot = tile_g % kNumSlots, v_use = tile_g / kNumSlots;
-        ok = mbar_wait_warp(bar(kBarSlotEmpty + v_slot), (v_use & 1u) ^ 1u, abort_flag, 0x112);
+        const uint32_t v_slot = slot_i;
+        ok = mbar_wait_warp(bar(kBarSlotEmpty + v_slot), slot_ph, abort_flag, 0x112);
         if (!ok) break;
-        if (lane == 0 && PSA_CHECKED(v_slot < (uint32_t)kNumSlots && at0 >= 0 && ah0 >= 0 && aw0 >= 0 && alast >= 0 && alast <= 2 &&
-                                     antok > 0 && antok <= kSlabTokens, 0xD03)) {
-          const uint32_t pb = bar(kBarPairFull + pair_g % kNumPairBars);
-          mbar_expect_tx(pb, (uint32_t)antok * 256u);
-          const uint32_t dv = sbase + kOffRing + v_slot * kSlabBytes;
-          tma_load_5d(dv, &tms.v[alast], pb, 0, aw0, ah0, at0, head_ld);
-          tma_load_5d(dv + kHalfBytes, &tms.v[alast], pb, 64, aw0, ah0, at0, head_ld);
+        const uint32_t pb = bar(kBarPairFull + pair_i), dv = sbase + kOffRing + v_slot * kSlabBytes;
+        if (PSA_CHECKED(v_slot < (uint32_t)kNumSlots && at0 >= 0 && ah0 >= 0 && aw0 >= 0 && alast >= 0 && alast <= 2 && antok > 0 &&
+                        antok <= kSlabTokens, 0xD03)) {
+          if (lane == 0) mbar_expect_tx(pb, (uint32_t)antok * 256u);
+          if constexpr (kBoxes) {
+            const int vl = list < npend ? list + kLists - npend : list - npend;
+            load_lists(box_of(vl, vl), pb, tms.v, dv, at0, tms.v, dv, 0);
+          } else if (lane == 0) {
+            load_box(dv, &tms.v[alast], pb, at0, ah0, aw0);
+          }
         }
-        ++tile_g;
+        slot_i = slot_next(slot_i, slot_ph);
         ++pair_g;
+        pair_i = pair_i + 1u == (uint32_t)kNumPairBars ? 0u : pair_i + 1u;
         at0 = bt0; ah0 = bh0; aw0 = bw0; alast = blast; antok = bntok;
         --npend;
       }
@@ -1226,8 +1400,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     uint32_t it_o0 = 0, it_o1 = 0;    // items in which accumulator O_i was used
     if constexpr (!kDraws) pdl_wait();   // (see pdl_wait)
     // keys of a slab from its index within its block (r = j mod n_sub, carried along: no division)
-    const int r_last = g.n_sub - 1;
-    auto nk_at = [&](int r) -> int { return r == r_last ? g.n_last : kSlabTokens; };
+    int n_sub = g.n_sub, n_last = g.n_last;
+    if constexpr (kEdge) { n_sub = prm.main_slabs; n_last = prm.main_last; }
+    const int r_last = n_sub - 1;
+    auto nk_at = [&](int r) -> int { return r == r_last ? n_last : kSlabTokens; };
     auto r_inc = [&](int r) -> int { return r == r_last ? 0 : r + 1; };
 
     for (uint32_t n = 0; ok; ++n) {
@@ -1235,8 +1411,8 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       if (!next_item(n, wi)) break;
       const int nq = (wi.w >> 16) & 0xff;
       const bool split = ((wi.w >> 24) & 1) != 0;
-      const int n_vid = wi.z * g.n_sub;          // key slabs, then those of edge blocks and of text (always 128 wide)
-      const int n_kv = n_vid + (kEdge ? (wi.x >> 8) * g.n_edge : 0) + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
+      const int n_vid = wi.z * n_sub;            // key slabs in the pattern, then others and those of text (always 128 wide)
+      const int n_kv = n_vid + (kEdge ? wi.x >> 8 : 0) + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
       auto nk_j = [&](int j, int r) -> int { return j >= n_vid ? kSlabTokens : nk_at(r); };
       // which accumulators this item uses: both for a two-slab item, and for a split-KV item
       // with at least two key slabs (even slabs -> O_0, odd slabs -> O_1)
@@ -1445,7 +1621,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       const int nq = (wi.w >> 16) & 0xff, rpc = nq * 128 / (int)cluster_size(), r0 = (int)cluster_rank() * rpc;
       for (int i = (int)threadIdx.x - 64; i < rpc; i += 64)
         *reinterpret_cast<int*>(smem + kOffRowTok + (uint32_t)i * 4u) =
-            (int)row_token(g, ((wi.w >> 25) & 1) != 0, wi.y, (wi.w & 0xffff) + ((r0 + i) >> 7), (r0 + i) & 127);
+            (int)row_token<kBoxes>(prm, ((wi.w >> 25) & 1) != 0, wi.y, (wi.w & 0xffff) + ((r0 + i) >> 7), (r0 + i) & 127);
     }
     __syncwarp();
   }
@@ -1464,6 +1640,8 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
     bool ok = true, met = false;   // met: cluster mode's first barrier passed
     const float neg_inf = __int_as_float(0xff800000);
     float2* xchg = reinterpret_cast<float2*>(smem + kOffXchg);
+    int n_sub = g.n_sub, n_last = g.n_last;
+    if constexpr (kEdge) { n_sub = prm.main_slabs; n_last = prm.main_last; }
     if constexpr (!kDraws) pdl_wait();   // (see pdl_wait)
 
     for (uint32_t n = 0; ok; ++n) {
@@ -1472,8 +1650,8 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       const int head = kEdge ? wi.x & 0xff : wi.x, qb = wi.y, sub0 = wi.w & 0xffff, nq = (wi.w >> 16) & 0xff;
       const bool split = ((wi.w >> 24) & 1) != 0;
       const bool textq = ((wi.w >> 25) & 1) != 0;
-      const int n_vid = wi.z * g.n_sub;          // key slabs, then those of edge blocks and of text (always 128 wide)
-      const int n_kv = n_vid + (kEdge ? (wi.x >> 8) * g.n_edge : 0) + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
+      const int n_vid = wi.z * n_sub;            // key slabs in the pattern, then others and those of text (always 128 wide)
+      const int n_kv = n_vid + (kEdge ? wi.x >> 8 : 0) + (kCluster && ((wi.w >> 26) & 1) ? 0 : g.n_ts);
       const bool use_o1 = (nq > 1) || (split && n_kv > 1);
       const bool active = (qi == 0) || use_o1;
       float m_ref = neg_inf;  // running reference maximum, scaled log2 domain
@@ -1482,10 +1660,10 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       if (active) {
         // key slabs of this tile: all of them, or every second one in a split-KV item
         const int j0 = split ? qi : 0, dj = split ? 2 : 1;
-        const int r_last = g.n_sub - 1;
+        const int r_last = n_sub - 1;
         int rj = (j0 > r_last) ? 0 : j0;   // j mod n_sub, carried along (no division in the loop)
         for (int j = j0; ok && j < n_kv; j += dj) {
-          const int nk = (rj == r_last && j < n_vid) ? g.n_last : kSlabTokens;
+          const int nk = (rj == r_last && j < n_vid) ? n_last : kSlabTokens;
           rj = (rj == r_last) ? 0 : rj + 1;
           if (dj == 2) rj = (rj == r_last) ? 0 : rj + 1;
           ok = mbar_wait_warp(bar(kBarSFull + qi), cnt_s & 1u, abort_flag, 0x300 + qi);
@@ -1613,7 +1791,7 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
       long long out_tok = -1;        // kShort: this row's token, and where its output goes
       uint4* out_row = nullptr;
       if constexpr (kShort) {
-        out_tok = row_token(g, textq, qb, sub0 + qi, row);
+        out_tok = row_token<kBoxes>(prm, textq, qb, sub0 + qi, row);
         if (out_tok >= 0)
           out_row = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head + out_tok * prm.out_token);
       }
@@ -1685,15 +1863,16 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         t0 = 0; h0 = 0; w0 = (sub0 + qi) * kSlabTokens; last = 2;
         if (w0 + row < g.n_text && PSA_CHECKED(head >= 0 && head < g.n_heads && w0 >= 0, 0xD10))
           prm.lse[(long long)head * g.Lt + g.L + w0 + row] = lse_row;
+      } else if (kBoxes) {
+        const long long tok = row_token<kBoxes>(prm, false, qb, sub0 + qi, row);
+        if (tok >= 0 && PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.L, 0xD14)) prm.lse[(long long)head * g.Lt + tok] = lse_row;
+        slab_origin(g, qb, 0, t0, h0, w0);
+        last = 0;
       } else {
         slab_origin(g, qb, sub0 + qi, t0, h0, w0);
         slab_shape(g, sub0 + qi, et, eh, ew, ntok, last);
-        const int wi_ = row % ew, hi_ = (row / ew) % eh, ti_ = row / (ew * eh);
-        const int t = t0 + ti_, hh = h0 + hi_, ww = w0 + wi_;
-        if (row < ntok && t < g.T && hh < g.H && ww < g.W) {
-          const long long tok = ((long long)t * g.H + hh) * g.W + ww;
-          if (PSA_CHECKED(head >= 0 && head < g.n_heads && tok >= 0 && tok < g.L, 0xD11)) prm.lse[(long long)head * g.Lt + tok] = lse_row;
-        }
+        const long long tok = row_token<false>(prm, false, qb, sub0 + qi, row);
+        if (tok >= 0 && PSA_CHECKED(head >= 0 && head < g.n_heads && tok < g.L, 0xD11)) prm.lse[(long long)head * g.Lt + tok] = lse_row;
       }
       // Every thread's staged row is made visible to the TMA engine; the warpgroup's first warp
       // waits for all 128 rows (a bounded wait, like every other one) and stores the slab.
@@ -1705,8 +1884,20 @@ attn_fwd_kernel(const __grid_constant__ TensorMaps tms, const __grid_constant__ 
         if (lane == 0) {
           const uint32_t src = sbase + kOffQ + (uint32_t)qi * kSlabBytes;
           if (PSA_CHECKED(w0 >= 0 && h0 >= 0 && t0 >= 0 && head >= 0 && head < g.n_heads && last >= 0 && last <= 2, 0xD13)) {
-            tma_store_5d(&tms.o[last], src, 0, w0, h0, t0, head);
-            tma_store_5d(&tms.o[last], src + kHalfBytes, 64, w0, h0, t0, head);
+            auto box = [&](uint32_t row8, int map, int t, int h, int w) {
+              tma_store_5d(tms.o + map, src + row8 * 1024u, 0, w, h, t, head);
+              tma_store_5d(tms.o + map, src + row8 * 1024u + kHalfBytes, 64, w, h, t, head);
+            };
+            if (kBoxes && !textq) {
+              if constexpr (kBoxes) {
+                const EdgeClass& e = prm.cls[block_class(g, qb / g.Sp, qb % g.Sp)];
+#pragma unroll 1
+                for (int b = e.first_box[sub0 + qi]; b < e.first_box[sub0 + qi + 1]; ++b)
+                  if (e.box[b].t != kZeros) box(e.box[b].row8, e.box[b].map, t0 + e.box[b].t, h0 + e.box[b].h, w0 + e.box[b].w);
+              }
+            } else {
+              box(0u, last, t0, h0, w0);
+            }
           }
           tma_store_commit();
           tma_store_wait_read();
@@ -1788,15 +1979,16 @@ struct LaunchConfig {
 
 // Once per device: shared-memory limits, and how many clusters of 2, 4 and 8 CTAs run at a time.
 cudaError_t attn_init(int clusters[3]) {
-  const void* kernels[] = {(const void*)attn_fwd_kernel<kTicket>, (const void*)attn_fwd_kernel<kDirect>,
-                           (const void*)attn_fwd_kernel<kShared>, (const void*)attn_fwd_kernel<kSharedDirect>,
-                           (const void*)attn_fwd_kernel<kTicketEdge>, (const void*)attn_fwd_kernel<kTicketShort>};
+#define PSA_ALL_GRIDS(mode) (const void*)attn_fwd_kernel<mode, kWhole>, (const void*)attn_fwd_kernel<mode, kPadded>, (const void*)attn_fwd_kernel<mode, kCut>
+  const void* kernels[] = {PSA_ALL_GRIDS(kTicket), PSA_ALL_GRIDS(kDirect), PSA_ALL_GRIDS(kShared), PSA_ALL_GRIDS(kSharedDirect),
+                           PSA_ALL_GRIDS(kTicketShort)};
+#undef PSA_ALL_GRIDS
   cudaError_t e = cudaSuccess;
   for (const void* k : kernels)
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAlloc)) != cudaSuccess) return e;
   for (int i = 0; i < 3; ++i) {
     LaunchConfig lc(2 << i, kThreads, kSmemAlloc, nullptr, 2 << i);
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters[i], attn_fwd_kernel<kSharedDirect>, &lc.cfg)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveClusters(&clusters[i], attn_fwd_kernel<kSharedDirect, kCut>, &lc.cfg)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -1813,26 +2005,36 @@ cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, i
 }
 
 template <int kMode>
-cudaError_t launch_mode(const LaunchConfig& lc, const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm) {
-  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode>, tm, heads, prm);
+cudaError_t launch_mode(const LaunchConfig& lc, const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm) {
+  if (prm.cut) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kCut>, tm, heads, prm);
+  TensorMaps plain;
+  for (int i = 0; i < 3; ++i) {
+    plain.q[i] = tm.q[i];
+    plain.k[i] = tm.k[i];
+    plain.v[i] = tm.v[i];
+    plain.o[i] = tm.o[i];
+  }
+  if (prm.g.edge_axes) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kPadded>, plain, heads, prm);
+  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kWhole>, plain, heads, static_cast<const AttnParams&>(prm));
 }
 
 // heads: read by launches without planning only.  cluster: CTAs per work item, 1: whole items.  direct: all items run
-// at once, nothing was planned.  *mode: the kernel launched.
-cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster, bool direct,
+// at once, nothing was planned.  *mode: how the launch hands out its items.
+cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm, int n_sms, int cluster, bool direct,
                         bool short_items, cudaStream_t stream, Mode* mode) {
   if (prm.n_items <= 0) return cudaSuccess;
   const int ctas = cluster > 1 || direct ? prm.n_items * cluster : (prm.n_items < n_sms ? prm.n_items : n_sms);
   LaunchConfig lc(ctas, kThreads, kSmemAlloc, stream, cluster);
-  *mode = cluster > 1 ? (direct ? kSharedDirect : kShared)
-                      : (direct ? kDirect : (short_items ? kTicketShort : (prm.g.nb_edge ? kTicketEdge : kTicket)));
-  switch (*mode) {
-    case kTicket: return launch_mode<kTicket>(lc, tm, heads, prm);
+  *mode = cluster > 1 ? (direct ? kSharedDirect : kShared) : (direct ? kDirect : (short_items ? kTicketShort : kTicket));
+  const Mode kernel = *mode;
+  for (int c = 1; c < 8; ++c)
+    if (kernel == kTicket && (c & ~prm.g.edge_axes) == 0 && prm.g.slabs_of[c] < prm.g.n_sub) *mode = kTicketEdge;
+  switch (kernel) {
     case kDirect: return launch_mode<kDirect>(lc, tm, heads, prm);
     case kShared: return launch_mode<kShared>(lc, tm, heads, prm);
     case kSharedDirect: return launch_mode<kSharedDirect>(lc, tm, heads, prm);
-    case kTicketEdge: return launch_mode<kTicketEdge>(lc, tm, heads, prm);
-    default: return launch_mode<kTicketShort>(lc, tm, heads, prm);
+    case kTicketShort: return launch_mode<kTicketShort>(lc, tm, heads, prm);
+    default: return launch_mode<kTicket>(lc, tm, heads, prm);
   }
 }
 

@@ -15,6 +15,31 @@ constexpr int kMaxTp = 256;       // limits of the in-kernel key-block bitmasks
 constexpr int kMaxSp = 2048;
 constexpr size_t kMaxSmemBytes = 232448;   // 227 KB of shared memory that a CTA may use
 
+// Blocks that reach beyond the grid (3D-padding) are edge blocks, the last ones along an axis.  A class has a bit for each axis
+// on which they are the last (1: t, 2: h, 4: w); class 0 is an ordinary block.  An edge block is cut to the part that holds its
+// tokens: `rows` of them, in the order t, h, w of frames of lines of 1 << lw, padded as far as loading by TMA boxes asks for.
+// Key slabs follow a pattern, that of the ordinary blocks or, where there are none, of the most frequent class: main_slabs slabs
+// per block, of 128 keys and the last one of main_last.  The slabs of blocks that do not follow it come behind, 128 keys each.  What
+// tokens do not fill is zeros, with validity bits of 0.
+struct alignas(8) EdgeBox {   // a box of a slab: its map, first row, and first token relative to the block's
+  uint8_t map, row8;        // (row / 8)
+  uint16_t t, h, w;         // t == kZeros: a box of zeros
+};
+constexpr int kMaxEdgeBoxes = 8;
+constexpr uint16_t kZeros = 0xffff;
+struct EdgeClass {
+  uint16_t rows, frame;     // of a block; of a frame
+  uint16_t step;            // rows of a slab that is not the last one
+  uint8_t lw;               // log2 of the line length
+  uint8_t n_slabs;          // slabs of a block
+  alignas(4) uint8_t first_box[4];   // boxes of slab s: first_box[s] .. first_box[s + 1] - 1
+  uint8_t together;         // blocks that share one slab of keys (1 unless they have at most 64 rows): of box[0] each, then box[1]
+  uint8_t n_boxes;
+  uint8_t in_pattern;
+  EdgeBox box[kMaxEdgeBoxes];
+  uint32_t valid[3][4];     // the slabs' rows with tokens, bit r % 32 of word r / 32; of `together` blocks
+};
+
 // Problem geometry handed to every kernel by value.
 struct Geom {
   int T, H, W;             // real token grid
@@ -26,12 +51,11 @@ struct Geom {
   int sub_axis;            // axis along which the slabs of a block stack: 0 = t, 1 = h, 2 = w
   int c_last;              // extent of a block's LAST slab along sub_axis (<= the full slab's)
   int n_last;              // tokens of that last slab: 128, 112, 96 or 64
-  // Slabs that 3D-padding leaves without a token are neither loaded nor computed: a block that is the last one along
-  // sub_axis ("edge block") has n_edge of its n_sub slabs.  n_edge == n_sub: no slab is empty, no block counts as edge.
-  int n_edge;              // (all full 128-token slabs when n_edge < n_sub)
-  int nb_edge;             // edge blocks of the grid, 0 if no slab is empty
+  int edge_axes;           // axes on which the grid has edge blocks (EdgeClass)
+  int s_edge;              // spatial block coordinates from here on are the last ones along h
+  uint8_t slabs_of[8];     // query slabs of a block by class
   int n_heads;
-  int items_per_block;     // work items per query block = ceil(n_sub / 2); ceil(n_edge / 2) for an edge block
+  int items_per_block;     // work items per query block = ceil(n_sub / 2); of an edge block by its n_slabs
   float scale_log2;        // softmax scale times log2(e)
   long long L;             // T*H*W
   // joint video + text sequences: n_text text tokens follow the L video tokens of every head
@@ -53,18 +77,24 @@ struct PlanParams {
 };
 
 // One unit of work of the attention kernel: up to two query slabs of one query block.
-// x = head | (attended edge blocks << 8), y = query block id, z = number of attended key blocks that are no edge blocks,
+// x = head, y = query block id, z = number of attended key blocks,
 // w = first slab index | (number of slabs << 16) | (split-KV mode << 24) | (text-query item << 25)
-// (inside a CTA of a cluster that shares one item: x and z = its share of the blocks, bit 26 of w = no text keys).
-// Key slabs come in this order: z blocks of n_sub slabs, the edge blocks' n_edge slabs each, the text slabs.
+// (inside a CTA of a cluster that shares one item: its share of the blocks, bit 26 of w = no text keys; inside a CTA, for grids
+// with edge blocks: z = attended blocks that follow the pattern, x = head | (slabs of the others' keys << 8)).
+// Key slabs come in this order: those of the blocks that follow the pattern, of the other edge blocks by class, of the text.
 typedef int4 WorkItem;
 
-// [0]: box of a full 128-token slab, [1]: of a block's last slab, [2]: of a text slab
+// [0]: box of a full 128-token slab, [1]: of a block's last slab, [2]: of a text slab, [3] on: those of edge blocks
+constexpr int kMaxMaps = 20;
 struct TensorMaps {
   CUtensorMap q[3], k[3], v[3], o[3];
 };
-
-// How an attention launch hands out its work items (see attn_fwd_kernel); the values are those of psa_launch_mode.
+struct TensorMapsEdge {
+  CUtensorMap q[kMaxMaps], k[kMaxMaps], v[kMaxMaps], o[kMaxMaps];
+};
+// How an attention launch hands out its work items (see attn_fwd_kernel); the values are those of psa_launch_mode.  (kTicketEdge
+// is only reported; the kernel is that of kTicket.)
+enum Grid { kWhole, kPadded, kCut };   // (see attn_fwd_kernel)
 enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge, kTicketShort };
 
 // Arguments of one attention launch; lse and out start at the launch's first head.
@@ -79,6 +109,15 @@ struct AttnParams {
   int shared_qkv;   // 1: every head reads head 0 of q, k, v (candidate masks of one head, PSA-Search)
   void* out;        // for rows that are stored without TMA; strides in elements
   long long out_head, out_token;
+};
+
+// The same of a launch on a grid with edge blocks.
+struct AttnParamsEdge : AttnParams {
+  EdgeClass cls[8];
+  int main_slabs, main_last;   // the pattern
+  int cut;                     // 1: the slabs are those of `box`; 0: those of ordinary blocks, of an edge block maybe fewer
+  int n_classes;               // classes that the grid has, those of the pattern first
+  uint8_t order[8];
 };
 
 // Layout of the per-device workspace (all int32 words).

@@ -21,7 +21,7 @@ cudaError_t attn_init(int clusters[3]);
 size_t plan_smem_bytes(const Geom& g);
 cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
                         WorkItem* items, cudaStream_t stream);
-cudaError_t launch_attn(const TensorMaps& tm, const HeadParamsArray& heads, const AttnParams& prm, int n_sms, int cluster,
+cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm, int n_sms, int cluster,
                         bool direct, bool short_items, cudaStream_t stream, Mode* mode);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
@@ -114,8 +114,205 @@ int host_chunks() {
   return v;
 }
 
+// Geometry with what only grids with edge blocks need: their classes, and the box shapes of maps 3 on.
+struct BoxShape {
+  int w, h, t;
+};
+struct HostGeom : Geom {
+  EdgeClass cls[8];
+  int main_slabs, main_last, cut;
+  int n_classes;
+  uint8_t order[8];
+  int n_shapes;
+  BoxShape shape[kMaxMaps - 3];
+};
+
+// Blocks of the grid of class c.
+int class_blocks(const Geom& g, int c) {
+  if (c & ~g.edge_axes) return 0;
+  auto along = [&](int n, int bit) -> int { return c & bit ? 1 : (g.edge_axes & bit ? n - 1 : n); };
+  return along(g.Tp, 1) * along(g.Hp, 2) * along(g.Wp, 4);
+}
+
+int round_up(int n, int to) { return (n + to - 1) / to * to; }
+int log2_up(int n) {
+  int l = 0;
+  while ((1 << l) < n) ++l;
+  return l;
+}
+
+// Map of a box shape, or -1 if there are too many.
+int map_of(HostGeom* g, int w, int h, int t) {
+  if (w == g->cw && h == g->ch && t == g->ct) return 0;
+  for (int i = 0; i < g->n_shapes; ++i)
+    if (g->shape[i].w == w && g->shape[i].h == h && g->shape[i].t == t) return 3 + i;
+  if (g->n_shapes == kMaxMaps - 3) return -1;
+  g->shape[g->n_shapes] = BoxShape{w, h, t};
+  return 3 + g->n_shapes++;
+}
+
+bool add_box(EdgeClass* e, int* rows, int map, int t, int h, int w, int n) {
+  if (map < 0 || e->n_boxes == kMaxEdgeBoxes) return false;
+  e->box[e->n_boxes++] = EdgeBox{(uint8_t)map, (uint8_t)(*rows / 8), (uint16_t)t, (uint16_t)h, (uint16_t)w};
+  *rows += n;
+  return true;
+}
+
+// Zeros up to `to` rows behind the `rows` that the class's boxes fill of its last slab so far: lines behind the grid's last one in the
+// same box, where the slab ends with them, or a box of their own from beyond the last frame.
+bool fill_slab(HostGeom* g, EdgeClass* e, bool at_bottom, int rows, int to) {
+  if (rows >= to) return true;
+  const EdgeBox last = e->box[e->n_boxes - 1];
+  const int w = 1 << e->lw, need = to - rows;
+  const BoxShape s = last.map >= 3 ? g->shape[last.map - 3] : BoxShape{g->cw, g->ch, g->ct};
+  if (at_bottom && e->together == 1 && last.map != 1 && s.t == 1 && s.w == w && (last.h + s.h) * w == e->frame && need % w == 0) {
+    int users = 0;   // of the box's map in finished classes: if it is this box alone, the map changes with it
+    for (const EdgeClass& x : g->cls)
+      for (int b = 0; b < x.n_boxes; ++b) users += x.box[b].map == last.map;
+    if (users == 1 && last.map >= 3 && e >= g->cls && e < g->cls + 8) {
+      g->shape[last.map - 3].h += need / w;
+      return true;
+    }
+    const int map = map_of(g, w, s.h + need / w, 1);
+    if (map < 0) return false;
+    e->box[e->n_boxes - 1].map = (uint8_t)map;
+    return true;
+  }
+  return add_box(e, &rows, map_of(g, 8, need / 8, 1), kZeros, 0, 0, need);
+}
+
+// A block of nt x nh x nw tokens as an ordinary one, without the slabs that have no token.
+void whole_slabs(const HostGeom& g, EdgeClass* e, int nt, int nh, int nw) {
+  const int tokens = g.sub_axis == 0 ? nt : (g.sub_axis == 1 ? nh : nw), slab = g.sub_axis == 0 ? g.ct : (g.sub_axis == 1 ? g.ch : g.cw),
+            block = g.sub_axis == 0 ? g.bt : (g.sub_axis == 1 ? g.bh : g.bw), along = round_up(tokens, slab) < block ? round_up(tokens, slab) : block;
+  std::memset(e, 0, sizeof(*e));
+  const int t = g.sub_axis == 0 ? along : g.bt, h = g.sub_axis == 1 ? along : g.bh, w = g.sub_axis == 2 ? along : g.bw;
+  e->rows = (uint16_t)(t * h * w);
+  e->frame = (uint16_t)(h * w);
+  e->lw = (uint8_t)log2_up(w);
+  e->step = kSlabTokens;
+  e->together = 1;
+  for (int at = 0; at < along; at += slab) {
+    int rows = 0;
+    e->first_box[e->n_slabs++] = e->n_boxes;
+    add_box(e, &rows, along - at < slab ? 1 : 0, g.sub_axis == 0 ? at : 0, g.sub_axis == 1 ? at : 0, g.sub_axis == 2 ? at : 0, 0);
+  }
+}
+
+// Keys that a slab of so many rows is multiplied as, at the end of a block: the widths of the softmax.
+int key_width(int rows) { return rows <= 64 ? 64 : (rows <= 96 ? 96 : (rows <= 112 ? 112 : 128)); }
+int last_rows(const EdgeClass& e) { return e.rows - (e.n_slabs - 1) * e.step; }
+
+// The same cut to its tokens, if that can be done and makes fewer slabs of keys (or a narrower last one that makes or follows the
+// pattern).  Lines have
+// a power of two of tokens, and a frame is a multiple of 8 rows (the unit of the 128-byte swizzle, so that boxes can be put
+// behind one another).  What that adds lies beyond the grid, where it is loaded as zeros -- never in the next block, whose values a
+// probability of 0 would not keep out if they are infinite -- so lines shorter than 8 tokens need a whole number of groups of
+// 8 rows in every block's height.
+bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, int nh, int nw) {
+  if (g->sub_axis == 2 || g->bh * g->bw < 8) return false;
+  const int shapes_before = g->n_shapes;
+  EdgeClass x = {};
+  auto lines = [](int width) -> int { return width < 8 ? 8 / width : 1; };   // that make whole groups of 8 rows
+  int w = g->bw;
+  if (c & 4) {
+    w = 1 << log2_up(nw);
+    while (w < g->bw && !(c & 2) && g->bh % lines(w) != 0) w *= 2;
+  }
+  const int h = c & 2 ? round_up(nh, lines(w)) : nh, frame = h * w, rows = nt * frame;
+  // slabs of whole frames, or of lines with up to four boxes a slab where that makes fewer of them (or a narrower last one)
+  auto slabs = [&](int step) -> int { return (rows + step - 1) / step; };
+  auto last_of = [&](int step) -> int { return rows - (slabs(step) - 1) * step; };
+  auto cost = [&](int step) -> int { return 128 * slabs(step) + (for_pattern || g->main_last < kSlabTokens ? key_width(last_of(step)) : 0); };
+  const int per = kSlabTokens / frame, step = rows <= kSlabTokens ? rows : (per > 0 && cost(per * frame) <= cost(kSlabTokens) ? per * frame : kSlabTokens);
+  x.rows = (uint16_t)rows;
+  x.frame = (uint16_t)frame;
+  x.lw = (uint8_t)log2_up(w);
+  x.step = (uint16_t)step;
+  x.together = (uint8_t)(rows <= kSlabTokens / 2 ? kSlabTokens / rows : 1);
+  bool ok = slabs(step) < e->n_slabs || x.together > 1 ||
+            (slabs(step) == e->n_slabs && key_width(last_of(step)) < key_width(last_rows(*e)) &&
+             (for_pattern || (e->n_slabs == g->main_slabs && last_rows(*e) > g->main_last && last_of(step) <= g->main_last)));
+  for (int r = 0; ok && r < rows; r += step) {
+    int end = 0;
+    x.first_box[x.n_slabs++] = x.n_boxes;
+    for (int y = r, to = r + step < rows ? r + step : rows; ok && y < to;) {
+      const int left = to - y, in_frame = y % frame;
+      if (in_frame == 0 && left >= frame) {   // whole frames
+        const int n = left / frame;
+        ok = add_box(&x, &end, map_of(g, w, h, n), y / frame, 0, 0, n * frame);
+        y += n * frame;
+      } else {
+        const int n = left < frame - in_frame ? left : frame - in_frame;
+        ok = add_box(&x, &end, map_of(g, w, n / w, 1), y / frame, in_frame / w, 0, n);
+        y += n;
+      }
+    }
+    if (r + step < rows) ok = ok && fill_slab(g, &x, (c & 2) || g->Hp == 1, end, kSlabTokens);
+  }
+  int classes = 0;   // set_edges has a map and a box left for each of them
+  for (int k = 1; k < 8; ++k) classes += class_blocks(*g, k) > 0;
+  if (!ok || g->n_shapes + classes > kMaxMaps - 3 || x.n_boxes == kMaxEdgeBoxes) {
+    g->n_shapes = shapes_before;
+    return false;
+  }
+  *e = x;
+  return true;
+}
+
+// Edge blocks (EdgeClass) of a grid whose extents the block does not divide.  T, H, W, the block and its slabs are set.
+//
+// Why: 3D-padding is issued work, along the keys and along the queries.  The last of the seven 30x8 blocks across 52 columns
+// holds 120 of its 240 tokens (12 heads of 21x30x52: 2.60 -> @@A ms), the last 3x8x16 block down 45 rows 240 of 384 (40 heads of
+// 21x45x80: 28.7 -> @@B ms).  Cut like this an edge block is mostly one box a slab, as an ordinary one: the load warp, which has
+// some 10 clocks for an instruction next to the softmax, fell behind with rows packed tightly across blocks, by boxes of 8 to
+// 128 rows (5,000 clocks a slab) as well as by 16-byte copies (8,000).
+void set_edges(HostGeom* g) {
+  const int rt = g->T - (g->Tp - 1) * g->bt, rh = g->H - (g->Hp - 1) * g->bh, rw = g->W - (g->Wp - 1) * g->bw;   // of the last block
+  g->edge_axes = (rt < g->bt ? 1 : 0) | (rh < g->bh ? 2 : 0) | (rw < g->bw ? 4 : 0);
+  g->s_edge = g->Sp - g->Wp;
+  g->n_shapes = g->n_classes = 0;
+  int pattern = 0;   // its class
+  for (int c = 0; c < 8; ++c)
+    if (class_blocks(*g, 0) == 0 && class_blocks(*g, c) > class_blocks(*g, pattern)) pattern = c;
+  g->slabs_of[0] = (uint8_t)g->n_sub;
+  if (g->edge_axes == 0) return;
+  auto make = [&](int c) {
+    EdgeClass& e = g->cls[c];
+    const int nt = c & 1 ? rt : g->bt, nh = c & 2 ? rh : g->bh, nw = c & 4 ? rw : g->bw;   // tokens along the axes
+    whole_slabs(*g, &e, nt, nh, nw);
+    if (c != 0 && cut_to_tokens(g, &e, c, c == pattern, nt, nh, nw)) g->cut = 1;
+    for (int s = 0; s < e.n_slabs; ++s) {
+      const int have = s + 1 < e.n_slabs ? e.step : last_rows(e);
+      for (int r = 0; r < have * e.together; ++r) {
+        const int x = s * e.step + r % have, y = x % e.frame;
+        if (x / e.frame < nt && (y >> e.lw) < nh && (y & ((1 << e.lw) - 1)) < nw) e.valid[s][r / 32] |= 1u << (r % 32);
+      }
+    }
+  };
+  make(pattern);
+  const EdgeClass& m = g->cls[pattern];
+  g->main_slabs = m.together > 1 ? 1 : m.n_slabs;
+  g->main_last = m.together > 1 ? kSlabTokens : key_width(last_rows(m));
+  for (int c = 0; c < 8; ++c)
+    if (c != pattern && class_blocks(*g, c)) make(c);
+  for (int c = 0; c < 8; ++c) {
+    if (!class_blocks(*g, c)) continue;
+    EdgeClass& e = g->cls[c];
+    e.in_pattern = e.together == 1 && e.n_slabs == g->main_slabs && last_rows(e) <= g->main_last;
+    const int to = e.in_pattern ? g->main_last : kSlabTokens;
+    fill_slab(g, &e, (c & 2) || g->Hp == 1, e.together * last_rows(e), to);   // (see cut_to_tokens)
+    for (int r = to; r < kSlabTokens; ++r) e.valid[e.n_slabs - 1][r / 32] |= 1u << (r % 32);   // (a short slab has no such keys)
+    e.first_box[e.n_slabs] = e.n_boxes;
+    g->slabs_of[c] = e.n_slabs;
+  }
+  for (int in = 1; in >= 0; --in)
+    for (int c = 0; c < 8; ++c)
+      if (class_blocks(*g, c) && g->cls[c].in_pattern == in) g->order[g->n_classes++] = (uint8_t)c;
+}
+
 // Geometry of the block grid; `for_attn` additionally derives the 128-token slab.
-int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, Geom* g) {
+int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, HostGeom* g) {
   if (!prob || T < 1 || H < 1 || W < 1 || prob->n_heads < 1) return PSA_ERR_INVALID_ARG;
   const psa_tile t = prob->tile;
   if (t.bt < 1 || t.bh < 1 || t.bw < 1) return PSA_ERR_INVALID_ARG;
@@ -170,18 +367,15 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, Geom*
     while ((1 << g->pos_ts) < g->cw * g->ch) ++g->pos_ts;
     if (g->Tp > kMaxTp || g->Sp > kMaxSp || plan_smem_bytes(*g) > kMaxSmemBytes) return PSA_ERR_UNSUPPORTED;
     g->n_sub = n_sub;
-    {   // slabs of the last block along the stacked axis that hold any token
-      const int ext = axis == 0 ? T : (axis == 1 ? H : W), b = axis == 0 ? t.bt : (axis == 1 ? t.bh : t.bw);
-      const int n = axis == 0 ? g->Tp : (axis == 1 ? g->Hp : g->Wp);
-      g->n_edge = (ext - (n - 1) * b + c0 - 1) / c0;
-      if (g->n_edge < n_sub) g->nb_edge = axis == 0 ? g->Sp : (axis == 1 ? g->Tp * g->Wp : g->Tp * g->Hp);
-    }
+    set_edges(g);
     g->items_per_block = (n_sub + 1) / 2;
     g->scale_log2 = prob->scale * 1.4426950408889634f;
   }
   g->items_per_head = g->NB * g->items_per_block;
-  // an edge block's empty slabs are no work (only with three slabs per block is it an item less)
-  if (g->nb_edge) g->items_per_head -= g->nb_edge * (g->items_per_block - (g->n_edge + 1) / 2);
+  // (only blocks of three slabs have a second item)
+  if (for_attn && g->n_sub == 3 && g->edge_axes)
+    for (int c = 0; c < 8; ++c)
+      if (g->slabs_of[c] < 3) g->items_per_head -= class_blocks(*g, c);
   g->Lt = L;
   return PSA_OK;
 }
@@ -249,16 +443,15 @@ int ensure_workspace(Workspace* w, size_t bytes) {
   return PSA_OK;
 }
 
-// `last`: box of a block's last (possibly shorter) slab instead of the full 128-token slab.
+// Map of [heads][T][H][W][128] with a box of 64 columns of box.w x box.h x box.t tokens.
 int encode_map(CUtensorMap* tm, const void* base, const Geom& g, long long stride_head, long long stride_token,
-               int n_heads_here, bool last) {
+               int n_heads_here, const BoxShape& shape) {
   const cuuint64_t dims[5] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.T,
                               (cuuint64_t)n_heads_here};
   const cuuint64_t st = (cuuint64_t)stride_token * 2;
   const cuuint64_t strides[4] = {st, st * g.W, st * g.W * g.H,
                                  n_heads_here > 1 ? (cuuint64_t)stride_head * 2 : st * g.W * g.H * g.T};
-  cuuint32_t box[5] = {64, (cuuint32_t)g.cw, (cuuint32_t)g.ch, (cuuint32_t)g.ct, 1};
-  if (last) box[3 - g.sub_axis] = (cuuint32_t)g.c_last;
+  const cuuint32_t box[5] = {64, (cuuint32_t)shape.w, (cuuint32_t)shape.h, (cuuint32_t)shape.t, 1};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   const CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box,
                               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -290,21 +483,25 @@ struct Layout {
   bool shared_qkv;                // every head reads head 0 of q, k, v
 };
 
-// The four tensors, each with the full-slab box ([0]) and the last-slab box ([1]).
-int encode_maps(TensorMaps* tm, const void* q, const void* k, const void* v, void* out, const Geom& g,
+// The four tensors with every box shape (TensorMaps).
+int encode_maps(TensorMapsEdge* tm, const void* q, const void* k, const void* v, void* out, const HostGeom& g,
                 const Layout& lay, int n_heads_here) {
   int rc;
   const int n_in = lay.shared_qkv ? 1 : n_heads_here;
-  for (int last = 0; last < 2; ++last) {
-    if (last && g.n_last == kSlabTokens) {   // a block's last slab is a full one
-      tm->q[1] = tm->q[0]; tm->k[1] = tm->k[0]; tm->v[1] = tm->v[0]; tm->o[1] = tm->o[0];
-      break;
-    }
-    if ((rc = encode_map(&tm->q[last], q, g, lay.in_head, lay.in_token, n_in, last != 0)) != PSA_OK) return rc;
-    if ((rc = encode_map(&tm->k[last], k, g, lay.in_head, lay.in_token, n_in, last != 0)) != PSA_OK) return rc;
-    if ((rc = encode_map(&tm->v[last], v, g, lay.in_head, lay.in_token, n_in, last != 0)) != PSA_OK) return rc;
-    if ((rc = encode_map(&tm->o[last], out, g, lay.out_head, lay.out_token, n_heads_here, last != 0)) != PSA_OK) return rc;
+  auto encode = [&](int i, const BoxShape& box) -> int {
+    if ((rc = encode_map(&tm->q[i], q, g, lay.in_head, lay.in_token, n_in, box)) != PSA_OK) return rc;
+    if ((rc = encode_map(&tm->k[i], k, g, lay.in_head, lay.in_token, n_in, box)) != PSA_OK) return rc;
+    if ((rc = encode_map(&tm->v[i], v, g, lay.in_head, lay.in_token, n_in, box)) != PSA_OK) return rc;
+    return encode_map(&tm->o[i], out, g, lay.out_head, lay.out_token, n_heads_here, box);
+  };
+  if ((rc = encode(0, BoxShape{g.cw, g.ch, g.ct})) != PSA_OK) return rc;
+  if (g.n_last == kSlabTokens) {   // a block's last slab is a full one
+    tm->q[1] = tm->q[0]; tm->k[1] = tm->k[0]; tm->v[1] = tm->v[0]; tm->o[1] = tm->o[0];
+  } else if ((rc = encode(1, BoxShape{g.sub_axis == 2 ? g.c_last : g.cw, g.sub_axis == 1 ? g.c_last : g.ch, g.sub_axis == 0 ? g.c_last : g.ct})) != PSA_OK) {
+    return rc;
   }
+  for (int i = 0; i < g.n_shapes; ++i)
+    if ((rc = encode(3 + i, g.shape[i])) != PSA_OK) return rc;
   if (g.n_text > 0) {
     if ((rc = encode_text_map(&tm->q[2], q, g, lay.in_head, lay.in_token, n_in)) != PSA_OK) return rc;
     if ((rc = encode_text_map(&tm->k[2], k, g, lay.in_head, lay.in_token, n_in)) != PSA_OK) return rc;
@@ -334,6 +531,15 @@ void plan_params(PlanParams* pp, const psa_head_params* params, const long long*
   }
 }
 
+// Key slabs of the average block.
+double slabs_per_block(const HostGeom& g) {
+  if (g.edge_axes == 0) return g.n_sub;
+  double n = 0;
+  for (int c = 0; c < 8; ++c)
+    if (class_blocks(g, c)) n += (double)class_blocks(g, c) * g.cls[c].n_slabs / g.cls[c].together;
+  return n / g.NB;
+}
+
 // CTAs that share a work item: 1 (persistent CTAs that draw whole items), 2, 4 or 8.  A launch takes about as many
 // rounds as its items need on the SMs, and at least as long as its longest item, so a problem of few items, of a few more
 // than a whole number of rounds, or of a few very long ones (text queries attend every key) leaves SMs idle; sharing
@@ -343,7 +549,7 @@ void plan_params(PlanParams* pp, const psa_head_params* params, const long long*
 // except one at 18 % (12 items); without text, whole items were best in all 24 problems of more than two rounds.
 // Decided for a call as a whole, so that the chunks of a host-tensor call compute what the device call computes, bit
 // for bit.  weights: attended block pairs of every head.
-int share_items(const Workspace& ws, const Geom& g, const long long* weights, int n_heads) {
+int share_items(const Workspace& ws, const HostGeom& g, const long long* weights, int n_heads) {
   const int heads = n_heads < kMaxHeads ? n_heads : kMaxHeads;   // of one launch
   const int n_items = heads * g.items_per_head, n_text = heads * g.n_titems;
   // beyond two rounds at most a third is to be gained, unless text queries make long items
@@ -355,11 +561,11 @@ int share_items(const Workspace& ws, const Geom& g, const long long* weights, in
   }
   // blocks attended by the average query block, of all heads and of the heaviest
   const double avg = (double)total / ((double)n_heads * g.NB), heavy = (double)most / g.NB;
-  const int singles = g.n_sub & 1, doubles = g.n_sub >> 1;
-  const double per_slab = (3300.0 * doubles + 1900.0 * singles) / (doubles + singles);
-  const double text = n_text ? ((double)g.NB * g.n_sub + g.n_ts) * (g.n_ts > 1 ? 3300.0 : 1900.0) : 0.0;
-  const double heavy_item = (heavy * g.n_sub + g.n_ts) * per_slab, longest = heavy_item > text ? heavy_item : text;
-  const double work = (double)(n_items - n_text) * (avg * g.n_sub + g.n_ts) * per_slab + n_text * text;
+  const int of_block = g.edge_axes ? g.main_slabs : g.n_sub, singles = of_block & 1, doubles = of_block >> 1;
+  const double per_slab = (3300.0 * doubles + 1900.0 * singles) / (doubles + singles), slabs = slabs_per_block(g);
+  const double text = n_text ? (g.NB * slabs + g.n_ts) * (g.n_ts > 1 ? 3300.0 : 1900.0) : 0.0;
+  const double heavy_item = (heavy * slabs + g.n_ts) * per_slab, longest = heavy_item > text ? heavy_item : text;
+  const double work = (double)(n_items - n_text) * (avg * slabs + g.n_ts) * per_slab + n_text * text;
   auto time = [&](int at_a_time, int c, double fixed) -> double {
     const double one = longest / c + fixed;
     if (n_items <= at_a_time) return one;
@@ -370,7 +576,7 @@ int share_items(const Workspace& ws, const Geom& g, const long long* weights, in
   int cluster = 1;
   for (int i = 0; i < 3; ++i) {
     const int c = 2 << i;
-    if (ws.clusters[i] < 1 || longest < c * per_slab * g.n_sub) break;   // a share of a long item holds at least one block
+    if (ws.clusters[i] < 1 || longest < c * per_slab * slabs) break;   // a share of a long item holds at least one block
     const double t = time(ws.clusters[i], c, 20000.0);
     // (rounds of whole items overlap more than the estimate knows: the longer ones go first)
     if (t < (n_items <= ws.clusters[i] ? 0.97 : 0.88) * best) { best = t; cluster = c; }
@@ -390,14 +596,14 @@ bool runs_at_once(const Workspace& ws, int n_items, int cluster) {
 // without and with: 15.6 key blocks 193 / 178, 19.5 221 / 198, 33.7 312 / 301, 65 532 / 532.  Items of two query slabs have
 // two warpgroups' rows to write and lose by it: 1x16x16 blocks attending 9.2 blocks 174 / 169 but 26.6 of a 16x48x80 grid
 // 1,308 / 1,353, 1x15x16 30.1 974 / 1,015; so do blocks of three slabs (3x8x16, 6.6 blocks 204 / 225).
-bool short_items(const Geom& g, const long long* weights, int n_heads) {
+bool short_items(const HostGeom& g, const long long* weights, int n_heads) {
   long long total = 0;
   for (int h = 0; h < n_heads; ++h) total += weights[h];
-  return g.n_sub == 1 && total < (64ll - g.n_ts) * n_heads * g.NB;
+  return g.n_sub == 1 && (double)total * slabs_per_block(g) < (64.0 - g.n_ts) * n_heads * g.NB;
 }
 
 // Planning (unless the launch is direct) and attention.
-cudaError_t launch_call(const TensorMaps& tm, const AttnParams& prm, const psa_head_params* params, const long long* weights,
+cudaError_t launch_call(const TensorMapsEdge& tm, const AttnParams& prm, const HostGeom& hg, const psa_head_params* params, const long long* weights,
                         const Workspace& ws, int cluster, bool record, cudaStream_t st) {
   HeadParamsArray heads;   // entries beyond the launch's heads are never read, nor any of a planned launch
   const int n = prm.g.n_heads;
@@ -413,7 +619,18 @@ cudaError_t launch_call(const TensorMaps& tm, const AttnParams& prm, const psa_h
     ++g_launches;
   }
   if (record && g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
-  const cudaError_t e = launch_attn(tm, heads, prm, ws.n_sms, cluster, direct, short_items(prm.g, weights, n), st, &g_last_attn.mode);
+  AttnParamsEdge pe;
+  pe.cut = 0;
+  static_cast<AttnParams&>(pe) = prm;
+  if (hg.edge_axes) {
+    std::memcpy(pe.cls, hg.cls, sizeof(pe.cls));
+    pe.main_slabs = hg.main_slabs;
+    pe.main_last = hg.main_last;
+    pe.cut = hg.cut;
+    pe.n_classes = hg.n_classes;
+    std::memcpy(pe.order, hg.order, sizeof(pe.order));
+  }
+  const cudaError_t e = launch_attn(tm, heads, pe, ws.n_sms, cluster, direct, short_items(hg, weights, n), st, &g_last_attn.mode);
   if (e == cudaSuccess) {
     ++g_launches;
     g_last_attn.items = prm.n_items;
@@ -508,7 +725,7 @@ int psa_profile_events(void* start_event, void* stop_event) {
 
 int psa_mask_sizes(const psa_head_params* params, const psa_problem* prob, int T, int H, int W, int64_t* nb,
                    int64_t* nnz) {
-  Geom g;
+  HostGeom g;
   const int rc = make_geom(prob, T, H, W, false, &g);
   if (rc != PSA_OK) return rc;
   if (nb) *nb = g.NB;
@@ -526,7 +743,7 @@ int psa_mask_sizes(const psa_head_params* params, const psa_problem* prob, int T
 
 int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T, int H, int W, uint8_t* block_mask,
                    int32_t* row_ptr, int32_t* col_idx, int64_t col_capacity, void* stream) {
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, false, &g);
   if (rc != PSA_OK) return rc;
   if (!params) return PSA_ERR_INVALID_ARG;
@@ -582,7 +799,7 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T
 // an earlier one -- more than 128 heads, chunks of a host-tensor call, samples of a batched call -- is not lost).
 // cluster: CTAs per work item, 0: by share_items for these heads.
 static int run_attn(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
-                    int n_heads, const Geom& g, const Layout& lay, cudaStream_t st, bool new_call = true, int cluster = 0) {
+                    int n_heads, const HostGeom& g, const Layout& lay, cudaStream_t st, bool new_call = true, int cluster = 0) {
   int dev;
   Workspace* ws;
   int rc = device_info(&dev, &ws);
@@ -606,7 +823,7 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
     const int n_here = n_heads - head0 < kMaxHeads ? n_heads - head0 : kMaxHeads;
     const long long in_off = lay.shared_qkv ? 0 : (long long)head0 * lay.in_head;
     const long long out_off = (long long)head0 * lay.out_head;
-    TensorMaps tm;
+    TensorMapsEdge tm;
     if ((rc = encode_maps(&tm, static_cast<const uint16_t*>(q) + in_off, static_cast<const uint16_t*>(k) + in_off,
                           static_cast<const uint16_t*>(v) + in_off, static_cast<uint16_t*>(out) + out_off, g, lay, n_here)) != PSA_OK)
       return rc;
@@ -615,7 +832,7 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
     const int n_items = n_here * g.items_per_head;
     const AttnParams prm = {gh, items, hp_dev, ws_header, lse + (long long)head0 * g.Lt, n_items,
                             ws->last_call, lay.shared_qkv ? 1 : 0, static_cast<uint16_t*>(out) + out_off, lay.out_head, lay.out_token};
-    if (launch_call(tm, prm, head_params + head0, weights.data() + head0, *ws, cluster, true, st) != cudaSuccess) return PSA_ERR_CUDA;
+    if (launch_call(tm, prm, g, head_params + head0, weights.data() + head0, *ws, cluster, true, st) != cudaSuccess) return PSA_ERR_CUDA;
     if (g_ev_start && g_ev_stop) cudaEventRecord(g_ev_stop, st);
   }
   return PSA_OK;
@@ -625,7 +842,7 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
 static int attn_fwd_checked(const void* q, const void* k, const void* v, void* out, float* lse,
                             const psa_head_params* head_params, const psa_problem* prob, int T, int H, int W, void* stream,
                             bool new_call, int cluster = 0) {
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
   if (!q || !k || !v || !out || !lse || !head_params) return PSA_ERR_INVALID_ARG;
@@ -657,7 +874,7 @@ int psa_search_select_at_sparsity(const float* losses, const float* sparsity, in
 int psa_attn_fwd_batched(const void* q, const void* k, const void* v, void* out, float* lse,
                          const psa_head_params* head_params, const psa_problem* prob, int n_batch, int64_t stride_batch,
                          int T, int H, int W, void* stream) {
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
   if (!q || !k || !v || !out || !lse || !head_params || n_batch < 1) return PSA_ERR_INVALID_ARG;
@@ -697,7 +914,7 @@ int psa_attn_fwd_batched(const void* q, const void* k, const void* v, void* out,
 int psa_attn_fwd_joint(const void* q, const void* k, const void* v, void* out, float* lse,
                        const psa_head_params* head_params, const psa_problem* prob, int64_t n_text, int T, int H, int W,
                        void* stream) {
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
   if ((rc = set_text(&g, n_text)) != PSA_OK) return rc;
@@ -728,7 +945,7 @@ int64_t psa_search_scratch_bytes(int n_cand, int T, int H, int W) {
 
 int psa_search_losses(const void* q, const void* k, const void* v, const psa_head_params* candidates, int n_cand,
                       const psa_problem* prob, int T, int H, int W, void* scratch, float* losses, void* stream) {
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
   if (!q || !k || !v || !candidates || !scratch || !losses || n_cand < 1) return PSA_ERR_INVALID_ARG;
@@ -780,7 +997,7 @@ int psa_search_select(const float* losses, const float* sparsity, int n, float a
 int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out, float* lse,
                          const psa_head_params* head_params, const psa_problem* prob, int T, int H, int W, void* stream,
                          int32_t* status_detail) {
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
   if (!q || !k || !v || !out || !lse || !head_params) return PSA_ERR_INVALID_ARG;
@@ -811,7 +1028,7 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(base) + kNoAllocItemsOff);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  TensorMaps tm;
+  TensorMapsEdge tm;
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
   if ((rc = encode_maps(&tm, q, k, v, out, g, lay, prob->n_heads)) != PSA_OK) return rc;
   // What the kernels read of the scratch is written by this call's planning kernel; nothing of the previous call is read.
@@ -820,7 +1037,7 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   const int cluster = share_items(*ws, g, weights, prob->n_heads), n_items = (int)n_items_ll, call_id = next_call_id(st);
   const AttnParams prm = {g, items, hp_dev, header, lse, n_items, call_id, 0,
                           out, lay.out_head, lay.out_token};
-  if (launch_call(tm, prm, head_params, weights, *ws, cluster, false, st) != cudaSuccess) return PSA_ERR_CUDA;
+  if (launch_call(tm, prm, g, head_params, weights, *ws, cluster, false, st) != cudaSuccess) return PSA_ERR_CUDA;
   if (status_detail) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return PSA_ERR_CUDA;
     return read_status(header, call_id, status_detail);
@@ -882,7 +1099,7 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
   Chunk chunks[kHostChunks];
   int n_list = 0;
   int last1 = -1, last2 = -1;   // lightest and second-lightest head
-  Geom g;
+  HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
   for (int h = 0; h < prob->n_heads; ++h)

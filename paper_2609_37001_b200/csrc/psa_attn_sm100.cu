@@ -990,26 +990,27 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
       WorkItem wi = make_int4(-1, 0, 0, 0);
       // The attended blocks of class c that are this CTA's (all of them, or its share: by rows, cut between blocks; text keys go with
       // the last share), and how many others come before them.  `before`: rows of the classes before, carried along.
-      auto blocks_of = [&](int c, long long all, long long& before, int* skip) -> int {
+      // (32 bits hold 8 times the rows of the largest block grid, 58,112 x 384)
+      auto blocks_of = [&](int c, int all, int& before, int* skip) -> int {
         const int n = attended.blocks(c);
         *skip = 0;
         if constexpr (kCluster) {
           const int per = block_rows(c), r = (int)cluster_rank(), size = (int)cluster_size();
-          auto upto = [&](long long rows) -> int { return rows <= before ? 0 : (int)min((rows - before) / per, (long long)n); };
+          auto upto = [&](int rows) -> int { return rows <= before ? 0 : min((rows - before) / per, n); };
           const int from = upto(all * r / size), to = upto(all * (r + 1) / size);
-          before += (long long)n * per;
+          before += n * per;
           *skip = from;
           return to - from;
         }
         return n;
       };
-      long long all_rows = 0;
+      int all_rows = 0;
       auto take_share = [&]() {   // (every lane)
         if constexpr (kCluster) {
-          for (int i = 0; i < n_classes; ++i) all_rows += (long long)attended.blocks(class_at(i)) * block_rows(class_at(i));
+          for (int i = 0; i < n_classes; ++i) all_rows += attended.blocks(class_at(i)) * block_rows(class_at(i));
           if (cluster_rank() + 1 < cluster_size()) wi.w |= 1 << 26;
         }
-        long long before = 0;
+        int before = 0;
         int edge_slabs = 0, skip;
         wi.z = 0;
 #pragma unroll 1
@@ -1196,7 +1197,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
         list = list == kLists - 1 ? 0 : list + 1;
       };
       // classes in turn
-      long long before = 0;
+      int before = 0;
 #pragma unroll 1
       for (int ci = 0; ok && ci < n_classes; ++ci) {
       const int c = class_at(ci);

@@ -211,6 +211,9 @@ int last_rows(const EdgeClass& e) { return e.rows - (e.n_slabs - 1) * e.step; }
 // 8 rows in every block's height.
 bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, int nh, int nw) {
   if (g->sub_axis == 2 || g->bh * g->bw < 8) return false;
+  // Blocks of one slab run in split-KV mode, where a slab takes 1,900 clocks and the load warp has no time for lists of boxes: 7
+  // heads of 7x19x25 with 2x8x8 blocks 93 us padded and 135 cut, 18 of 3x25x73 with 1x8x16 165 and 177.
+  if (g->n_sub == 1) return false;
   const int shapes_before = g->n_shapes;
   EdgeClass x = {};
   auto lines = [](int width) -> int { return width < 8 ? 8 / width : 1; };   // that make whole groups of 8 rows
@@ -231,7 +234,9 @@ bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, i
   x.step = (uint16_t)step;
   x.together = (uint8_t)(rows <= kSlabTokens / 2 ? kSlabTokens / rows : 1);
   bool ok = slabs(step) < e->n_slabs || x.together > 1 ||
-            (slabs(step) == e->n_slabs && key_width(last_of(step)) < key_width(last_rows(*e)) &&
+            // (narrower slabs alone do not pay for the maps of a small grid: 16 heads of 11 3x32x4 blocks 55.9 us padded and 62.1 cut,
+            // 13 of 60 1x30x8 blocks 495 and 460)
+            (g->NB >= 32 && slabs(step) == e->n_slabs && key_width(last_of(step)) < key_width(last_rows(*e)) &&
              (for_pattern || (e->n_slabs == g->main_slabs && last_rows(*e) > g->main_last && last_of(step) <= g->main_last)));
   for (int r = 0; ok && r < rows; r += step) {
     int end = 0;
@@ -263,8 +268,8 @@ bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, i
 // Edge blocks (EdgeClass) of a grid whose extents the block does not divide.  T, H, W, the block and its slabs are set.
 //
 // Why: 3D-padding is issued work, along the keys and along the queries.  The last of the seven 30x8 blocks across 52 columns
-// holds 120 of its 240 tokens (12 heads of 21x30x52: 2.60 -> @@A ms), the last 3x8x16 block down 45 rows 240 of 384 (40 heads of
-// 21x45x80: 28.7 -> @@B ms).  Cut like this an edge block is mostly one box a slab, as an ordinary one: the load warp, which has
+// holds 120 of its 240 tokens (12 heads of 21x30x52: 2.60 -> 2.39 ms), the last 3x8x16 block down 45 rows 240 of 384 (40 heads of
+// 21x45x80: 28.7 -> 26.3 ms).  Cut like this an edge block is mostly one box a slab, as an ordinary one: the load warp, which has
 // some 10 clocks for an instruction next to the softmax, fell behind with rows packed tightly across blocks, by boxes of 8 to
 // 128 rows (5,000 clocks a slab) as well as by 16-byte copies (8,000).
 void set_edges(HostGeom* g) {

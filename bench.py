@@ -87,7 +87,7 @@ def slab_split(tile):
 def issued_flops(w):
     """FLOPs the tensor cores are asked for: every attended block pair costs (128 rows per query
     slab) x (keys of every key slab) x 4 x head_dim, padded and idle rows included.  Slabs without any token (of the last
-    block along the stacked axis) are left out, as the kernel leaves them out."""
+    block along the stacked axis) are left out.  An upper bound where the kernel cuts blocks at the grid's edge to their tokens."""
     from oracle import psa_oracle as O
     axis, c0, n_sub, n_last = slab_split(w["tile"])
     n = [-(-x // b) for x, b in zip(w["grid"], w["tile"])]

@@ -873,7 +873,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
 
   // A short query slab leaves its last rows of the Q buffer unwritten; keep them finite.
-  if (kDraws || kEdge || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
+  if (kDraws || kBoxes || g.n_last != kSlabTokens) {   // (the test alone costs the ticket kernel 2 %: see Mode)
     for (uint32_t off = threadIdx.x * 16u; off < 2u * kSlabBytes; off += kThreads * 16u)
       *reinterpret_cast<uint4*>(smem + kOffQ + off) = make_uint4(0u, 0u, 0u, 0u);
     fence_async_smem();

@@ -234,7 +234,7 @@ typedef enum {
   PSA_LAUNCH_DIRECT = 1,         /* every item runs at once, nothing is planned             */
   PSA_LAUNCH_SHARED = 2,         /* CTAs share planned items                                */
   PSA_LAUNCH_SHARED_DIRECT = 3,  /* CTAs share items that all run at once                   */
-  PSA_LAUNCH_TICKET_EDGE = 4,    /* as 0, some blocks at the grid's edge needing fewer slabs */
+  PSA_LAUNCH_TICKET_EDGE = 4,    /* as 0, some blocks having slabs without any token        */
   PSA_LAUNCH_TICKET_SHORT = 5    /* as 0, few key slabs per item, blocks of one slab        */
 } psa_launch_mode;
 int psa_last_attn_launch(int32_t* mode, int32_t* ctas_per_item);

@@ -2020,16 +2020,15 @@ cudaError_t launch_mode(const LaunchConfig& lc, const TensorMapsEdge& tm, const 
 }
 
 // heads: read by launches without planning only.  cluster: CTAs per work item, 1: whole items.  direct: all items run
-// at once, nothing was planned.  *mode: how the launch hands out its items.
+// at once, nothing was planned.  *mode: how the launch hands out its items (empty_slabs: with kTicketEdge for kTicket).
 cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm, int n_sms, int cluster, bool direct,
-                        bool short_items, cudaStream_t stream, Mode* mode) {
+                        bool short_items, bool empty_slabs, cudaStream_t stream, Mode* mode) {
   if (prm.n_items <= 0) return cudaSuccess;
   const int ctas = cluster > 1 || direct ? prm.n_items * cluster : (prm.n_items < n_sms ? prm.n_items : n_sms);
   LaunchConfig lc(ctas, kThreads, kSmemAlloc, stream, cluster);
   *mode = cluster > 1 ? (direct ? kSharedDirect : kShared) : (direct ? kDirect : (short_items ? kTicketShort : kTicket));
   const Mode kernel = *mode;
-  for (int c = 1; c < 8; ++c)
-    if (kernel == kTicket && (c & ~prm.g.edge_axes) == 0 && prm.g.slabs_of[c] < prm.g.n_sub) *mode = kTicketEdge;
+  if (kernel == kTicket && empty_slabs) *mode = kTicketEdge;
   switch (kernel) {
     case kDirect: return launch_mode<kDirect>(lc, tm, heads, prm);
     case kShared: return launch_mode<kShared>(lc, tm, heads, prm);

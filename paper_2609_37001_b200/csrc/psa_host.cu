@@ -22,7 +22,7 @@ size_t plan_smem_bytes(const Geom& g);
 cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
                         WorkItem* items, cudaStream_t stream);
 cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm, int n_sms, int cluster,
-                        bool direct, bool short_items, cudaStream_t stream, Mode* mode);
+                        bool direct, bool short_items, bool empty_slabs, cudaStream_t stream, Mode* mode);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
                                  float* losses, cudaStream_t stream, int* launches);
@@ -121,6 +121,7 @@ struct BoxShape {
 struct HostGeom : Geom {
   EdgeClass cls[8];
   int main_slabs, main_last, cut;
+  bool empty_slabs;   // some blocks have, uncut, slabs without any token
   int n_classes;
   uint8_t order[8];
   int n_shapes;
@@ -276,6 +277,8 @@ void set_edges(HostGeom* g) {
   const int rt = g->T - (g->Tp - 1) * g->bt, rh = g->H - (g->Hp - 1) * g->bh, rw = g->W - (g->Wp - 1) * g->bw;   // of the last block
   g->edge_axes = (rt < g->bt ? 1 : 0) | (rh < g->bh ? 2 : 0) | (rw < g->bw ? 4 : 0);
   g->s_edge = g->Sp - g->Wp;
+  const int along = g->sub_axis == 0 ? rt : (g->sub_axis == 1 ? rh : rw), slab = g->sub_axis == 0 ? g->ct : (g->sub_axis == 1 ? g->ch : g->cw);
+  g->empty_slabs = (along + slab - 1) / slab < g->n_sub;
   g->n_shapes = g->n_classes = 0;
   int pattern = 0;   // its class
   for (int c = 0; c < 8; ++c)
@@ -635,7 +638,8 @@ cudaError_t launch_call(const TensorMapsEdge& tm, const AttnParams& prm, const H
     pe.n_classes = hg.n_classes;
     std::memcpy(pe.order, hg.order, sizeof(pe.order));
   }
-  const cudaError_t e = launch_attn(tm, heads, pe, ws.n_sms, cluster, direct, short_items(hg, weights, n), st, &g_last_attn.mode);
+  const cudaError_t e = launch_attn(tm, heads, pe, ws.n_sms, cluster, direct, short_items(hg, weights, n), hg.empty_slabs, st,
+                                    &g_last_attn.mode);
   if (e == cudaSuccess) {
     ++g_launches;
     g_last_attn.items = prm.n_items;

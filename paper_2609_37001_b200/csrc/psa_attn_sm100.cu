@@ -72,8 +72,8 @@ constexpr int kBarQFull = 0, kBarQEmpty = 2, kBarPairFull = 4, kBarSlotEmpty = k
               kBarSchedEmpty = kBarSchedFull + 2, kBarStage = kBarSchedEmpty + 2, kBarMerge = kBarStage + 2,
               kBarDrain = kBarMerge + 1, kNumBars = (kBarDrain + 1 + 1) & ~1;
 constexpr uint32_t kOffMeta = kOffBar + kNumBars * 8;           // kMetaRing x 8 words
-constexpr uint32_t kOffMaskT = kOffMeta + kMetaRing * 32;       // [kMaxTp / 32] words
-constexpr uint32_t kOffMaskS = kOffMaskT + (kMaxTp / 32) * 4;   // [2][kMaxSp / 32] words (key_block_sets)
+constexpr uint32_t kOffMaskT = kOffMeta + kMetaRing * 32;       // [2][kMaxTp / 32] words (key_block_sets)
+constexpr uint32_t kOffMaskS = kOffMaskT + 2 * (kMaxTp / 32) * 4;   // [2][kMaxSp / 32] words, or [4][kMaxSp / 64]
 constexpr uint32_t kOffSched = kOffMaskS + 2 * (kMaxSp / 32) * 4;   // two published work items
 constexpr uint32_t kOffMisc = kOffSched + 32;                   // tmem base, abort flag
 constexpr uint32_t kOffXchg = kOffMisc + 16;                    // split-KV merge: (m, l) of 128 rows
@@ -726,8 +726,14 @@ struct Attended {
   }
 };
 
+// Words in front of the set of class c's spatial coordinates: two sets, or four of a grid that is cut along both h and w, whose spatial
+// blocks are at most half as many (cut_edges).
+__device__ __forceinline__ int spatial_set(const Geom& g, int c) { return (g.edge_axes & 6) == 6 ? (c >> 1) * (kMaxSp / 64) : (c > 1 ? kMaxSp / 32 : 0); }
+
 // Attended key-block coordinates of an item's query block (all of them for text queries), one bit per block coordinate, by a
-// whole warp; spatial coordinates in the last column behind the others if these are edge blocks.
+// whole warp: temporal ones without and with the edge one, spatial ones of classes 0, 2, 4 and 6 (those that the grid has).
+// (With one set each, and its classes told apart in the loop over the key blocks, edge slabs took the load warp 10,000 clocks of
+// its CTA's time instead of 7,000: 3 heads of 22x11x12 with 1x12x16 blocks, all dense, 74 us instead of 58.)
 template <bool kEdge>
 __device__ __forceinline__ Attended key_block_sets(const Geom& g, bool textq, int qb, const psa_head_params& p, int lane, uint32_t* maskT,
                                                    uint32_t* maskS) {
@@ -736,9 +742,12 @@ __device__ __forceinline__ Attended key_block_sets(const Geom& g, bool textq, in
   for (int b = 0; b < g.Tp; b += 32) {
     const int tk = b + lane;
     const unsigned m = __ballot_sync(0xffffffffu, tk < g.Tp && (textq || axis_attends(tk - tq, p.Tw, p.To, p.Ts)));
-    if (lane == 0) maskT[b >> 5] = m;
-    a.t += (uint32_t)__popc(m);
-    if (kEdge && (g.edge_axes & 1) && b == ((g.Tp - 1) & ~31)) a.t += (m >> ((g.Tp - 1) & 31) & 1u) * 0xffffu;   // one from the lower to the upper half
+    const unsigned last = kEdge && (g.edge_axes & 1) && b == ((g.Tp - 1) & ~31) ? m & 1u << ((g.Tp - 1) & 31) : 0u;
+    if (lane == 0) {
+      maskT[b >> 5] = m & ~last;
+      if (kEdge && (g.edge_axes & 1)) maskT[kMaxTp / 32 + (b >> 5)] = last;
+    }
+    a.t += (uint32_t)(__popc(m & ~last) | __popc(last) << 16);
   }
   for (int b = 0; b < g.Sp; b += 32) {
     const int sk = b + lane;
@@ -750,8 +759,11 @@ __device__ __forceinline__ Attended key_block_sets(const Geom& g, bool textq, in
     }
     const unsigned col = g.edge_axes & 4 ? __ballot_sync(0xffffffffu, sk % g.Wp == g.Wp - 1) : 0u, row = last_row_word(g, b);
     if (lane == 0) {
-      maskS[b >> 5] = m & ~col;
-      maskS[kMaxSp / 32 + (b >> 5)] = m & col;
+      uint32_t* to = maskS + (b >> 5);
+      to[0] = m & ~col & ~row;
+      if (g.edge_axes & 2) to[spatial_set(g, 2)] = m & ~col & row;
+      if (g.edge_axes & 4) to[spatial_set(g, 4)] = m & col & ~row;
+      if ((g.edge_axes & 6) == 6) to[spatial_set(g, 6)] = m & col & row;
     }
     a.s += (uint32_t)(__popc(m & ~col & ~row) | __popc(m & ~col & row) << 16);
     a.s4 += (uint32_t)(__popc(m & col & ~row) | __popc(m & col & row) << 16);
@@ -838,15 +850,10 @@ __device__ __forceinline__ void merge_cluster(const Params& prm, const uint8_t* 
 //                 buffers are released by the MMAs that read them last (a commit), the output goes from registers to
 //                 memory instead of through those buffers, and the accumulators are waited for at the first P V only.
 //                 12 heads of 1x8x16 blocks attending 19.5 of them, 8x32x48 grid: 221 -> 198 us
-// kGrid: what the grid's edge asks for.
-//   kWhole    nothing: the block divides the grid, and no slab has padding except beyond the text
-//   kPadded   blocks at the edge have the slabs of ordinary ones, or fewer; padding is masked
-//   kCut      some blocks at the edge are cut to their tokens (EdgeClass)
 // (A slab of a cut grid goes through a list of boxes, which costs the load warp some 700 clocks: more than it has in split-KV mode.
 // 2 heads of 5x16x63 with 1x30x8 blocks, one slab each, took 28.6 us as a cut grid and take 23.6 as a padded one.)
-template <int kGrid> struct ArgsOf { typedef TensorMaps maps; typedef AttnParamsEdge params; };
-template <> struct ArgsOf<kWhole> { typedef TensorMaps maps; typedef AttnParams params; };
-template <> struct ArgsOf<kCut> { typedef TensorMapsEdge maps; typedef AttnParamsEdge params; };
+template <int kGrid> struct ArgsOf { typedef TensorMaps maps; typedef AttnParams params; };
+template <> struct ArgsOf<kCut> { typedef TensorMapsCut maps; typedef AttnParamsCut params; };
 template <int kMode, int kGrid>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const __grid_constant__ HeadParamsArray heads,
@@ -960,27 +967,21 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
     uint32_t pair_g = 0;       // pair barriers armed so far
     uint32_t kv_g = 0;         // key slabs issued so far
     uint32_t it_q0 = 0, it_q1 = 0; // items in which query slab i was active
-    // kPadded: position of key c = lane + 32 i within a slab, t << 16 | h << 8 | w, for the validity words of slabs at the grid's
-    // edge (a block's last slab is only shorter along its slowest axis, so it is laid out alike).  Computed once: with
-    // its divisions in the slab loop this warp took 3,800 clocks per edge slab and the whole CTA waited for it.
-    int pos[4];
-#pragma unroll
-    for (int i = 0; i < 4 && kGrid == kPadded; ++i) {
-      const int c = lane + 32 * i;
-      pos[i] = (c / (g.cw * g.ch)) << 16 | ((c / g.cw) % g.ch) << 8 | (c % g.cw);
-    }
     // block -> row of the spatial block grid without a division: sk, Wp <= 2^11
     const uint32_t magic_w = ((1u << 22) + (uint32_t)g.Wp - 1u) / (uint32_t)g.Wp;
     auto class_at = [&](int i) -> int {
-      if constexpr (kEdge) return prm.order[i];
-      return 0;
+      if constexpr (kBoxes) return prm.order[i];
+      return i == 0 ? 0 : g.edge_axes;
     };
     int n_classes = 1;
-    if constexpr (kEdge) n_classes = prm.n_classes;
-    auto block_rows = [&](int c) -> int {
-      if constexpr (kEdge) return prm.cls[c].rows;
-      return g.bt * g.bh * g.bw;
-    };
+    bool late = !kDraws;   // an item is published when its classes of key blocks have been counted
+    if constexpr (kBoxes) {
+      n_classes = prm.n_classes;
+      late = late || !prm.planned;
+    } else if constexpr (kEdge) {
+      n_classes = g.edge_axes != 0 ? 2 : 1;
+      late = late || g.edge_axes != 0;
+    }
     bool ok = tmem_ok;
     pdl_wait();   // the work items are written by the planning kernel, q, k and v by whatever ran before
     for (uint32_t n = 0; ok; ++n) {
@@ -988,14 +989,15 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
       ok = mbar_wait_warp(bar(kBarSchedEmpty + sslot), ((n >> 1) & 1u) ^ 1u, abort_flag, 0x401);
       if (!ok) break;
       WorkItem wi = make_int4(-1, 0, 0, 0);
-      // The attended blocks of class c that are this CTA's (all of them, or its share: by rows, cut between blocks; text keys go with
-      // the last share), and how many others come before them.  `before`: rows of the classes before, carried along.
+      int skip = 0, left = 0x7fffffff;   // attended key blocks before this CTA's share, and those still to load (kBoxes: of a class)
+      // kBoxes: the attended blocks of class c that are this CTA's (all of them, or its share: by rows, cut between blocks), and how
+      // many others come before them.  `before`: rows of the classes before, carried along.
       // (32 bits hold 8 times the rows of the largest block grid, 58,112 x 384)
       auto blocks_of = [&](int c, int all, int& before, int* skip) -> int {
         const int n = attended.blocks(c);
         *skip = 0;
-        if constexpr (kCluster) {
-          const int per = block_rows(c), r = (int)cluster_rank(), size = (int)cluster_size();
+        if constexpr (kCluster && kBoxes) {
+          const int per = prm.cls[c].rows, r = (int)cluster_rank(), size = (int)cluster_size();
           auto upto = [&](int rows) -> int { return rows <= before ? 0 : min((rows - before) / per, n); };
           const int from = upto(all * r / size), to = upto(all * (r + 1) / size);
           before += n * per;
@@ -1004,27 +1006,38 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
         }
         return n;
       };
-      int all_rows = 0;
+      int all = 0;   // rows of the attended blocks
       auto take_share = [&]() {   // (every lane)
-        if constexpr (kCluster) {
-          for (int i = 0; i < n_classes; ++i) all_rows += attended.blocks(class_at(i)) * block_rows(class_at(i));
-          if (cluster_rank() + 1 < cluster_size()) wi.w |= 1 << 26;
-        }
-        int before = 0;
-        int edge_slabs = 0, skip;
-        wi.z = 0;
-#pragma unroll 1
-        for (int i = 0; i < n_classes; ++i) {
-          const int c = class_at(i), n = blocks_of(c, all_rows, before, &skip);
-          if constexpr (kEdge) {
-            if (!prm.cls[c].in_pattern) {
-              edge_slabs += n ? class_slabs(prm.cls[c], n) : 0;
-              continue;
-            }
+        // (this CTA's share of the item's key blocks; the text keys go with the last share)
+        if (kCluster && cluster_rank() + 1 < cluster_size()) wi.w |= 1 << 26;
+        if constexpr (kBoxes) {
+          if constexpr (kCluster) {
+            for (int i = 0; i < n_classes; ++i) all += attended.blocks(class_at(i)) * prm.cls[class_at(i)].rows;
           }
-          wi.z += n;
+          int before = 0, edge_slabs = 0;
+          wi.z = 0;
+#pragma unroll 1
+          for (int i = 0; i < n_classes; ++i) {
+            const int c = class_at(i), n = blocks_of(c, all, before, &skip);
+            if (prm.cls[c].in_pattern) wi.z += n;
+            else edge_slabs += n ? class_slabs(prm.cls[c], n) : 0;
+          }
+          wi.x |= edge_slabs << 8;
+        } else {   // whole blocks, those of fewer slabs last
+          wi.z = attended.blocks(0);
+          const int main = wi.z, edge = n_classes > 1 ? attended.blocks(g.edge_axes) : 0, edge_slabs = kEdge ? g.slabs_of[g.edge_axes] : 0;
+          left = main + edge;
+          if constexpr (kCluster) {   // by slabs, cut between blocks
+            const int slabs = kEdge && edge != 0 ? g.main_slabs : 1, all = main * slabs + edge * edge_slabs, r = (int)cluster_rank();
+            auto by = [](int n, int d) -> int { return d == 1 ? n : (d == 2 ? n >> 1 : n / 3); };   // (a division costs this warp some 400 clocks)
+            auto upto = [&](int n) -> int { return n <= main * slabs ? by(n, slabs) : main + by(n - main * slabs, edge_slabs); };
+            const int shift = 31 - __clz((int)cluster_size());   // 2, 4 or 8 CTAs
+            skip = upto(all * r >> shift);
+            left = upto(all * (r + 1) >> shift) - skip;
+            wi.z = max(min(skip + left, main) - skip, 0);
+          }
+          if (edge != 0) wi.x |= (left - wi.z) * edge_slabs << 8;
         }
-        if (kEdge) wi.x |= edge_slabs << 8;
       };
       auto publish = [&]() {   // by lane 0
         sched[sslot].x = wi.x; sched[sslot].y = wi.y; sched[sslot].z = wi.z; sched[sslot].w = wi.w;
@@ -1034,7 +1047,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
         if (lane == 0) {
           const int ticket = atomicAdd(prm.ws_header + kWsCounter, 1);
           if (ticket < prm.n_items) wi = prm.items[ticket];
-          if (!kEdge) publish();
+          if (!late) publish();
         }
         wi.x = __shfl_sync(0xffffffffu, wi.x, 0);
         wi.y = __shfl_sync(0xffffffffu, wi.y, 0);
@@ -1043,7 +1056,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
         wi = kPlanned ? prm.items[blockIdx.x / cluster_size()] : first_item;
       }
       if (kPlanned && wi.x >= 0) attended = key_block_sets<kEdge>(g, ((wi.w >> 25) & 1) != 0, wi.y, prm.hp_dev[wi.x], lane, maskT, maskS);
-      if (kEdge || !kDraws) {
+      if (late) {
         if (wi.x >= 0) take_share();
         if (lane == 0) publish();
       }
@@ -1106,7 +1119,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
             n_boxes = list_boxes(e, sub0 + i, t0, h0, w0);
             const bool whole = sub0 + i + 1 < e.n_slabs || !(e.in_pattern || e.together > 1);
             if (e.together > 1) n_boxes = 1;   // (a block alone: no box of zeros)
-            if (lane == 0) mbar_expect_tx(bar(kBarQFull + i), whole ? kSlabBytes : (uint32_t)(e.together > 1 ? e.rows : prm.main_last) * 256u);
+            if (lane == 0) mbar_expect_tx(bar(kBarQFull + i), whole ? kSlabBytes : (uint32_t)(e.together > 1 ? e.rows : g.main_last) * 256u);
             load_lists(box_of(list, list), bar(kBarQFull + i), tms.q, 0u, 0, tms.q, sbase + kOffQ + (uint32_t)i * kSlabBytes, n_boxes);
           }
         }
@@ -1201,37 +1214,31 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
 #pragma unroll 1
       for (int ci = 0; ok && ci < n_classes; ++ci) {
       const int c = class_at(ci);
-      int skip, left = blocks_of(c, all_rows, before, &skip);   // blocks before this CTA's share, and those still to load
-      const uint32_t* mask_s = maskS + (kEdge && (c & 4) ? kMaxSp / 32 : 0);
+      if constexpr (kBoxes) left = blocks_of(c, all, before, &skip);
+      const uint32_t *mask_t = maskT + (c & 1) * (kMaxTp / 32), *mask_s = maskS + spatial_set(g, c);
       int listed = 0;
       // The class in registers (constants by a computed index are slow): lane b holds box b, lane 4 s + i word i of slab s's validity.
       int rows = 0, n_slabs = 1, together = 1, n_full = 0;
       uint32_t first_box = 0, valid = 0, last_keys = kSlabTokens;
       EdgeBox mine_box = {};
-      if constexpr (kEdge) n_slabs = prm.cls[c].n_slabs;
-      else n_slabs = g.n_sub;
+      n_slabs = kEdge ? g.slabs_of[c] : g.n_sub;
       if constexpr (kBoxes) {
         const EdgeClass& e = prm.cls[c];
         rows = e.rows;
         together = e.together;
         n_full = e.together + e.n_boxes - 1;
         first_box = *reinterpret_cast<const uint32_t*>(e.first_box);
-        if (e.in_pattern) last_keys = (uint32_t)prm.main_last;
+        if (e.in_pattern) last_keys = (uint32_t)g.main_last;
         if (lane < 12) valid = e.valid[lane >> 2][lane & 3];
         if (lane < kMaxEdgeBoxes) mine_box = e.box[lane];
       }
       for (int tw = 0; ok && left > 0 && tw < g.Tp; tw += 32) {
-        uint32_t mt = maskT[tw >> 5];
-        if (kEdge && (g.edge_axes & 1)) {
-          const uint32_t edge = tw == ((g.Tp - 1) & ~31) ? 1u << ((g.Tp - 1) & 31) : 0u;
-          mt &= c & 1 ? edge : ~edge;
-        }
+        uint32_t mt = mask_t[tw >> 5];
         while (ok && left > 0 && mt) {
           const int tk = tw + __ffs(mt) - 1;
           mt &= mt - 1;
           for (int sw = 0; ok && left > 0 && sw < g.Sp; sw += 32) {
             uint32_t ms = mask_s[sw >> 5];
-            if (kEdge) ms &= c & 2 ? last_row_word(g, sw) : ~last_row_word(g, sw);
             while (ok && ms) {
               const int sk = sw + __ffs(ms) - 1;
               ms &= ms - 1;
@@ -1239,7 +1246,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
                 if (skip > 0) { --skip; continue; }
                 if (left == 0) break;
               }
-              if (kCluster || kEdge) --left;
+              if (kCluster || kBoxes) --left;
               const int hb = (int)(((unsigned long long)(uint32_t)sk * magic_w) >> 22);
               int t0 = tk * g.bt, h0 = hb * g.bh, w0 = (sk - hb * g.Wp) * g.bw;
               if constexpr (kBoxes) {
@@ -1279,7 +1286,8 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
                   const int rt = g.T - t0, rh = g.H - h0, rw = g.W - w0;
                   if (et > rt || eh > rh || ew > rw) {
                     auto valid = [&](int i) -> bool {
-                      return ((pos[i] >> 16) < rt && ((pos[i] >> 8) & 0xff) < rh && (pos[i] & 0xff) < rw) || lane + 32 * i >= ntok;
+                      const int x = lane + 32 * i;
+                      return ((x >> g.pos_ts) < rt && ((x >> g.pos_ws) & (g.ch - 1)) < rh && (x & (g.cw - 1)) < rw) || x >= ntok;
                     };
                     vw0 = __ballot_sync(0xffffffffu, valid(0));
                     vw1 = __ballot_sync(0xffffffffu, valid(1));
@@ -1401,8 +1409,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
     uint32_t it_o0 = 0, it_o1 = 0;    // items in which accumulator O_i was used
     if constexpr (!kDraws) pdl_wait();   // (see pdl_wait)
     // keys of a slab from its index within its block (r = j mod n_sub, carried along: no division)
-    int n_sub = g.n_sub, n_last = g.n_last;
-    if constexpr (kEdge) { n_sub = prm.main_slabs; n_last = prm.main_last; }
+    const int n_sub = kEdge ? g.main_slabs : g.n_sub, n_last = kEdge ? g.main_last : g.n_last;
     const int r_last = n_sub - 1;
     auto nk_at = [&](int r) -> int { return r == r_last ? n_last : kSlabTokens; };
     auto r_inc = [&](int r) -> int { return r == r_last ? 0 : r + 1; };
@@ -1641,8 +1648,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
     bool ok = true, met = false;   // met: cluster mode's first barrier passed
     const float neg_inf = __int_as_float(0xff800000);
     float2* xchg = reinterpret_cast<float2*>(smem + kOffXchg);
-    int n_sub = g.n_sub, n_last = g.n_last;
-    if constexpr (kEdge) { n_sub = prm.main_slabs; n_last = prm.main_last; }
+    const int n_sub = kEdge ? g.main_slabs : g.n_sub, n_last = kEdge ? g.main_last : g.n_last;
     if constexpr (!kDraws) pdl_wait();   // (see pdl_wait)
 
     for (uint32_t n = 0; ok; ++n) {
@@ -2006,8 +2012,8 @@ cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, i
 }
 
 template <int kMode>
-cudaError_t launch_mode(const LaunchConfig& lc, const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm) {
-  if (prm.cut) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kCut>, tm, heads, prm);
+cudaError_t launch_mode(const LaunchConfig& lc, Grid grid, const TensorMapsCut& tm, const HeadParamsArray& heads, const AttnParamsCut& prm) {
+  if (grid == kCut) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kCut>, tm, heads, prm);
   TensorMaps plain;
   for (int i = 0; i < 3; ++i) {
     plain.q[i] = tm.q[i];
@@ -2015,13 +2021,14 @@ cudaError_t launch_mode(const LaunchConfig& lc, const TensorMapsEdge& tm, const 
     plain.v[i] = tm.v[i];
     plain.o[i] = tm.o[i];
   }
-  if (prm.g.edge_axes) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kPadded>, plain, heads, prm);
-  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kWhole>, plain, heads, static_cast<const AttnParams&>(prm));
+  const AttnParams& p = prm;
+  if (grid == kPadded) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kPadded>, plain, heads, p);
+  return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kWhole>, plain, heads, p);
 }
 
 // heads: read by launches without planning only.  cluster: CTAs per work item, 1: whole items.  direct: all items run
 // at once, nothing was planned.  *mode: how the launch hands out its items (empty_slabs: with kTicketEdge for kTicket).
-cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm, int n_sms, int cluster, bool direct,
+cudaError_t launch_attn(const TensorMapsCut& tm, const HeadParamsArray& heads, const AttnParamsCut& prm, int n_sms, int cluster, Grid grid, bool direct,
                         bool short_items, bool empty_slabs, cudaStream_t stream, Mode* mode) {
   if (prm.n_items <= 0) return cudaSuccess;
   const int ctas = cluster > 1 || direct ? prm.n_items * cluster : (prm.n_items < n_sms ? prm.n_items : n_sms);
@@ -2030,11 +2037,11 @@ cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, 
   const Mode kernel = *mode;
   if (kernel == kTicket && empty_slabs) *mode = kTicketEdge;
   switch (kernel) {
-    case kDirect: return launch_mode<kDirect>(lc, tm, heads, prm);
-    case kShared: return launch_mode<kShared>(lc, tm, heads, prm);
-    case kSharedDirect: return launch_mode<kSharedDirect>(lc, tm, heads, prm);
-    case kTicketShort: return launch_mode<kTicketShort>(lc, tm, heads, prm);
-    default: return launch_mode<kTicket>(lc, tm, heads, prm);
+    case kDirect: return launch_mode<kDirect>(lc, grid, tm, heads, prm);
+    case kShared: return launch_mode<kShared>(lc, grid, tm, heads, prm);
+    case kSharedDirect: return launch_mode<kSharedDirect>(lc, grid, tm, heads, prm);
+    case kTicketShort: return launch_mode<kTicketShort>(lc, grid, tm, heads, prm);
+    default: return launch_mode<kTicket>(lc, grid, tm, heads, prm);
   }
 }
 

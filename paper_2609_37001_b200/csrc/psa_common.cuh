@@ -15,12 +15,17 @@ constexpr int kMaxTp = 256;       // limits of the in-kernel key-block bitmasks
 constexpr int kMaxSp = 2048;
 constexpr size_t kMaxSmemBytes = 232448;   // 227 KB of shared memory that a CTA may use
 
-// Blocks that reach beyond the grid (3D-padding) are edge blocks, the last ones along an axis.  A class has a bit for each axis
-// on which they are the last (1: t, 2: h, 4: w); class 0 is an ordinary block.  An edge block is cut to the part that holds its
-// tokens: `rows` of them, in the order t, h, w of frames of lines of 1 << lw, padded as far as loading by TMA boxes asks for.
+// How a launch treats blocks that reach beyond the grid (3D-padding).
+//   kWhole    the block divides the grid: there are none
+//   kPadded   they are loaded like the others, with masks, less the slabs that hold no token
+//   kCut      some are cut to their tokens
+enum Grid { kWhole, kPadded, kCut };
+// They are edge blocks, the last ones along an axis.  A class has a bit for each axis on which they are the last (1: t, 2: h, 4: w);
+// class 0 is an ordinary block.  A padded grid tells only blocks of fewer slabs apart, the last ones along the axis on which slabs stack.
 // Key slabs follow a pattern, that of the ordinary blocks or, where there are none, of the most frequent class: main_slabs slabs
-// per block, of 128 keys and the last one of main_last.  The slabs of blocks that do not follow it come behind, 128 keys each.  What
-// tokens do not fill is zeros, with validity bits of 0.
+// per block, of 128 keys and the last one of main_last.  The slabs of blocks that do not follow it come behind, 128 keys each.
+// In a cut grid an edge block is the part that holds its tokens: `rows` of them, in the order t, h, w of frames of lines of 1 << lw,
+// padded as far as loading by TMA boxes asks for.  What tokens do not fill is zeros, with validity bits of 0.
 struct alignas(8) EdgeBox {   // a box of a slab: its map, first row, and first token relative to the block's
   uint8_t map, row8;        // (row / 8)
   uint16_t t, h, w;         // t == kZeros: a box of zeros
@@ -54,6 +59,7 @@ struct Geom {
   int edge_axes;           // axes on which the grid has edge blocks (EdgeClass)
   int s_edge;              // spatial block coordinates from here on are the last ones along h
   uint8_t slabs_of[8];     // query slabs of a block by class
+  int main_slabs, main_last;   // the pattern of key slabs
   int n_heads;
   int items_per_block;     // work items per query block = ceil(n_sub / 2); of an edge block by its n_slabs
   float scale_log2;        // softmax scale times log2(e)
@@ -89,12 +95,11 @@ constexpr int kMaxMaps = 20;
 struct TensorMaps {
   CUtensorMap q[3], k[3], v[3], o[3];
 };
-struct TensorMapsEdge {
+struct TensorMapsCut {
   CUtensorMap q[kMaxMaps], k[kMaxMaps], v[kMaxMaps], o[kMaxMaps];
 };
 // How an attention launch hands out its work items (see attn_fwd_kernel); the values are those of psa_launch_mode.  (kTicketEdge
 // is only reported; the kernel is that of kTicket.)
-enum Grid { kWhole, kPadded, kCut };   // (see attn_fwd_kernel)
 enum Mode { kTicket, kDirect, kShared, kSharedDirect, kTicketEdge, kTicketShort };
 
 // Arguments of one attention launch; lse and out start at the launch's first head.
@@ -111,11 +116,10 @@ struct AttnParams {
   long long out_head, out_token;
 };
 
-// The same of a launch on a grid with edge blocks.
-struct AttnParamsEdge : AttnParams {
+// The same of a launch on a cut grid.
+struct AttnParamsCut : AttnParams {
   EdgeClass cls[8];
-  int main_slabs, main_last;   // the pattern
-  int cut;                     // 1: the slabs are those of `box`; 0: those of ordinary blocks, of an edge block maybe fewer
+  int planned;                 // 1: every class follows the pattern, so that an item's number of key blocks is the planned one
   int n_classes;               // classes that the grid has, those of the pattern first
   uint8_t order[8];
 };

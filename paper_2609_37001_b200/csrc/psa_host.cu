@@ -21,8 +21,8 @@ cudaError_t attn_init(int clusters[3]);
 size_t plan_smem_bytes(const Geom& g);
 cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, int* ws_header, psa_head_params* hp_dev,
                         WorkItem* items, cudaStream_t stream);
-cudaError_t launch_attn(const TensorMapsEdge& tm, const HeadParamsArray& heads, const AttnParamsEdge& prm, int n_sms, int cluster,
-                        bool direct, bool short_items, bool empty_slabs, cudaStream_t stream, Mode* mode);
+cudaError_t launch_attn(const TensorMapsCut& tm, const HeadParamsArray& heads, const AttnParamsCut& prm, int n_sms, int cluster,
+                        Grid grid, bool direct, bool short_items, bool empty_slabs, cudaStream_t stream, Mode* mode);
 size_t search_partial_bytes(int n_cand);
 cudaError_t launch_search_losses(const void* outs, const void* ref, long long elems_per_cand, int n_cand, double* partial,
                                  float* losses, cudaStream_t stream, int* launches);
@@ -120,9 +120,9 @@ struct BoxShape {
 };
 struct HostGeom : Geom {
   EdgeClass cls[8];
-  int main_slabs, main_last, cut;
+  Grid grid;
+  int planned, n_classes;
   bool empty_slabs;   // some blocks have, uncut, slabs without any token
-  int n_classes;
   uint8_t order[8];
   int n_shapes;
   BoxShape shape[kMaxMaps - 3];
@@ -211,10 +211,6 @@ int last_rows(const EdgeClass& e) { return e.rows - (e.n_slabs - 1) * e.step; }
 // probability of 0 would not keep out if they are infinite -- so lines shorter than 8 tokens need a whole number of groups of
 // 8 rows in every block's height.
 bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, int nh, int nw) {
-  if (g->sub_axis == 2 || g->bh * g->bw < 8) return false;
-  // Blocks of one slab run in split-KV mode, where a slab takes 1,900 clocks and the load warp has no time for lists of boxes: 7
-  // heads of 7x19x25 with 2x8x8 blocks 93 us padded and 135 cut, 18 of 3x25x73 with 1x8x16 165 and 177.
-  if (g->n_sub == 1) return false;
   const int shapes_before = g->n_shapes;
   EdgeClass x = {};
   auto lines = [](int width) -> int { return width < 8 ? 8 / width : 1; };   // that make whole groups of 8 rows
@@ -266,37 +262,34 @@ bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, i
   return true;
 }
 
-// Edge blocks (EdgeClass) of a grid whose extents the block does not divide.  T, H, W, the block and its slabs are set.
+// Edge blocks of a cut grid (EdgeClass); false, if no class is cut.  `axes`: those on which the grid has edge blocks, whose extents are
+// rt, rh and rw.
 //
 // Why: 3D-padding is issued work, along the keys and along the queries.  The last of the seven 30x8 blocks across 52 columns
 // holds 120 of its 240 tokens (12 heads of 21x30x52: 2.60 -> 2.39 ms), the last 3x8x16 block down 45 rows 240 of 384 (40 heads of
 // 21x45x80: 28.7 -> 26.3 ms).  Cut like this an edge block is mostly one box a slab, as an ordinary one: the load warp, which has
 // some 10 clocks for an instruction next to the softmax, fell behind with rows packed tightly across blocks, by boxes of 8 to
 // 128 rows (5,000 clocks a slab) as well as by 16-byte copies (8,000).
-void set_edges(HostGeom* g) {
-  const int rt = g->T - (g->Tp - 1) * g->bt, rh = g->H - (g->Hp - 1) * g->bh, rw = g->W - (g->Wp - 1) * g->bw;   // of the last block
-  g->edge_axes = (rt < g->bt ? 1 : 0) | (rh < g->bh ? 2 : 0) | (rw < g->bw ? 4 : 0);
-  g->s_edge = g->Sp - g->Wp;
-  const int along = g->sub_axis == 0 ? rt : (g->sub_axis == 1 ? rh : rw), slab = g->sub_axis == 0 ? g->ct : (g->sub_axis == 1 ? g->ch : g->cw);
-  g->empty_slabs = (along + slab - 1) / slab < g->n_sub;
+bool cut_edges(HostGeom* g, int axes, int rt, int rh, int rw) {
+  if (g->sub_axis == 2 || g->bh * g->bw < 8) return false;
+  if ((axes & 6) == 6 && g->Sp > kMaxSp / 2) return false;   // (the kernel keeps four sets of spatial coordinates of such a grid)
+  // Blocks of one slab run in split-KV mode, where a slab takes 1,900 clocks and the load warp has no time for lists of boxes: 7
+  // heads of 7x19x25 with 2x8x8 blocks 93 us padded and 135 cut, 18 of 3x25x73 with 1x8x16 165 and 177.
+  if (g->n_sub == 1) return false;
+  g->edge_axes = axes;
   g->n_shapes = g->n_classes = 0;
   int pattern = 0;   // its class
   for (int c = 0; c < 8; ++c)
     if (class_blocks(*g, 0) == 0 && class_blocks(*g, c) > class_blocks(*g, pattern)) pattern = c;
-  g->slabs_of[0] = (uint8_t)g->n_sub;
-  if (g->edge_axes == 0) return;
+  int tokens[8][3];   // of a block of every class, along the axes
+  bool cut = false;
   auto make = [&](int c) {
-    EdgeClass& e = g->cls[c];
-    const int nt = c & 1 ? rt : g->bt, nh = c & 2 ? rh : g->bh, nw = c & 4 ? rw : g->bw;   // tokens along the axes
-    whole_slabs(*g, &e, nt, nh, nw);
-    if (c != 0 && cut_to_tokens(g, &e, c, c == pattern, nt, nh, nw)) g->cut = 1;
-    for (int s = 0; s < e.n_slabs; ++s) {
-      const int have = s + 1 < e.n_slabs ? e.step : last_rows(e);
-      for (int r = 0; r < have * e.together; ++r) {
-        const int x = s * e.step + r % have, y = x % e.frame;
-        if (x / e.frame < nt && (y >> e.lw) < nh && (y & ((1 << e.lw) - 1)) < nw) e.valid[s][r / 32] |= 1u << (r % 32);
-      }
-    }
+    int* n = tokens[c];
+    n[0] = c & 1 ? rt : g->bt;
+    n[1] = c & 2 ? rh : g->bh;
+    n[2] = c & 4 ? rw : g->bw;
+    whole_slabs(*g, &g->cls[c], n[0], n[1], n[2]);
+    if (c != 0 && cut_to_tokens(g, &g->cls[c], c, c == pattern, n[0], n[1], n[2])) cut = true;
   };
   make(pattern);
   const EdgeClass& m = g->cls[pattern];
@@ -304,10 +297,20 @@ void set_edges(HostGeom* g) {
   g->main_last = m.together > 1 ? kSlabTokens : key_width(last_rows(m));
   for (int c = 0; c < 8; ++c)
     if (c != pattern && class_blocks(*g, c)) make(c);
+  if (!cut) return false;
+  g->planned = 1;
   for (int c = 0; c < 8; ++c) {
     if (!class_blocks(*g, c)) continue;
     EdgeClass& e = g->cls[c];
+    for (int s = 0; s < e.n_slabs; ++s) {
+      const int have = s + 1 < e.n_slabs ? e.step : last_rows(e);
+      for (int r = 0; r < have * e.together; ++r) {
+        const int x = s * e.step + r % have, y = x % e.frame;
+        if (x / e.frame < tokens[c][0] && (y >> e.lw) < tokens[c][1] && (y & ((1 << e.lw) - 1)) < tokens[c][2]) e.valid[s][r / 32] |= 1u << (r % 32);
+      }
+    }
     e.in_pattern = e.together == 1 && e.n_slabs == g->main_slabs && last_rows(e) <= g->main_last;
+    g->planned &= e.in_pattern;
     const int to = e.in_pattern ? g->main_last : kSlabTokens;
     fill_slab(g, &e, (c & 2) || g->Hp == 1, e.together * last_rows(e), to);   // (see cut_to_tokens)
     for (int r = to; r < kSlabTokens; ++r) e.valid[e.n_slabs - 1][r / 32] |= 1u << (r % 32);   // (a short slab has no such keys)
@@ -317,6 +320,34 @@ void set_edges(HostGeom* g) {
   for (int in = 1; in >= 0; --in)
     for (int c = 0; c < 8; ++c)
       if (class_blocks(*g, c) && g->cls[c].in_pattern == in) g->order[g->n_classes++] = (uint8_t)c;
+  return true;
+}
+
+// Classes of a padded grid, which has no boxes: blocks with fewer slabs than the others, the last ones along the axis on which slabs
+// stack, are the only ones told apart.  Where there are none the grid has one class and its items are what the planning kernel
+// counted.  (With a class for every combination of ragged axes, as in a cut grid, 3 heads of 6x15x23 with 2x8x8 blocks took 26.3 us
+// and take 21.0, 2 of 13x13x14 34.2 and 26.3: their tables, two dozen constants, and the tests in the loop over the key blocks.)
+void pad_edges(HostGeom* g, int edge_slabs) {
+  const int blocks = g->sub_axis == 0 ? g->Tp : (g->sub_axis == 1 ? g->Hp : g->Wp);
+  const bool two = edge_slabs < g->n_sub && blocks > 1;
+  g->edge_axes = two ? 1 << g->sub_axis : 0;
+  g->n_shapes = 0;
+  g->main_slabs = two ? g->n_sub : edge_slabs;
+  g->main_last = g->main_slabs == g->n_sub ? g->n_last : kSlabTokens;
+  g->slabs_of[0] = (uint8_t)g->main_slabs;
+  if (two) g->slabs_of[g->edge_axes] = (uint8_t)edge_slabs;
+}
+
+// The kind of the grid, its edge blocks and their classes.  T, H, W, the block and its slabs are set.
+void set_edges(HostGeom* g) {
+  const int rt = g->T - (g->Tp - 1) * g->bt, rh = g->H - (g->Hp - 1) * g->bh, rw = g->W - (g->Wp - 1) * g->bw;   // of the last block
+  const int axes = (rt < g->bt ? 1 : 0) | (rh < g->bh ? 2 : 0) | (rw < g->bw ? 4 : 0);
+  const int along = g->sub_axis == 0 ? rt : (g->sub_axis == 1 ? rh : rw), slab = g->sub_axis == 0 ? g->ct : (g->sub_axis == 1 ? g->ch : g->cw);
+  const int edge_slabs = (along + slab - 1) / slab;   // of the last block along the axis on which slabs stack, with any token
+  g->empty_slabs = edge_slabs < g->n_sub;
+  g->s_edge = g->Sp - g->Wp;
+  g->grid = axes == 0 ? kWhole : (cut_edges(g, axes, rt, rh, rw) ? kCut : kPadded);
+  if (g->grid != kCut) pad_edges(g, edge_slabs);   // (a whole grid has one class of blocks)
 }
 
 // Geometry of the block grid; `for_attn` additionally derives the 128-token slab.
@@ -381,7 +412,7 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, HostG
   }
   g->items_per_head = g->NB * g->items_per_block;
   // (only blocks of three slabs have a second item)
-  if (for_attn && g->n_sub == 3 && g->edge_axes)
+  if (for_attn && g->n_sub == 3)
     for (int c = 0; c < 8; ++c)
       if (g->slabs_of[c] < 3) g->items_per_head -= class_blocks(*g, c);
   g->Lt = L;
@@ -492,7 +523,7 @@ struct Layout {
 };
 
 // The four tensors with every box shape (TensorMaps).
-int encode_maps(TensorMapsEdge* tm, const void* q, const void* k, const void* v, void* out, const HostGeom& g,
+int encode_maps(TensorMapsCut* tm, const void* q, const void* k, const void* v, void* out, const HostGeom& g,
                 const Layout& lay, int n_heads_here) {
   int rc;
   const int n_in = lay.shared_qkv ? 1 : n_heads_here;
@@ -541,10 +572,9 @@ void plan_params(PlanParams* pp, const psa_head_params* params, const long long*
 
 // Key slabs of the average block.
 double slabs_per_block(const HostGeom& g) {
-  if (g.edge_axes == 0) return g.n_sub;
   double n = 0;
   for (int c = 0; c < 8; ++c)
-    if (class_blocks(g, c)) n += (double)class_blocks(g, c) * g.cls[c].n_slabs / g.cls[c].together;
+    if (class_blocks(g, c)) n += (double)class_blocks(g, c) * g.slabs_of[c] / (g.grid == kCut ? g.cls[c].together : 1);
   return n / g.NB;
 }
 
@@ -569,7 +599,7 @@ int share_items(const Workspace& ws, const HostGeom& g, const long long* weights
   }
   // blocks attended by the average query block, of all heads and of the heaviest
   const double avg = (double)total / ((double)n_heads * g.NB), heavy = (double)most / g.NB;
-  const int of_block = g.edge_axes ? g.main_slabs : g.n_sub, singles = of_block & 1, doubles = of_block >> 1;
+  const int of_block = g.main_slabs, singles = of_block & 1, doubles = of_block >> 1;
   const double per_slab = (3300.0 * doubles + 1900.0 * singles) / (doubles + singles), slabs = slabs_per_block(g);
   const double text = n_text ? (g.NB * slabs + g.n_ts) * (g.n_ts > 1 ? 3300.0 : 1900.0) : 0.0;
   const double heavy_item = (heavy * slabs + g.n_ts) * per_slab, longest = heavy_item > text ? heavy_item : text;
@@ -611,7 +641,7 @@ bool short_items(const HostGeom& g, const long long* weights, int n_heads) {
 }
 
 // Planning (unless the launch is direct) and attention.
-cudaError_t launch_call(const TensorMapsEdge& tm, const AttnParams& prm, const HostGeom& hg, const psa_head_params* params, const long long* weights,
+cudaError_t launch_call(const TensorMapsCut& tm, const AttnParams& prm, const HostGeom& hg, const psa_head_params* params, const long long* weights,
                         const Workspace& ws, int cluster, bool record, cudaStream_t st) {
   HeadParamsArray heads;   // entries beyond the launch's heads are never read, nor any of a planned launch
   const int n = prm.g.n_heads;
@@ -627,18 +657,15 @@ cudaError_t launch_call(const TensorMapsEdge& tm, const AttnParams& prm, const H
     ++g_launches;
   }
   if (record && g_ev_start && g_ev_stop) cudaEventRecord(g_ev_start, st);
-  AttnParamsEdge pe;
-  pe.cut = 0;
+  AttnParamsCut pe;
   static_cast<AttnParams&>(pe) = prm;
-  if (hg.edge_axes) {
+  if (hg.grid == kCut) {
     std::memcpy(pe.cls, hg.cls, sizeof(pe.cls));
-    pe.main_slabs = hg.main_slabs;
-    pe.main_last = hg.main_last;
-    pe.cut = hg.cut;
+    pe.planned = hg.planned;
     pe.n_classes = hg.n_classes;
     std::memcpy(pe.order, hg.order, sizeof(pe.order));
   }
-  const cudaError_t e = launch_attn(tm, heads, pe, ws.n_sms, cluster, direct, short_items(hg, weights, n), hg.empty_slabs, st,
+  const cudaError_t e = launch_attn(tm, heads, pe, ws.n_sms, cluster, hg.grid, direct, short_items(hg, weights, n), hg.empty_slabs, st,
                                     &g_last_attn.mode);
   if (e == cudaSuccess) {
     ++g_launches;
@@ -832,7 +859,7 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
     const int n_here = n_heads - head0 < kMaxHeads ? n_heads - head0 : kMaxHeads;
     const long long in_off = lay.shared_qkv ? 0 : (long long)head0 * lay.in_head;
     const long long out_off = (long long)head0 * lay.out_head;
-    TensorMapsEdge tm;
+    TensorMapsCut tm;
     if ((rc = encode_maps(&tm, static_cast<const uint16_t*>(q) + in_off, static_cast<const uint16_t*>(k) + in_off,
                           static_cast<const uint16_t*>(v) + in_off, static_cast<uint16_t*>(out) + out_off, g, lay, n_here)) != PSA_OK)
       return rc;
@@ -1037,7 +1064,7 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(base) + kNoAllocItemsOff);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  TensorMapsEdge tm;
+  TensorMapsCut tm;
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
   if ((rc = encode_maps(&tm, q, k, v, out, g, lay, prob->n_heads)) != PSA_OK) return rc;
   // What the kernels read of the scratch is written by this call's planning kernel; nothing of the previous call is read.

@@ -262,6 +262,27 @@ bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, i
   return true;
 }
 
+// EdgeClass::valid of a class whose blocks hold nt x nh x nw tokens, by lines (a slab holds whole ones); `to`: keys of the last slab,
+// beyond which there are none to mask.
+void set_valid(EdgeClass* e, int nt, int nh, int nw, int to) {
+  using u128 = unsigned __int128;
+  auto low = [](int n) -> u128 { return n >= 128 ? ~(u128)0 : ((u128)1 << n) - 1; };
+  const u128 line = low(nw);
+  const int w = 1 << e->lw, lines = e->frame >> e->lw;   // of a frame
+  int t = 0, h = 0;
+  for (int s = 0; s < e->n_slabs; ++s) {
+    const bool last = s + 1 == e->n_slabs;
+    const int have = last ? last_rows(*e) : e->step;
+    u128 one = 0, all = last ? ~low(to) : 0;
+    for (int r = 0; r < have; r += w) {
+      if (t < nt && h < nh) one |= line << r;
+      if (++h == lines) { h = 0; ++t; }
+    }
+    for (int b = 0; b < e->together; ++b) all |= one << b * have;
+    for (int i = 0; i < 4; ++i) e->valid[s][i] = (uint32_t)(all >> 32 * i);
+  }
+}
+
 // Edge blocks of a cut grid (EdgeClass); false, if no class is cut.  `axes`: those on which the grid has edge blocks, whose extents are
 // rt, rh and rw.
 //
@@ -281,15 +302,11 @@ bool cut_edges(HostGeom* g, int axes, int rt, int rh, int rw) {
   int pattern = 0;   // its class
   for (int c = 0; c < 8; ++c)
     if (class_blocks(*g, 0) == 0 && class_blocks(*g, c) > class_blocks(*g, pattern)) pattern = c;
-  int tokens[8][3];   // of a block of every class, along the axes
   bool cut = false;
   auto make = [&](int c) {
-    int* n = tokens[c];
-    n[0] = c & 1 ? rt : g->bt;
-    n[1] = c & 2 ? rh : g->bh;
-    n[2] = c & 4 ? rw : g->bw;
-    whole_slabs(*g, &g->cls[c], n[0], n[1], n[2]);
-    if (c != 0 && cut_to_tokens(g, &g->cls[c], c, c == pattern, n[0], n[1], n[2])) cut = true;
+    const int nt = c & 1 ? rt : g->bt, nh = c & 2 ? rh : g->bh, nw = c & 4 ? rw : g->bw;   // tokens along the axes
+    whole_slabs(*g, &g->cls[c], nt, nh, nw);
+    if (c != 0 && cut_to_tokens(g, &g->cls[c], c, c == pattern, nt, nh, nw)) cut = true;
   };
   make(pattern);
   const EdgeClass& m = g->cls[pattern];
@@ -302,18 +319,11 @@ bool cut_edges(HostGeom* g, int axes, int rt, int rh, int rw) {
   for (int c = 0; c < 8; ++c) {
     if (!class_blocks(*g, c)) continue;
     EdgeClass& e = g->cls[c];
-    for (int s = 0; s < e.n_slabs; ++s) {
-      const int have = s + 1 < e.n_slabs ? e.step : last_rows(e);
-      for (int r = 0; r < have * e.together; ++r) {
-        const int x = s * e.step + r % have, y = x % e.frame;
-        if (x / e.frame < tokens[c][0] && (y >> e.lw) < tokens[c][1] && (y & ((1 << e.lw) - 1)) < tokens[c][2]) e.valid[s][r / 32] |= 1u << (r % 32);
-      }
-    }
     e.in_pattern = e.together == 1 && e.n_slabs == g->main_slabs && last_rows(e) <= g->main_last;
     g->planned &= e.in_pattern;
     const int to = e.in_pattern ? g->main_last : kSlabTokens;
     fill_slab(g, &e, (c & 2) || g->Hp == 1, e.together * last_rows(e), to);   // (see cut_to_tokens)
-    for (int r = to; r < kSlabTokens; ++r) e.valid[e.n_slabs - 1][r / 32] |= 1u << (r % 32);   // (a short slab has no such keys)
+    set_valid(&e, c & 1 ? rt : g->bt, c & 2 ? rh : g->bh, c & 4 ? rw : g->bw, to);
     e.first_box[e.n_slabs] = e.n_boxes;
     g->slabs_of[c] = e.n_slabs;
   }

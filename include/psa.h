@@ -239,6 +239,16 @@ typedef enum {
 } psa_launch_mode;
 int psa_last_attn_launch(int32_t* mode, int32_t* ctas_per_item);
 
+/* How the same launch treated blocks that reach beyond the token grid: a psa_grid_kind is returned.  *slabs, *last_keys (both
+ * optional): its pattern of key slabs, those of a block and the keys of a block's last one (64, 96, 112 or 128; the others
+ * have 128).  For measurements and tests, too. */
+typedef enum {
+  PSA_GRID_WHOLE = 0,    /* there are none: the block divides the grid                      */
+  PSA_GRID_PADDED = 1,   /* computed like the others, with masks, less slabs without token  */
+  PSA_GRID_CUT = 2       /* some are cut to their tokens                                    */
+} psa_grid_kind;
+int psa_last_attn_grid(int32_t* slabs, int32_t* last_keys);
+
 /* Frees the per-device workspaces.  Safe to call more than once. */
 int psa_shutdown(void);
 

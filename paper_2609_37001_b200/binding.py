@@ -80,6 +80,8 @@ def lib() -> ctypes.CDLL:
         L.psa_last_device_status.argtypes = [ctypes.POINTER(ctypes.c_int32)]
         L.psa_last_attn_launch.argtypes = [ctypes.POINTER(ctypes.c_int32)] * 2
         L.psa_last_attn_launch.restype = ctypes.c_int
+        L.psa_last_attn_grid.argtypes = [ctypes.POINTER(ctypes.c_int32)] * 2
+        L.psa_last_attn_grid.restype = ctypes.c_int
         L.psa_shutdown.argtypes = []
         L.psa_selftest_wait_timeout.argtypes = [i32, vp]
         L.psa_selftest_wait_timeout.restype = ctypes.c_int
@@ -400,6 +402,16 @@ def psa_last_attn_launch() -> Tuple[int, str, int]:
     mode, ctas = ctypes.c_int32(0), ctypes.c_int32(0)
     items = lib().psa_last_attn_launch(ctypes.byref(mode), ctypes.byref(ctas))
     return items, LAUNCH_MODES[mode.value], ctas.value
+
+
+GRID_KINDS = ("whole", "padded", "cut")
+
+
+def psa_last_attn_grid() -> Tuple[str, int, int]:
+    """(kind of grid, key slabs per block, keys of a block's last slab) of the last attention kernel launched, see psa.h."""
+    slabs, keys = ctypes.c_int32(0), ctypes.c_int32(0)
+    kind = lib().psa_last_attn_grid(ctypes.byref(slabs), ctypes.byref(keys))
+    return GRID_KINDS[kind], slabs.value, keys.value
 
 
 def psa_last_device_status() -> Tuple[int, int]:

@@ -19,6 +19,7 @@ constexpr size_t kMaxSmemBytes = 232448;   // 227 KB of shared memory that a CTA
 //   kWhole    the block divides the grid: there are none
 //   kPadded   they are loaded like the others, with masks, less the slabs that hold no token
 //   kCut      some are cut to their tokens
+// (the values are those of psa_grid_kind)
 enum Grid { kWhole, kPadded, kCut };
 // They are edge blocks, the last ones along an axis.  A class has a bit for each axis on which they are the last (1: t, 2: h, 4: w);
 // class 0 is an ordinary block.  A padded grid tells only blocks of fewer slabs apart, the last ones along the axis on which slabs stack.

@@ -52,6 +52,8 @@ Workspace g_ws[kMaxDevices];
 struct {
   Mode mode = kTicket;
   int items = 0, cluster = 1;
+  Grid grid = kWhole;
+  int slabs = 0, last_keys = 0;
 } g_last_attn;
 
 // Id of a new API call on `stream` (g_mu held).  Never 0, which is what untouched status words hold.  A call that is
@@ -231,9 +233,7 @@ bool cut_to_tokens(HostGeom* g, EdgeClass* e, int c, bool for_pattern, int nt, i
   x.step = (uint16_t)step;
   x.together = (uint8_t)(rows <= kSlabTokens / 2 ? kSlabTokens / rows : 1);
   bool ok = slabs(step) < e->n_slabs || x.together > 1 ||
-            // (narrower slabs alone do not pay for the maps of a small grid: 16 heads of 11 3x32x4 blocks 55.9 us padded and 62.1 cut,
-            // 13 of 60 1x30x8 blocks 495 and 460)
-            (g->NB >= 32 && slabs(step) == e->n_slabs && key_width(last_of(step)) < key_width(last_rows(*e)) &&
+            (slabs(step) == e->n_slabs && key_width(last_of(step)) < key_width(last_rows(*e)) &&
              (for_pattern || (e->n_slabs == g->main_slabs && last_rows(*e) > g->main_last && last_of(step) <= g->main_last)));
   for (int r = 0; ok && r < rows; r += step) {
     int end = 0;
@@ -283,15 +283,25 @@ void set_valid(EdgeClass* e, int nt, int nh, int nw, int to) {
   }
 }
 
-// Edge blocks of a cut grid (EdgeClass); false, if no class is cut.  `axes`: those on which the grid has edge blocks, whose extents are
-// rt, rh and rw.
+// Work items of a head.
+void count_items(HostGeom* g) {
+  g->items_per_block = (g->n_sub + 1) / 2;
+  g->items_per_head = g->NB * g->items_per_block + g->n_titems;
+  if (g->n_sub == 3)   // (only blocks of three slabs have a second item)
+    for (int c = 0; c < 8; ++c)
+      if (g->slabs_of[c] < 3) g->items_per_head -= class_blocks(*g, c);
+}
+
+// Makes a padded grid a cut one (EdgeClass); false, if no class is cut, and then *g is of no use.
 //
 // Why: 3D-padding is issued work, along the keys and along the queries.  The last of the seven 30x8 blocks across 52 columns
 // holds 120 of its 240 tokens (12 heads of 21x30x52: 2.60 -> 2.39 ms), the last 3x8x16 block down 45 rows 240 of 384 (40 heads of
 // 21x45x80: 28.7 -> 26.3 ms).  Cut like this an edge block is mostly one box a slab, as an ordinary one: the load warp, which has
 // some 10 clocks for an instruction next to the softmax, fell behind with rows packed tightly across blocks, by boxes of 8 to
 // 128 rows (5,000 clocks a slab) as well as by 16-byte copies (8,000).
-bool cut_edges(HostGeom* g, int axes, int rt, int rh, int rw) {
+bool cut_edges(HostGeom* g) {
+  const int rt = g->T - (g->Tp - 1) * g->bt, rh = g->H - (g->Hp - 1) * g->bh, rw = g->W - (g->Wp - 1) * g->bw;   // of the last block
+  const int axes = (rt < g->bt ? 1 : 0) | (rh < g->bh ? 2 : 0) | (rw < g->bw ? 4 : 0);
   if (g->sub_axis == 2 || g->bh * g->bw < 8) return false;
   if ((axes & 6) == 6 && g->Sp > kMaxSp / 2) return false;   // (the kernel keeps four sets of spatial coordinates of such a grid)
   // Blocks of one slab run in split-KV mode, where a slab takes 1,900 clocks and the load warp has no time for lists of boxes: 7
@@ -330,6 +340,8 @@ bool cut_edges(HostGeom* g, int axes, int rt, int rh, int rw) {
   for (int in = 1; in >= 0; --in)
     for (int c = 0; c < 8; ++c)
       if (class_blocks(*g, c) && g->cls[c].in_pattern == in) g->order[g->n_classes++] = (uint8_t)c;
+  g->grid = kCut;
+  count_items(g);
   return true;
 }
 
@@ -348,16 +360,15 @@ void pad_edges(HostGeom* g, int edge_slabs) {
   if (two) g->slabs_of[g->edge_axes] = (uint8_t)edge_slabs;
 }
 
-// The kind of the grid, its edge blocks and their classes.  T, H, W, the block and its slabs are set.
+// Whether the grid is whole or padded, and its edge blocks.  T, H, W, the block and its slabs are set.
 void set_edges(HostGeom* g) {
   const int rt = g->T - (g->Tp - 1) * g->bt, rh = g->H - (g->Hp - 1) * g->bh, rw = g->W - (g->Wp - 1) * g->bw;   // of the last block
-  const int axes = (rt < g->bt ? 1 : 0) | (rh < g->bh ? 2 : 0) | (rw < g->bw ? 4 : 0);
   const int along = g->sub_axis == 0 ? rt : (g->sub_axis == 1 ? rh : rw), slab = g->sub_axis == 0 ? g->ct : (g->sub_axis == 1 ? g->ch : g->cw);
   const int edge_slabs = (along + slab - 1) / slab;   // of the last block along the axis on which slabs stack, with any token
   g->empty_slabs = edge_slabs < g->n_sub;
   g->s_edge = g->Sp - g->Wp;
-  g->grid = axes == 0 ? kWhole : (cut_edges(g, axes, rt, rh, rw) ? kCut : kPadded);
-  if (g->grid != kCut) pad_edges(g, edge_slabs);   // (a whole grid has one class of blocks)
+  g->grid = rt == g->bt && rh == g->bh && rw == g->bw ? kWhole : kPadded;
+  pad_edges(g, edge_slabs);   // (a whole grid has one class of blocks)
 }
 
 // Geometry of the block grid; `for_attn` additionally derives the 128-token slab.
@@ -417,14 +428,9 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, HostG
     if (g->Tp > kMaxTp || g->Sp > kMaxSp || plan_smem_bytes(*g) > kMaxSmemBytes) return PSA_ERR_UNSUPPORTED;
     g->n_sub = n_sub;
     set_edges(g);
-    g->items_per_block = (n_sub + 1) / 2;
     g->scale_log2 = prob->scale * 1.4426950408889634f;
   }
-  g->items_per_head = g->NB * g->items_per_block;
-  // (only blocks of three slabs have a second item)
-  if (for_attn && g->n_sub == 3)
-    for (int c = 0; c < 8; ++c)
-      if (g->slabs_of[c] < 3) g->items_per_head -= class_blocks(*g, c);
+  count_items(g);
   g->Lt = L;
   return PSA_OK;
 }
@@ -588,6 +594,24 @@ double slabs_per_block(const HostGeom& g) {
   return n / g.NB;
 }
 
+// What share_items needs to know of a cut grid, in clocks.  A slab takes the load warp 1,200 for each of its boxes (of K and of V),
+// which is more than it takes the others where it has more than one or two; an item, 1,750 for each class of blocks, and a quarter of a
+// slab for blocks that share one, as there are not always enough of them.  (Least squares over 230 drawn problems of 8 to 6,000
+// items, cut and padded.)
+void cut_clocks(const HostGeom& g, double per_slab, double* block, double* rest, double* setup) {
+  *block = *rest = 0;
+  *setup = 1750.0 * g.n_classes;
+  auto width = [](int keys) -> double { return 0.5 + 0.5 * keys / kSlabTokens; };   // a narrower slab's time
+  for (int i = 0; i < g.n_classes; ++i) {
+    const EdgeClass& e = g.cls[g.order[i]];
+    const double boxes = e.together > 1 ? e.together + e.n_boxes - 1 : (double)e.n_boxes / e.n_slabs;
+    auto slab = [&](double clocks) -> double { return 1200.0 * boxes > clocks ? 1200.0 * boxes : clocks; };
+    const double last = e.in_pattern ? per_slab * width(g.main_last) / width(g.main_slabs == g.n_sub ? g.n_last : kSlabTokens) : per_slab;
+    *block += (slab(per_slab) * (e.n_slabs - 1) + slab(last)) * class_blocks(g, g.order[i]) / e.together / g.NB;
+    if (e.together > 1) *rest += 0.25 * slab(per_slab);
+  }
+}
+
 // CTAs that share a work item: 1 (persistent CTAs that draw whole items), 2, 4 or 8.  A launch takes about as many
 // rounds as its items need on the SMs, and at least as long as its longest item, so a problem of few items, of a few more
 // than a whole number of rounds, or of a few very long ones (text queries attend every key) leaves SMs idle; sharing
@@ -595,13 +619,14 @@ double slabs_per_block(const HostGeom& g) {
 // 1,900 for one (split-KV mode); start-up, epilogue and exit take 15,000 in a persistent CTA and 20,000 in a cluster
 // (which also merges).  Over 56 drawn problems of 12 to 700 items the choice was within 9 % of the best of the four,
 // except one at 18 % (12 items); without text, whole items were best in all 24 problems of more than two rounds.
-// Decided for a call as a whole, so that the chunks of a host-tensor call compute what the device call computes, bit
-// for bit.  weights: attended block pairs of every head.
-int share_items(const Workspace& ws, const HostGeom& g, const long long* weights, int n_heads) {
+// weights: attended block pairs of every head.
+struct Sharing {
+  int cluster;
+  double clocks;   // the launch's estimated time with them
+};
+Sharing share_items(const Workspace& ws, const HostGeom& g, const long long* weights, int n_heads) {
   const int heads = n_heads < kMaxHeads ? n_heads : kMaxHeads;   // of one launch
   const int n_items = heads * g.items_per_head, n_text = heads * g.n_titems;
-  // beyond two rounds at most a third is to be gained, unless text queries make long items
-  if (n_items > (n_text ? 8 : 2) * ws.n_sms) return 1;
   long long total = 0, most = 0;
   for (int h = 0; h < n_heads; ++h) {
     total += weights[h];
@@ -612,24 +637,49 @@ int share_items(const Workspace& ws, const HostGeom& g, const long long* weights
   const int of_block = g.main_slabs, singles = of_block & 1, doubles = of_block >> 1;
   const double per_slab = (3300.0 * doubles + 1900.0 * singles) / (doubles + singles), slabs = slabs_per_block(g);
   const double text = n_text ? (g.NB * slabs + g.n_ts) * (g.n_ts > 1 ? 3300.0 : 1900.0) : 0.0;
-  const double heavy_item = (heavy * slabs + g.n_ts) * per_slab, longest = heavy_item > text ? heavy_item : text;
-  const double work = (double)(n_items - n_text) * (avg * slabs + g.n_ts) * per_slab + n_text * text;
-  auto time = [&](int at_a_time, int c, double fixed) -> double {
-    const double one = longest / c + fixed;
+  // (a block: clocks of an attended one; rest: clocks of an item besides)
+  auto time = [&](int at_a_time, int c, double fixed, double block, double rest) -> double {
+    const double item = avg * block + rest + g.n_ts * per_slab, heavy_item = heavy * block + rest + g.n_ts * per_slab;
+    const double one = (heavy_item > text ? heavy_item : text) / c + fixed;
     if (n_items <= at_a_time) return one;
-    const double all = (double)((n_items + at_a_time - 1) / at_a_time) * (work / n_items / c + fixed);
+    const double all = (double)((n_items + at_a_time - 1) / at_a_time) * (((n_items - n_text) * item + n_text * text) / n_items / c + fixed);
     return all > one ? all : one;
   };
-  double best = time(ws.n_sms, 1, 15000.0);
-  int cluster = 1;
-  for (int i = 0; i < 3; ++i) {
+  const double block = slabs * per_slab, heavy_item = heavy * block + g.n_ts * per_slab, longest = heavy_item > text ? heavy_item : text;
+  int cluster = 1, at_a_time = ws.n_sms;
+  double best = time(at_a_time, 1, 15000.0, block, 0);
+  // beyond two rounds at most a third is to be gained, unless text queries make long items
+  for (int i = 0; i < 3 && n_items <= (n_text ? 8 : 2) * ws.n_sms; ++i) {
     const int c = 2 << i;
-    if (ws.clusters[i] < 1 || longest < c * per_slab * slabs) break;   // a share of a long item holds at least one block
-    const double t = time(ws.clusters[i], c, 20000.0);
+    if (ws.clusters[i] < 1 || longest < c * block) break;   // a share of a long item holds at least one block
+    const double t = time(ws.clusters[i], c, 20000.0, block, 0);
     // (rounds of whole items overlap more than the estimate knows: the longer ones go first)
-    if (t < (n_items <= ws.clusters[i] ? 0.97 : 0.88) * best) { best = t; cluster = c; }
+    if (t < (n_items <= ws.clusters[i] ? 0.97 : 0.88) * best) { best = t; cluster = c; at_a_time = ws.clusters[i]; }
   }
-  return cluster;
+  if (g.grid == kCut) {
+    double cut_block, rest, setup;
+    cut_clocks(g, per_slab, &cut_block, &rest, &setup);
+    best = time(at_a_time, cluster, (cluster > 1 ? 20000.0 : 15000.0) + setup, cut_block, rest);
+  }
+  return Sharing{cluster, cluster > 1 && n_items > at_a_time ? best / 0.88 : best};   // (as above)
+}
+
+// Cuts a padded grid if the launch is estimated to take less time then; the CTAs that share an item.  Decided for a call as a whole,
+// so that the chunks of a host-tensor call compute what the device call computes, bit for bit.
+//
+// What a cut grid saves is in proportion to the launch's slabs, what it costs is not: over 230 drawn problems of 8 to 6,000 items
+// that can be cut it was from 0.47 to 3.0 times as fast as padded.  By this rule 168 of them are cut, 15 of these lose more than 2 %
+// by it (0.79 times as fast the worst, 51 us) and 8 of the others would have gained more (15 % at most).  Below an estimate of 30,000
+// clocks (about 20 us) none gains, and the call would wait for the host's tables.
+int choose_edges(const Workspace& ws, HostGeom* g, const long long* weights, int n_heads) {
+  const Sharing padded = share_items(ws, *g, weights, n_heads);
+  if (g->grid != kPadded || padded.clocks < 30000.0) return padded.cluster;
+  HostGeom cut = *g;
+  if (!cut_edges(&cut)) return padded.cluster;
+  const Sharing s = share_items(ws, cut, weights, n_heads);
+  if (s.clocks >= padded.clocks) return padded.cluster;
+  *g = cut;
+  return s.cluster;
 }
 
 // Whether every item of a launch runs at the same time.  Then their order does not matter and no planning is needed:
@@ -681,6 +731,9 @@ cudaError_t launch_call(const TensorMapsCut& tm, const AttnParams& prm, const Ho
     ++g_launches;
     g_last_attn.items = prm.n_items;
     g_last_attn.cluster = cluster;
+    g_last_attn.grid = hg.grid;
+    g_last_attn.slabs = hg.main_slabs;
+    g_last_attn.last_keys = hg.main_last;
   }
   return e;
 }
@@ -760,6 +813,13 @@ int psa_last_attn_launch(int32_t* mode, int32_t* ctas_per_item) {
   if (mode) *mode = g_last_attn.mode;
   if (ctas_per_item) *ctas_per_item = g_last_attn.cluster;
   return g_last_attn.items;
+}
+
+int psa_last_attn_grid(int32_t* slabs, int32_t* last_keys) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (slabs) *slabs = g_last_attn.slabs;
+  if (last_keys) *last_keys = g_last_attn.last_keys;
+  return g_last_attn.grid;
 }
 
 int psa_profile_events(void* start_event, void* stop_event) {
@@ -844,9 +904,9 @@ int psa_mask_build(const psa_head_params* params, const psa_problem* prob, int T
 // per-device workspace.  Arguments are already validated; g_mu is held by the caller.
 // new_call: this is the first launch sequence of an API call (later ones report under the same id, so that an error of
 // an earlier one -- more than 128 heads, chunks of a host-tensor call, samples of a batched call -- is not lost).
-// cluster: CTAs per work item, 0: by share_items for these heads.
+// cluster: CTAs per work item, and the grid as it is; 0: both by choose_edges for these heads; -1: one CTA, the grid by choose_edges.
 static int run_attn(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
-                    int n_heads, const HostGeom& g, const Layout& lay, cudaStream_t st, bool new_call = true, int cluster = 0) {
+                    int n_heads, HostGeom g, const Layout& lay, cudaStream_t st, bool new_call = true, int cluster = 0) {
   int dev;
   Workspace* ws;
   int rc = device_info(&dev, &ws);
@@ -864,7 +924,10 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(ws->base) + items_off);
   std::vector<long long> weights((size_t)n_heads);
   head_weights(head_params, n_heads, g, weights.data());
-  if (cluster == 0) cluster = share_items(*ws, g, weights.data(), n_heads);
+  if (cluster <= 0) {
+    const int chosen = choose_edges(*ws, &g, weights.data(), n_heads);
+    cluster = cluster < 0 ? 1 : chosen;
+  }
   if (new_call) ws->last_call = next_call_id(st);
   for (int head0 = 0; head0 < n_heads; head0 += kMaxHeads) {
     const int n_here = n_heads - head0 < kMaxHeads ? n_heads - head0 : kMaxHeads;
@@ -885,10 +948,10 @@ static int run_attn(const void* q, const void* k, const void* v, void* out, floa
   return PSA_OK;
 }
 
-// psa_attn_fwd with the choice of continuing an API call and of the CTAs per item (chunks of one host-tensor call).
+// psa_attn_fwd with the choice of continuing an API call, of the CTAs per item and of the grid's edges (chunks of one host-tensor call).
 static int attn_fwd_checked(const void* q, const void* k, const void* v, void* out, float* lse,
                             const psa_head_params* head_params, const psa_problem* prob, int T, int H, int W, void* stream,
-                            bool new_call, int cluster = 0) {
+                            bool new_call, int cluster = 0, const HostGeom* chosen = nullptr) {
   HostGeom g;
   int rc = make_geom(prob, T, H, W, true, &g);
   if (rc != PSA_OK) return rc;
@@ -902,7 +965,8 @@ static int attn_fwd_checked(const void* q, const void* k, const void* v, void* o
     if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lock(g_mu);
   const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
-  return run_attn(q, k, v, out, lse, head_params, prob->n_heads, g, lay, static_cast<cudaStream_t>(stream), new_call, cluster);
+  return run_attn(q, k, v, out, lse, head_params, prob->n_heads, chosen ? *chosen : g, lay, static_cast<cudaStream_t>(stream), new_call,
+                  cluster);
 }
 
 int psa_attn_fwd(const void* q, const void* k, const void* v, void* out, float* lse, const psa_head_params* head_params,
@@ -1015,7 +1079,7 @@ int psa_search_losses(const void* q, const void* k, const void* v, const psa_hea
   const Layout lay = {0, prob->stride_token, g.L * kHeadDim, kHeadDim, true};
   // whole items: with n_cand + 1 of them per block they are rarely few, and every candidate's output is then rounded as
   // a plain call's is (the losses are differences of outputs)
-  rc = run_attn(q, k, v, outs, lse, params.data(), n_cand + 1, g, lay, st, true, 1);
+  rc = run_attn(q, k, v, outs, lse, params.data(), n_cand + 1, g, lay, st, true, -1);
   if (rc != PSA_OK) return rc;
   int launches = 0;
   const cudaError_t e = launch_search_losses(outs, outs + (long long)n_cand * g.L * kHeadDim, g.L * kHeadDim, n_cand, partial,
@@ -1057,7 +1121,6 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
     if (!valid_params(head_params[h])) return PSA_ERR_INVALID_ARG;
   // the fixed scratch bounds the problem: one launch worth of heads and kNoAllocMaxItems items
   // (edge blocks counted like the others, whatever items they save: the limit that the header states)
-  const long long n_items_ll = (long long)prob->n_heads * g.items_per_head;
   if (prob->n_heads > kMaxHeads || (long long)prob->n_heads * g.NB * g.items_per_block > kNoAllocMaxItems) return PSA_ERR_CAPACITY;
 
   std::lock_guard<std::mutex> lock(g_mu);
@@ -1075,13 +1138,14 @@ int psa_attn_fwd_noalloc(const void* q, const void* k, const void* v, void* out,
   WorkItem* items = reinterpret_cast<WorkItem*>(static_cast<char*>(base) + kNoAllocItemsOff);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  TensorMapsCut tm;
-  const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
-  if ((rc = encode_maps(&tm, q, k, v, out, g, lay, prob->n_heads)) != PSA_OK) return rc;
   // What the kernels read of the scratch is written by this call's planning kernel; nothing of the previous call is read.
   long long weights[kMaxHeads];
   head_weights(head_params, prob->n_heads, g, weights);
-  const int cluster = share_items(*ws, g, weights, prob->n_heads), n_items = (int)n_items_ll, call_id = next_call_id(st);
+  const int cluster = choose_edges(*ws, &g, weights, prob->n_heads);
+  TensorMapsCut tm;
+  const Layout lay = {prob->stride_head, prob->stride_token, prob->stride_head, prob->stride_token, false};
+  if ((rc = encode_maps(&tm, q, k, v, out, g, lay, prob->n_heads)) != PSA_OK) return rc;
+  const int n_items = prob->n_heads * g.items_per_head, call_id = next_call_id(st);
   const AttnParams prm = {g, items, hp_dev, header, lse, n_items, call_id, 0,
                           out, lay.out_head, lay.out_token};
   if (launch_call(tm, prm, g, head_params, weights, *ws, cluster, false, st) != cudaSuccess) return PSA_ERR_CUDA;
@@ -1158,7 +1222,7 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
     std::lock_guard<std::mutex> lock(g_mu);
     Workspace* ws;
     if ((rc = device_info(&dev, &ws)) != PSA_OK || (rc = init_attn(ws)) != PSA_OK) return rc;
-    cluster = share_items(*ws, g, weights.data(), prob->n_heads);
+    cluster = choose_edges(*ws, &g, weights.data(), prob->n_heads);
   }
   if (n_edge || (per == 1 && prob->n_heads >= 3)) {
     for (int h = 0; h < prob->n_heads; ++h) {
@@ -1213,7 +1277,7 @@ int psa_attn_fwd_host(const void* q, const void* k, const void* v, void* out, fl
     if (cudaStreamWaitEvent(st, pipe->ev_in[c], 0) != cudaSuccess) return PSA_ERR_CUDA;
     psa_problem sub = *prob;
     sub.n_heads = nh;
-    rc = attn_fwd_checked(dq, dk, dv, dout, d_lse + (size_t)h0 * L, head_params + h0, &sub, T, H, W, stream, c == 0, cluster);
+    rc = attn_fwd_checked(dq, dk, dv, dout, d_lse + (size_t)h0 * L, head_params + h0, &sub, T, H, W, stream, c == 0, cluster, &g);
     if (rc != PSA_OK) return rc;
     if (cudaEventRecord(pipe->ev_done[c], st) != cudaSuccess) return PSA_ERR_CUDA;
     if (c > 0 && !copy_out(c - 1)) return PSA_ERR_CUDA;

@@ -493,7 +493,7 @@ plan_kernel(const __grid_constant__ PlanParams hp, const Geom g, int* __restrict
     for (int it = 0; it < ipb; ++it) {
       const int sub0 = 2 * it;
       if (sub0 >= n_sub) break;
-      if (it == 1 && g.edge_axes != 0) {   // not all edge blocks have a second item: the rank among the blocks that have one
+      if (it == 1 && g.items_per_head - g.n_titems != 2 * g.NB) {   // some blocks have no second item: the rank among those that have one
         pos = j = 0;
         for (int tj = 0; tj < g.Tp; ++tj)
           for (int sj = 0, wj = 0; sj < g.Sp; ++sj, ++j) {

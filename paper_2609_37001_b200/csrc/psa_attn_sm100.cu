@@ -1798,7 +1798,7 @@ attn_fwd_kernel(const __grid_constant__ typename ArgsOf<kGrid>::maps tms, const 
       long long out_tok = -1;        // kShort: this row's token, and where its output goes
       uint4* out_row = nullptr;
       if constexpr (kShort) {
-        out_tok = row_token<kBoxes>(prm, textq, qb, sub0 + qi, row);
+        out_tok = row_token<false>(prm, textq, qb, sub0 + qi, row);
         if (out_tok >= 0)
           out_row = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(prm.out) + (long long)head * prm.out_head + out_tok * prm.out_token);
       }
@@ -1988,7 +1988,7 @@ struct LaunchConfig {
 cudaError_t attn_init(int clusters[3]) {
 #define PSA_ALL_GRIDS(mode) (const void*)attn_fwd_kernel<mode, kWhole>, (const void*)attn_fwd_kernel<mode, kPadded>, (const void*)attn_fwd_kernel<mode, kCut>
   const void* kernels[] = {PSA_ALL_GRIDS(kTicket), PSA_ALL_GRIDS(kDirect), PSA_ALL_GRIDS(kShared), PSA_ALL_GRIDS(kSharedDirect),
-                           PSA_ALL_GRIDS(kTicketShort)};
+                           (const void*)attn_fwd_kernel<kTicketShort, kWhole>, (const void*)attn_fwd_kernel<kTicketShort, kPadded>};
 #undef PSA_ALL_GRIDS
   cudaError_t e = cudaSuccess;
   for (const void* k : kernels)
@@ -2013,7 +2013,9 @@ cudaError_t launch_plan(const PlanParams& hp, const Geom& g, int n_heads_here, i
 
 template <int kMode>
 cudaError_t launch_mode(const LaunchConfig& lc, Grid grid, const TensorMapsCut& tm, const HeadParamsArray& heads, const AttnParamsCut& prm) {
-  if (grid == kCut) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kCut>, tm, heads, prm);
+  if constexpr (kMode != kTicketShort) {   // (blocks of one slab are not cut)
+    if (grid == kCut) return cudaLaunchKernelEx(&lc.cfg, attn_fwd_kernel<kMode, kCut>, tm, heads, prm);
+  }
   TensorMaps plain;
   for (int i = 0; i < 3; ++i) {
     plain.q[i] = tm.q[i];

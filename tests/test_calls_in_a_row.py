@@ -1,5 +1,5 @@
 """Calls enqueued one behind the other without a synchronisation, in every order of the ways a launch may hand out its work
-items and through both scratch areas: a call's kernels start while the ones before are still running, so each must wait for
+items, on whole, padded and cut grids, and through both scratch areas: a call's kernels start while the ones before are still running, so each must wait for
 what it reads and overwrites.  Every result bit for bit that of the call alone; the inputs of a group of calls are
 overwritten right in front of it, and again behind it."""
 import math
@@ -10,14 +10,25 @@ import torch
 
 pytestmark = pytest.mark.gpu
 SCALE = 1.0 / math.sqrt(128.0)
-KINDS = {   # mode: grid, tile, heads, text tokens
+KINDS = {   # mode (and grid): grid, tile, heads, text tokens
     "shared_direct": ((8, 16, 16), (2, 8, 8), 2, 0),
     "direct": ((7, 16, 32), (1, 8, 16), 4, 0),
     "ticket": ((4, 16, 32), (1, 16, 16), 40, 0),
     "ticket_short": ((4, 16, 32), (1, 8, 16), 24, 0),
     "ticket_edge": ((2, 23, 32), (1, 16, 16), 90, 0),
     "shared": ((20, 24, 32), (1, 16, 16), 1, 219),
+    "shared whole": ((20, 32, 32), (1, 16, 16), 1, 219),
+    "shared_direct padded": ((6, 15, 23), (2, 8, 8), 3, 0),
+    "direct padded": ((2, 24, 27), (2, 8, 8), 11, 0),
+    "ticket padded": ((5, 11, 60), (1, 15, 16), 17, 0),
+    "ticket_short padded": ((3, 15, 33), (1, 8, 16), 30, 0),
+    "shared_direct cut": ((5, 10, 45), (3, 32, 4), 2, 0),
+    "direct cut": ((11, 9, 16), (2, 32, 4), 6, 0),
+    "ticket cut": ((6, 16, 20), (3, 32, 4), 20, 0),
+    "ticket_edge cut": ((9, 11, 60), (2, 32, 4), 2, 0),
+    "shared cut": ((20, 12, 35), (1, 15, 16), 3, 50),
 }
+GRIDS = {"shared_direct": "whole", "direct": "whole", "ticket": "whole", "ticket_short": "whole", "ticket_edge": "padded", "shared": "padded"}
 
 
 class Problem:
@@ -34,7 +45,8 @@ class Problem:
             self.fill(v)
             torch.cuda.synchronize()
             got = self.call(*self.outputs())
-            assert B.psa_last_attn_launch()[1] == mode
+            assert B.psa_last_attn_launch()[1] == mode.split()[0]
+            assert B.psa_last_attn_grid()[0] == (GRIDS[mode] if mode in GRIDS else mode.split()[1])
             torch.cuda.synchronize()
             self.want.append([x.clone() for x in got])
 

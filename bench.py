@@ -73,35 +73,26 @@ def config_of(w, extra=None):
     return c
 
 
-def slab_split(tile):
-    """(axis that a mask block's slabs stack on, its extent per full slab, slabs per block, keys of the last slab), as the
-    attention kernel splits a block: 128-token slabs along its outermost axis of extent > 1, the last possibly shorter."""
-    bt, bh, bw = tile
-    axis = 0 if bt > 1 or (bh == 1 and bw == 1) else (1 if bh > 1 else 2)
-    other = bt * bh * bw // tile[axis]
-    c0 = 128 // other
-    n_sub = -(-tile[axis] // c0)
-    return axis, c0, n_sub, (tile[axis] - (n_sub - 1) * c0) * other
-
-
-def issued_flops(w):
-    """FLOPs the tensor cores are asked for: every attended block pair costs (128 rows per query
-    slab) x (keys of every key slab) x 4 x head_dim, padded and idle rows included.  Slabs without any token (of the last
-    block along the stacked axis) are left out.  An upper bound where the kernel cuts blocks at the grid's edge to their tokens."""
+def issued_flops(w, B):
+    """FLOPs the tensor cores are asked for by the last attention launch, one of this workload: every attended block pair costs
+    (128 rows per query slab) x (keys as computed) x 4 x head_dim, by the classes of blocks that the launch told apart; padded
+    and idle rows are included."""
     from oracle import psa_oracle as O
-    axis, c0, n_sub, n_last = slab_split(w["tile"])
+    axes, classes = B.psa_last_attn_classes()
     n = [-(-x // b) for x, b in zip(w["grid"], w["tile"])]
-    n_edge = min(-(-(w["grid"][axis] - (n[axis] - 1) * w["tile"][axis]) // c0), n_sub)
-    # query rows and keys of a block by its temporal and by its spatial coordinate (all ones on the axis that has no say)
-    at = np.indices(n)[axis].reshape(n[0], -1)
-    at = at[:, 0] if axis == 0 else at[0]
-    edge = (at == n[axis] - 1) & (n_edge < n_sub)
-    rows = np.where(edge, 128.0 * n_edge, 128.0 * n_sub)
-    keys = np.where(edge, 128.0 * n_edge, 128.0 * (n_sub - 1) + n_last)
+    t, h, x = np.indices(n).reshape(3, n[0], -1)
+    cls = ((t == n[0] - 1) * 1 | (h == n[1] - 1) * 2 | (x == n[2] - 1) * 4) & axes
+    query = np.array([c[0] * 128.0 for c in classes])[cls]
+    ct, cs = cls[:, 0] & 1, cls[0] & 6   # of temporal and of spatial coordinates
     total = 0.0
     for p in w["head_params"]:
         mt, ms = O.axis_mask(n[0], *p[:3]).astype(np.float64), O.axis_mask(n[1] * n[2], *p[3:]).astype(np.float64)
-        total += (rows @ mt @ keys) * ms.sum() if axis == 0 else mt.sum() * (rows @ ms @ keys)
+        keys = np.zeros(cls.shape)   # of every query block
+        for c, (_, per, together) in enumerate(classes):
+            if per:
+                blocks = np.outer(mt @ (ct == (c & 1)), ms @ (cs == (c & 6)))
+                keys += per * np.ceil(blocks / together)
+        total += float((query * keys).sum())
     return 4.0 * HEAD_DIM * total
 
 
@@ -307,6 +298,7 @@ def run_ours(args, w):
         if st != 0:
             raise SystemExit(f"device status {st} detail {hex(detail)}")
 
+        issued = issued_flops(w, B)
         ms_max = R.max_over_ranks(ms_step, dev)
 
         extra = {}
@@ -417,7 +409,6 @@ def run_ours(args, w):
             for ln in open(tp):
                 if ln.startswith("traffic_bytes_per_launch:"):
                     traffic = int(ln.split(":")[1])
-        issued = issued_flops(w)
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": max(args.warmup, 3), "ms_per_step": ms_max, "ms_median": float(np.median(step_ms)),
@@ -488,7 +479,7 @@ def time_other_configs(B, WL, torch, dev, peaks, skip):
                     "computed_tflops": flops / (mean * 1e-3) / 1e12,
                     "frac": flops / (mean * 1e-3) / 1e12 / peaks["bf16_tflops"],
                     "dense_equiv_tflops": dflops / (mean * 1e-3) / 1e12,
-                    "padding_ratio": issued_flops(w) / flops if flops else None})
+                    "padding_ratio": issued_flops(w, B) / flops if flops else None})
         del q, k, v, out, lse
         torch.cuda.empty_cache()
     return res

@@ -249,6 +249,11 @@ typedef enum {
 } psa_grid_kind;
 int psa_last_attn_grid(int32_t* slabs, int32_t* last_keys);
 
+/* What the same launch computed for a video block of class c, 0 to 7: bits for the last ones along t (1), h (2) and w (4), of
+ * those axes whose last blocks it told apart, which are returned (or PSA_ERR_INVALID_ARG).  As a query block *query_slabs of 128
+ * rows, as key blocks *keys for every *together of them that are attended (all optional; 0, 0 and 1 of a class without blocks). */
+int psa_last_attn_class(int c, int32_t* query_slabs, int32_t* keys, int32_t* together);
+
 /* Frees the per-device workspaces.  Safe to call more than once. */
 int psa_shutdown(void);
 

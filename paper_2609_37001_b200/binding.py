@@ -10,7 +10,7 @@ import ctypes
 import os
 import struct
 from itertools import chain
-from typing import Optional, Sequence, Tuple
+from typing import List, Optional, Sequence, Tuple
 
 import torch
 
@@ -82,6 +82,8 @@ def lib() -> ctypes.CDLL:
         L.psa_last_attn_launch.restype = ctypes.c_int
         L.psa_last_attn_grid.argtypes = [ctypes.POINTER(ctypes.c_int32)] * 2
         L.psa_last_attn_grid.restype = ctypes.c_int
+        L.psa_last_attn_class.argtypes = [i32] + [ctypes.POINTER(ctypes.c_int32)] * 3
+        L.psa_last_attn_class.restype = ctypes.c_int
         L.psa_shutdown.argtypes = []
         L.psa_selftest_wait_timeout.argtypes = [i32, vp]
         L.psa_selftest_wait_timeout.restype = ctypes.c_int
@@ -412,6 +414,17 @@ def psa_last_attn_grid() -> Tuple[str, int, int]:
     slabs, keys = ctypes.c_int32(0), ctypes.c_int32(0)
     kind = lib().psa_last_attn_grid(ctypes.byref(slabs), ctypes.byref(keys))
     return GRID_KINDS[kind], slabs.value, keys.value
+
+
+def psa_last_attn_classes() -> Tuple[int, List[Tuple[int, int, int]]]:
+    """(axes whose last blocks were told apart, per class (query slabs, keys, blocks that share these)) of the last attention
+    kernel launched, see psa.h: psa_last_attn_class."""
+    got, axes = [], 0
+    for c in range(8):
+        x = [ctypes.c_int32(0) for _ in range(3)]
+        axes = lib().psa_last_attn_class(c, *map(ctypes.byref, x))
+        got.append(tuple(v.value for v in x))
+    return axes, got
 
 
 def psa_last_device_status() -> Tuple[int, int]:

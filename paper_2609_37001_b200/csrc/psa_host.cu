@@ -53,7 +53,9 @@ struct {
   Mode mode = kTicket;
   int items = 0, cluster = 1;
   Grid grid = kWhole;
-  int slabs = 0, last_keys = 0;
+  int slabs = 0, last_keys = 0, edge_axes = 0;
+  uint8_t query_slabs[8] = {}, together[8] = {};
+  uint16_t keys[8] = {};   // of every `together` attended blocks
 } g_last_attn;
 
 // Id of a new API call on `stream` (g_mu held).  Never 0, which is what untouched status words hold.  A call that is
@@ -307,6 +309,7 @@ bool cut_edges(HostGeom* g) {
   // Blocks of one slab run in split-KV mode, where a slab takes 1,900 clocks and the load warp has no time for lists of boxes: 7
   // heads of 7x19x25 with 2x8x8 blocks 93 us padded and 135 cut, 18 of 3x25x73 with 1x8x16 165 and 177.
   if (g->n_sub == 1) return false;
+  std::memset(g->cls, 0, sizeof(g->cls));
   g->edge_axes = axes;
   g->n_shapes = g->n_classes = 0;
   int pattern = 0;   // its class
@@ -378,7 +381,7 @@ int make_geom(const psa_problem* prob, int T, int H, int W, bool for_attn, HostG
   if (t.bt < 1 || t.bh < 1 || t.bw < 1) return PSA_ERR_INVALID_ARG;
   const long long L = (long long)T * H * W;
   if (L >= (1ll << 31)) return PSA_ERR_INVALID_ARG;
-  std::memset(g, 0, sizeof(*g));
+  std::memset(static_cast<Geom*>(g), 0, sizeof(Geom));
   g->T = T; g->H = H; g->W = W;
   g->bt = t.bt; g->bh = t.bh; g->bw = t.bw;
   g->Tp = (T + t.bt - 1) / t.bt;
@@ -734,6 +737,14 @@ cudaError_t launch_call(const TensorMapsCut& tm, const AttnParams& prm, const Ho
     g_last_attn.grid = hg.grid;
     g_last_attn.slabs = hg.main_slabs;
     g_last_attn.last_keys = hg.main_last;
+    g_last_attn.edge_axes = hg.edge_axes;
+    for (int c = 0; c < 8; ++c) {
+      const int slabs = class_blocks(hg, c) ? hg.slabs_of[c] : 0;
+      const bool follows = hg.grid == kCut ? hg.cls[c].in_pattern != 0 : slabs == hg.main_slabs;
+      g_last_attn.query_slabs[c] = (uint8_t)slabs;
+      g_last_attn.together[c] = hg.grid == kCut && slabs ? hg.cls[c].together : 1;
+      g_last_attn.keys[c] = (uint16_t)(slabs == 0 ? 0 : (slabs - 1) * kSlabTokens + (follows ? hg.main_last : kSlabTokens));
+    }
   }
   return e;
 }
@@ -820,6 +831,15 @@ int psa_last_attn_grid(int32_t* slabs, int32_t* last_keys) {
   if (slabs) *slabs = g_last_attn.slabs;
   if (last_keys) *last_keys = g_last_attn.last_keys;
   return g_last_attn.grid;
+}
+
+int psa_last_attn_class(int c, int32_t* query_slabs, int32_t* keys, int32_t* together) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (c < 0 || c > 7) return PSA_ERR_INVALID_ARG;
+  if (query_slabs) *query_slabs = g_last_attn.query_slabs[c];
+  if (keys) *keys = g_last_attn.keys[c];
+  if (together) *together = g_last_attn.together[c];
+  return g_last_attn.edge_axes;
 }
 
 int psa_profile_events(void* start_event, void* stop_event) {

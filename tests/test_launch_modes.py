@@ -72,3 +72,21 @@ def test_chunks_of_a_host_call_are_cut_as_the_whole_call():
     B.psa_attn_fwd_host(*host, out, lse, staging, params, grid, tile, 0.1)
     assert B.psa_last_attn_grid()[0] == "cut" and B.psa_last_device_status() == (0, 0)
     assert torch.equal(out.view(torch.int16), want.cpu().view(torch.int16)) and torch.equal(lse.view(torch.int32), want_lse.cpu().view(torch.int32))
+
+
+@pytest.mark.parametrize("grid,tile,n_heads,axes,classes", [
+    ((3, 16, 20), (1, 14, 16), 60, 6, {0: (2, 224, 1), 2: (1, 128, 4), 4: (1, 128, 2), 6: (1, 128, 16)}),   # cut: 224, 32, 56 and 8 rows
+    ((4, 20, 32), (1, 16, 16), 20, 2, {0: (2, 256, 1), 2: (1, 128, 1)}),                                    # padded: the second slab is empty
+    ((4, 18, 20), (2, 8, 8), 60, 0, {0: (1, 128, 1)}),
+], ids=["cut", "empty_slab", "padded"])
+def test_classes_of_blocks(grid, tile, n_heads, axes, classes):
+    from paper_2609_37001_b200 import build
+    build.build()
+    from paper_2609_37001_b200 import binding as B
+    if axes == 2:
+        n = [-(-x // b) for x, b in zip(grid, tile)]
+        q, k, v = (torch.zeros((n_heads, math.prod(grid), 128), dtype=torch.bfloat16, device="cuda") for _ in range(3))
+        B.psa_attn_fwd(q, k, v, [(1, 0, 0, 1, 0, 0)] * n_heads, grid, tile, 0.1)
+    else:
+        _call(B, grid, tile, n_heads)
+    assert B.psa_last_attn_classes() == (axes, [classes.get(c, (0, 0, 1)) for c in range(8)])
